@@ -57,6 +57,7 @@ struct TcPlan {
     int m_pairs;          // 256-row tile rows of the two-SM kernel
     int units;            // 128-row B halves over all segments (non-SwiGLU) or ffn/128 (SwiGLU)
     int group_n;          // two-SM kernel, whole tiles: weight tiles per group of the tile order
+    int whole;            // two-SM kernel, whole tiles: no tile is cut (the stream-K fields do not apply)
     int w_keep;           // weights loaded with the evict-last policy (every row tile re-reads them from L2) instead of evict-first
 };
 
@@ -1105,8 +1106,8 @@ __global__ void __launch_bounds__(256) logit_reduce_kernel(const GemmArgs g, con
     const int row = blockIdx.x, mt = row / TC_BM;
     LogitAcc a{-INFINITY, 0.f, 0x7fffffff};
     for (int nt = threadIdx.x; nt < p.n_tiles; nt += 256) {
-        int c_first, c_last;
-        tile_cover(p, nt * p.m_tiles + mt, c_first, c_last);
+        int c_first = 0, c_last = 0;
+        if (!p.whole) tile_cover(p, nt * p.m_tiles + mt, c_first, c_last);
         const int n_entries = c_first == c_last ? 1 : 16;
         const float4* e = g.logit_stats + ((int64_t)row * p.n_tiles + nt) * 16;
         for (int i = 0; i < n_entries; ++i) {
@@ -1239,23 +1240,111 @@ TcPlan make_plan(int M, int K, int units, bool swiglu) {
     return p;
 }
 
+// How a projection is launched: kernel, work split and the tiles that the finish kernel completes.
+struct GemmLaunch {
+    TcPlan p;
+    bool pair;                // gemm_tc2_kernel
+    int clusters;
+    SplitTiles split;
+};
+
+cudaLaunchConfig_t pair_config(cudaLaunchAttribute* at, int clusters, cudaStream_t stream) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(clusters * 2);
+    cfg.blockDim = dim3(TC_THREADS);
+    cfg.dynamicSmemBytes = TC2_SMEM;
+    cfg.stream = stream;
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = 2; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 2;
+    return cfg;
+}
+
+// Clusters of the two-SM kernel that are resident at once (phase 0 ends in a grid-wide barrier); 0: none fits.
+int pair_max_clusters() {
+    static const int n = [] {
+        cudaFuncSetAttribute(gemm_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, TC_SMEM);
+        cudaFuncSetAttribute(gemm_tc2_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, TC2_SMEM);
+        cudaLaunchAttribute at[2];
+        const cudaLaunchConfig_t cfg = pair_config(at, sm_count() / 2, nullptr);
+        int c = 0;
+        if (cudaOccupancyMaxActiveClusters(&c, gemm_tc2_kernel, &cfg) != cudaSuccess || c < 0) {
+            (void)cudaGetLastError();
+            c = 0;
+        }
+        return std::min(c, sm_count() / 2);
+    }();
+    return n;
+}
+
+GemmLaunch plan_gemm(const GemmArgs& g) {
+    const bool swiglu = g.epilogue == kEpiSwiGLU;
+    const int n_total = swiglu ? g.n[0] : g.n[0] + g.n[1] + g.n[2];
+    GemmLaunch gl{};
+    gl.p = make_plan(g.M, g.K, n_total / 128, swiglu);
+    TcPlan& p = gl.p;
+    if (g.prefetch_blocks > 0) p.prefetch = g.prefetch_blocks;
+    // Two or more row tiles: two SMs per 256 x 256 tile.  With many tiles per cluster every tile is whole
+    // and the clusters walk them round-robin; with few, the (tile, K block) iterations are cut into equal
+    // contiguous ranges, one per cluster (stream-K), and the cut tiles go through the finish kernel.
+    // The LM head comes here as well: on the one-SM kernel, which reads every weight tile once per 128 rows and moves twice
+    // the shared-memory bytes per flop, 512 rows x 126 464 x 4096 took 670 us with its finish, here 379 us (decode
+    // pass of 16 requests, 4 layers: 2349 -> 2025 us).
+    static const int pair_min_tiles = [] { const char* e = getenv("ACACHE_GEMM_PAIR_MIN_MTILES"); return e ? atoi(e) : 2; }();
+    const int max_clusters = pair_max_clusters();
+    if (p.m_tiles >= pair_min_tiles && (p.units % 2 == 0 || swiglu) && max_clusters >= 1) {
+        gl.pair = true;
+        const int m_pairs = (p.m_tiles + 1) / 2;
+        const int tiles = m_pairs * p.n_tiles;
+        p.m_pairs = m_pairs;
+        static const int group_n = [] { const char* e = getenv("ACACHE_GEMM_GROUP_N"); return e && atoi(e) > 0 ? atoi(e) : kTileGroupN; }();
+        p.group_n = group_n;
+        static const int w_keep_from = [] { const char* e = getenv("ACACHE_GEMM_WKEEP_PAIRS"); return e ? atoi(e) : kKeepWeightsFromPairs; }();
+        gl.clusters = std::min(max_clusters, tiles);
+        // measured: cutting tiles pays (partial tiles + finish kernel included) up to about two thirds of a wave
+        static const int stream_k_pct = [] { const char* e = getenv("ACACHE_GEMM_PAIR_STREAMK_PCT"); return e ? atoi(e) : 66; }();
+        if (tiles * 100 <= stream_k_pct * max_clusters) {
+            const int64_t total = (int64_t)tiles * p.KB;
+            gl.clusters = (int)std::min<int64_t>(max_clusters, total);
+            p.pair_u = (int)((total + gl.clusters - 1) / gl.clusters);
+            gl.clusters = (int)((total + p.pair_u - 1) / p.pair_u);
+            // pair tiles cut by a boundary between two clusters: both of their 128-row tiles go to the finish
+            int last = -1;
+            for (int c = 1; c < gl.clusters; ++c) {
+                const int64_t cut = (int64_t)c * p.pair_u;
+                if (cut % p.KB == 0) continue;
+                const int tp = (int)(cut / p.KB);
+                if (tp == last) continue;
+                last = tp;
+                const int nt = tp / m_pairs, mp = tp - nt * m_pairs;
+                for (int r = 0; r < 2; ++r)
+                    if (mp * 2 + r < p.m_tiles && gl.split.n < 160) gl.split.tile[gl.split.n++] = nt * p.m_tiles + mp * 2 + r;
+            }
+            if (gl.split.n >= 159) { p.pair_u = 0; gl.split.n = 0; gl.clusters = std::min(max_clusters, tiles); }
+        }
+        p.whole = p.pair_u == 0;
+        p.w_keep = (m_pairs >= w_keep_from && p.whole) ? 1 : 0;      // whole tiles, walked by three or more row pairs
+        return gl;
+    }
+    // tiles whose K range is cut by a boundary between two CTAs, each listed once
+    for (int c = 1; c < p.ctas && gl.split.n < 160; ++c) {
+        const int64_t cut = (int64_t)c * p.U;
+        if (cut % p.KB == 0) continue;
+        const int t = (int)(cut / p.KB);
+        if (gl.split.n == 0 || gl.split.tile[gl.split.n - 1] != t) gl.split.tile[gl.split.n++] = t;
+    }
+    return gl;
+}
+
 }  // namespace
 
 size_t gemm_partial_bytes(int M, int K, int n_total, bool swiglu) {
     (void)M; (void)K; (void)n_total; (void)swiglu;
     // two fp32 partial tiles per CTA, at most one CTA per SM, whatever the problem size
     return (size_t)sm_count() * 2 * TC_SLOT_FLOATS * sizeof(float);
-}
-
-int launch_predict_commit(const GemmArgs& g, int batch, int n_blk, float threshold, int32_t* token, float* confidence,
-                          int32_t* commit, cudaStream_t stream) {
-    if (g.M == 0) return 0;
-    const TcPlan p = make_plan(g.M, g.K, g.n[0] / 128, false);
-    if (launch_pdl(logit_reduce_kernel, dim3(g.M), dim3(256), 0, stream, g, p, token, confidence) != cudaSuccess) return -1;
-    if (launch_pdl(commit_kernel, dim3(batch), dim3(32), 0, stream, (const float*)confidence, n_blk, threshold, commit) !=
-        cudaSuccess)
-        return -1;
-    return 2;
 }
 
 static int launch_gemm_impl(const GemmArgs& g, cudaStream_t stream);
@@ -1277,9 +1366,8 @@ int launch_gemm(const GemmArgs& g, cudaStream_t stream) {
 
 static int launch_gemm_impl(const GemmArgs& g, cudaStream_t stream) {
     const bool swiglu = g.epilogue == kEpiSwiGLU;
-    const int n_total = swiglu ? g.n[0] : g.n[0] + g.n[1] + g.n[2];
-    TcPlan p = make_plan(g.M, g.K, n_total / 128, swiglu);
-    if (g.prefetch_blocks > 0) p.prefetch = g.prefetch_blocks;
+    const GemmLaunch gl = plan_gemm(g);
+    const TcPlan& p = gl.p;
     std::lock_guard<std::mutex> lock(g_map_mutex);
     CUtensorMap map_a, map_b[3];
     {
@@ -1296,100 +1384,40 @@ static int launch_gemm_impl(const GemmArgs& g, cudaStream_t stream) {
     if (!have_b[0]) return -1;
     const CUtensorMap* mA = &map_a;
     const CUtensorMap* mB[3] = {&map_b[0], have_b[1] ? &map_b[1] : &map_b[0], have_b[2] ? &map_b[2] : &map_b[0]};
-    static bool attr = false;
-    if (!attr) {
-        cudaFuncSetAttribute(gemm_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, TC_SMEM);
-        cudaFuncSetAttribute(gemm_tc2_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, TC2_SMEM);
-        attr = true;
-    }
-    // Two or more row tiles: two SMs per 256 x 256 tile.  With many tiles per cluster every tile is whole
-    // and the clusters walk them round-robin; with few, the (tile, K block) iterations are cut into equal
-    // contiguous ranges, one per cluster (stream-K), and the cut tiles go through the finish kernel.
-    static const int pair_min_tiles = [] { const char* e = getenv("ACACHE_GEMM_PAIR_MIN_MTILES"); return e ? atoi(e) : 2; }();
-    if (p.m_tiles >= pair_min_tiles && g.epilogue != kEpiLogits && (p.units % 2 == 0 || swiglu) && sm_count() >= 2) {
-        const int m_pairs = (p.m_tiles + 1) / 2;
-        const int tiles = m_pairs * p.n_tiles;
-        cudaLaunchConfig_t cfg{};
-        cfg.gridDim = dim3(sm_count() / 2 * 2);
-        cfg.blockDim = dim3(TC_THREADS);
-        cfg.dynamicSmemBytes = TC2_SMEM;
-        cfg.stream = stream;
+    if (gl.pair) {
         cudaLaunchAttribute at[2];
-        at[0].id = cudaLaunchAttributeClusterDimension;
-        at[0].val.clusterDim.x = 2; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
-        at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        at[1].val.programmaticStreamSerializationAllowed = 1;
-        cfg.attrs = at;
-        cfg.numAttrs = 2;
-        // all clusters must be resident at once (phase 0 ends in a grid-wide barrier)
-        static int max_clusters = 0;
-        if (!max_clusters) {
-            int n = 0;
-            if (cudaOccupancyMaxActiveClusters(&n, gemm_tc2_kernel, &cfg) != cudaSuccess || n <= 0) {
-                (void)cudaGetLastError();
-                n = -1;
-            }
-            max_clusters = n;
-        }
-        if (max_clusters < 1) goto single_cta;
-        TcPlan pp = p;
-        pp.m_pairs = m_pairs;
-        static const int group_n = [] { const char* e = getenv("ACACHE_GEMM_GROUP_N"); return e && atoi(e) > 0 ? atoi(e) : kTileGroupN; }();
-        pp.group_n = group_n;
-        static const int w_keep_from = [] { const char* e = getenv("ACACHE_GEMM_WKEEP_PAIRS"); return e ? atoi(e) : kKeepWeightsFromPairs; }();
-        int clusters = std::min(std::min(max_clusters, sm_count() / 2), tiles);
-        // measured: cutting tiles pays (partial tiles + finish kernel included) up to about two thirds of a wave
-        static const int stream_k_pct = [] { const char* e = getenv("ACACHE_GEMM_PAIR_STREAMK_PCT"); return e ? atoi(e) : 66; }();
-        SplitTiles split{};
-        if (tiles * 100 <= stream_k_pct * std::min(max_clusters, sm_count() / 2)) {
-            const int64_t total = (int64_t)tiles * p.KB;
-            clusters = (int)std::min<int64_t>(std::min(max_clusters, sm_count() / 2), total);
-            pp.pair_u = (int)((total + clusters - 1) / clusters);
-            clusters = (int)((total + pp.pair_u - 1) / pp.pair_u);
-            // pair tiles cut by a boundary between two clusters: both of their 128-row tiles go to the finish
-            int last = -1;
-            for (int c = 1; c < clusters; ++c) {
-                const int64_t cut = (int64_t)c * pp.pair_u;
-                if (cut % p.KB == 0) continue;
-                const int tp = (int)(cut / p.KB);
-                if (tp == last) continue;
-                last = tp;
-                const int nt = tp / m_pairs, mp = tp - nt * m_pairs;
-                for (int r = 0; r < 2; ++r)
-                    if (mp * 2 + r < p.m_tiles && split.n < 160) split.tile[split.n++] = nt * p.m_tiles + mp * 2 + r;
-            }
-            if (split.n >= 159) { pp.pair_u = 0; split.n = 0; clusters = std::min(std::min(max_clusters, sm_count() / 2), tiles); }
-        }
-        pp.w_keep = (m_pairs >= w_keep_from && pp.pair_u == 0) ? 1 : 0;      // whole tiles, walked by three or more row pairs
-        cfg.gridDim = dim3(clusters * 2);
-        if (cudaLaunchKernelEx(&cfg, gemm_tc2_kernel, g, pp, clusters, *mA, *mB[0], *mB[1], *mB[2]) != cudaSuccess) return -1;
-        if (split.n == 0) return 1;
+        const cudaLaunchConfig_t cfg = pair_config(at, gl.clusters, stream);
+        if (cudaLaunchKernelEx(&cfg, gemm_tc2_kernel, g, p, gl.clusters, *mA, *mB[0], *mB[1], *mB[2]) != cudaSuccess) return -1;
+        if (gl.split.n == 0) return 1;
         const int per_tile = finish_items_per_tile(g.epilogue) * TC_BM;
-        if (launch_pdl(gemm_finish_kernel<2>, dim3((per_tile + 255) / 256, split.n), dim3(256), 0, stream, g, pp, split) != cudaSuccess)
+        if (launch_pdl(gemm_finish_kernel<2>, dim3((per_tile + 255) / 256, gl.split.n), dim3(256), 0, stream, g, p, gl.split) !=
+            cudaSuccess)
             return -1;
         return 2;
     }
-single_cta:
     // a plain launch: a cooperative one measured ~2.5 us slower and cannot overlap the previous
     // kernel's tail; the grid never exceeds the SM count at one CTA per SM and the barrier is bounded
     if (launch_pdl(gemm_tc_kernel, dim3(p.ctas), dim3(TC_THREADS), TC_SMEM, stream, g, p, *mA, *mB[0], *mB[1], *mB[2]) !=
         cudaSuccess)
         return -1;
-    // tiles whose K range is cut by a boundary between two CTAs, each listed once
-    SplitTiles split{};
-    for (int c = 1; c < p.ctas && split.n < 160; ++c) {
-        const int64_t cut = (int64_t)c * p.U;
-        if (cut % p.KB == 0) continue;
-        const int t = (int)(cut / p.KB);
-        if (split.n == 0 || split.tile[split.n - 1] != t) split.tile[split.n++] = t;
-    }
-    if (split.n == 0) return 1;
+    if (gl.split.n == 0) return 1;
     const int rows_per = p.m_tiles == 1 ? ((g.M + 31) & ~31) : TC_BM;
     const int per_tile = finish_items_per_tile(g.epilogue) * rows_per;
-    const dim3 fgrid((per_tile + 255) / 256, split.n);
+    const dim3 fgrid((per_tile + 255) / 256, gl.split.n);
     const bool wide = g.epilogue == kEpiQKV && (int)(fgrid.x * fgrid.y) <= sm_count();
-    if ((wide ? launch_pdl(gemm_finish_kernel<4>, fgrid, dim3(256), 0, stream, g, p, split)
-              : launch_pdl(gemm_finish_kernel<2>, fgrid, dim3(256), 0, stream, g, p, split)) != cudaSuccess)
+    if ((wide ? launch_pdl(gemm_finish_kernel<4>, fgrid, dim3(256), 0, stream, g, p, gl.split)
+              : launch_pdl(gemm_finish_kernel<2>, fgrid, dim3(256), 0, stream, g, p, gl.split)) != cudaSuccess)
+        return -1;
+    return 2;
+}
+
+int launch_predict_commit(const GemmArgs& g, int batch, int n_blk, float threshold, int32_t* token, float* confidence,
+                          int32_t* commit, cudaStream_t stream) {
+    if (g.M == 0) return 0;
+    const TcPlan p = plan_gemm(g).p;
+    if (launch_pdl(logit_reduce_kernel, dim3(g.M), dim3(256), 0, stream, g, p, token, confidence) != cudaSuccess) return -1;
+    if (launch_pdl(commit_kernel, dim3(batch), dim3(32), 0, stream, (const float*)confidence, n_blk, threshold, commit) !=
+        cudaSuccess)
         return -1;
     return 2;
 }
