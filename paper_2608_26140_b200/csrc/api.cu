@@ -22,7 +22,7 @@ struct acache_ctx {
     unsigned char* ws = nullptr;
     size_t ws_have = 0;
     // workspace offsets (bytes)
-    size_t o_status, o_row_pos, o_row_pos2, o_row_src, o_xn, o_q, o_o, o_h1, o_xn2, o_act, o_knew, o_vnew;
+    size_t o_status, o_row_pos, o_row_src, o_xn, o_q, o_o, o_h1, o_xn2, o_act, o_knew, o_vnew;
     size_t o_mrow_pos, o_mrow_src, o_xn_mask, o_qmask, o_stats, o_partial, o_slot;
     size_t o_rowmask, partial_bytes;
     size_t o_xstage, o_ystage, o_sstage, o_astage, o_gemm, o_attn, o_gridbar, o_mcidx, o_lstats, o_lxn, o_keymask;
@@ -245,28 +245,19 @@ acache_status run_recompute(acache_ctx* c, const acache_layer_weights* w, const 
         // the rows that serve their positions from k_new / v_new: the rows recomputed now, or the whole private
         // slot array of which they refreshed a part
         const int fresh = priv ? priv->k + priv->e : rows;
-        const int32_t* fresh_pos = row_pos;
-        if (priv) {
-            int32_t* rp2 = wsp<int32_t>(c, c->o_row_pos2);
-            if (!maps.reuse) {
-                launch_row_positions(priv->anchor_idx, priv->k, priv->extra_rows, priv->e, r->affix_start, r->affix_len,
-                                     r->ctx_len, r->batch, rp2, status, st);
-                c->launches += 1;
-            }
-            fresh_pos = rp2;
-            at.n_fresh = fresh;
-        }
+        if (priv) at.n_fresh = fresh;
         int32_t* slot = wsp<int32_t>(c, c->o_slot);
         at.k_new = k_new; at.v_new = v_new; at.slot = slot;
         // key masks of the same map, for the kernel that reads cache and fresh rows as two sources
         at.excl_words = (r->ctx_len + 31) / 32; at.keep_words = (fresh + 31) / 32;
         uint32_t* km = wsp<uint32_t>(c, c->o_keymask);
-        at.pos_excl = km; at.row_keep = km + (size_t)r->batch * at.excl_words;
+        uint32_t* keep = km + (size_t)r->batch * at.excl_words;
+        at.pos_excl = km; at.row_keep = keep;
         if (!maps.reuse) {
-            launch_build_slot_map(slot, r->ctx_len, fresh_pos, fresh, r->batch, st);
-            launch_key_masks(slot, r->ctx_len, fresh_pos, fresh, r->batch, km, at.excl_words,
-                             km + (size_t)r->batch * at.excl_words, at.keep_words, st);
-            c->launches += 2;
+            launch_fresh_map(priv ? priv->anchor_idx : anchor_idx, priv ? priv->k : k, priv ? priv->extra_rows : r->extra_rows,
+                             priv ? priv->e : r->n_extra, r->affix_start, r->affix_len, r->ctx_len, r->batch, slot, km,
+                             at.excl_words, keep, at.keep_words, status, st);
+            c->launches += 1;
         }
     }
     if (drop_non_anchor) {
@@ -365,7 +356,6 @@ acache_status acache_create(const acache_model_desc* desc, acache_ctx** out) {
     c->o_status = take(cur, 256);
     c->o_gridbar = take(cur, 256);
     c->o_row_pos = take(cur, nr * 4);
-    c->o_row_pos2 = take(cur, nr * 4);
     c->o_row_src = take(cur, nr * 8);
     c->o_xn = take(cur, nr * d.hidden * 2);
     c->o_q = take(cur, nr * qd * 2);
@@ -608,7 +598,7 @@ acache_status layer_step_impl(acache_ctx* ctx, const acache_layer_weights* w, co
         (size_t)req->batch * d.n_heads * ((req->n_extra + 127) / 128) * req->affix_len * 4 <= ctx->partial_bytes) {
         fs.rm_words = (req->n_extra + 31) / 32;
         uint32_t* rm = wsp<uint32_t>(ctx, ctx->o_rowmask);
-        launch_row_mask(req->masked_pos, req->n_masked, req->extra_rows, req->n_extra, 0, req->batch, rm, fs.rm_words,
+        launch_row_mask(req->masked_pos, req->n_masked, req->extra_rows, req->n_extra, 0, req->ctx_len, req->batch, rm, fs.rm_words,
                         wsp<uint32_t>(ctx, ctx->o_status), stream);
         ctx->launches += 1;
         fs.rowmask = rm; fs.scores = scores; fs.accumulate = (flags & ACACHE_F_ACCUMULATE) ? 1 : 0;
@@ -632,7 +622,7 @@ acache_status layer_step_impl(acache_ctx* ctx, const acache_layer_weights* w, co
                 if (x_is_compact) {
                     // the masked rows are among the extra rows of the compact input: find where
                     int32_t* cidx = wsp<int32_t>(ctx, ctx->o_mcidx);
-                    launch_match_rows(req->masked_pos, req->n_masked, req->extra_rows, req->n_extra, k, req->batch, cidx,
+                    launch_match_rows(req->masked_pos, req->n_masked, req->extra_rows, req->n_extra, k, req->ctx_len, req->batch, cidx,
                                       wsp<uint32_t>(ctx, ctx->o_status), stream);
                     ctx->launches += 1;
                     g.prep.compact_idx = cidx;

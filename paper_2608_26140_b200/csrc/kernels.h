@@ -13,7 +13,7 @@ void launch_scatter_kv(void* cache_k, void* cache_v, int64_t batch_stride, int c
                        uint32_t* status, cudaStream_t stream);
 
 // idx[b, i] = compact row (k + j) whose position extra_rows[b, j] equals masked_pos[b, i], or -1.
-void launch_match_rows(const int32_t* masked_pos, int m, const int32_t* extra_rows, int e, int k, int batch,
+void launch_match_rows(const int32_t* masked_pos, int m, const int32_t* extra_rows, int e, int k, int ctx_len, int batch,
                        int32_t* idx, uint32_t* status, cudaStream_t stream);
 
 // Eq. 3 on the sequence state: the block's still-masked positions whose confidence exceeds the threshold
@@ -22,17 +22,12 @@ void launch_commit_update(int32_t* token_ids, int ctx_len, const int32_t* block_
                           const int32_t* token, const float* confidence, int mask_id, float threshold,
                           int32_t* remaining, uint32_t* status, cudaStream_t stream);
 
-// slot[b, t] = compact row index whose fresh K/V replaces position t, or -1.
-// Positions of the rows of a private slot array (k anchors, then e extra rows per request).
-void launch_row_positions(const int32_t* anchor_idx, int k, const int32_t* extra_rows, int e, int affix_start, int affix_len,
-                          int ctx_len, int batch, int32_t* row_pos, uint32_t* status, cudaStream_t stream);
-void launch_build_slot_map(int32_t* slot, int ctx_len, const int32_t* row_pos, int rows_per_req, int batch,
-                           cudaStream_t stream);
-
-// pos_excl[b, t / 32] bit t % 32 = position t is served by a fresh row; row_keep[b, i / 32] bit i % 32 = fresh
-// row i serves its position (built from the position -> row map, so duplicates resolve the same way).
-void launch_key_masks(const int32_t* slot, int ctx_len, const int32_t* row_pos, int rows_per_req, int batch,
-                      uint32_t* pos_excl, int excl_words, uint32_t* row_keep, int keep_words, cudaStream_t stream);
+// The fresh rows (k anchors, then e extra rows per request) and the positions they serve: slot[b, t] = compact row whose
+// fresh K/V replaces position t, or -1 (the last of several rows naming a position); pos_excl[b, t / 32] bit t % 32 =
+// position t is served by a fresh row; row_keep[b, i / 32] bit i % 32 = fresh row i serves its position.
+void launch_fresh_map(const int32_t* anchor_idx, int k, const int32_t* extra_rows, int e, int affix_start, int affix_len,
+                      int ctx_len, int batch, int32_t* slot, uint32_t* pos_excl, int excl_words, uint32_t* row_keep,
+                      int keep_words, uint32_t* status, cudaStream_t stream);
 
 // scores[b, j] (+)= ||K_full[b, l + j] - K_ref[b, l + j]||^2 + ||V_full[b, l + j] - V_ref[b, l + j]||^2 (batch strides in
 // elements, 0 = one cache shared by the batch).
@@ -47,8 +42,8 @@ void launch_drop_mask(const int32_t* anchor_idx, int k, int affix_start, int aff
 
 // rowmask[b, i / 32] bit i % 32 = compact row i (k anchors, then the e extra rows) of request b is one of its masked
 // positions; a masked position that is not among the extra rows raises kFlagBadIndex.
-void launch_row_mask(const int32_t* masked_pos, int m, const int32_t* extra_rows, int e, int k, int batch, uint32_t* rowmask,
-                     int words, uint32_t* status, cudaStream_t stream);
+void launch_row_mask(const int32_t* masked_pos, int m, const int32_t* extra_rows, int e, int k, int ctx_len, int batch,
+                     uint32_t* rowmask, int words, uint32_t* status, cudaStream_t stream);
 
 // scores[b, j] (+)= sum over heads and over the query tiles that hold a flagged row of partial[b, h, qt, j], in a fixed order.
 void launch_score_reduce_tiles(const float* partial, const uint32_t* rowmask, int rm_words, float* scores, int batch, int n_heads,
@@ -186,7 +181,7 @@ struct AttnArgs {
     const void* v_new;
     int n_fresh;              // rows per request in k_new / v_new; 0 = n (the rows being recomputed are the fresh rows)
     const int32_t* slot;      // [B, ctx_len] or null: >= 0 => read k_new/v_new row slot
-    const uint32_t* pos_excl; // optional key masks of the same map (launch_key_masks): with them the tensor-core
+    const uint32_t* pos_excl; // optional key masks of the same map (launch_fresh_map): with them the tensor-core
     const uint32_t* row_keep; //   kernel reads the cache and k_new / v_new as two key sources instead of gathering
     int excl_words, keep_words;
     const uint32_t* key_drop; // optional [B, excl_words]: bit t = position t does not exist as a key (DropNA, Section 5.3)

@@ -34,76 +34,107 @@ __global__ void __launch_bounds__(128) scatter_kv_kernel(
     }
 }
 
-__global__ void __launch_bounds__(1024) slot_map_kernel(int32_t* __restrict__ slot, int ctx_len,
-                                                        const int32_t* __restrict__ row_pos, int rows_per_req) {
-    pdl_wait();
-    pdl_launch_dependents();
-    const int b = blockIdx.x;
-    int32_t* s = slot + (int64_t)b * ctx_len;
-    for (int t = threadIdx.x; t < ctx_len; t += blockDim.x) s[t] = -1;
-    __syncthreads();
-    // later rows win on duplicates, the same order a sequential scatter would give
-    if (threadIdx.x == 0) {
-        for (int i = 0; i < rows_per_req; ++i) {
-            int p = row_pos[(int64_t)b * rows_per_req + i];
-            if (p >= 0) s[p] = i;
-        }
-    }
-}
-
-// Bit masks over keys for the attention that reads the cache and the fresh rows as two sources
-// (Section 4.1: shared storage + private slots): pos_excl[b] bit t = position t is served by a fresh
-// row (skip it in the cache); row_keep[b] bit i = fresh row i is the one that serves its position
-// (the last one wins if two rows name the same position, as in the position -> row map).
-__global__ void __launch_bounds__(1024) key_mask_kernel(const int32_t* __restrict__ slot, int ctx_len,
-                                                        const int32_t* __restrict__ row_pos, int rows_per_req,
-                                                        uint32_t* __restrict__ pos_excl, int excl_words,
-                                                        uint32_t* __restrict__ row_keep, int keep_words) {
+// Which fresh row serves which position, for the attention that reads the cache and the fresh rows as two sources
+// (Section 4.1: shared storage + private slots), one CTA per request, one launch:
+//   slot[b, t]     = the compact row whose K/V replace position t, -1 if the cache serves it (the last row wins if two
+//                    name the same position, the order a sequential scatter would give);
+//   pos_excl[b]    bit t = position t is served by a fresh row (skip it in the cache);
+//   row_keep[b]    bit i = fresh row i is the one that serves its position.
+// Bound by a few dependent trips to L2.  The map is built in shared memory by atomicMax on the row index (one thread
+// writing the rows in order, between two other launches: 41 us for 922 rows x 16 requests; this 4.5).  Contexts past the shared memory build it in place
+// in global memory.
+constexpr int kMapSmemBytes = 200 * 1024;
+__global__ void __launch_bounds__(1024) fresh_map_kernel(const int32_t* __restrict__ anchor_idx, int k,
+                                                         const int32_t* __restrict__ extra_rows, int e, int affix_start,
+                                                         int affix_len, int ctx_len, int32_t* __restrict__ slot,
+                                                         uint32_t* __restrict__ pos_excl, int excl_words,
+                                                         uint32_t* __restrict__ row_keep, int keep_words, uint32_t* status,
+                                                         int use_smem) {
+    extern __shared__ int32_t map_s[];
     pdl_wait();
     pdl_launch_dependents();
     const int b = blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-    const int32_t* s = slot + (int64_t)b * ctx_len;
+    int32_t* out = slot + (int64_t)b * ctx_len;
+    int32_t* s = use_smem ? map_s : out;
+    for (int t = threadIdx.x; t < ctx_len; t += blockDim.x) s[t] = -1;
+    __syncthreads();
+    for (int i = threadIdx.x; i < k + e; i += blockDim.x) {
+        const int p = row_position(anchor_idx, k, extra_rows, e, b, i, affix_start, affix_len, ctx_len);
+        if (p >= 0) atomicMax(&s[p], i);
+        else atomicOr(status, kFlagBadIndex);
+    }
+    __syncthreads();
+    auto serves = [&](int t) { return use_smem ? map_s[t] : __ldcg(out + t); };
     for (int w = warp; w < excl_words; w += nw) {
         const int t = w * 32 + lane;
-        const uint32_t bits = __ballot_sync(0xffffffffu, t < ctx_len && s[t] >= 0);
+        const int r = t < ctx_len ? serves(t) : -1;
+        if (use_smem && t < ctx_len) out[t] = r;
+        const uint32_t bits = __ballot_sync(0xffffffffu, r >= 0);
         if (lane == 0) pos_excl[(int64_t)b * excl_words + w] = bits;
     }
     for (int w = warp; w < keep_words; w += nw) {
         const int i = w * 32 + lane;
         bool ok = false;
-        if (i < rows_per_req) {
-            const int p = row_pos[(int64_t)b * rows_per_req + i];
-            ok = p >= 0 && p < ctx_len && s[p] == i;
+        if (i < k + e) {
+            const int p = row_position(anchor_idx, k, extra_rows, e, b, i, affix_start, affix_len, ctx_len);
+            ok = p >= 0 && serves(p) == i;
         }
         const uint32_t bits = __ballot_sync(0xffffffffu, ok);
         if (lane == 0) row_keep[(int64_t)b * keep_words + w] = bits;
     }
 }
 
-void launch_key_masks(const int32_t* slot, int ctx_len, const int32_t* row_pos, int rows_per_req, int batch,
-                      uint32_t* pos_excl, int excl_words, uint32_t* row_keep, int keep_words, cudaStream_t stream) {
+void launch_fresh_map(const int32_t* anchor_idx, int k, const int32_t* extra_rows, int e, int affix_start, int affix_len,
+                      int ctx_len, int batch, int32_t* slot, uint32_t* pos_excl, int excl_words, uint32_t* row_keep,
+                      int keep_words, uint32_t* status, cudaStream_t stream) {
     if (batch == 0) return;
-    launch_pdl(key_mask_kernel, batch, 1024, 0, stream, slot, ctx_len, row_pos, rows_per_req, pos_excl, excl_words, row_keep,
-               keep_words);
+    const size_t need = (size_t)ctx_len * sizeof(int32_t);
+    const int use_smem = need <= kMapSmemBytes;
+    const size_t smem = use_smem ? need : 0;
+    if (smem > 48 * 1024) cudaFuncSetAttribute(fresh_map_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMapSmemBytes);
+    launch_pdl(fresh_map_kernel, batch, 1024, smem, stream, anchor_idx, k, extra_rows, e, affix_start, affix_len, ctx_len, slot,
+               pos_excl, excl_words, row_keep, keep_words, status, use_smem);
+}
+
+// The first of a request's extra rows at position `want`, -1 if there is none.  With the context in shared memory the
+// extra rows are entered by position once (first_extra_rows) and looked up (a linear search per masked position:
+// 40 us for 256 of 512 rows x 32 requests; this 4-5).  Contexts past the shared memory are searched.
+__device__ __forceinline__ void first_extra_rows(int32_t* map, int ctx_len, const int32_t* extra_rows, int e) {
+    for (int t = threadIdx.x; t < ctx_len; t += blockDim.x) map[t] = 0x7fffffff;
+    __syncthreads();
+    for (int j = threadIdx.x; j < e; j += blockDim.x) {
+        const int p = extra_rows[j];
+        if ((unsigned)p < (unsigned)ctx_len) atomicMin(&map[p], j);
+    }
+    __syncthreads();
+}
+__device__ __forceinline__ int find_extra_row(const int32_t* map, int ctx_len, const int32_t* extra_rows, int e, int want) {
+    if (map) {
+        const int j = (unsigned)want < (unsigned)ctx_len ? map[want] : 0x7fffffff;
+        return j == 0x7fffffff ? -1 : j;
+    }
+    for (int j = 0; j < e; ++j)
+        if (extra_rows[j] == want) return j;
+    return -1;
 }
 
 // idx[b, i] = k + j where extra_rows[b, j] == masked_pos[b, i]: the compact row that holds a
 // masked position when the layer input is given in compact row order; -1 (and kFlagBadIndex)
 // if the position is not among the extra rows.
-__global__ void __launch_bounds__(256) match_rows_kernel(const int32_t* __restrict__ masked_pos, int m,
-                                                         const int32_t* __restrict__ extra_rows, int e, int k,
-                                                         int32_t* __restrict__ idx, uint32_t* status) {
+__global__ void __launch_bounds__(512) match_rows_kernel(const int32_t* __restrict__ masked_pos, int m,
+                                                         const int32_t* __restrict__ extra_rows, int e, int k, int ctx_len,
+                                                         int32_t* __restrict__ idx, uint32_t* status, int use_smem) {
+    extern __shared__ int32_t map_s[];
     pdl_wait();
     pdl_launch_dependents();
-    const int b = blockIdx.y;
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= m) return;
-    const int want = masked_pos[(int64_t)b * m + i];
-    int found = -1;
-    for (int j = 0; j < e; ++j)
-        if (extra_rows[(int64_t)b * e + j] == want) { found = k + j; break; }
-    idx[(int64_t)b * m + i] = found;
-    if (found < 0) atomicOr(status, kFlagBadIndex);
+    const int b = blockIdx.x;
+    const int32_t* rows = extra_rows + (int64_t)b * e;
+    if (use_smem) first_extra_rows(map_s, ctx_len, rows, e);
+    for (int i = threadIdx.x; i < m; i += blockDim.x) {
+        const int j = find_extra_row(use_smem ? map_s : nullptr, ctx_len, rows, e, masked_pos[(int64_t)b * m + i]);
+        idx[(int64_t)b * m + i] = j < 0 ? -1 : k + j;
+        if (j < 0) atomicOr(status, kFlagBadIndex);
+    }
 }
 
 // Eq. 3 on the sequence state: among the block's positions that still hold the mask id, those whose
@@ -165,11 +196,15 @@ void launch_commit_update(int32_t* token_ids, int ctx_len, const int32_t* block_
                mask_id, threshold, remaining, status);
 }
 
-void launch_match_rows(const int32_t* masked_pos, int m, const int32_t* extra_rows, int e, int k, int batch,
+void launch_match_rows(const int32_t* masked_pos, int m, const int32_t* extra_rows, int e, int k, int ctx_len, int batch,
                        int32_t* idx, uint32_t* status, cudaStream_t stream) {
     if (batch == 0 || m == 0) return;
-    launch_pdl(match_rows_kernel, dim3((m + 255) / 256, batch), dim3(256), 0, stream, masked_pos, m, extra_rows, e, k, idx,
-               status);
+    const size_t need = (size_t)ctx_len * sizeof(int32_t);
+    const int use_smem = need <= kMapSmemBytes;
+    const size_t smem = use_smem ? need : 0;
+    if (smem > 48 * 1024) cudaFuncSetAttribute(match_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMapSmemBytes);
+    launch_pdl(match_rows_kernel, dim3(batch), dim3(512), smem, stream, masked_pos, m, extra_rows, e, k, ctx_len, idx, status,
+               use_smem);
 }
 
 void launch_scatter_kv(void* cache_k, void* cache_v, int64_t batch_stride, int ctx_len, const int32_t* anchor_idx,
@@ -182,34 +217,6 @@ void launch_scatter_kv(void* cache_k, void* cache_v, int64_t batch_stride, int c
                                              anchor_idx, k, extra_rows, e, affix_start, affix_len, kv_dim,
                                              static_cast<const __nv_bfloat16*>(k_new),
                                              static_cast<const __nv_bfloat16*>(v_new), status);
-}
-
-// row_pos[b, i] = position of private row i of request b (anchors first, then the extra rows); -1 and
-// kFlagBadIndex for an index out of range.
-__global__ void __launch_bounds__(256) row_pos_kernel(const int32_t* __restrict__ anchor_idx, int k,
-                                                      const int32_t* __restrict__ extra_rows, int e, int affix_start,
-                                                      int affix_len, int ctx_len, int32_t* __restrict__ row_pos,
-                                                      uint32_t* status) {
-    pdl_wait();
-    pdl_launch_dependents();
-    const int b = blockIdx.y, i = blockIdx.x * 256 + threadIdx.x;
-    if (i >= k + e) return;
-    const int pos = row_position(anchor_idx, k, extra_rows, e, b, i, affix_start, affix_len, ctx_len);
-    if (pos < 0) atomicOr(status, kFlagBadIndex);
-    row_pos[(int64_t)b * (k + e) + i] = pos;
-}
-
-void launch_row_positions(const int32_t* anchor_idx, int k, const int32_t* extra_rows, int e, int affix_start, int affix_len,
-                          int ctx_len, int batch, int32_t* row_pos, uint32_t* status, cudaStream_t stream) {
-    if (batch == 0 || k + e == 0) return;
-    launch_pdl(row_pos_kernel, dim3((k + e + 255) / 256, batch), dim3(256), 0, stream, anchor_idx, k, extra_rows, e, affix_start,
-               affix_len, ctx_len, row_pos, status);
-}
-
-void launch_build_slot_map(int32_t* slot, int ctx_len, const int32_t* row_pos, int rows_per_req, int batch,
-                           cudaStream_t stream) {
-    if (batch == 0) return;
-    launch_pdl(slot_map_kernel, batch, 1024, 0, stream, slot, ctx_len, row_pos, rows_per_req);
 }
 
 // ---- KV-deviation selector (the CacheBlend-style variant of the paper's appendix) ------------------
@@ -311,35 +318,38 @@ void launch_drop_mask(const int32_t* anchor_idx, int k, int affix_start, int aff
 }
 
 // ---- Eq. 4-5 from the probe's own attention logits: which compact rows are masked positions, and the final sum --------
-__global__ void __launch_bounds__(256) row_mask_kernel(const int32_t* __restrict__ masked_pos, int m,
-                                                       const int32_t* __restrict__ extra_rows, int e, int k,
-                                                       uint32_t* __restrict__ rowmask, int words, uint32_t* status) {
-    extern __shared__ uint32_t bits[];          // [words] the mask, then [e] the request's extra rows
-    int32_t* rows_s = reinterpret_cast<int32_t*>(bits + words);
+__global__ void __launch_bounds__(512) row_mask_kernel(const int32_t* __restrict__ masked_pos, int m,
+                                                       const int32_t* __restrict__ extra_rows, int e, int k, int ctx_len,
+                                                       uint32_t* __restrict__ rowmask, int words, uint32_t* status,
+                                                       int use_smem) {
+    extern __shared__ int32_t map_s[];          // [words] the mask, then [ctx_len] the first extra row at a position
+    uint32_t* bits = reinterpret_cast<uint32_t*>(map_s);
+    int32_t* map = map_s + words;
     pdl_wait();
     pdl_launch_dependents();
     const int b = blockIdx.x;
+    const int32_t* rows = extra_rows + (int64_t)b * e;
     for (int w = threadIdx.x; w < words; w += blockDim.x) bits[w] = 0u;
-    for (int j = threadIdx.x; j < e; j += blockDim.x) rows_s[j] = extra_rows[(int64_t)b * e + j];
-    __syncthreads();
+    if (use_smem) first_extra_rows(map, ctx_len, rows, e);
+    else __syncthreads();
     for (int i = threadIdx.x; i < m; i += blockDim.x) {
-        const int want = masked_pos[(int64_t)b * m + i];
-        int found = -1;
-        for (int j = 0; j < e; ++j)
-            if (rows_s[j] == want) { found = k + j; break; }
-        if (found < 0 || (found >> 5) >= words) atomicOr(status, kFlagBadIndex);
-        else atomicOr(&bits[found >> 5], 1u << (found & 31));
+        const int j = find_extra_row(use_smem ? map : nullptr, ctx_len, rows, e, masked_pos[(int64_t)b * m + i]);
+        if (j < 0 || ((k + j) >> 5) >= words) atomicOr(status, kFlagBadIndex);
+        else atomicOr(&bits[(k + j) >> 5], 1u << ((k + j) & 31));
     }
     __syncthreads();
     for (int w = threadIdx.x; w < words; w += blockDim.x) rowmask[(int64_t)b * words + w] = bits[w];
 }
 
-void launch_row_mask(const int32_t* masked_pos, int m, const int32_t* extra_rows, int e, int k, int batch, uint32_t* rowmask,
-                     int words, uint32_t* status, cudaStream_t stream) {
+void launch_row_mask(const int32_t* masked_pos, int m, const int32_t* extra_rows, int e, int k, int ctx_len, int batch,
+                     uint32_t* rowmask, int words, uint32_t* status, cudaStream_t stream) {
     if (batch == 0) return;
-    const size_t smem = (size_t)(words + e) * sizeof(uint32_t);
-    if (smem > 48 * 1024) cudaFuncSetAttribute(row_mask_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    launch_pdl(row_mask_kernel, dim3(batch), dim3(256), smem, stream, masked_pos, m, extra_rows, e, k, rowmask, words, status);
+    const size_t need = (size_t)(words + ctx_len) * sizeof(uint32_t);
+    const int use_smem = need <= kMapSmemBytes;
+    const size_t smem = use_smem ? need : (size_t)words * sizeof(uint32_t);
+    if (smem > 48 * 1024) cudaFuncSetAttribute(row_mask_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMapSmemBytes);
+    launch_pdl(row_mask_kernel, dim3(batch), dim3(512), smem, stream, masked_pos, m, extra_rows, e, k, ctx_len, rowmask, words,
+               status, use_smem);
 }
 
 // Two small results of a step (scores, anchor indices: 4-byte words) copied to page-locked host memory by plain

@@ -1,8 +1,13 @@
 """Sizes at the edges of the kernels' dispatch rules and tiles, against the oracle."""
+import numpy as np
 import pytest
+import torch
 
+from paper_2608_26140_b200 import binding as ab
 from paper_2608_26140_b200 import workloads as wl
 
+from helpers import DEV, DeviceCase, assert_close_bf16, oracle_step
+from test_gpu_parity import MID128, run_layer_step, run_split_calls
 from test_gpu_predict_commit import test_predict_commit as check_predict_commit
 
 pytestmark = pytest.mark.gpu
@@ -17,3 +22,41 @@ pytestmark = pytest.mark.gpu
 ])
 def test_lm_head_tiles(V, B, n_blk):
     check_predict_commit(wl.TINY, V, B, 64, n_blk)
+
+
+@pytest.mark.parametrize("T", [51200, 51201])     # the last context whose position map fits shared memory, the first past it
+def test_position_maps_of_long_contexts(T):
+    # slot map of the split call (with two rows naming one position), lookup of the masked rows in a compact input
+    lay = wl.make_layout(1, 5, T - 5 - 40, 8, 32, 32, "masked")
+    lay.extra_rows = lay.extra_rows.copy()
+    lay.extra_rows[0, 3] = lay.extra_rows[0, 20]
+    case = wl.make_case(wl.TINY, lay, 0.0, cfg_id=71)
+    dc = DeviceCase(case, max_rows=64)
+    K = 7
+    anchors = np.sort(np.random.default_rng(T).choice(lay.affix_len, K, replace=False)).astype(np.int32)[None]
+    k_new, v_new, y = run_split_calls(dc, torch.from_numpy(anchors).to(DEV), K)
+    assert dc.ctx.poll_status() == 0
+    ref = oracle_step(case, 0, anchor_idx=anchors[0])
+    assert_close_bf16(ab.to_host_bits(y[0]), ref["y"], "y")
+
+    lay.extra_rows[0] = lay.masked_pos[0]
+    dc = DeviceCase(case, max_rows=64)
+    compact = dc.x[:, torch.from_numpy(lay.extra_rows[0]).long().to(DEV)].contiguous()
+    scores = torch.zeros((2, lay.affix_len), dtype=torch.float32, device=DEV)
+    y = torch.zeros((1, lay.n_extra, case.shape.hidden), dtype=torch.bfloat16, device=DEV)
+    for i, (x, is_compact) in enumerate(((dc.x, 0), (compact, 1))):
+        dc.ctx.layer_step(dc.lw, dc.req, dc.kv(), x, is_compact, 0.0, ab.F_SCORE | ab.F_NO_RECOMPUTE, scores[i:i + 1], None, y)
+    assert dc.ctx.poll_status() == 0
+    assert scores[0].sum().item() > 0 and torch.equal(scores[0], scores[1])
+
+
+@pytest.mark.parametrize("T", [51198, 51199])     # with the two mask words of 40 rows: the map just fits, just does not
+def test_probe_row_mask_of_long_contexts(T):
+    lay = wl.make_layout(1, 0, T - 40, 8, 32, 32, "all")
+    case = wl.make_case(MID128, lay, 0.0, cfg_id=72)
+    dc = DeviceCase(case)
+    K, s_gpu, _, _ = run_layer_step(dc, 0.0, ab.F_SCORE)
+    assert dc.ctx.poll_status() == 0
+    ref = oracle_step(case, 0, ratio=0.0)["scores"]
+    # Eq. 4-5 from bf16 products summed in fp32: the bound the other scoring tests use
+    assert np.all(np.abs(s_gpu[0] - ref) <= 1e-3 * np.maximum(ref, ref.mean()))
