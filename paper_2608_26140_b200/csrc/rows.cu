@@ -371,52 +371,63 @@ void launch_copy_out_words(const void* a, void* a_out, int n_a, const void* b, v
                static_cast<uint32_t*>(a_out), n_a, static_cast<const uint32_t*>(b), static_cast<uint32_t*>(b_out), n_b);
 }
 
+// A CTA takes 64 affix keys of a request; its four groups of 64 threads take every fourth head each, eight loads in
+// flight per thread, and meet in a fixed order.  Bound by L2 latency: which query tiles wrote sums is found by a
+// warp, a tile per lane (one thread reading the words one after the other and a thread per key over all heads and
+// tiles: 54 us for 32 requests x 28 heads x 2 tiles x 1024 keys; this 13.5).
 __global__ void __launch_bounds__(256) score_reduce_tiles_kernel(const float* __restrict__ partial,
                                                                  const uint32_t* __restrict__ rowmask, int rm_words,
                                                                  float* __restrict__ scores, int n_heads, int q_tiles, int L,
                                                                  int accumulate) {
     __shared__ int live[256];                    // the query tiles that hold a flagged row (they wrote their partial sums)
-    __shared__ int n_live;
+    __shared__ int n_live_s;
+    __shared__ float group_sum[4][64];
     pdl_wait();
     pdl_launch_dependents();
-    const int b = blockIdx.y;
-    if (threadIdx.x == 0) {
+    const int b = blockIdx.y, lane = threadIdx.x & 31;
+    if (threadIdx.x < 32) {
         int n = 0;
-        for (int qt = 0; qt < q_tiles && qt < 256; ++qt) {
+        for (int q0 = 0; q0 < q_tiles && q0 < 256; q0 += 32) {
+            const int qt = q0 + lane;
             uint32_t any = 0u;
-            for (int w = qt * 4; w < min(qt * 4 + 4, rm_words); ++w) any |= rowmask[(int64_t)b * rm_words + w];
-            if (any) live[n++] = qt;
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+                if (qt * 4 + i < rm_words) any |= __ldg(rowmask + (int64_t)b * rm_words + qt * 4 + i);
+            const bool hit = any != 0u && qt < q_tiles;
+            const uint32_t hits = __ballot_sync(0xffffffffu, hit);
+            if (hit) live[n + __popc(hits & ((1u << lane) - 1u))] = qt;
+            n += __popc(hits);
         }
-        n_live = n;
+        if (lane == 0) n_live_s = n;
     }
     __syncthreads();
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= L) return;
-    // (head, live tile) pairs in a fixed order, eight loads in flight at a time
-    const int total = n_heads * n_live;
+    const int n_live = n_live_s, grp = threadIdx.x >> 6, j = blockIdx.x * 64 + (threadIdx.x & 63);
     float s = 0.f;
-    for (int i0 = 0; i0 < total; i0 += 8) {
-        float t[8];
+    if (j < L) {
+        for (int q = 0; q < n_live; ++q) {
+            const float* src = partial + ((int64_t)b * n_heads * q_tiles + live[q]) * L + j;
+            for (int h0 = grp; h0 < n_heads; h0 += 32) {
+                float t[8];
 #pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            const int i = i0 + u;
-            t[u] = 0.f;
-            if (i < total) {
-                const int h = i / n_live, qt = live[i - h * n_live];
-                t[u] = __ldcg(partial + (((int64_t)b * n_heads + h) * q_tiles + qt) * L + j);
+                for (int u = 0; u < 8; ++u) t[u] = h0 + 4 * u < n_heads ? __ldcg(src + (int64_t)(h0 + 4 * u) * q_tiles * L) : 0.f;
+#pragma unroll
+                for (int u = 0; u < 8; ++u) s += t[u];
             }
         }
-#pragma unroll
-        for (int u = 0; u < 8; ++u) s += t[u];
     }
-    float* out = scores + (int64_t)b * L + j;
-    *out = accumulate ? *out + s : s;
+    group_sum[grp][threadIdx.x & 63] = s;
+    __syncthreads();
+    if (grp == 0 && j < L) {
+        s = (s + group_sum[1][threadIdx.x]) + (group_sum[2][threadIdx.x] + group_sum[3][threadIdx.x]);
+        float* out = scores + (int64_t)b * L + j;
+        *out = accumulate ? *out + s : s;
+    }
 }
 
 void launch_score_reduce_tiles(const float* partial, const uint32_t* rowmask, int rm_words, float* scores, int batch, int n_heads,
                                int q_tiles, int affix_len, int accumulate, cudaStream_t stream) {
     if (batch == 0 || affix_len == 0) return;
-    launch_pdl(score_reduce_tiles_kernel, dim3((affix_len + 255) / 256, batch), dim3(256), 0, stream, partial, rowmask, rm_words,
+    launch_pdl(score_reduce_tiles_kernel, dim3((affix_len + 63) / 64, batch), dim3(256), 0, stream, partial, rowmask, rm_words,
                scores, n_heads, q_tiles, affix_len, accumulate);
 }
 
