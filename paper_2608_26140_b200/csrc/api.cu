@@ -1013,19 +1013,24 @@ acache_status acache_layer_step_host(acache_ctx* ctx, const acache_layer_weights
                                         ys, stream);
     ctx->stash_rows = nullptr;
     if (s != ACACHE_OK) return s;
-    // Results: y through the copy engine (written over the bus by the projection's epilogue it cost 40 us more); scores
-    // and anchors, when page-locked, by one small copy kernel instead of two more transfers.
+    // Results, when page-locked: one copy kernel for all of them (written over the bus by the projection's epilogue, in
+    // 32-byte pieces, y cost 40 us more), unless y is so large that the copy engine's start no longer counts and the SMs
+    // have better to do.
+    constexpr size_t kCopyKernelBytes = 4u << 20;
     void* s_map = const_cast<void*>(mapped_device_pointer(scores_host));
     void* a_map = k ? const_cast<void*>(mapped_device_pointer(anchor_idx_host)) : nullptr;
     const size_t rows = (size_t)req->batch * (k + req->n_extra);
     const size_t n_s = (size_t)req->batch * req->affix_len, n_a = (size_t)req->batch * k;
+    const size_t y_bytes = (flags & ACACHE_F_NO_RECOMPUTE) ? 0 : rows * d.hidden * 2;
     bool ok = true;
-    if (!(flags & ACACHE_F_NO_RECOMPUTE) && rows)
-        ok &= cudaMemcpyAsync(y_host, ys, rows * d.hidden * 2, cudaMemcpyDeviceToHost, stream) == cudaSuccess;
     if (s_map && (a_map || !k) && n_s + n_a < (1u << 30)) {
-        launch_copy_out_words(ss, s_map, (int)n_s, as, a_map, (int)n_a, stream);
+        void* y_map = y_bytes && y_bytes <= kCopyKernelBytes ? const_cast<void*>(mapped_device_pointer(y_host)) : nullptr;
+        if (!aligned16(y_map)) y_map = nullptr;
+        launch_copy_out(ys, y_map, y_map ? (int64_t)(y_bytes / 16) : 0, ss, s_map, (int)n_s, as, a_map, (int)n_a, stream);
         ++ctx->launches;
+        if (y_bytes && !y_map) ok &= cudaMemcpyAsync(y_host, ys, y_bytes, cudaMemcpyDeviceToHost, stream) == cudaSuccess;
     } else {
+        if (y_bytes) ok &= cudaMemcpyAsync(y_host, ys, y_bytes, cudaMemcpyDeviceToHost, stream) == cudaSuccess;
         if (k) ok &= cudaMemcpyAsync(anchor_idx_host, as, n_a * 4, cudaMemcpyDeviceToHost, stream) == cudaSuccess;
         ok &= cudaMemcpyAsync(scores_host, ss, n_s * 4, cudaMemcpyDeviceToHost, stream) == cudaSuccess;
     }

@@ -49,8 +49,10 @@ void launch_row_mask(const int32_t* masked_pos, int m, const int32_t* extra_rows
 void launch_score_reduce_tiles(const float* partial, const uint32_t* rowmask, int rm_words, float* scores, int batch, int n_heads,
                                int q_tiles, int affix_len, int accumulate, cudaStream_t stream);
 
-// a_out[0, n_a) = a, b_out[0, n_b) = b (4-byte words); the outputs may be page-locked host memory seen from the device.
-void launch_copy_out_words(const void* a, void* a_out, int n_a, const void* b, void* b_out, int n_b, cudaStream_t stream);
+// big_out = big (n_big 16-byte pieces), a_out[0, n_a) = a, b_out[0, n_b) = b (4-byte words); the outputs may be page-locked
+// host memory seen from the device.
+void launch_copy_out(const void* big, void* big_out, int64_t n_big, const void* a, void* a_out, int n_a, const void* b, void* b_out,
+                     int n_b, cudaStream_t stream);
 
 // ---- score.cu ---------------------------------------------------------------------------
 struct ScoreArgs {
