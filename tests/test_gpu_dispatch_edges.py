@@ -3,6 +3,7 @@ import numpy as np
 import pytest
 import torch
 
+from oracle import acache_oracle as orc
 from paper_2608_26140_b200 import binding as ab
 from paper_2608_26140_b200 import workloads as wl
 
@@ -60,3 +61,23 @@ def test_probe_row_mask_of_long_contexts(T):
     ref = oracle_step(case, 0, ratio=0.0)["scores"]
     # Eq. 4-5 from bf16 products summed in fp32: the bound the other scoring tests use
     assert np.all(np.abs(s_gpu[0] - ref) <= 1e-3 * np.maximum(ref, ref.mean()))
+
+
+@pytest.mark.parametrize("L", [255, 256, 257, 1025, 2047, 8192, 16385])
+def test_topk_score_distributions(L):
+    """Histogram ranges and candidate counts the selection's passes depend on: a few huge scores over many small ones,
+    a narrow band, zeros and denormals, more equal scores around the threshold than are ranked directly."""
+    g = np.random.default_rng(L)
+    ctx = ab.Context.for_shape(wl.TINY, 1, 256, 128, 1, 1, DEV)
+    spread = np.exp(4.0 * g.standard_normal(L))
+    narrow = 1.0 + 1e-6 * g.random(L)
+    sparse = np.where(g.random(L) < 0.05, g.random(L), 0.0)
+    sparse[::7] = 1e-41
+    bands = np.where(g.random(L) < 0.5, 0.5, g.random(L))
+    signs = g.standard_normal(L) * 1e30
+    for name, s in (("spread", spread), ("narrow", narrow), ("sparse", sparse), ("bands", bands), ("signs", signs)):
+        s = s.astype(np.float32)
+        for K in sorted({1, L // 10, L // 2, L - 1}):
+            out = torch.full((1, K), -7, dtype=torch.int32, device=DEV)
+            ctx.select_topk(torch.from_numpy(s).to(DEV), 1, L, K, out)
+            assert np.array_equal(out[0].cpu().numpy(), orc.select_topk(s, K)[0]), (name, L, K)
