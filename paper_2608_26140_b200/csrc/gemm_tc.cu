@@ -125,12 +125,26 @@ __device__ __forceinline__ void out_residual(const GemmArgs& g, int grow, int co
     }
 }
 
+// x / (1 + exp(-x)).  The quotient is an approximate reciprocal with one Newton step and one correction by the remainder
+// (Newton-Raphson division): as accurate as the division operator to the last bit or two, but without its check for
+// special operands, whose branch kept a thread from working on more than one element at a time (one warp per scheduler: a
+// 256-column tile's SwiGLU took 10 us).  The divisor is kept finite; below
+// x = -87.3 the result is 0 (the true value is under 1e-36 there).  Epilogue of a 128 x 256 tile: 10 -> 4.5 us, of the last
+// one, which nothing hides, 9.5 -> 3.4.
+__device__ __forceinline__ float silu(float x) {
+    const float d = fminf(1.f + __expf(-x), 3e38f);
+    float r = __fdividef(1.f, d);
+    r = fmaf(fmaf(-d, r, 1.f), r, r);
+    const float q = x * r;
+    return fmaf(fmaf(-q, d, x), r, q);
+}
+
 // out[grow, col..col+W) = bf16(silu(gate) * up)
 template <int W>
 __device__ __forceinline__ void out_swiglu(const GemmArgs& g, int grow, int col, float (&gate)[W], const float (&up)[W]) {
     uint4* o = reinterpret_cast<uint4*>(static_cast<__nv_bfloat16*>(g.c) + (int64_t)grow * g.n[0] + col);
 #pragma unroll
-    for (int i = 0; i < W; ++i) gate[i] = gate[i] / (1.f + __expf(-gate[i])) * up[i];
+    for (int i = 0; i < W; ++i) gate[i] = silu(gate[i]) * up[i];
 #pragma unroll
     for (int j = 0; j < W / 8; ++j) o[j] = pack8(gate + 8 * j);
 }
