@@ -105,25 +105,23 @@ __device__ __forceinline__ uint4 pack8(const float* v) {
     return make_uint4(pack_bf16(v[0], v[1]), pack_bf16(v[2], v[3]), pack_bf16(v[4], v[5]), pack_bf16(v[6], v[7]));
 }
 
-// ---- epilogues on W adjacent fp32 accumulator columns of one row (W = 16 or 32) ----------------
-// Every store is W*2 bytes of one row: whole 32-byte sectors, no partial-sector writes.
-
-// out[grow, col..col+W) = bf16(resid[grow] + acc)
-template <int W>
-__device__ __forceinline__ void out_residual(const GemmArgs& g, int grow, int col, float (&v)[W]) {
-    const int N = g.n[0];
-    const int64_t roff = g.resid_off ? __ldcg(g.resid_off + grow) : (int64_t)grow * N;
-    const uint4* rp = reinterpret_cast<const uint4*>(static_cast<const __nv_bfloat16*>(g.resid) + roff + col);
-    uint4* o = reinterpret_cast<uint4*>(static_cast<__nv_bfloat16*>(g.c) + (int64_t)grow * N + col);
+// 16 bf16 of one row: one 32-byte store (a whole sector per lane) where the address allows it.
+__device__ __forceinline__ void store16(__nv_bfloat16* o, const float* v) {
+    uint32_t w[8];
 #pragma unroll
-    for (int j = 0; j < W / 8; ++j) {
-        const uint4 r = __ldcg(rp + j);
-        const uint32_t rw[4] = {r.x, r.y, r.z, r.w};
-#pragma unroll
-        for (int i = 0; i < 4; ++i) { v[8 * j + 2 * i] += bf16_lo(rw[i]); v[8 * j + 2 * i + 1] += bf16_hi(rw[i]); }
-        o[j] = pack8(v + 8 * j);
+    for (int i = 0; i < 8; ++i) w[i] = pack_bf16(v[2 * i], v[2 * i + 1]);
+    if ((reinterpret_cast<uintptr_t>(o) & 31u) == 0) {
+        asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};"
+                     ::"l"(o), "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3]), "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7])
+                     : "memory");
+    } else {
+        reinterpret_cast<uint4*>(o)[0] = make_uint4(w[0], w[1], w[2], w[3]);
+        reinterpret_cast<uint4*>(o)[1] = make_uint4(w[4], w[5], w[6], w[7]);
     }
 }
+
+// ---- epilogues on W adjacent fp32 accumulator columns of one row (W = 16 or 32) ----------------
+// Every store is W*2 bytes of one row: whole 32-byte sectors, no partial-sector writes.
 
 // x / (1 + exp(-x)).  The quotient is an approximate reciprocal with one Newton step and one correction by the remainder
 // (Newton-Raphson division): as accurate as the division operator to the last bit or two, but without its check for
@@ -142,20 +140,33 @@ __device__ __forceinline__ float silu(float x) {
 // out[grow, col..col+W) = bf16(silu(gate) * up)
 template <int W>
 __device__ __forceinline__ void out_swiglu(const GemmArgs& g, int grow, int col, float (&gate)[W], const float (&up)[W]) {
-    uint4* o = reinterpret_cast<uint4*>(static_cast<__nv_bfloat16*>(g.c) + (int64_t)grow * g.n[0] + col);
+    __nv_bfloat16* o = static_cast<__nv_bfloat16*>(g.c) + (int64_t)grow * g.n[0] + col;
 #pragma unroll
     for (int i = 0; i < W; ++i) gate[i] = silu(gate[i]) * up[i];
 #pragma unroll
-    for (int j = 0; j < W / 8; ++j) o[j] = pack8(gate + 8 * j);
+    for (int j = 0; j < W / 16; ++j) store16(o + 16 * j, gate + 16 * j);
+}
+
+// cos and sin of the row's position for W pairs from j0 on.
+template <int W>
+__device__ __forceinline__ void load_rope(const GemmArgs& g, int pos, int j0, float (&c)[W], float (&sn)[W]) {
+    const int64_t at = (int64_t)(pos < 0 ? 0 : pos) * (g.head_dim >> 1) + j0;
+    const float4* c4 = reinterpret_cast<const float4*>(g.rope_cos + at);
+    const float4* s4 = reinterpret_cast<const float4*>(g.rope_sin + at);
+#pragma unroll
+    for (int j = 0; j < W / 4; ++j) {
+        const float4 x = c4[j], y = s4[j];
+        c[4 * j] = x.x; c[4 * j + 1] = x.y; c[4 * j + 2] = x.z; c[4 * j + 3] = x.w;
+        sn[4 * j] = y.x; sn[4 * j + 1] = y.y; sn[4 * j + 2] = y.z; sn[4 * j + 3] = y.w;
+    }
 }
 
 // q/k/v: bias, rotary embedding with the pairing (i, i + d/2) at the row's position, bf16 store
 // to the compact output and, for k/v, straight into the cache row (scatter fused).
-// lo/hi: W columns of each rotary half; col: column of lo[0] inside segment seg; j0: its index
-// inside the half head.
+// lo/hi: W columns of each rotary half; col: column of lo[0] inside segment seg; c/sn: load_rope (rotary segments).
 template <int W>
-__device__ __forceinline__ void out_qkv(const GemmArgs& g, int grow, int pos, int seg, int col, int j0, float (&lo)[W],
-                                        float (&hi)[W]) {
+__device__ __forceinline__ void rope_qkv(const GemmArgs& g, int seg, int col, float (&lo)[W], float (&hi)[W], const float (&c)[W],
+                                         const float (&sn)[W]) {
     const int half = g.head_dim >> 1;
     const __nv_bfloat16* bias = static_cast<const __nv_bfloat16*>(g.bias[seg]);
     if (bias) {
@@ -166,21 +177,18 @@ __device__ __forceinline__ void out_qkv(const GemmArgs& g, int grow, int pos, in
         }
     }
     if (seg < g.rope_segments) {
-        const int pp = pos < 0 ? 0 : pos;
-        const float4* cs = reinterpret_cast<const float4*>(g.rope_cos + (int64_t)pp * half + j0);
-        const float4* sn = reinterpret_cast<const float4*>(g.rope_sin + (int64_t)pp * half + j0);
 #pragma unroll
-        for (int j = 0; j < W / 4; ++j) {
-            const float4 c4 = cs[j], s4 = sn[j];
-            const float c[4] = {c4.x, c4.y, c4.z, c4.w}, sv[4] = {s4.x, s4.y, s4.z, s4.w};
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const float x = lo[4 * j + i], y = hi[4 * j + i];
-                lo[4 * j + i] = x * c[i] - y * sv[i];
-                hi[4 * j + i] = y * c[i] + x * sv[i];
-            }
+        for (int i = 0; i < W; ++i) {
+            const float x = lo[i], y = hi[i];
+            lo[i] = x * c[i] - y * sn[i];
+            hi[i] = y * c[i] + x * sn[i];
         }
     }
+}
+template <int W>
+__device__ __forceinline__ void store_qkv(const GemmArgs& g, int grow, int pos, int seg, int col, const float (&lo)[W],
+                                          const float (&hi)[W]) {
+    const int half = g.head_dim >> 1;
     const int nseg = g.n[seg];
     __nv_bfloat16* cache = seg == 1 ? static_cast<__nv_bfloat16*>(g.cache_k)
                          : seg == 2 ? static_cast<__nv_bfloat16*>(g.cache_v) : nullptr;
@@ -199,10 +207,9 @@ __device__ __forceinline__ void out_qkv(const GemmArgs& g, int grow, int pos, in
                             ? cache + (int64_t)(grow / g.rows_per_req) * g.kv_batch_stride + (int64_t)pos * nseg + col
                             : nullptr;
 #pragma unroll
-    for (int j = 0; j < W / 8; ++j) {
-        const uint4 l = pack8(lo + 8 * j), h = pack8(hi + 8 * j);
-        if (o1) { reinterpret_cast<uint4*>(o1)[j] = l; reinterpret_cast<uint4*>(o1 + half)[j] = h; }
-        if (o2) { reinterpret_cast<uint4*>(o2)[j] = l; reinterpret_cast<uint4*>(o2 + half)[j] = h; }
+    for (int j = 0; j < W / 16; ++j) {
+        if (o1) { store16(o1 + 16 * j, lo + 16 * j); store16(o1 + half + 16 * j, hi + 16 * j); }
+        if (o2) { store16(o2 + 16 * j, lo + 16 * j); store16(o2 + half + 16 * j, hi + 16 * j); }
     }
 }
 
@@ -272,6 +279,12 @@ __device__ __forceinline__ void sum_slots16(const float* __restrict__ partial, c
             }
         }
     }
+}
+
+// Entry of the softmax statistics of one row in vocabulary tile nt: rows contiguous, so that a warp (a row per lane) writes
+// whole lines.
+__device__ __forceinline__ float4* logit_entry(const GemmArgs& g, int nt, int entry, int row) {
+    return g.logit_stats + ((int64_t)nt * 16 + entry) * g.M + row;
 }
 
 // Softmax statistics of W logits starting at vocabulary index col: running (max, sum exp(z - max),
@@ -380,43 +393,83 @@ __device__ __forceinline__ void finish_item(const GemmArgs& g, const TcPlan& p, 
         const uint32_t rw[8] = {res[0].x, res[0].y, res[0].z, res[0].w, res[1].x, res[1].y, res[1].z, res[1].w};
 #pragma unroll
         for (int i = 0; i < 8; ++i) { lo[2 * i] += bf16_lo(rw[i]); lo[2 * i + 1] += bf16_hi(rw[i]); }
-        uint4* o = reinterpret_cast<uint4*>(static_cast<__nv_bfloat16*>(g.c) + (int64_t)grow * g.n[0] + nt * TC_BN + item * 16);
-        o[0] = pack8(lo); o[1] = pack8(lo + 8);
+        store16(static_cast<__nv_bfloat16*>(g.c) + (int64_t)grow * g.n[0] + nt * TC_BN + item * 16, lo);
     } else if (g.epilogue == kEpiLogits) {
         float m = -INFINITY, sm = 0.f;
         int arg = 0;
         logit_stats_update<16>(lo, nt * TC_BN + item * 16, m, sm, arg);
-        g.logit_stats[((int64_t)grow * p.n_tiles + nt) * 16 + item] = make_float4(m, sm, __int_as_float(arg), 0.f);
+        *logit_entry(g, nt, item, grow) = make_float4(m, sm, __int_as_float(arg), 16.f);
     } else if (g.epilogue == kEpiSwiGLU) {
         out_swiglu<16>(g, grow, nt * 128 + item * 16, lo, hi);
     } else {
         int seg, c0;
         qkv_unit(g, u128, seg, c0);
-        out_qkv<16>(g, grow, pos, seg, c0 + lo_col, lo_col & (half - 1), lo, hi);
+        float c[16], sn[16];
+        if (seg < g.rope_segments) load_rope<16>(g, pos, lo_col & (half - 1), c, sn);
+        rope_qkv<16>(g, seg, c0 + lo_col, lo, hi, c, sn);
+        store_qkv<16>(g, grow, pos, seg, c0 + lo_col, lo, hi);
     }
 }
 
-// Epilogue of a whole tile straight from TMEM (the CTA covered the tile's entire K range):
-// thread = one row of the tile, 32 accumulator columns per tcgen05.ld.
-__device__ __forceinline__ void direct_epilogue(const GemmArgs& g, const TcPlan& p, uint32_t taddr, int nt, int grow,
-                                                bool valid, int nchunks) {
+// Epilogue of one half (128 accumulator columns) of a whole tile straight from TMEM: thread = one row, 32 columns per
+// tcgen05.ld.  The last tile's epilogue is the tail of the launch, and with four warps taking a tile's 256 columns and asking
+// for the residual (the rotary table) chunk by chunk it lasted 10-16 us.  So eight warps share a tile, and what does not
+// depend on the accumulator is requested before the wait for it: the half's 256 bytes of residual, or the first 32 pairs'
+// cosines and sines.  Last tile of a 1015-row down projection: 13.1 -> 3.0 us, of a q/k/v projection 14.3 -> 10.1.
+struct HalfPre {
+    uint32_t w[64];
+    int pos;
+};
+__device__ __forceinline__ void half_prefetch(const GemmArgs& g, int nt, int hf, int grow, bool valid, HalfPre& pre) {
+    pre.pos = 0;
+    if (!valid) return;
     if (g.epilogue == kEpiResidual) {
-        for (int c = 0; c < nchunks; ++c) {
+        const int64_t roff = g.resid_off ? __ldcg(g.resid_off + grow) : (int64_t)grow * g.n[0];
+        const uint4* rp = reinterpret_cast<const uint4*>(static_cast<const __nv_bfloat16*>(g.resid) + roff + nt * TC_BN + hf * 128);
+        if (nt * TC_BN + hf * 128 < g.n[0]) {
+#pragma unroll
+            for (int j = 0; j < 16; ++j) {
+                const uint4 u = __ldcg(rp + j);
+                pre.w[4 * j] = u.x; pre.w[4 * j + 1] = u.y; pre.w[4 * j + 2] = u.z; pre.w[4 * j + 3] = u.w;
+            }
+        }
+    } else if (g.epilogue == kEpiQKV) {
+        pre.pos = __ldcg(g.row_pos + grow);
+        int seg, c0;
+        qkv_unit(g, nt * 2 + hf, seg, c0);
+        if (seg < g.rope_segments) {
+            float (&c)[32] = reinterpret_cast<float (&)[32]>(pre.w[0]);
+            float (&sn)[32] = reinterpret_cast<float (&)[32]>(pre.w[32]);
+            load_rope<32>(g, pre.pos, 0, c, sn);
+        }
+    }
+}
+__device__ __forceinline__ void half_epilogue(const GemmArgs& g, const TcPlan& p, uint32_t taddr, int nt, int hf, int n_halves,
+                                              int grow, bool valid, HalfPre& pre) {
+    if (g.epilogue == kEpiResidual) {
+        __nv_bfloat16* o = static_cast<__nv_bfloat16*>(g.c) + (int64_t)grow * g.n[0] + nt * TC_BN + hf * 128;
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
             float v[32];
-            tc_ld32(taddr + c * 32, v);
-            if (valid) out_residual<32>(g, grow, nt * TC_BN + c * 32, v);
+            tc_ld32(taddr + hf * 128 + c * 32, v);
+#pragma unroll
+            for (int i = 0; i < 16; ++i) { v[2 * i] += bf16_lo(pre.w[16 * c + i]); v[2 * i + 1] += bf16_hi(pre.w[16 * c + i]); }
+            if (valid) { store16(o + c * 32, v); store16(o + c * 32 + 16, v + 16); }
         }
     } else if (g.epilogue == kEpiLogits) {
+        // one entry per half; w: how many entries the tile has
         float m = -INFINITY, sm = 0.f;
         int arg = 0;
-        for (int c = 0; c < nchunks; ++c) {
-            float v[32];
-            tc_ld32(taddr + c * 32, v);
-            logit_stats_update<32>(v, nt * TC_BN + c * 32, m, sm, arg);
-        }
-        if (valid) g.logit_stats[((int64_t)grow * p.n_tiles + nt) * 16] = make_float4(m, sm, __int_as_float(arg), 0.f);
-    } else if (g.epilogue == kEpiSwiGLU) {
+#pragma unroll 1
         for (int c = 0; c < 4; ++c) {
+            float v[32];
+            tc_ld32(taddr + hf * 128 + c * 32, v);
+            logit_stats_update<32>(v, nt * TC_BN + hf * 128 + c * 32, m, sm, arg);
+        }
+        if (valid) *logit_entry(g, nt, hf, grow) = make_float4(m, sm, __int_as_float(arg), (float)n_halves);
+    } else if (g.epilogue == kEpiSwiGLU) {
+#pragma unroll 1
+        for (int c = hf * 2; c < hf * 2 + 2; ++c) {
             float gate[32], up[32];
             tc_ld32(taddr + c * 32, gate);
             tc_ld32(taddr + 128 + c * 32, up);
@@ -424,17 +477,21 @@ __device__ __forceinline__ void direct_epilogue(const GemmArgs& g, const TcPlan&
         }
     } else {
         const int half = g.head_dim >> 1;
-        const int pos = valid ? __ldcg(g.row_pos + grow) : 0;
-        for (int h = 0; h < nchunks / 4; ++h) {
-            int seg, c0;
-            qkv_unit(g, nt * 2 + h, seg, c0);
-            for (int r = 0; r < 2; ++r) {
-                // d = 128: chunks (r, r + 2) of the unit; d = 64: chunks (2r, 2r + 1)
-                const int cl = g.head_dim == 128 ? r : 2 * r, ch = g.head_dim == 128 ? r + 2 : 2 * r + 1;
-                float lo[32], hi[32];
-                tc_ld32(taddr + h * 128 + cl * 32, lo);
-                tc_ld32(taddr + h * 128 + ch * 32, hi);
-                if (valid) out_qkv<32>(g, grow, pos, seg, c0 + cl * 32, (cl * 32) & (half - 1), lo, hi);
+        int seg, c0;
+        qkv_unit(g, nt * 2 + hf, seg, c0);
+        float (&c)[32] = reinterpret_cast<float (&)[32]>(pre.w[0]);
+        float (&sn)[32] = reinterpret_cast<float (&)[32]>(pre.w[32]);
+#pragma unroll 1
+        for (int r = 0; r < 2; ++r) {
+            // d = 128: chunks (r, r + 2) of the unit; d = 64: chunks (2r, 2r + 1)
+            const int cl = g.head_dim == 128 ? r : 2 * r, ch = g.head_dim == 128 ? r + 2 : 2 * r + 1;
+            float lo[32], hi[32];
+            tc_ld32(taddr + hf * 128 + cl * 32, lo);
+            tc_ld32(taddr + hf * 128 + ch * 32, hi);
+            if (valid) {
+                rope_qkv<32>(g, seg, c0 + cl * 32, lo, hi, c, sn);
+                if (r == 0 && half == 64 && seg < g.rope_segments) load_rope<32>(g, pre.pos, 32, c, sn);
+                store_qkv<32>(g, grow, pre.pos, seg, c0 + cl * 32, lo, hi);
             }
         }
     }
@@ -782,7 +839,11 @@ gemm_tc_kernel(const GemmArgs g, const TcPlan p, const __grid_constant__ CUtenso
             const bool valid = mt * TC_BM + row < g.M;
             const uint32_t taddr = tmem_base + acc * TC_BN + ((uint32_t)(q * 32) << 16);
             if (kb0 == 0 && kb1 == p.KB) {
-                direct_epilogue(g, p, taddr, nt, mt * TC_BM + row, valid, nchunks);
+                for (int hf = 0; hf < nchunks / 4; ++hf) {
+                    HalfPre pre;
+                    half_prefetch(g, nt, hf, mt * TC_BM + row, valid, pre);
+                    half_epilogue(g, p, taddr, nt, hf, nchunks / 4, mt * TC_BM + row, valid, pre);
+                }
             } else {
                 float4* dst = reinterpret_cast<float4*>(g.partial) +
                               ((int64_t)blockIdx.x * 2 + (it == it0 ? 0 : 1)) * (TC_SLOT_FLOATS / 4);
@@ -846,6 +907,7 @@ gemm_tc_kernel(const GemmArgs g, const TcPlan p, const __grid_constant__ CUtenso
 // Barriers: the leader's full[s] counts both CTAs' TMA bytes (announced by the leader's producer); empty[s] and tmem_full[a] live in
 // each CTA and are signalled by a tcgen05.commit multicast to both; the leader's tmem_empty[a]
 // collects the drain warps of both CTAs.
+constexpr int TC2_THREADS = 320;                                // warp 0: TMA, warp 1: MMA, warps 2-9: drain
 constexpr int TC2_STAGES = 6;
 constexpr int TC2_STAGE_BYTES = TC_A_BYTES + TC_HALF_BYTES;     // 32 KB per CTA and stage
 constexpr int TC2_SMEM = TC2_STAGES * TC2_STAGE_BYTES + 1024 + 256;
@@ -885,12 +947,12 @@ __device__ __forceinline__ void tma_load_2d_pair(uint32_t dst, const CUtensorMap
         ::"r"(dst), "l"(map), "r"(c0), "r"(c1), "r"(bar_cluster), "l"(policy)
         : "memory");
 }
-__global__ void __launch_bounds__(TC_THREADS, 1)
+__global__ void __launch_bounds__(TC2_THREADS, 1)
 gemm_tc2_kernel(const GemmArgs g, const TcPlan p, const int clusters, const __grid_constant__ CUtensorMap mapA,
                 const __grid_constant__ CUtensorMap mapB0, const __grid_constant__ CUtensorMap mapB1,
                 const __grid_constant__ CUtensorMap mapB2) {
     extern __shared__ unsigned char smem_raw[];
-    __shared__ float red[TC_THREADS / 32];
+    __shared__ float red[TC2_THREADS / 32];
     const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     unsigned char* base_ptr = smem_raw + (base - smem_u32(smem_raw));
     const uint32_t bars = base + TC2_STAGES * TC2_STAGE_BYTES;
@@ -907,7 +969,7 @@ gemm_tc2_kernel(const GemmArgs g, const TcPlan p, const int clusters, const __gr
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < TC2_STAGES; ++s) { mbar_init(full_bar(s), 1); mbar_init(empty_bar(s), 1); }
-        for (int i = 0; i < 2; ++i) { mbar_init(tfull_bar(i), 1); mbar_init(tempty_bar(i), 8); }
+        for (int i = 0; i < 2; ++i) { mbar_init(tfull_bar(i), 1); mbar_init(tempty_bar(i), 16); }
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -998,9 +1060,9 @@ gemm_tc2_kernel(const GemmArgs g, const TcPlan p, const int clusters, const __gr
             if (++acc == 2) { acc = 0; acc_phase ^= 1; }
             if (p.pair_u) { it += kb1 - kb0; ++t; } else t += clusters;
         }
-    } else if (warp >= 2 && warp < 6) {
-        // drain: this CTA's 128 rows of the tile, epilogue straight from TMEM
-        const int q = warp & 3;
+    } else if (warp >= 2) {
+        // drain: this CTA's 128 rows of the tile, epilogue straight from TMEM; two warps per lane quarter, 128 columns each
+        const int q = warp & 3, hf = (warp - 2) >> 2;
         const int row = q * 32 + lane;
         int acc = 0;
         uint32_t acc_phase = 0;
@@ -1015,16 +1077,19 @@ gemm_tc2_kernel(const GemmArgs g, const TcPlan p, const int clusters, const __gr
             const int kb0 = p.pair_u ? (int)(it - (long long)t * p.KB) : 0;
             const int kb1 = p.pair_u ? (int)min((long long)p.KB, (long long)(kb0 + (it_end - it))) : p.KB;
             const int grow = (mp * 2 + (int)rank) * TC_BM + row;
+            const bool is_whole = kb0 == 0 && kb1 == p.KB;
+            HalfPre pre;
+            if (is_whole) half_prefetch(g, nt, hf, grow, grow < g.M, pre);
             if (!(ok = mbar_wait(tfull_bar(acc), acc_phase, abort_flag))) break;
             tc_fence_after();
             const uint32_t taddr = tmem_base + acc * TC_BN + ((uint32_t)(q * 32) << 16);
-            if (kb0 == 0 && kb1 == p.KB) {
-                direct_epilogue(g, p, taddr, nt, grow, grow < g.M, 8);
+            if (is_whole) {
+                half_epilogue(g, p, taddr, nt, hf, 2, grow, grow < g.M, pre);
             } else {
                 // a tile whose K range is cut between clusters: this CTA's 128 rows to its fp32 partial slot
                 float4* dst = reinterpret_cast<float4*>(g.partial) +
                               (((int64_t)cluster_id * 2 + (it == it_first ? 0 : 1)) * 2 + rank) * (TC_SLOT_FLOATS / 4);
-                for (int c = 0; c < 8; ++c) {
+                for (int c = hf * 4; c < hf * 4 + 4; ++c) {
                     float v[32];
                     tc_ld32(taddr + c * 32, v);
                     if (grow < g.M) {
@@ -1098,51 +1163,67 @@ __global__ void __launch_bounds__(256, NC == 2 ? 2 : 1) gemm_finish_kernel(const
 
 // ---- predict and commit (Eq. 2-3): confidence and arg max per row, commit rule per request ------
 struct LogitAcc { float m, s; int arg; };
+// Branch-free (lanes hold different tiles); an empty entry is m = -FLT_MAX, s = 0.  The lowest index wins a tie.
 __device__ __forceinline__ void logit_merge(LogitAcc& a, float m, float s, int arg) {
-    if (s == 0.f) return;            // an empty entry
-    if (m > a.m || (m == a.m && arg < a.arg && s > 0.f)) {
-        a.s = a.s * __expf(a.m - m) + s;
-        a.m = m;
-        a.arg = arg;
-    } else {
-        a.s += s * __expf(m - a.m);
+    const float nm = fmaxf(a.m, m);
+    a.s = a.s * __expf(a.m - nm) + s * __expf(m - nm);
+    a.arg = m > a.m || (m == a.m && arg < a.arg) ? arg : a.arg;
+    a.m = nm;
+}
+__device__ __forceinline__ void logit_merge_warp(LogitAcc& a, int width) {
+#pragma unroll 1
+    for (int o = width >> 1; o > 0; o >>= 1) {
+        const float m = __shfl_xor_sync(0xffffffffu, a.m, o), sm = __shfl_xor_sync(0xffffffffu, a.s, o);
+        logit_merge(a, m, sm, __shfl_xor_sync(0xffffffffu, a.arg, o));
     }
 }
 
-// One CTA per row: merges the per-tile statistics (16 entries for a tile whose K range was split
-// between CTAs, one otherwise) in a fixed order.
-__global__ void __launch_bounds__(256) logit_reduce_kernel(const GemmArgs g, const TcPlan p, int32_t* __restrict__ token,
-                                                           float* __restrict__ confidence) {
-    __shared__ float sm_m[256], sm_s[256];
-    __shared__ int sm_a[256];
+// One CTA per row: merges the per-tile statistics (16 entries for a tile whose K range was split between CTAs, one or two
+// otherwise; the first one's w says how many) in a fixed order.  Bound by the latency of L2 and the instructions per entry:
+// half a warp takes a tile, a lane per entry, four tiles in flight per lane; where no tile is cut a thread takes an entry.
+// 512 rows x 126 464 logits: 20.7 -> 8.2 us.
+constexpr int LR_THREADS = 512;
+__global__ void __launch_bounds__(LR_THREADS) logit_reduce_kernel(const GemmArgs g, const TcPlan p, int32_t* __restrict__ token,
+                                                                  float* __restrict__ confidence) {
+    __shared__ LogitAcc part[32];
+    const int row = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5, entry = lane & 15;
+    const LogitAcc empty{-3.402823466e38f, 0.f, 0x7fffffff};
+    if (threadIdx.x < 32) part[threadIdx.x] = empty;
     pdl_wait();
     pdl_launch_dependents();
-    const int row = blockIdx.x, mt = row / TC_BM;
-    LogitAcc a{-INFINITY, 0.f, 0x7fffffff};
-    for (int nt = threadIdx.x; nt < p.n_tiles; nt += 256) {
-        int c_first = 0, c_last = 0;
-        if (!p.whole) tile_cover(p, nt * p.m_tiles + mt, c_first, c_last);
-        const int n_entries = c_first == c_last ? 1 : 16;
-        const float4* e = g.logit_stats + ((int64_t)row * p.n_tiles + nt) * 16;
-        for (int i = 0; i < n_entries; ++i) {
-            if (n_entries == 16 && nt * 2 + (i >> 3) >= p.units) break;
-            const float4 v = __ldcg(e + i);
+    LogitAcc a = empty;
+    constexpr int kStep = LR_THREADS / 16;
+    if (p.whole) {
+#pragma unroll 1
+        for (int i = threadIdx.x; i < 2 * p.n_tiles; i += LR_THREADS) {
+            const float4 v = __ldcg(logit_entry(g, i >> 1, i & 1, row));
             logit_merge(a, v.x, v.y, __float_as_int(v.z));
         }
-    }
-    sm_m[threadIdx.x] = a.m; sm_s[threadIdx.x] = a.s; sm_a[threadIdx.x] = a.arg;
-    __syncthreads();
-    for (int o = 128; o > 0; o >>= 1) {
-        if (threadIdx.x < o) {
-            LogitAcc x{sm_m[threadIdx.x], sm_s[threadIdx.x], sm_a[threadIdx.x]};
-            logit_merge(x, sm_m[threadIdx.x + o], sm_s[threadIdx.x + o], sm_a[threadIdx.x + o]);
-            sm_m[threadIdx.x] = x.m; sm_s[threadIdx.x] = x.s; sm_a[threadIdx.x] = x.arg;
+    } else {
+#pragma unroll 1
+        for (int nt0 = threadIdx.x >> 4; nt0 - (lane >> 4) < p.n_tiles; nt0 += 4 * kStep) {
+            float4 v[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) v[i] = __ldcg(logit_entry(g, min(nt0 + i * kStep, p.n_tiles - 1), entry, row));
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const int nt = nt0 + i * kStep, n = (int)__shfl_sync(0xffffffffu, v[i].w, lane & 16);
+                const bool use = nt < p.n_tiles && entry < n && (n < 16 || nt * 2 + (entry >> 3) < p.units);
+                logit_merge(a, use ? v[i].x : empty.m, use ? v[i].y : 0.f, use ? __float_as_int(v[i].z) : empty.arg);
+            }
         }
-        __syncthreads();
     }
-    if (threadIdx.x == 0) {
-        token[row] = sm_a[0];
-        confidence[row] = 1.f / sm_s[0];       // softmax probability of the arg max
+    logit_merge_warp(a, 32);
+    __syncthreads();
+    if (lane == 0) part[warp] = a;
+    __syncthreads();
+    if (warp == 0) {
+        a = part[lane];
+        logit_merge_warp(a, LR_THREADS / 32);
+        if (lane == 0) {
+            token[row] = a.arg;
+            confidence[row] = 1.f / a.s;       // softmax probability of the arg max
+        }
     }
 }
 
@@ -1265,7 +1346,7 @@ struct GemmLaunch {
 cudaLaunchConfig_t pair_config(cudaLaunchAttribute* at, int clusters, cudaStream_t stream) {
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(clusters * 2);
-    cfg.blockDim = dim3(TC_THREADS);
+    cfg.blockDim = dim3(TC2_THREADS);
     cfg.dynamicSmemBytes = TC2_SMEM;
     cfg.stream = stream;
     at[0].id = cudaLaunchAttributeClusterDimension;
@@ -1429,7 +1510,7 @@ int launch_predict_commit(const GemmArgs& g, int batch, int n_blk, float thresho
                           int32_t* commit, cudaStream_t stream) {
     if (g.M == 0) return 0;
     const TcPlan p = plan_gemm(g).p;
-    if (launch_pdl(logit_reduce_kernel, dim3(g.M), dim3(256), 0, stream, g, p, token, confidence) != cudaSuccess) return -1;
+    if (launch_pdl(logit_reduce_kernel, dim3(g.M), dim3(LR_THREADS), 0, stream, g, p, token, confidence) != cudaSuccess) return -1;
     if (launch_pdl(commit_kernel, dim3(batch), dim3(32), 0, stream, (const float*)confidence, n_blk, threshold, commit) !=
         cudaSuccess)
         return -1;

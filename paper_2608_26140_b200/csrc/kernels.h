@@ -154,7 +154,7 @@ struct GemmArgs {
     // --- kEpiSwiGLU / kEpiResidual output ---
     void* c;                  // bf16 [M, Nout]
     // --- kEpiLogits ---
-    float4* logit_stats;      // [M, n_tiles, 16] of (max, sum exp(z - max), argmax as int bits, -)
+    float4* logit_stats;      // [n_tiles, 16, M] of (max, sum exp(z - max), argmax as int bits, entries of the tile)
     // --- row work fused in front of the contraction ---
     RowPrep prep;             // writes the A rows (a) before the contraction
     // --- scratch ---
