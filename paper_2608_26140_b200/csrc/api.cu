@@ -1,7 +1,6 @@
 // C-ABI entry points (see include/acache.h): argument validation, workspace layout and the
 // kernel sequences of the affix-cache refresh path.  Everything is enqueued on the caller's
 // stream; nothing here allocates device memory or synchronises (except acache_poll_status).
-#include <array>
 #include <algorithm>
 #include <cmath>
 #include <cstdarg>
@@ -145,19 +144,6 @@ acache_status run_score(acache_ctx* c, const acache_request* r, const void* q_ma
 // The private slot array a decode pass over shared storage works against: k anchors and e extra rows per
 // request as an earlier refresh pass over the same storage wrote them; out_rows[b, i] = the slot row that
 // holds row i of the rows recomputed now.
-// K blocks past the shared-memory ring that each projection asks into L2 before its dependency wait (masked-row
-// queries, q/k/v, output, gate/up, down).  Worth it only behind kernels that leave memory idle for a while: the
-// previous step's last finish, and scoring + selection (measured at 103 rows: 168.8 us per layer-step with none,
-// 167.9 with 8 blocks for the first two, 170.7 with 8 for the down projection).  ACACHE_GEMM_PREFETCH_BY="a,b,c,d,e"
-// overrides.
-static int prefetch_by(int which) {
-    static const std::array<int, 5> v = [] {
-        std::array<int, 5> r{8, 8, 0, 0, 0};
-        if (const char* e = getenv("ACACHE_GEMM_PREFETCH_BY")) sscanf(e, "%d,%d,%d,%d,%d", &r[0], &r[1], &r[2], &r[3], &r[4]);
-        return r;
-    }();
-    return v[which];
-}
 // Eq. 4-5 taken from the attention of the rows being recomputed (the probe of Section 3.2: the masked rows are among them)
 struct FusedScore {
     const uint32_t* rowmask;
@@ -228,7 +214,6 @@ acache_status run_recompute(acache_ctx* c, const acache_layer_weights* w, const 
     g.kv_batch_stride = kv->batch_stride; g.rows_per_req = rows;
     if (priv) { g.kv_out_rows = priv->out_rows; g.kv_out_stride = priv->k + priv->e; }
     g.partial = partial; g.status = status; g.grid_bar = grid_bar;
-    g.prefetch_blocks = prefetch_by(1);
     g.debug_expire = c->debug_expire_once;
     c->debug_expire_once = 0;
     { int nl = launch_gemm(g, st); if (nl < 0) return check_cuda(c, "qkv projection") == ACACHE_OK ? fail(c, ACACHE_ERR_CUDA, "qkv projection launch failed") : ACACHE_ERR_CUDA;
@@ -293,7 +278,6 @@ acache_status run_recompute(acache_ctx* c, const acache_layer_weights* w, const 
     go.a = o; go.M = n; go.K = qd; go.b[0] = w->wo; go.n[0] = d.hidden;
     go.epilogue = kEpiResidual; go.resid = x_rows ? x_rows : x; go.resid_off = x_rows ? nullptr : row_src; go.c = h1;
     go.partial = partial; go.status = status; go.grid_bar = grid_bar;
-    go.prefetch_blocks = prefetch_by(2);
     { int nl = launch_gemm(go, st); if (nl < 0) return check_cuda(c, "output projection") == ACACHE_OK ? fail(c, ACACHE_ERR_CUDA, "output projection launch failed") : ACACHE_ERR_CUDA;
     c->launches += nl; }
     mark(c, ACACHE_STAGE_GATE_UP, st);
@@ -303,7 +287,6 @@ acache_status run_recompute(acache_ctx* c, const acache_layer_weights* w, const 
     gu.a = xn2; gu.M = n; gu.K = d.hidden; gu.b[0] = w->w_gate; gu.b[1] = w->w_up; gu.n[0] = d.ffn; gu.n[1] = d.ffn;
     gu.epilogue = kEpiSwiGLU; gu.c = act;
     gu.partial = partial; gu.status = status; gu.grid_bar = grid_bar;
-    gu.prefetch_blocks = prefetch_by(3);
     { int nl = launch_gemm(gu, st); if (nl < 0) return check_cuda(c, "gate/up projection") == ACACHE_OK ? fail(c, ACACHE_ERR_CUDA, "gate/up projection launch failed") : ACACHE_ERR_CUDA;
     c->launches += nl; }
 
@@ -312,7 +295,6 @@ acache_status run_recompute(acache_ctx* c, const acache_layer_weights* w, const 
     gd.a = act; gd.M = n; gd.K = d.ffn; gd.b[0] = w->w_down; gd.n[0] = d.hidden;
     gd.epilogue = kEpiResidual; gd.resid = h1; gd.resid_off = nullptr; gd.c = y;
     gd.partial = partial; gd.status = status; gd.grid_bar = grid_bar;
-    gd.prefetch_blocks = prefetch_by(4);
     { int nl = launch_gemm(gd, st); if (nl < 0) return check_cuda(c, "down projection") == ACACHE_OK ? fail(c, ACACHE_ERR_CUDA, "down projection launch failed") : ACACHE_ERR_CUDA;
     c->launches += nl; }
     mark(c, ACACHE_N_STAGES, st);
@@ -645,7 +627,6 @@ acache_status layer_step_impl(acache_ctx* ctx, const acache_layer_weights* w, co
                 g.head_dim = d.head_dim; g.rope_segments = 1; g.out[0] = qmask; g.rows_per_req = req->n_masked;
                 g.partial = wsp<float>(ctx, ctx->o_gemm); g.status = wsp<uint32_t>(ctx, ctx->o_status);
                 g.grid_bar = wsp<unsigned int>(ctx, ctx->o_gridbar);
-                g.prefetch_blocks = prefetch_by(0);
                 { int nl = launch_gemm(g, stream); if (nl < 0) return check_cuda(ctx, "masked-row query projection") == ACACHE_OK ? fail(ctx, ACACHE_ERR_CUDA, "masked-row query projection launch failed") : ACACHE_ERR_CUDA;
                 ctx->launches += nl; }
             }

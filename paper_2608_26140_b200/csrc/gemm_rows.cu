@@ -1,0 +1,524 @@
+// Projections of few rows (C[M, N] = A[M, K] B[N, K]^T with M <= 128) as one launch without partial tiles in global memory.
+//
+// At these sizes the weights' stream from HBM is the floor and everything around it is latency.  The general one-SM kernel
+// (gemm_tc.cu) cuts (tile, K block) ranges so that every SM streams the same bytes, and pays with fp32 partial tiles through
+// L2 and a finish kernel behind every projection.  Here a tile of TN weight rows (TN chosen from N, not fixed) belongs to
+// one CTA or to a cluster of S = 2 or 4 CTAs that split K; the cluster's partial accumulators meet in distributed shared
+// memory, every CTA finishing its share of the columns, and the epilogue follows in the same kernel.
+//
+// A ring stage holds CP panels of 64 K columns, loaded by one TMA instruction per operand box (3-d and 4-d tensor maps: the
+// panel is a dimension of the box), so that a stage's fixed cost of waits and issue is shared by more bytes.
+//
+// Roles of the 256 threads: warp 0 TMA producer, warp 1 tcgen05.mma issuer, then all eight warps the epilogue (warp = TMEM
+// lane quarter x column half).  All eight take part in the row preparation before (prep_phase).  Every wait on an mbarrier
+// or the grid barrier is bounded as in gemm_tc.cu; the cluster barriers are passed by every CTA whatever happened before.
+#include <algorithm>
+
+#include "common.cuh"
+#include "gemm_common.cuh"
+#include "kernels.h"
+#include "launch.h"
+#include "tc_ptx.cuh"
+
+namespace acache {
+
+constexpr int RW_THREADS = 256;
+constexpr int RW_MAX_STAGES = 16;
+constexpr int RW_MAX_UNITS = 4;
+
+struct RowsPlan {
+    int TN, n_tiles;
+    int CP, blocks;           // K panels (64 columns) per ring stage, stages' worth of K in all
+    int S;                    // CTAs per tile, splitting K
+    int rows_pad;             // M rounded up to 8: rows of an A panel
+    int R, n_units;           // weight rows per box, boxes per stage
+    int mma_n, mma_count;     // columns per instruction, instructions per 16 K columns (one panel: the boxes lie side by side)
+    int stages, stage_bytes;
+    int tmem_cols;
+    int groups;               // q/k/v: groups of 32 rotary pairs over all segments
+    int smem_bytes;
+};
+
+__device__ __forceinline__ void tc_ld16(uint32_t taddr, float (&v)[16]) {
+    uint32_t r[16];
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
+        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+        : "r"(taddr)
+        : "memory");
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+    for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
+}
+__device__ __forceinline__ void tc_ld8x2(uint32_t ta, uint32_t tb, float (&a)[8], float (&b)[8]) {
+    uint32_t r[16];
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+                 : "r"(ta)
+                 : "memory");
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+                 : "r"(tb)
+                 : "memory");
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+    for (int i = 0; i < 8; ++i) { a[i] = __uint_as_float(r[i]); b[i] = __uint_as_float(r[8 + i]); }
+}
+__device__ __forceinline__ float4 ld_cluster_f4(uint32_t cluster_addr) {
+    float4 v;
+    asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
+                 : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+                 : "r"(cluster_addr)
+                 : "memory");
+    return v;
+}
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+__device__ __forceinline__ void prefetch_l1(const void* p) { asm volatile("prefetch.global.L1 [%0];" ::"l"(p)); }
+__device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map, int c1, int c2, uint32_t bar, uint64_t policy) {
+    asm volatile(
+        "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint "
+        "[%0], [%1, {%2, %3, %4}], [%5], %6;"
+        ::"r"(dst), "l"(map), "r"(0), "r"(c1), "r"(c2), "r"(bar), "l"(policy)
+        : "memory");
+}
+__device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap* map, int c1, int c2, int c3, uint32_t bar, uint64_t policy) {
+    asm volatile(
+        "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint "
+        "[%0], [%1, {%2, %3, %4, %5}], [%6], %7;"
+        ::"r"(dst), "l"(map), "r"(0), "r"(c1), "r"(c2), "r"(c3), "r"(bar), "l"(policy)
+        : "memory");
+}
+
+// q/k/v: segment of the grp-th group of 32 rotary pairs, row of its first pair inside the segment (the partners sit
+// head_dim / 2 rows further).
+__device__ __forceinline__ int pair_group(const GemmArgs& g, int grp, int& row) {
+    int r = g.head_dim == 128 ? (grp >> 1) * 128 + (grp & 1) * 32 : grp * 64;
+    int seg = 0;
+    while (seg < 2 && r >= g.n[seg]) { r -= g.n[seg]; ++seg; }
+    row = r;
+    return seg;
+}
+
+// The boxes of weight rows of tile `nt`.  q/k/v: a box is the two halves of a group, 32 rows each (past the last group the
+// last one is loaded again and ignored); SwiGLU: gate rows, then as many up rows; residual: the tile's rows.  Rows past a
+// matrix's end read as zero.
+template <int EPI>
+struct WeightBoxes {
+    int seg[RW_MAX_UNITS], row[RW_MAX_UNITS];
+    __device__ __forceinline__ WeightBoxes(const GemmArgs& g, const RowsPlan& p, int nt) {
+#pragma unroll
+        for (int u = 0; u < RW_MAX_UNITS; ++u) {
+            if (EPI == kEpiQKV) seg[u] = pair_group(g, min(nt * p.n_units + u, p.groups - 1), row[u]);
+            else { seg[u] = EPI == kEpiSwiGLU ? u : 0; row[u] = nt * p.R; }
+        }
+    }
+};
+
+// 16 adjacent accumulator columns of this thread's row, summed over the cluster: own tensor memory first, then the peers in
+// rank order (fixed, hence bitwise reproducible).  slice_col: the columns' place inside the slice this CTA finishes;
+// peers: where it lies in each peer's staging area (cluster addresses).
+template <int S>
+__device__ __forceinline__ void sum_cluster16(uint32_t taddr, const uint32_t (&peers)[S > 1 ? S - 1 : 1], int slice_col, int rows_pad,
+                                              int row, float (&v)[16]) {
+    float4 t[S > 1 ? S - 1 : 1][4];
+    if (S > 1) {
+        const int r = min(row, rows_pad - 1);
+#pragma unroll
+        for (int i = 0; i < S - 1; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) t[i][j] = ld_cluster_f4(peers[i] + ((((slice_col >> 2) + j) * rows_pad + r) << 4));
+    }
+    tc_ld16(taddr, v);
+    if (S > 1) {
+#pragma unroll
+        for (int i = 0; i < S - 1; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                v[4 * j] += t[i][j].x; v[4 * j + 1] += t[i][j].y; v[4 * j + 2] += t[i][j].z; v[4 * j + 3] += t[i][j].w;
+            }
+    }
+}
+
+template <int S, int EPI>
+__global__ void __launch_bounds__(RW_THREADS, 1)
+gemm_rows_kernel(const GemmArgs g, const RowsPlan p, const __grid_constant__ CUtensorMap mapA,
+                 const __grid_constant__ CUtensorMap mapB0, const __grid_constant__ CUtensorMap mapB1,
+                 const __grid_constant__ CUtensorMap mapB2) {
+    extern __shared__ unsigned char smem_raw[];
+    __shared__ uint64_t bar_s[2 * RW_MAX_STAGES + 1];
+    __shared__ uint32_t tmem_slot;
+    __shared__ volatile int abort_s;
+    __shared__ float red[RW_THREADS / 32];
+    const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
+    volatile int* abort_flag = &abort_s;
+    const uint32_t bars = smem_u32(bar_s);
+    auto full_bar = [&](int s) { return bars + 8 * s; };
+    auto empty_bar = [&](int s) { return bars + 8 * (RW_MAX_STAGES + s); };
+    const uint32_t done_bar = bars + 8 * 2 * RW_MAX_STAGES;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int rank = S > 1 ? (int)cluster_ctarank() : 0;
+    const int nt = blockIdx.x / S;
+    const int blk0 = rank * p.blocks / S, blk1 = (rank + 1) * p.blocks / S;
+    const int n_blk = blk1 - blk0;
+    unsigned int nbar = 0;
+
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < p.stages; ++s) { mbar_init(full_bar(s), 1); mbar_init(empty_bar(s), 1); }
+        mbar_init(done_bar, 1);
+        *abort_flag = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    // The weights are constant inputs: the ring's weight halves are requested before the previous kernel has finished; the
+    // activation rows follow once they are there.
+    const uint64_t pol_a = policy_evict_last(), pol_w = g.keep_weights ? pol_a : policy_evict_first();
+    const uint32_t a_bytes = p.CP * p.rows_pad * 128, box_bytes = p.CP * p.R * 128;
+    const WeightBoxes<EPI> boxes(g, p, nt);
+    auto load_weights = [&](int stage, int blk) {
+        const uint32_t dst = base + stage * p.stage_bytes + a_bytes;
+#pragma unroll
+        for (int u = 0; u < RW_MAX_UNITS; ++u) {
+            if (u >= p.n_units) break;
+            const CUtensorMap* map = boxes.seg[u] == 0 ? &mapB0 : boxes.seg[u] == 1 ? &mapB1 : &mapB2;
+            if (EPI == kEpiQKV) {
+                const int half = g.head_dim >> 1;
+                const int h = boxes.row[u] / half;
+                tma_load_4d(dst + u * box_bytes, map, boxes.row[u] - h * half, h, blk * p.CP, full_bar(stage), pol_w);
+            } else {
+                tma_load_3d(dst + u * box_bytes, map, boxes.row[u], blk * p.CP, full_bar(stage), pol_w);
+            }
+        }
+    };
+    int prefilled = 0;
+    if (threadIdx.x == 0) {
+        for (; prefilled < p.stages && prefilled < n_blk; ++prefilled) {
+            mbar_expect_tx(full_bar(prefilled), p.stage_bytes);
+            load_weights(prefilled, blk0 + prefilled);
+        }
+    }
+    __syncwarp();
+    if (warp == 1) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
+                     ::"r"(smem_u32(&tmem_slot)), "r"(p.tmem_cols) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem_base = tmem_slot;
+    pdl_wait();
+    pdl_launch_dependents();
+
+    if (g.prep.enabled) prep_phase(g, red, abort_flag, nbar);
+
+    // ---------------- the contraction ----------------
+    if (threadIdx.x == 0) {
+        bool ok = !*abort_flag;
+        int stage = 0;
+        uint32_t phase = 0;
+        for (int i = 0; i < n_blk && ok; ++i) {
+            if (prefilled > 0) {
+                --prefilled;              // this stage's weights are already on their way
+            } else {
+                if (!(ok = mbar_wait(empty_bar(stage), phase ^ 1, abort_flag))) break;
+                mbar_expect_tx(full_bar(stage), p.stage_bytes);
+                load_weights(stage, blk0 + i);
+            }
+            tma_load_3d(base + stage * p.stage_bytes, &mapA, 0, (blk0 + i) * p.CP, full_bar(stage), pol_a);
+            if (++stage == p.stages) { stage = 0; phase ^= 1; }
+        }
+    } else if (threadIdx.x == 32) {
+        bool ok = !*abort_flag;
+        int stage = 0;
+        uint32_t phase = 0;
+        const uint32_t idesc = idesc_bf16(p.mma_n);
+        for (int i = 0; i < n_blk && ok; ++i) {
+            if (!(ok = mbar_wait(full_bar(stage), phase, abort_flag))) break;
+            tc_fence_after();
+            const uint32_t sA = base + stage * p.stage_bytes, sB = sA + a_bytes;
+            for (int c = 0; c < p.CP; ++c) {
+                const uint64_t da = smem_desc_sw128(sA + c * p.rows_pad * 128);
+                for (int u = 0; u < p.mma_count; ++u) {
+                    const uint64_t db = smem_desc_sw128(sB + u * box_bytes + c * p.R * 128);
+#pragma unroll
+                    for (int k = 0; k < 4; ++k)
+                        tc_mma(tmem_base + u * p.mma_n, da + (uint64_t)(k * 2), db + (uint64_t)(k * 2), idesc,
+                               (i > 0 || c > 0 || k > 0) ? 1u : 0u);
+                }
+            }
+            tc_commit(empty_bar(stage));
+            if (++stage == p.stages) { stage = 0; phase ^= 1; }
+        }
+        if (ok) tc_commit(done_bar);
+    }
+    __syncwarp();
+
+    // ---------------- epilogue: thread = one row, warp = lane quarter x column half ----------------
+    const int q = warp & 3, hf = warp >> 2, row = q * 32 + lane;
+    const bool live = q * 32 < p.rows_pad;                 // warp-uniform: the tensor-memory accesses are collective
+    const bool valid = row < g.M;
+    const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16);
+    // the columns this CTA finishes: items of 16 + 16 rotary pairs (q/k/v), of 16 columns (residual), of 8 + 8 (SwiGLU)
+    constexpr int UNIT = EPI == kEpiQKV ? 32 : 16;
+    const int items = p.TN / UNIT, item0 = rank * items / S, item1 = (rank + 1) * items / S;
+    const int region = (items + S - 1) / S * UNIT * p.rows_pad * 4;
+
+    // what does not depend on the sums is requested while the weights stream
+    int pos = 0;
+    uint4 res[2] = {make_uint4(0u, 0u, 0u, 0u), make_uint4(0u, 0u, 0u, 0u)};
+    const uint4* res_row = nullptr;
+    if (EPI == kEpiResidual && valid) {
+        const int64_t roff = g.resid_off ? __ldcg(g.resid_off + row) : (int64_t)row * g.n[0];
+        res_row = reinterpret_cast<const uint4*>(static_cast<const __nv_bfloat16*>(g.resid) + roff);
+        const int col = nt * p.TN + (item0 + hf) * UNIT;
+        if (item0 + hf < item1 && col < g.n[0]) { res[0] = __ldcg(res_row + (col >> 3)); res[1] = __ldcg(res_row + (col >> 3) + 1); }
+    }
+    if (EPI == kEpiQKV && valid) {
+        pos = __ldcg(g.row_pos + row);
+        if (g.rope_segments > 0) {
+            const int64_t at = (int64_t)(pos < 0 ? 0 : pos) * (g.head_dim >> 1);
+            for (int i = hf * 32; i < (g.head_dim >> 1); i += 64) { prefetch_l1(g.rope_cos + at + i); prefetch_l1(g.rope_sin + at + i); }
+        }
+    }
+
+    bool ok = !*abort_flag;
+    if (ok) ok = mbar_wait(done_bar, 0, abort_flag);
+    ok = __all_sync(0xffffffffu, ok);
+    tc_fence_after();
+    uint32_t peers[S > 1 ? S - 1 : 1] = {};
+    if (S > 1) {
+        // the other CTAs' slices to the staging area (the ring: every MMA that read it has completed), layout
+        // [destination][column / 4][row][4]
+        if (ok && live) {
+            int at = 0;
+            for (int d = 0; d < S; ++d) {
+                if (d == rank) continue;
+                const int u0 = d * items / S, u1 = (d + 1) * items / S;
+                for (int u = u0 + hf; u < u1; u += 2) {
+#pragma unroll
+                    for (int part = 0; part < UNIT / 16; ++part) {
+                        const int col = EPI == kEpiQKV ? (u >> 1) * 64 + (u & 1) * 16 + part * 32 : u * 16;
+                        float v[16];
+                        tc_ld16(taddr + col, v);
+                        const int sc = ((u - u0) * UNIT + part * 16) >> 2;
+                        if (row < p.rows_pad) {
+#pragma unroll
+                            for (int j = 0; j < 4; ++j)
+                                asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};"
+                                             ::"r"(base + at * region + (((sc + j) * p.rows_pad + row) << 4)), "f"(v[4 * j]),
+                                               "f"(v[4 * j + 1]), "f"(v[4 * j + 2]), "f"(v[4 * j + 3])
+                                             : "memory");
+                        }
+                    }
+                }
+                ++at;
+            }
+        }
+        __syncwarp();
+        cluster_arrive();
+        cluster_wait();
+#pragma unroll
+        for (int i = 0; i < S - 1; ++i) {
+            const int r = i < rank ? i : i + 1;            // peer; its staging area holds this CTA's slice at place ...
+            peers[i] = mapa_u32(base + (rank < r ? rank : rank - 1) * region, r);
+        }
+    }
+    if (ok && live) {
+        for (int u = item0 + hf; u < item1; u += 2) {
+            const int sc = (u - item0) * UNIT;
+            if (EPI == kEpiResidual) {
+                const int col = nt * p.TN + u * 16;
+                float v[16];
+                sum_cluster16<S>(taddr + u * 16, peers, sc, p.rows_pad, row, v);
+                if (valid && col < g.n[0]) {
+                    if (u != item0 + hf) { res[0] = __ldcg(res_row + (col >> 3)); res[1] = __ldcg(res_row + (col >> 3) + 1); }
+                    const uint32_t rw[8] = {res[0].x, res[0].y, res[0].z, res[0].w, res[1].x, res[1].y, res[1].z, res[1].w};
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) { v[2 * i] += bf16_lo(rw[i]); v[2 * i + 1] += bf16_hi(rw[i]); }
+                    store16(static_cast<__nv_bfloat16*>(g.c) + (int64_t)row * g.n[0] + col, v);
+                }
+            } else if (EPI == kEpiSwiGLU) {
+                const int col = nt * (p.TN >> 1) + u * 8;
+                float gate[8], up[8];
+                tc_ld8x2(taddr + u * 8, taddr + (p.TN >> 1) + u * 8, gate, up);
+                if (valid && col < g.n[0]) {
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) gate[i] = silu(gate[i]) * up[i];
+                    *reinterpret_cast<uint4*>(static_cast<__nv_bfloat16*>(g.c) + (int64_t)row * g.n[0] + col) = pack8(gate);
+                }
+            } else {
+                const int grp = nt * p.n_units + (u >> 1);
+                int col;
+                const int seg = pair_group(g, min(grp, p.groups - 1), col);
+                col += (u & 1) * 16;
+                float lo[16], hi[16], c[16], sn[16];
+                if (valid && seg < g.rope_segments) load_rope<16>(g, pos, col & ((g.head_dim >> 1) - 1), c, sn);
+                sum_cluster16<S>(taddr + (u >> 1) * 64 + (u & 1) * 16, peers, sc, p.rows_pad, row, lo);
+                sum_cluster16<S>(taddr + (u >> 1) * 64 + (u & 1) * 16 + 32, peers, sc + 16, p.rows_pad, row, hi);
+                if (valid && grp < p.groups) {
+                    rope_qkv<16>(g, seg, col, lo, hi, c, sn);
+                    store_qkv<16>(g, row, pos, seg, col, lo, hi);
+                }
+            }
+        }
+    }
+    // ---------------- teardown ----------------
+    tc_fence_before();
+    __syncthreads();
+    if (*abort_flag) {
+        if (threadIdx.x == 0) {
+            atomicOr(g.status, kFlagWaitExpired);
+            // ring stages whose weights were requested before the dependency wait but whose activation rows never were:
+            // send those now, so that each stage's full barrier completes when all of its copies have landed
+            for (int i = 0; i < prefilled; ++i) tma_load_3d(base + i * p.stage_bytes, &mapA, 0, 0, full_bar(i), pol_a);
+            for (int i = 0; i < prefilled; ++i)
+                for (uint32_t n = 0; n < TC_WAIT_LIMIT && !mbar_try_wait(full_bar(i), 0); ++n) __nanosleep(40);
+            for (int i = 0; i < 4096; ++i) __nanosleep(64);   // copies of stages that were complete when a role gave up
+        }
+        __syncthreads();
+    } else if (threadIdx.x == 0 && nbar > 0) {
+        // the last CTA to leave re-arms the barrier words for the next launch
+        __threadfence();
+        if (atomicAdd(&g.grid_bar[1], 1u) == gridDim.x - 1) {
+            g.grid_bar[0] = 0u;
+            __threadfence();
+            g.grid_bar[1] = 0u;
+        }
+    }
+    __syncwarp();
+    if (S > 1) { cluster_arrive(); cluster_wait(); }          // no CTA leaves while a peer may still read its staging area
+    if (warp == 1) {
+        tc_fence_after();
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(p.tmem_cols) : "memory");
+    }
+}
+
+// ---- host side ------------------------------------------------------------------------------
+namespace {
+
+template <int S, int EPI>
+cudaError_t launch_rows(const GemmArgs& g, const RowsPlan& p, const CUtensorMap& a, const CUtensorMap* b, cudaStream_t stream) {
+    static const cudaError_t attr =
+        cudaFuncSetAttribute(gemm_rows_kernel<S, EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024);
+    if (attr != cudaSuccess) return attr;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(p.n_tiles * S);
+    cfg.blockDim = dim3(RW_THREADS);
+    cfg.dynamicSmemBytes = p.smem_bytes;
+    cfg.stream = stream;
+    cudaLaunchAttribute at[2];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    at[1].id = cudaLaunchAttributeClusterDimension;
+    at[1].val.clusterDim.x = S; at[1].val.clusterDim.y = 1; at[1].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = S > 1 ? 2 : 1;
+    return cudaLaunchKernelEx(&cfg, gemm_rows_kernel<S, EPI>, g, p, a, b[0], b[1], b[2]);
+}
+
+// Clusters of S CTAs that are resident at once with one CTA per SM (the SM counts of the GPCs are not multiples of S).
+template <int S>
+int resident_clusters() {
+    static const int n = [] {
+        if (S == 1) return sm_count();
+        cudaFuncSetAttribute(gemm_rows_kernel<S, kEpiResidual>, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024);
+        cudaLaunchConfig_t cfg{};
+        cfg.gridDim = dim3(sm_count() / S * S);
+        cfg.blockDim = dim3(RW_THREADS);
+        cfg.dynamicSmemBytes = 200 * 1024;
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = S; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+        cfg.attrs = at;
+        cfg.numAttrs = 1;
+        int c = 0;
+        if (cudaOccupancyMaxActiveClusters(&c, gemm_rows_kernel<S, kEpiResidual>, &cfg) != cudaSuccess) { (void)cudaGetLastError(); c = 0; }
+        return c;
+    }();
+    return n;
+}
+
+// Tile width and K split: the least estimated time of one wave.  The weights cannot stream faster than HBM delivers them
+// (6.5 TB/s); a CTA not faster than about 60 GB/s (its weight rows and, once per tile, all rows of A; measured 45-60 with
+// this ring); a split costs an exchange per doubling, 1.5 us where rotary pairs are finished and 1 us otherwise.  A stage
+// takes as many panels as leave three stages in the ring (fewer, larger stages lost, two stages of any size did too).
+// Measured at 103 rows (us per launch, finish included | here): q/k/v 30.2 | 29.6, output 16.3 | 13.0, gate/up 47.7 | 43,
+// down 25.7 | 23.4; at 32 rows output 14.3 | 10.9, down 25.0 | 20.4, masked rows' queries 20.6 | 18.8.
+constexpr int kRingBytes = 200 * 1024;
+bool plan_rows(const GemmArgs& g, RowsPlan& best) {
+    if (g.M > 128 || g.epilogue == kEpiLogits || g.K < 64) return false;
+    const bool qkv = g.epilogue == kEpiQKV, swiglu = g.epilogue == kEpiSwiGLU;
+    const int n_total = swiglu ? 2 * g.n[0] : g.n[0] + g.n[1] + g.n[2];
+    const int KB = g.K / 64, rows_pad = (g.M + 7) & ~7;
+    const int step = qkv ? 64 : swiglu ? 16 : 32;
+    const int limit[3] = {resident_clusters<1>(), resident_clusters<2>(), resident_clusters<4>()};
+    double t_best = 1e30;
+    for (int si = 0; si < (swiglu ? 1 : 3); ++si) {
+        const int S = 1 << si;
+        for (int TN = step; TN <= 256; TN += step) {
+            const int items = TN / (qkv ? 32 : 16);
+            const int n_tiles = (n_total + TN - 1) / TN;
+            if (items < S || n_tiles > limit[si]) continue;
+            const int panel = (rows_pad + TN) * 128;
+            int CP = 1;         // an instruction spans 16 columns' multiples: half a SwiGLU tile has to be one to take more panels
+            while (CP < 8 && (!swiglu || TN % 32 == 0) && 2 * CP * 3 * panel <= kRingBytes && 2 * CP * S <= KB) CP *= 2;
+            const int blocks = (KB + CP - 1) / CP;
+            if (blocks < S) continue;
+            const int my_blocks = (blocks + S - 1) / S;
+            const int stages = std::min(std::min(kRingBytes / (CP * panel), RW_MAX_STAGES), my_blocks);
+            const int region = (items + S - 1) / S * (qkv ? 32 : 16) * rows_pad * 4;
+            const double t_hbm = 2.0 * n_total * g.K / 6.5e6, t_sm = (double)my_blocks * CP * panel / 60e3;
+            const double t = std::max(std::max(t_hbm, t_sm), my_blocks * 0.15) + si * (qkv ? 1.5 : 1.0);
+            if (t >= t_best * 0.999) continue;
+            t_best = t;
+            best = RowsPlan{};
+            best.TN = TN; best.n_tiles = n_tiles; best.CP = CP; best.blocks = blocks; best.S = S; best.rows_pad = rows_pad;
+            best.R = qkv ? 64 : swiglu ? TN / 2 : TN;
+            best.n_units = TN / best.R;
+            best.mma_n = CP == 1 ? TN : best.R;
+            best.mma_count = CP == 1 ? 1 : best.n_units;
+            best.stages = stages; best.stage_bytes = CP * panel;
+            best.tmem_cols = TN <= 32 ? 32 : TN <= 64 ? 64 : TN <= 128 ? 128 : 256;
+            best.groups = n_total / 64;
+            // the MMA reads 128 rows of A whatever M is: the last panel's read may run past the ring
+            const int ring = std::max(stages * CP * panel, (stages - 1) * CP * panel + (CP - 1) * rows_pad * 128 + 128 * 128);
+            best.smem_bytes = std::max(ring, (S - 1) * region) + 1024;
+        }
+    }
+    return t_best < 1e29;
+}
+
+}  // namespace
+
+int launch_gemm_rows(const GemmArgs& g, cudaStream_t stream) {
+    RowsPlan p;
+    if (!plan_rows(g, p)) return 0;
+    CUtensorMap map_a, map_b[3];
+    {
+        std::lock_guard<std::mutex> lock(g_map_mutex);
+        const CUtensorMap* m = get_panel_map(g.a, g.M, g.K, p.rows_pad, p.CP, 0);
+        if (!m) return -1;
+        map_a = *m;
+        const bool qkv = g.epilogue == kEpiQKV;
+        for (int i = 0; i < 3; ++i) {
+            if (!g.b[i]) { if (i == 0) return -1; map_b[i] = map_b[0]; continue; }
+            if (!(m = get_panel_map(g.b[i], g.n[i], g.K, qkv ? 32 : p.R, p.CP, qkv ? g.head_dim / 2 : 0))) return -1;
+            map_b[i] = *m;
+        }
+    }
+    cudaError_t e = cudaErrorInvalidValue;
+    if (g.epilogue == kEpiSwiGLU) e = launch_rows<1, kEpiSwiGLU>(g, p, map_a, map_b, stream);
+    else if (g.epilogue == kEpiResidual)
+        e = p.S == 1 ? launch_rows<1, kEpiResidual>(g, p, map_a, map_b, stream)
+          : p.S == 2 ? launch_rows<2, kEpiResidual>(g, p, map_a, map_b, stream)
+                     : launch_rows<4, kEpiResidual>(g, p, map_a, map_b, stream);
+    else
+        e = p.S == 1 ? launch_rows<1, kEpiQKV>(g, p, map_a, map_b, stream)
+          : p.S == 2 ? launch_rows<2, kEpiQKV>(g, p, map_a, map_b, stream)
+                     : launch_rows<4, kEpiQKV>(g, p, map_a, map_b, stream);
+    return e == cudaSuccess ? 1 : -1;
+}
+
+}  // namespace acache

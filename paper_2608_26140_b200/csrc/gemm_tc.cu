@@ -1,6 +1,9 @@
 // C[M, N] = A[M, K] * B[N, K]^T (bf16 in, fp32 accumulate) on the 5th-generation tensor
 // cores for the projections of the selective recomputation (Section 3.3).
 //
+// Projections of at most 128 rows run on gemm_rows.cu where their tiles fit the SMs at once; here, the rest of them (the LM
+// head, very wide ones) and everything above.
+//
 // gemm_tc_kernel (at most one CTA per SM):
 //   phase 0 (optional)  gather the rows of R (or take compact rows) and RMSNorm them into the
 //                       A operand, then a grid-wide barrier
@@ -33,6 +36,7 @@
 #include <mutex>
 
 #include "common.cuh"
+#include "gemm_common.cuh"
 #include "kernels.h"
 #include "launch.h"
 #include "rows.cuh"
@@ -47,11 +51,9 @@ constexpr int TC_STAGE_BYTES = TC_A_BYTES + 2 * TC_HALF_BYTES;
 constexpr int TC_THREADS = 192;                        // warp 0: TMA, warp 1: MMA, warps 2-5: drain; all six warps do phase 0
 constexpr int TC_SMEM = TC_STAGES * TC_STAGE_BYTES + 1024 /*alignment slack*/ + 256 /*barriers*/;
 constexpr int TC_SLOT_FLOATS = TC_BM * TC_BN;          // one fp32 partial tile
-constexpr uint32_t GRID_WAIT_LIMIT = 1u << 21;
 
 struct TcPlan {
     int m_tiles, n_tiles, KB, tiles, U, ctas, smax;
-    int prefetch;         // K blocks past the ring whose weight tiles are requested into L2 before the dependency wait
     int prefill;          // ring stages whose weight halves are loaded before the dependency wait
     int pair_u;           // two-SM kernel, stream-K mode: (pair tile, K block) iterations per cluster (0: whole tiles)
     int m_pairs;          // 256-row tile rows of the two-SM kernel
@@ -73,150 +75,6 @@ __device__ __forceinline__ int half_source(const GemmArgs& g, const TcPlan& p, i
     while (seg < 2 && r >= g.n[seg]) { r -= g.n[seg]; ++seg; }
     row = r;
     return seg;
-}
-
-// Grid-wide barrier number `k` (1, 2, ...) of this launch on a pair of counters in global
-// memory: arrivals only ever add to bar[0], so barrier k is passed at k * gridDim.x.  Bounded;
-// returns false (and raises the CTA's abort flag) if the others do not arrive.
-// self_test: the failure-detection self-test (acache_debug_expire_next_wait): the target is one arrival more than
-// the grid can deliver and the poll limit is short, so the wait runs out and the abort path below is taken.
-__device__ __forceinline__ bool grid_barrier(unsigned int* bar, unsigned int k, volatile int* abort_flag, bool self_test = false) {
-    __syncthreads();
-    if (threadIdx.x == 0 && !*abort_flag) {
-        __threadfence();
-        atomicAdd(&bar[0], 1u);
-        const unsigned int target = k * gridDim.x + (self_test ? 1u : 0u);
-        const uint32_t limit = self_test ? (1u << 12) : GRID_WAIT_LIMIT;
-        bool ok = false;
-        for (uint32_t i = 0; i < limit; ++i) {
-            unsigned int v;
-            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(bar) : "memory");
-            if (v >= target) { ok = true; break; }
-            __nanosleep(i < 64 ? 20 : 100);
-        }
-        if (!ok) *abort_flag = 1;
-        __threadfence();
-    }
-    __syncthreads();
-    return !*abort_flag;
-}
-
-__device__ __forceinline__ uint4 pack8(const float* v) {
-    return make_uint4(pack_bf16(v[0], v[1]), pack_bf16(v[2], v[3]), pack_bf16(v[4], v[5]), pack_bf16(v[6], v[7]));
-}
-
-// 16 bf16 of one row: one 32-byte store (a whole sector per lane) where the address allows it.
-__device__ __forceinline__ void store16(__nv_bfloat16* o, const float* v) {
-    uint32_t w[8];
-#pragma unroll
-    for (int i = 0; i < 8; ++i) w[i] = pack_bf16(v[2 * i], v[2 * i + 1]);
-    if ((reinterpret_cast<uintptr_t>(o) & 31u) == 0) {
-        asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};"
-                     ::"l"(o), "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3]), "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7])
-                     : "memory");
-    } else {
-        reinterpret_cast<uint4*>(o)[0] = make_uint4(w[0], w[1], w[2], w[3]);
-        reinterpret_cast<uint4*>(o)[1] = make_uint4(w[4], w[5], w[6], w[7]);
-    }
-}
-
-// ---- epilogues on W adjacent fp32 accumulator columns of one row (W = 16 or 32) ----------------
-// Every store is W*2 bytes of one row: whole 32-byte sectors, no partial-sector writes.
-
-// x / (1 + exp(-x)).  The quotient is an approximate reciprocal with one Newton step and one correction by the remainder
-// (Newton-Raphson division): as accurate as the division operator to the last bit or two, but without its check for
-// special operands, whose branch kept a thread from working on more than one element at a time (one warp per scheduler: a
-// 256-column tile's SwiGLU took 10 us).  The divisor is kept finite; below
-// x = -87.3 the result is 0 (the true value is under 1e-36 there).  Epilogue of a 128 x 256 tile: 10 -> 4.5 us, of the last
-// one, which nothing hides, 9.5 -> 3.4.
-__device__ __forceinline__ float silu(float x) {
-    const float d = fminf(1.f + __expf(-x), 3e38f);
-    float r = __fdividef(1.f, d);
-    r = fmaf(fmaf(-d, r, 1.f), r, r);
-    const float q = x * r;
-    return fmaf(fmaf(-q, d, x), r, q);
-}
-
-// out[grow, col..col+W) = bf16(silu(gate) * up)
-template <int W>
-__device__ __forceinline__ void out_swiglu(const GemmArgs& g, int grow, int col, float (&gate)[W], const float (&up)[W]) {
-    __nv_bfloat16* o = static_cast<__nv_bfloat16*>(g.c) + (int64_t)grow * g.n[0] + col;
-#pragma unroll
-    for (int i = 0; i < W; ++i) gate[i] = silu(gate[i]) * up[i];
-#pragma unroll
-    for (int j = 0; j < W / 16; ++j) store16(o + 16 * j, gate + 16 * j);
-}
-
-// cos and sin of the row's position for W pairs from j0 on.
-template <int W>
-__device__ __forceinline__ void load_rope(const GemmArgs& g, int pos, int j0, float (&c)[W], float (&sn)[W]) {
-    const int64_t at = (int64_t)(pos < 0 ? 0 : pos) * (g.head_dim >> 1) + j0;
-    const float4* c4 = reinterpret_cast<const float4*>(g.rope_cos + at);
-    const float4* s4 = reinterpret_cast<const float4*>(g.rope_sin + at);
-#pragma unroll
-    for (int j = 0; j < W / 4; ++j) {
-        const float4 x = c4[j], y = s4[j];
-        c[4 * j] = x.x; c[4 * j + 1] = x.y; c[4 * j + 2] = x.z; c[4 * j + 3] = x.w;
-        sn[4 * j] = y.x; sn[4 * j + 1] = y.y; sn[4 * j + 2] = y.z; sn[4 * j + 3] = y.w;
-    }
-}
-
-// q/k/v: bias, rotary embedding with the pairing (i, i + d/2) at the row's position, bf16 store
-// to the compact output and, for k/v, straight into the cache row (scatter fused).
-// lo/hi: W columns of each rotary half; col: column of lo[0] inside segment seg; c/sn: load_rope (rotary segments).
-template <int W>
-__device__ __forceinline__ void rope_qkv(const GemmArgs& g, int seg, int col, float (&lo)[W], float (&hi)[W], const float (&c)[W],
-                                         const float (&sn)[W]) {
-    const int half = g.head_dim >> 1;
-    const __nv_bfloat16* bias = static_cast<const __nv_bfloat16*>(g.bias[seg]);
-    if (bias) {
-#pragma unroll
-        for (int i = 0; i < W; ++i) {
-            lo[i] += __bfloat162float(bias[col + i]);
-            hi[i] += __bfloat162float(bias[col + half + i]);
-        }
-    }
-    if (seg < g.rope_segments) {
-#pragma unroll
-        for (int i = 0; i < W; ++i) {
-            const float x = lo[i], y = hi[i];
-            lo[i] = x * c[i] - y * sn[i];
-            hi[i] = y * c[i] + x * sn[i];
-        }
-    }
-}
-template <int W>
-__device__ __forceinline__ void store_qkv(const GemmArgs& g, int grow, int pos, int seg, int col, const float (&lo)[W],
-                                          const float (&hi)[W]) {
-    const int half = g.head_dim >> 1;
-    const int nseg = g.n[seg];
-    __nv_bfloat16* cache = seg == 1 ? static_cast<__nv_bfloat16*>(g.cache_k)
-                         : seg == 2 ? static_cast<__nv_bfloat16*>(g.cache_v) : nullptr;
-    int64_t orow = grow;
-    bool o1_ok = g.out[seg] != nullptr;
-    if (seg >= 1 && g.kv_out_rows && o1_ok) {          // the row's place in its request's private slot array
-        const int r = __ldg(g.kv_out_rows + grow);
-        if ((unsigned)r >= (unsigned)g.kv_out_stride) {
-            atomicOr(g.status, kFlagBadIndex);
-            o1_ok = false;
-        }
-        orow = (int64_t)(grow / g.rows_per_req) * g.kv_out_stride + r;
-    }
-    __nv_bfloat16* o1 = o1_ok ? static_cast<__nv_bfloat16*>(g.out[seg]) + orow * nseg + col : nullptr;
-    __nv_bfloat16* o2 = (cache && pos >= 0)
-                            ? cache + (int64_t)(grow / g.rows_per_req) * g.kv_batch_stride + (int64_t)pos * nseg + col
-                            : nullptr;
-#pragma unroll
-    for (int j = 0; j < W / 16; ++j) {
-        if (o1) { store16(o1 + 16 * j, lo + 16 * j); store16(o1 + half + 16 * j, hi + 16 * j); }
-        if (o2) { store16(o2 + 16 * j, lo + 16 * j); store16(o2 + half + 16 * j, hi + 16 * j); }
-    }
-}
-
-// Segment and in-segment column of the 128-wide column unit u128 of a q/k/v projection.
-__device__ __forceinline__ void qkv_unit(const GemmArgs& g, int u128, int& seg, int& c0) {
-    seg = 0; c0 = u128 * 128;
-    while (seg < 2 && c0 >= g.n[seg]) { c0 -= g.n[seg]; ++seg; }
 }
 
 // ---- split tiles: partial slots and their ordered sum -------------------------------------------
@@ -249,11 +107,11 @@ __device__ __forceinline__ int64_t slot_of(const TcPlan& p, int t, int c) {
 // starting at column group pc0 and, if pc1 >= 0, 16 more starting at pc1.  Loads are issued two
 // CTAs at a time for all eight column groups (16 independent 16-byte loads in flight per thread)
 // and added in ascending CTA order, which keeps the result bitwise reproducible.
-template <int NC>      // contributing CTAs per round of loads: 2, or 4 where the kernel may use 255 registers
 __device__ __forceinline__ void sum_slots16(const float* __restrict__ partial, const TcPlan& p, int t, int c_first,
                                             int c_last, int pc0, int pc1, int row, float (&lo)[16], float (&hi)[16]) {
 #pragma unroll
     for (int i = 0; i < 16; ++i) { lo[i] = 0.f; hi[i] = 0.f; }
+    constexpr int NC = 2;      // contributing CTAs per round of loads
     const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
     const int o0 = pc0 * TC_BM + row, o1 = (pc1 < 0 ? pc0 : pc1) * TC_BM + row;
     for (int c = c_first; c <= c_last; c += NC) {
@@ -377,7 +235,6 @@ __device__ __forceinline__ FinishItem finish_plan(const GemmArgs& g, const TcPla
 }
 
 // res: the residual, loaded by the caller (kEpiResidual only).
-template <int NC>
 __device__ __forceinline__ void finish_item(const GemmArgs& g, const TcPlan& p, int t, int item, int row, const FinishItem& f,
                                             const uint4 (&res)[2]) {
     if (f.skip) return;
@@ -388,7 +245,7 @@ __device__ __forceinline__ void finish_item(const GemmArgs& g, const TcPlan& p, 
     if (g.epilogue == kEpiQKV) pos = __ldcg(g.row_pos + grow);     // independent of the sums: overlaps their loads
     float lo[16], hi[16];
     if (pc1 < 0) sum_slots16_single(g.partial, p, t, c_first, c_last, pc0, row, lo);
-    else sum_slots16<NC>(g.partial, p, t, c_first, c_last, pc0, pc1, row, lo, hi);
+    else sum_slots16(g.partial, p, t, c_first, c_last, pc0, pc1, row, lo, hi);
     if (g.epilogue == kEpiResidual) {
         const uint32_t rw[8] = {res[0].x, res[0].y, res[0].z, res[0].w, res[1].x, res[1].y, res[1].z, res[1].w};
 #pragma unroll
@@ -497,176 +354,6 @@ __device__ __forceinline__ void half_epilogue(const GemmArgs& g, const TcPlan& p
     }
 }
 
-// Where row `row` of the A operand comes from (element offset inside rp.x); `writer` (one thread per
-// row) records the row's position and source for the later kernels and raises the bad-index flag.
-__device__ __forceinline__ int64_t prep_row_source(const GemmArgs& g, int row, bool writer) {
-    const RowPrep& rp = g.prep;
-    const int rows_per_req = rp.k + rp.e;
-    int64_t src = (int64_t)row * g.K;
-    if (rp.enabled == 3) {       // compact rows picked by index
-        const int b = row / rows_per_req;
-        const int ci = rp.compact_idx[row];
-        if (ci < 0 || ci >= rp.compact_rows) {
-            if (writer) atomicOr(g.status, kFlagBadIndex);
-        }
-        src = ((int64_t)b * rp.compact_rows + (ci < 0 || ci >= rp.compact_rows ? 0 : ci)) * g.K;
-    }
-    if (rp.enabled == 1) {       // rows of R: position from the anchor / extra-row lists
-        const int b = row / rows_per_req, i = row - b * rows_per_req;
-        const int pos = row_position(rp.anchor_idx, rp.k, rp.extra_rows, rp.e, b, i, rp.affix_start,
-                                     rp.affix_len, rp.ctx_len);
-        if (!rp.x_is_compact) {
-            if (rp.token_ids) {       // x is an embedding table: the row of the token at that position
-                int id = rp.token_ids[(int64_t)b * rp.ctx_len + (pos < 0 ? 0 : pos)];
-                if (id < 0 || id >= rp.table_rows) {
-                    if (writer) atomicOr(g.status, kFlagBadIndex);
-                    id = 0;
-                }
-                src = (int64_t)id * g.K;
-            } else {
-                src = (int64_t)b * rp.x_batch_stride + (int64_t)(pos < 0 ? 0 : pos) * g.K;
-            }
-        } else if (rp.compact_idx) {
-            const int ci = rp.compact_idx[row];
-            src = ((int64_t)b * rp.compact_rows + (ci < 0 ? 0 : ci)) * g.K;
-        }
-        if (writer) {
-            rp.row_pos[row] = pos;
-            rp.row_src[row] = src;
-            if (pos < 0) atomicOr(g.status, kFlagBadIndex);
-        }
-    }
-    return src;
-}
-
-// out = bf16(x * rsqrt(mean(x^2) + eps) * g) for one row, by one warp: rows of up to 4096 values in one pass from
-// registers; longer ones in two passes with eight independent 16-byte loads in flight per lane (the second pass hits
-// L1 / L2).
-__device__ __forceinline__ void rmsnorm_row_warp(const uint4* __restrict__ xr, const uint4* __restrict__ gn,
-                                                 uint4* __restrict__ out, int hidden, float eps, int lane,
-                                                 uint4* __restrict__ raw) {
-    const int nchunk = hidden >> 3;
-    if (nchunk <= 512) {
-        // rows of up to 4096 values: one pass, the row stays in registers (sixteen 16-byte loads in flight per lane,
-        // one trip to memory per row instead of two), the gain is requested before the warp-wide sum
-        uint4 u[16];
-        float s1 = 0.f;
-#pragma unroll
-        for (int i = 0; i < 16; ++i) {
-            const int c = i * 32 + lane;
-            u[i] = c < nchunk ? __ldcg(xr + c) : make_uint4(0, 0, 0, 0);
-        }
-        if (raw) {
-#pragma unroll
-            for (int i = 0; i < 16; ++i) {
-                const int c = i * 32 + lane;
-                if (c < nchunk) raw[c] = u[i];
-            }
-        }
-#pragma unroll
-        for (int i = 0; i < 16; ++i) {
-            const uint32_t w[4] = {u[i].x, u[i].y, u[i].z, u[i].w};
-#pragma unroll
-            for (int e = 0; e < 4; ++e) { const float a = bf16_lo(w[e]), b = bf16_hi(w[e]); s1 += a * a + b * b; }
-        }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) s1 += __shfl_xor_sync(0xffffffffu, s1, o);
-        const float rstd1 = rsqrtf(s1 / (float)hidden + eps);
-#pragma unroll
-        for (int i = 0; i < 16; ++i) {
-            const int c = i * 32 + lane;
-            if (c < nchunk) {
-                const uint4 gg = __ldg(gn + c);
-                const uint32_t w[4] = {u[i].x, u[i].y, u[i].z, u[i].w};
-                const uint32_t gw[4] = {gg.x, gg.y, gg.z, gg.w};
-                uint32_t r[4];
-#pragma unroll
-                for (int e = 0; e < 4; ++e)
-                    r[e] = pack_bf16(bf16_lo(w[e]) * rstd1 * bf16_lo(gw[e]), bf16_hi(w[e]) * rstd1 * bf16_hi(gw[e]));
-                out[c] = make_uint4(r[0], r[1], r[2], r[3]);
-            }
-        }
-        return;
-    }
-    float ss = 0.f;
-    for (int c0 = 0; c0 < nchunk; c0 += 256) {
-        uint4 u[8];
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            const int c = c0 + i * 32 + lane;
-            u[i] = c < nchunk ? __ldcg(xr + c) : make_uint4(0, 0, 0, 0);
-            if (raw && c < nchunk) raw[c] = u[i];
-        }
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            const uint32_t w[4] = {u[i].x, u[i].y, u[i].z, u[i].w};
-#pragma unroll
-            for (int e = 0; e < 4; ++e) { const float a = bf16_lo(w[e]), b = bf16_hi(w[e]); ss += a * a + b * b; }
-        }
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
-    const float rstd = rsqrtf(ss / (float)hidden + eps);
-    for (int c0 = 0; c0 < nchunk; c0 += 256) {
-        uint4 u[8];
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            const int c = c0 + i * 32 + lane;
-            u[i] = c < nchunk ? __ldcg(xr + c) : make_uint4(0, 0, 0, 0);
-        }
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            const int c = c0 + i * 32 + lane;
-            if (c < nchunk) {
-                const uint4 gg = __ldg(gn + c);
-                const uint32_t w[4] = {u[i].x, u[i].y, u[i].z, u[i].w};
-                const uint32_t gw[4] = {gg.x, gg.y, gg.z, gg.w};
-                uint32_t r[4];
-#pragma unroll
-                for (int e = 0; e < 4; ++e)
-                    r[e] = pack_bf16(bf16_lo(w[e]) * rstd * bf16_lo(gw[e]), bf16_hi(w[e]) * rstd * bf16_hi(gw[e]));
-                out[c] = make_uint4(r[0], r[1], r[2], r[3]);
-            }
-        }
-    }
-}
-
-// Phase 0 of the projection kernels: the rows of R (or compact rows) -> RMSNorm -> the A operand,
-// then a grid-wide barrier; the rows are read back through TMA.  With no more rows than CTAs a
-// whole CTA takes a row (shortest latency); with many rows every warp takes rows of its own, which
-// keeps six rows in flight per SM instead of one.
-__device__ __forceinline__ void prep_phase(const GemmArgs& g, float* red, volatile int* abort_flag, unsigned int& nbar) {
-    const RowPrep& rp = g.prep;
-    const __nv_bfloat16* x = static_cast<const __nv_bfloat16*>(rp.x);
-    __nv_bfloat16* a_out = static_cast<__nv_bfloat16*>(const_cast<void*>(g.a));
-    __nv_bfloat16* raw = static_cast<__nv_bfloat16*>(rp.raw_out);
-    if (g.M <= (int)gridDim.x) {
-        for (int row = blockIdx.x; row < g.M; row += gridDim.x) {
-            const int64_t src = prep_row_source(g, row, threadIdx.x == 0);
-            rmsnorm_row(reinterpret_cast<const uint4*>(x + src), reinterpret_cast<const uint4*>(rp.gain),
-                        reinterpret_cast<uint4*>(a_out + (int64_t)row * g.K), g.K, rp.eps, red,
-                        raw ? reinterpret_cast<uint4*>(raw + (int64_t)row * g.K) : nullptr);
-        }
-    } else {
-        const int nw = blockDim.x >> 5, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-        // the source of the next row (index lookups: a dependent trip to memory) is asked for before this row is read
-        int row = blockIdx.x * nw + warp;
-        int64_t src = row < g.M ? prep_row_source(g, row, lane == 0) : 0;
-        while (row < g.M) {
-            const int next = row + gridDim.x * nw;
-            const int64_t src_next = next < g.M ? prep_row_source(g, next, lane == 0) : 0;
-            rmsnorm_row_warp(reinterpret_cast<const uint4*>(x + src), reinterpret_cast<const uint4*>(rp.gain),
-                             reinterpret_cast<uint4*>(a_out + (int64_t)row * g.K), g.K, rp.eps, lane,
-                             raw ? reinterpret_cast<uint4*>(raw + (int64_t)row * g.K) : nullptr);
-            row = next;
-            src = src_next;
-        }
-    }
-    asm volatile("fence.proxy.async;" ::: "memory");   // the rows are read back through TMA
-    grid_barrier(g.grid_bar, ++nbar, abort_flag, g.debug_expire != 0);
-    asm volatile("fence.proxy.async;" ::: "memory");
-}
-
 // The same row preparation as a kernel of its own, for many rows: inside the projection kernel only the CTA's six warps
 // work on it (one CTA per SM: 14 752 rows took 88-95 us per launch, 2.5 TB/s); here sixteen warps per SM do, and the
 // projection starts without the grid-wide barrier.
@@ -727,27 +414,21 @@ gemm_tc_kernel(const GemmArgs g, const TcPlan p, const __grid_constant__ CUtenso
     const int it0 = blockIdx.x * p.U;
     const int it1 = min(it0 + p.U, p.tiles * p.KB);
     // The weights are constant inputs (no earlier kernel writes them), so their loads may start
-    // before the previous kernel has finished: fill the ring's weight halves now and ask L2 for the
-    // k-blocks after that.  The activation halves follow once the producer kernel is done.
-    const int kPrefetchL2 = p.prefetch;
+    // before the previous kernel has finished: fill the ring's weight halves now.  The activation halves
+    // follow once the producer kernel is done.
     int prefilled = 0;
     if (warp == 0 && lane == 0) {
         const CUtensorMap* maps[3] = {&mapB0, &mapB1, &mapB2};
         const uint64_t pol_w = g.keep_weights ? policy_evict_last() : policy_evict_first();
-        for (int i = 0; i < p.prefill + kPrefetchL2 && it0 + i < it1; ++i) {
+        for (int i = 0; i < p.prefill && it0 + i < it1; ++i) {
             const int it = it0 + i, t = it / p.KB, kb = it - t * p.KB, nt = t / p.m_tiles;
             int row0, row1;
             const int s0 = half_source(g, p, nt, 0, row0), s1 = half_source(g, p, nt, 1, row1);
-            if (i < p.prefill) {
-                const uint32_t sB = base + i * TC_STAGE_BYTES + TC_A_BYTES;
-                mbar_expect_tx(full_bar(i), TC_A_BYTES + TC_HALF_BYTES * (1 + (s1 >= 0)));
-                tma_load_2d(sB, maps[s0], kb * TC_BK, row0, full_bar(i), pol_w);
-                if (s1 >= 0) tma_load_2d(sB + TC_HALF_BYTES, maps[s1], kb * TC_BK, row1, full_bar(i), pol_w);
-                prefilled = i + 1;
-            } else {
-                tma_prefetch_2d(maps[s0], kb * TC_BK, row0);
-                if (s1 >= 0) tma_prefetch_2d(maps[s1], kb * TC_BK, row1);
-            }
+            const uint32_t sB = base + i * TC_STAGE_BYTES + TC_A_BYTES;
+            mbar_expect_tx(full_bar(i), TC_A_BYTES + TC_HALF_BYTES * (1 + (s1 >= 0)));
+            tma_load_2d(sB, maps[s0], kb * TC_BK, row0, full_bar(i), pol_w);
+            if (s1 >= 0) tma_load_2d(sB + TC_HALF_BYTES, maps[s1], kb * TC_BK, row1, full_bar(i), pol_w);
+            prefilled = i + 1;
         }
     }
     // everything above overlaps the previous kernel's tail; its outputs are touched only below
@@ -1136,10 +817,7 @@ struct SplitTiles {
     int tile[160];     // one per CTA boundary that cuts a tile (at most SM count - 1)
 };
 
-// NC = 4 (255 registers, one block per SM) serves finishes of at most one block per SM with two column groups per
-// item: the masked rows' query projection has nine or ten contributors per tile and every round is a trip to L2.
-template <int NC>
-__global__ void __launch_bounds__(256, NC == 2 ? 2 : 1) gemm_finish_kernel(const GemmArgs g, const TcPlan p, const SplitTiles split) {
+__global__ void __launch_bounds__(256, 2) gemm_finish_kernel(const GemmArgs g, const TcPlan p, const SplitTiles split) {
     const int t = split.tile[blockIdx.y];
     const int mt = t % p.m_tiles;
     const int rows_per = p.m_tiles == 1 ? ((g.M + 31) & ~31) : TC_BM;
@@ -1158,7 +836,7 @@ __global__ void __launch_bounds__(256, NC == 2 ? 2 : 1) gemm_finish_kernel(const
     pdl_wait();
     pdl_launch_dependents();
     if (!active) return;
-    finish_item<NC>(g, p, t, item, row, f, res);
+    finish_item(g, p, t, item, row, f, res);
 }
 
 // ---- predict and commit (Eq. 2-3): confidence and arg max per row, commit rule per request ------
@@ -1274,33 +952,58 @@ EncodeTiledFn encode_fn() {
     return fn;
 }
 
-// bf16 [rows, cols] row-major, box = 128 rows x 64 cols, 128-byte swizzle, zero fill out of bounds.
-struct MapKey { const void* ptr; int rows, cols; };
+struct MapKey { const void* ptr; int rows, cols, box_rows, panels, half; };
 struct MapEntry { MapKey key; CUtensorMap map; };
 constexpr int kMapCache = 1024;   // a 32-layer model has over 200 weight matrices
-std::mutex g_map_mutex;
 MapEntry g_maps[kMapCache];
 int g_map_count = 0, g_map_next = 0;
 
-// The pointer is only good until the next call (a miss may replace any entry): callers copy the map.
-const CUtensorMap* get_map(const void* ptr, int rows, int cols) {
-    for (int i = 0; i < g_map_count; ++i)
-        if (g_maps[i].key.ptr == ptr && g_maps[i].key.rows == rows && g_maps[i].key.cols == cols) return &g_maps[i].map;
+const CUtensorMap* lookup_map(const MapKey& want, int rank, const cuuint64_t* dims, const cuuint64_t* strides, const cuuint32_t* box) {
+    for (int i = 0; i < g_map_count; ++i) {
+        const MapKey& k = g_maps[i].key;
+        if (k.ptr == want.ptr && k.rows == want.rows && k.cols == want.cols && k.box_rows == want.box_rows &&
+            k.panels == want.panels && k.half == want.half)
+            return &g_maps[i].map;
+    }
     EncodeTiledFn fn = encode_fn();
     if (!fn) return nullptr;
     MapEntry& e = g_maps[g_map_next];
-    cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
-    cuuint64_t strides[1] = {(cuuint64_t)cols * 2};
-    cuuint32_t box[2] = {64, 128};
-    cuuint32_t estr[2] = {1, 1};
-    CUresult r = fn(&e.map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(ptr), dims, strides, box, estr,
-                    CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    if (r != CUDA_SUCCESS) return nullptr;
-    e.key = MapKey{ptr, rows, cols};
+    const cuuint32_t estr[4] = {1, 1, 1, 1};
+    if (fn(&e.map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, rank, const_cast<void*>(want.ptr), dims, strides, box, estr,
+           CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+           CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+        return nullptr;
+    e.key = want;
     g_map_next = (g_map_next + 1) % kMapCache;
     if (g_map_count < kMapCache) ++g_map_count;
     return &e.map;
+}
+
+// bf16 [rows, cols] row-major, box = 128 rows x 64 cols, 128-byte swizzle, zero fill out of bounds; like every lookup here,
+// the pointer is only good until the next one (a miss may replace any entry): callers copy the map.
+const CUtensorMap* get_map(const void* ptr, int rows, int cols) {
+    const cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows}, strides[1] = {(cuuint64_t)cols * 2};
+    const cuuint32_t box[2] = {64, 128};
+    return lookup_map(MapKey{ptr, rows, cols, 128, 0, 0}, 2, dims, strides, box);
+}
+
+}  // namespace
+
+std::mutex g_map_mutex;
+
+const CUtensorMap* get_panel_map(const void* ptr, int rows, int cols, int box_rows, int panels, int half) {
+    const cuuint64_t row = (cuuint64_t)cols * 2;
+    const MapKey key{ptr, rows, cols, box_rows, panels, half};
+    if (half) {
+        const cuuint64_t dims[4] = {64, (cuuint64_t)half, (cuuint64_t)(rows / half), (cuuint64_t)(cols / 64)};
+        const cuuint64_t strides[3] = {row, row * half, 128};
+        const cuuint32_t box[4] = {64, (cuuint32_t)box_rows, 2, (cuuint32_t)panels};
+        return lookup_map(key, 4, dims, strides, box);
+    }
+    const cuuint64_t dims[3] = {64, (cuuint64_t)rows, (cuuint64_t)(cols / 64)};
+    const cuuint64_t strides[2] = {row, 128};
+    const cuuint32_t box[3] = {64, (cuuint32_t)box_rows, (cuuint32_t)panels};
+    return lookup_map(key, 3, dims, strides, box);
 }
 
 int sm_count() {
@@ -1314,6 +1017,8 @@ int sm_count() {
     return n;
 }
 
+namespace {
+
 TcPlan make_plan(int M, int K, int units, bool swiglu) {
     TcPlan p{};
     p.units = units;
@@ -1326,11 +1031,7 @@ TcPlan make_plan(int M, int K, int units, bool swiglu) {
     p.U = (int)((total + g - 1) / g);
     p.ctas = (int)((total + p.U - 1) / p.U);
     p.smax = 2;   // partial slots per CTA
-    // K blocks past the ring asked into L2 before the dependency wait: none by default (measured at configuration 2:
-    // 168.1 us per layer-step at 0, 170.1 at 12, 175.7 at 28: with neighbours this short the requests compete with the
-    // stream that follows); GemmArgs::prefetch_blocks sets it per projection.  The ring itself is filled before the
-    // wait (174.9 us per layer-step with no stage prefilled, 169.1 with two, 167.9-168.6 with three or four).
-    p.prefetch = 0;
+    // measured: 174.9 us per layer-step of 103 rows with no stage prefilled, 169.1 with two, 167.9-168.6 with three or four
     p.prefill = TC_STAGES;
     return p;
 }
@@ -1381,7 +1082,6 @@ GemmLaunch plan_gemm(const GemmArgs& g) {
     GemmLaunch gl{};
     gl.p = make_plan(g.M, g.K, n_total / 128, swiglu);
     TcPlan& p = gl.p;
-    if (g.prefetch_blocks > 0) p.prefetch = g.prefetch_blocks;
     // Two or more row tiles: two SMs per 256 x 256 tile.  With many tiles per cluster every tile is whole
     // and the clusters walk them round-robin; with few, the (tile, K block) iterations are cut into equal
     // contiguous ranges, one per cluster (stream-K), and the cut tiles go through the finish kernel.
@@ -1460,6 +1160,7 @@ int launch_gemm(const GemmArgs& g, cudaStream_t stream) {
 }
 
 static int launch_gemm_impl(const GemmArgs& g, cudaStream_t stream) {
+    if (const int n = launch_gemm_rows(g, stream)) return n;
     const bool swiglu = g.epilogue == kEpiSwiGLU;
     const GemmLaunch gl = plan_gemm(g);
     const TcPlan& p = gl.p;
@@ -1485,7 +1186,7 @@ static int launch_gemm_impl(const GemmArgs& g, cudaStream_t stream) {
         if (cudaLaunchKernelEx(&cfg, gemm_tc2_kernel, g, p, gl.clusters, *mA, *mB[0], *mB[1], *mB[2]) != cudaSuccess) return -1;
         if (gl.split.n == 0) return 1;
         const int per_tile = finish_items_per_tile(g.epilogue) * TC_BM;
-        if (launch_pdl(gemm_finish_kernel<2>, dim3((per_tile + 255) / 256, gl.split.n), dim3(256), 0, stream, g, p, gl.split) !=
+        if (launch_pdl(gemm_finish_kernel, dim3((per_tile + 255) / 256, gl.split.n), dim3(256), 0, stream, g, p, gl.split) !=
             cudaSuccess)
             return -1;
         return 2;
@@ -1498,10 +1199,7 @@ static int launch_gemm_impl(const GemmArgs& g, cudaStream_t stream) {
     if (gl.split.n == 0) return 1;
     const int rows_per = p.m_tiles == 1 ? ((g.M + 31) & ~31) : TC_BM;
     const int per_tile = finish_items_per_tile(g.epilogue) * rows_per;
-    const dim3 fgrid((per_tile + 255) / 256, gl.split.n);
-    const bool wide = g.epilogue == kEpiQKV && (int)(fgrid.x * fgrid.y) <= sm_count();
-    if ((wide ? launch_pdl(gemm_finish_kernel<4>, fgrid, dim3(256), 0, stream, g, p, gl.split)
-              : launch_pdl(gemm_finish_kernel<2>, fgrid, dim3(256), 0, stream, g, p, gl.split)) != cudaSuccess)
+    if (launch_pdl(gemm_finish_kernel, dim3((per_tile + 255) / 256, gl.split.n), dim3(256), 0, stream, g, p, gl.split) != cudaSuccess)
         return -1;
     return 2;
 }

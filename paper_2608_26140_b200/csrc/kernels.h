@@ -143,9 +143,6 @@ struct GemmArgs {
     int kv_out_stride;
     // the weights are read again by the next projection (the masked rows' queries before Q/K/V): keep them in L2
     int keep_weights;
-    // K blocks past the ring asked into L2 before the dependency wait (0: the default; worth it only behind a long
-    // kernel that leaves memory idle)
-    int prefetch_blocks;
     // failure-detection self-test: the grid barrier of the row-preparation phase is given a target it cannot reach
     int debug_expire;
     // --- kEpiResidual ---

@@ -7,8 +7,8 @@ from oracle import acache_oracle as orc
 from paper_2608_26140_b200 import binding as ab
 from paper_2608_26140_b200 import workloads as wl
 
-from helpers import DEV, DeviceCase, assert_close_bf16, oracle_step
-from test_gpu_parity import MID128, run_layer_step, run_split_calls
+from helpers import DEV, DeviceCase, assert_close_bf16, cached_weights, oracle_step
+from test_gpu_parity import MID128, check_against_oracle, run_layer_step, run_split_calls
 from test_gpu_predict_commit import test_predict_commit as check_predict_commit
 
 pytestmark = pytest.mark.gpu
@@ -81,3 +81,19 @@ def test_topk_score_distributions(L):
             out = torch.full((1, K), -7, dtype=torch.int32, device=DEV)
             ctx.select_topk(torch.from_numpy(s).to(DEV), 1, L, K, out)
             assert np.array_equal(out[0].cpu().numpy(), orc.select_topk(s, K)[0]), (name, L, K)
+
+
+# K is cut between 1, 2 or 4 CTAs of a cluster depending on rows and shape; a ring stage takes 1 to 8 panels of K
+DEEP128 = wl.LayerShape(3584, 4, 1, 128, 8192, 1e-6, True, 1e6, "deep-d128")
+ODD64 = wl.LayerShape(1024, 6, 2, 64, 640, 1e-5, False, 5e5, "odd-d64")
+
+
+@pytest.mark.parametrize("shape,rows", [(DEEP128, n) for n in (1, 8, 33, 103, 128, 129)] + [(ODD64, n) for n in (1, 7, 9, 64, 127)])
+def test_few_row_projections(shape, rows):
+    lay = wl.make_layout(1, 3, 160, 8, 8, 8, "none")
+    case = wl.make_case(shape, lay, 0.0, cfg_id=73, weights=cached_weights(shape, 73))
+    dc = DeviceCase(case)
+    anchors = np.sort(np.random.default_rng(rows).choice(160, rows, replace=False)).astype(np.int32)[None]
+    k_new, v_new, y = run_split_calls(dc, torch.from_numpy(anchors).to(DEV), rows)
+    assert dc.ctx.poll_status() == 0
+    check_against_oracle(dc, anchors, k_new, v_new, y, None, None, rows)
