@@ -59,7 +59,6 @@ struct TcPlan {
     int m_pairs;          // 256-row tile rows of the two-SM kernel
     int units;            // 128-row B halves over all segments (non-SwiGLU) or ffn/128 (SwiGLU)
     int group_n;          // two-SM kernel, whole tiles: weight tiles per group of the tile order
-    int whole;            // two-SM kernel, whole tiles: no tile is cut (the stream-K fields do not apply)
     int w_keep;           // weights loaded with the evict-last policy (every row tile re-reads them from L2) instead of evict-first
 };
 
@@ -205,6 +204,12 @@ __device__ __forceinline__ void load_residual16(const GemmArgs& g, int grow, int
     const uint4* rp = reinterpret_cast<const uint4*>(static_cast<const __nv_bfloat16*>(g.resid) + roff + col);
     res[0] = __ldcg(rp); res[1] = __ldcg(rp + 1);
 }
+
+// Tiles whose K range is cut, each listed once.
+struct SplitTiles {
+    int n;
+    int tile[160];     // one per CTA boundary that cuts a tile (at most SM count - 1)
+};
 
 // Where an item of the finish lives: everything that can be worked out before the projection has finished.
 struct FinishItem {
@@ -812,10 +817,6 @@ gemm_tc2_kernel(const GemmArgs g, const TcPlan p, const int clusters, const __gr
 
 // Finish of the split tiles: grid row y finishes tile split.tile[y]; blockIdx.x * 256 +
 // threadIdx.x -> (item, row).
-struct SplitTiles {
-    int n;
-    int tile[160];     // one per CTA boundary that cuts a tile (at most SM count - 1)
-};
 
 __global__ void __launch_bounds__(256, 2) gemm_finish_kernel(const GemmArgs g, const TcPlan p, const SplitTiles split) {
     const int t = split.tile[blockIdx.y];
@@ -858,38 +859,31 @@ __device__ __forceinline__ void logit_merge_warp(LogitAcc& a, int width) {
 
 // One CTA per row: merges the per-tile statistics (16 entries for a tile whose K range was split between CTAs, one or two
 // otherwise; the first one's w says how many) in a fixed order.  Bound by the latency of L2 and the instructions per entry:
-// half a warp takes a tile, a lane per entry, four tiles in flight per lane; where no tile is cut a thread takes an entry.
-// 512 rows x 126 464 logits: 20.7 -> 8.2 us.
+// a thread takes a tile's first entry (and second); then half a warp takes one of the cut tiles, which the launch lists, a lane
+// per entry.  32 rows x 126 464 logits with 147 cut tiles: 17.5 -> 9.7 us against reading sixteen entries of every tile.
 constexpr int LR_THREADS = 512;
-__global__ void __launch_bounds__(LR_THREADS) logit_reduce_kernel(const GemmArgs g, const TcPlan p, int32_t* __restrict__ token,
-                                                                  float* __restrict__ confidence) {
+__global__ void __launch_bounds__(LR_THREADS) logit_reduce_kernel(const GemmArgs g, const TcPlan p, const SplitTiles split,
+                                                                  int32_t* __restrict__ token, float* __restrict__ confidence) {
     __shared__ LogitAcc part[32];
-    const int row = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5, entry = lane & 15;
+    const int row = blockIdx.x, mt = row / TC_BM, lane = threadIdx.x & 31, warp = threadIdx.x >> 5, entry = lane & 15;
     const LogitAcc empty{-3.402823466e38f, 0.f, 0x7fffffff};
     if (threadIdx.x < 32) part[threadIdx.x] = empty;
     pdl_wait();
     pdl_launch_dependents();
     LogitAcc a = empty;
-    constexpr int kStep = LR_THREADS / 16;
-    if (p.whole) {
 #pragma unroll 1
-        for (int i = threadIdx.x; i < 2 * p.n_tiles; i += LR_THREADS) {
-            const float4 v = __ldcg(logit_entry(g, i >> 1, i & 1, row));
-            logit_merge(a, v.x, v.y, __float_as_int(v.z));
-        }
-    } else {
-#pragma unroll 1
-        for (int nt0 = threadIdx.x >> 4; nt0 - (lane >> 4) < p.n_tiles; nt0 += 4 * kStep) {
-            float4 v[4];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) v[i] = __ldcg(logit_entry(g, min(nt0 + i * kStep, p.n_tiles - 1), entry, row));
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const int nt = nt0 + i * kStep, n = (int)__shfl_sync(0xffffffffu, v[i].w, lane & 16);
-                const bool use = nt < p.n_tiles && entry < n && (n < 16 || nt * 2 + (entry >> 3) < p.units);
-                logit_merge(a, use ? v[i].x : empty.m, use ? v[i].y : 0.f, use ? __float_as_int(v[i].z) : empty.arg);
-            }
-        }
+    for (int nt = threadIdx.x; nt < p.n_tiles; nt += LR_THREADS) {
+        const float4 v = __ldcg(logit_entry(g, nt, 0, row)), u = __ldcg(logit_entry(g, nt, 1, row));
+        const bool one = v.w <= 2.f, two = v.w == 2.f;
+        logit_merge(a, one ? v.x : empty.m, one ? v.y : 0.f, one ? __float_as_int(v.z) : empty.arg);
+        logit_merge(a, two ? u.x : empty.m, two ? u.y : 0.f, two ? __float_as_int(u.z) : empty.arg);
+    }
+#pragma unroll 4
+    for (int i = threadIdx.x >> 4; i < split.n; i += LR_THREADS / 16) {
+        const int nt = split.tile[i] / p.m_tiles;
+        const bool use = nt * p.m_tiles + mt == split.tile[i] && nt * 2 + (entry >> 3) < p.units;
+        const float4 v = __ldcg(logit_entry(g, nt, entry, row));
+        logit_merge(a, use ? v.x : empty.m, use ? v.y : 0.f, use ? __float_as_int(v.z) : empty.arg);
     }
     logit_merge_warp(a, 32);
     __syncthreads();
@@ -1120,8 +1114,7 @@ GemmLaunch plan_gemm(const GemmArgs& g) {
             }
             if (gl.split.n >= 159) { p.pair_u = 0; gl.split.n = 0; gl.clusters = std::min(max_clusters, tiles); }
         }
-        p.whole = p.pair_u == 0;
-        p.w_keep = (m_pairs >= w_keep_from && p.whole) ? 1 : 0;      // whole tiles, walked by three or more row pairs
+        p.w_keep = (m_pairs >= w_keep_from && p.pair_u == 0) ? 1 : 0;      // whole tiles, walked by three or more row pairs
         return gl;
     }
     // tiles whose K range is cut by a boundary between two CTAs, each listed once
@@ -1207,8 +1200,8 @@ static int launch_gemm_impl(const GemmArgs& g, cudaStream_t stream) {
 int launch_predict_commit(const GemmArgs& g, int batch, int n_blk, float threshold, int32_t* token, float* confidence,
                           int32_t* commit, cudaStream_t stream) {
     if (g.M == 0) return 0;
-    const TcPlan p = plan_gemm(g).p;
-    if (launch_pdl(logit_reduce_kernel, dim3(g.M), dim3(LR_THREADS), 0, stream, g, p, token, confidence) != cudaSuccess) return -1;
+    const GemmLaunch gl = plan_gemm(g);
+    if (launch_pdl(logit_reduce_kernel, dim3(g.M), dim3(LR_THREADS), 0, stream, g, gl.p, gl.split, token, confidence) != cudaSuccess) return -1;
     if (launch_pdl(commit_kernel, dim3(batch), dim3(32), 0, stream, (const float*)confidence, n_blk, threshold, commit) !=
         cudaSuccess)
         return -1;
