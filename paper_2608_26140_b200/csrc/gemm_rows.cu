@@ -222,7 +222,7 @@ gemm_rows_kernel(const GemmArgs g, const RowsPlan p, const __grid_constant__ CUt
             if (prefilled > 0) {
                 --prefilled;              // this stage's weights are already on their way
             } else {
-                if (!(ok = mbar_wait(empty_bar(stage), phase ^ 1, abort_flag))) break;
+                if (!(ok = mbar_poll(empty_bar(stage), phase ^ 1, abort_flag))) break;
                 mbar_expect_tx(full_bar(stage), p.stage_bytes);
                 load_weights(stage, blk0 + i);
             }
@@ -235,7 +235,7 @@ gemm_rows_kernel(const GemmArgs g, const RowsPlan p, const __grid_constant__ CUt
         uint32_t phase = 0;
         const uint32_t idesc = idesc_bf16(p.mma_n);
         for (int i = 0; i < n_blk && ok; ++i) {
-            if (!(ok = mbar_wait(full_bar(stage), phase, abort_flag))) break;
+            if (!(ok = mbar_poll(full_bar(stage), phase, abort_flag))) break;
             tc_fence_after();
             const uint32_t sA = base + stage * p.stage_bytes, sB = sA + a_bytes;
             for (int c = 0; c < p.CP; ++c) {

@@ -465,7 +465,7 @@ gemm_tc_kernel(const GemmArgs g, const TcPlan p, const __grid_constant__ CUtenso
                     --prefilled;
                     tma_load_2d(sA, &mapA, kb * TC_BK, mt * TC_BM, full_bar(stage), pol_a);
                 } else {
-                    if (!(ok = mbar_wait(empty_bar(stage), phase ^ 1, abort_flag))) break;
+                    if (!(ok = mbar_poll(empty_bar(stage), phase ^ 1, abort_flag))) break;
                     mbar_expect_tx(full_bar(stage), bytes);
                     tma_load_2d(sA, &mapA, kb * TC_BK, mt * TC_BM, full_bar(stage), pol_a);
                     tma_load_2d(sB, maps[s0], kb * TC_BK, row0, full_bar(stage), pol_w);
@@ -486,11 +486,11 @@ gemm_tc_kernel(const GemmArgs g, const TcPlan p, const __grid_constant__ CUtenso
             const int nt = t / p.m_tiles;
             int row1;
             const uint32_t idesc = idesc_bf16(half_source(g, p, nt, 1, row1) >= 0 ? 256 : 128);
-            if (!(ok = mbar_wait(tempty_bar(acc), acc_phase ^ 1, abort_flag))) break;
+            if (!(ok = mbar_poll(tempty_bar(acc), acc_phase ^ 1, abort_flag))) break;
             tc_fence_after();
             const uint32_t d_tmem = tmem_base + acc * TC_BN;
             for (int kb = kb0; kb < kb1; ++kb) {
-                if (!(ok = mbar_wait(full_bar(stage), phase, abort_flag))) break;
+                if (!(ok = mbar_poll(full_bar(stage), phase, abort_flag))) break;
                 tc_fence_after();
                 const uint32_t sA = base + stage * TC_STAGE_BYTES, sB = sA + TC_A_BYTES;
                 const uint64_t da = smem_desc_sw128(sA), db = smem_desc_sw128(sB);
@@ -698,7 +698,7 @@ gemm_tc2_kernel(const GemmArgs g, const TcPlan p, const int clusters, const __gr
             const int bs = half_source(g, p, nt, (int)rank, brow);
             const int arow = (mp * 2 + (int)rank) * TC_BM;
             for (int kb = kb0; kb < kb1; ++kb) {
-                if (!(ok = mbar_wait(empty_bar(stage), phase ^ 1, abort_flag))) break;
+                if (!(ok = mbar_poll(empty_bar(stage), phase ^ 1, abort_flag))) break;
                 const uint32_t sA = base + stage * TC2_STAGE_BYTES, sB = sA + TC_A_BYTES;
                 const uint32_t lead_full = mapa_u32(full_bar(stage), 0);
                 // the leader announces the bytes of both CTAs; the peer's copies only report completion
@@ -713,7 +713,7 @@ gemm_tc2_kernel(const GemmArgs g, const TcPlan p, const int clusters, const __gr
         // wait until the MMAs have consumed everything this CTA loaded, so that no signal from the
         // leader can arrive after this CTA has left
         for (int i = 0; i < min(issued, TC2_STAGES) && ok; ++i) {
-            ok = mbar_wait(empty_bar(stage), phase ^ 1, abort_flag);
+            ok = mbar_poll(empty_bar(stage), phase ^ 1, abort_flag);
             if (++stage == TC2_STAGES) { stage = 0; phase ^= 1; }
         }
     } else if (warp == 1 && lane == 0 && rank == 0) {
@@ -727,11 +727,11 @@ gemm_tc2_kernel(const GemmArgs g, const TcPlan p, const int clusters, const __gr
         for (int t = p.pair_u ? (int)(it / p.KB) : cluster_id; ok && (p.pair_u ? it < it_end : t < tiles);) {
             const int kb0 = p.pair_u ? (int)(it - (long long)t * p.KB) : 0;
             const int kb1 = p.pair_u ? (int)min((long long)p.KB, (long long)(kb0 + (it_end - it))) : p.KB;
-            if (!(ok = mbar_wait_cluster(tempty_bar(acc), acc_phase ^ 1, abort_flag))) break;
+            if (!(ok = mbar_poll_cluster(tempty_bar(acc), acc_phase ^ 1, abort_flag))) break;
             tc_fence_after();
             const uint32_t d_tmem = tmem_base + acc * TC_BN;
             for (int kb = kb0; kb < kb1; ++kb) {
-                if (!(ok = mbar_wait_cluster(full_bar(stage), phase, abort_flag))) break;
+                if (!(ok = mbar_poll_cluster(full_bar(stage), phase, abort_flag))) break;
                 tc_fence_after();
                 const uint32_t sA = base + stage * TC2_STAGE_BYTES, sB = sA + TC_A_BYTES;
                 const uint64_t da = smem_desc_sw128(sA), db = smem_desc_sw128(sB);
