@@ -10,30 +10,36 @@ namespace acache {
 
 constexpr uint32_t GRID_WAIT_LIMIT = 1u << 21;
 
-// Grid-wide barrier number `k` (1, 2, ...) of this launch on a pair of counters in global
-// memory: arrivals only ever add to bar[0], so barrier k is passed at k * gridDim.x.  Bounded;
-// returns false (and raises the CTA's abort flag) if the others do not arrive.
+// Grid-wide barrier on a pair of counters in global memory: every CTA adds to bar[0] and waits for gridDim.x arrivals;
+// those who have passed add to bar[1], and the last of them re-arms both words for the next launch.  One round trip to L2
+// for the arrival and its view of the others: the arrival releases what the CTA wrote (the threads met at the block barrier
+// before), the polls acquire, and the re-arming is left to a thread that has nothing to do until the epilogue (with fences
+// around an atomic and the re-arming at the kernel's end, 1-2 us more per launch).  Bounded; returns false (and raises the CTA's abort flag) if the others do not arrive.
 // self_test: the failure-detection self-test (acache_debug_expire_next_wait): the target is one arrival more than
 // the grid can deliver and the poll limit is short, so the wait runs out and the abort path below is taken.
-__device__ __forceinline__ bool grid_barrier(unsigned int* bar, unsigned int k, volatile int* abort_flag, bool self_test = false) {
+__device__ __forceinline__ bool grid_barrier(unsigned int* bar, volatile int* abort_flag, bool self_test = false) {
     __syncthreads();
     if (threadIdx.x == 0 && !*abort_flag) {
-        __threadfence();
-        atomicAdd(&bar[0], 1u);
-        const unsigned int target = k * gridDim.x + (self_test ? 1u : 0u);
+        asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(bar) : "memory");
+        const unsigned int target = gridDim.x + (self_test ? 1u : 0u);
         const uint32_t limit = self_test ? (1u << 12) : GRID_WAIT_LIMIT;
         bool ok = false;
         for (uint32_t i = 0; i < limit; ++i) {
             unsigned int v;
             asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(bar) : "memory");
             if (v >= target) { ok = true; break; }
-            __nanosleep(i < 64 ? 20 : 100);
+            if (i >= 64) __nanosleep(100);
         }
         if (!ok) *abort_flag = 1;
-        __threadfence();
     }
     __syncthreads();
-    return !*abort_flag;
+    const bool passed = !*abort_flag;
+    if (passed && threadIdx.x == 64 && atomicAdd(&bar[1], 1u) == gridDim.x - 1) {
+        bar[0] = 0u;
+        __threadfence();
+        bar[1] = 0u;
+    }
+    return passed;
 }
 
 __device__ __forceinline__ uint4 pack8(const float* v) {
@@ -292,7 +298,7 @@ __device__ __forceinline__ void rmsnorm_row_warp(const uint4* __restrict__ xr, c
 // then a grid-wide barrier; the rows are read back through TMA.  With no more rows than CTAs a
 // whole CTA takes a row (shortest latency); with many rows every warp takes rows of its own, which
 // keeps six rows in flight per SM instead of one.
-__device__ __forceinline__ void prep_phase(const GemmArgs& g, float* red, volatile int* abort_flag, unsigned int& nbar) {
+__device__ __forceinline__ void prep_phase(const GemmArgs& g, float* red, volatile int* abort_flag) {
     const RowPrep& rp = g.prep;
     const __nv_bfloat16* x = static_cast<const __nv_bfloat16*>(rp.x);
     __nv_bfloat16* a_out = static_cast<__nv_bfloat16*>(const_cast<void*>(g.a));
@@ -320,7 +326,7 @@ __device__ __forceinline__ void prep_phase(const GemmArgs& g, float* red, volati
         }
     }
     asm volatile("fence.proxy.async;" ::: "memory");   // the rows are read back through TMA
-    grid_barrier(g.grid_bar, ++nbar, abort_flag, g.debug_expire != 0);
+    grid_barrier(g.grid_bar, abort_flag, g.debug_expire != 0);
     asm volatile("fence.proxy.async;" ::: "memory");
 }
 

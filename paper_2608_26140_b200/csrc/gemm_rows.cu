@@ -163,7 +163,6 @@ gemm_rows_kernel(const GemmArgs g, const RowsPlan p, const __grid_constant__ CUt
     const int nt = blockIdx.x / S;
     const int blk0 = rank * p.blocks / S, blk1 = (rank + 1) * p.blocks / S;
     const int n_blk = blk1 - blk0;
-    unsigned int nbar = 0;
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < p.stages; ++s) { mbar_init(full_bar(s), 1); mbar_init(empty_bar(s), 1); }
@@ -211,7 +210,7 @@ gemm_rows_kernel(const GemmArgs g, const RowsPlan p, const __grid_constant__ CUt
     pdl_wait();
     pdl_launch_dependents();
 
-    if (g.prep.enabled) prep_phase(g, red, abort_flag, nbar);
+    if (g.prep.enabled) prep_phase(g, red, abort_flag);
 
     // ---------------- the contraction ----------------
     if (threadIdx.x == 0) {
@@ -378,14 +377,6 @@ gemm_rows_kernel(const GemmArgs g, const RowsPlan p, const __grid_constant__ CUt
             for (int i = 0; i < 4096; ++i) __nanosleep(64);   // copies of stages that were complete when a role gave up
         }
         __syncthreads();
-    } else if (threadIdx.x == 0 && nbar > 0) {
-        // the last CTA to leave re-arms the barrier words for the next launch
-        __threadfence();
-        if (atomicAdd(&g.grid_bar[1], 1u) == gridDim.x - 1) {
-            g.grid_bar[0] = 0u;
-            __threadfence();
-            g.grid_bar[1] = 0u;
-        }
     }
     __syncwarp();
     if (S > 1) { cluster_arrive(); cluster_wait(); }          // no CTA leaves while a peer may still read its staging area

@@ -399,7 +399,6 @@ gemm_tc_kernel(const GemmArgs g, const TcPlan p, const __grid_constant__ CUtenso
     auto tfull_bar = [&](int i) { return bars + 8 * (2 * TC_STAGES + i); };
     auto tempty_bar = [&](int i) { return bars + 8 * (2 * TC_STAGES + 2 + i); };
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    unsigned int nbar = 0;
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < TC_STAGES; ++s) { mbar_init(full_bar(s), 1); mbar_init(empty_bar(s), 1); }
@@ -441,7 +440,7 @@ gemm_tc_kernel(const GemmArgs g, const TcPlan p, const __grid_constant__ CUtenso
     pdl_launch_dependents();
 
     // ---------------- phase 0: gather the rows of R and RMSNorm them into A ----------------
-    if (g.prep.enabled) prep_phase(g, red, abort_flag, nbar);
+    if (g.prep.enabled) prep_phase(g, red, abort_flag);
 
     // ---------------- phase 1: the contraction ----------------
 
@@ -569,14 +568,6 @@ gemm_tc_kernel(const GemmArgs g, const TcPlan p, const __grid_constant__ CUtenso
             for (int i = 0; i < 4096; ++i) __nanosleep(64);   // copies of stages that were complete when a role gave up
         }
         __syncthreads();
-    } else if (threadIdx.x == 0 && nbar > 0) {
-        // the last CTA to leave re-arms the barrier words for the next launch
-        __threadfence();
-        if (atomicAdd(&g.grid_bar[1], 1u) == gridDim.x - 1) {
-            g.grid_bar[0] = 0u;
-            __threadfence();
-            g.grid_bar[1] = 0u;
-        }
     }
     if (warp == 1) {
         tc_fence_after();
@@ -651,7 +642,6 @@ gemm_tc2_kernel(const GemmArgs g, const TcPlan p, const int clusters, const __gr
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t rank = cluster_ctarank();
     const int cluster_id = blockIdx.x >> 1;
-    unsigned int nbar = 0;
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < TC2_STAGES; ++s) { mbar_init(full_bar(s), 1); mbar_init(empty_bar(s), 1); }
@@ -672,7 +662,7 @@ gemm_tc2_kernel(const GemmArgs g, const TcPlan p, const int clusters, const __gr
     pdl_wait();
     pdl_launch_dependents();
 
-    if (g.prep.enabled) prep_phase(g, red, abort_flag, nbar);
+    if (g.prep.enabled) prep_phase(g, red, abort_flag);
 
     const int m_pairs = (p.m_tiles + 1) >> 1;
     const int tiles = m_pairs * p.n_tiles;
@@ -800,13 +790,6 @@ gemm_tc2_kernel(const GemmArgs g, const TcPlan p, const int clusters, const __gr
             for (int i = 0; i < 4096; ++i) __nanosleep(64);
         }
         __syncthreads();
-    } else if (threadIdx.x == 0 && nbar > 0) {
-        __threadfence();
-        if (atomicAdd(&g.grid_bar[1], 1u) == gridDim.x - 1) {
-            g.grid_bar[0] = 0u;
-            __threadfence();
-            g.grid_bar[1] = 0u;
-        }
     }
     cluster_sync_all();          // neither CTA leaves while its peer may still signal it
     if (warp == 1) {
