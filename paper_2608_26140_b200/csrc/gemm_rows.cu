@@ -76,7 +76,6 @@ __device__ __forceinline__ float4 ld_cluster_f4(uint32_t cluster_addr) {
 }
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
-__device__ __forceinline__ void prefetch_l1(const void* p) { asm volatile("prefetch.global.L1 [%0];" ::"l"(p)); }
 __device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map, int c1, int c2, uint32_t bar, uint64_t policy) {
     asm volatile(
         "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint "
@@ -274,12 +273,15 @@ gemm_rows_kernel(const GemmArgs g, const RowsPlan p, const __grid_constant__ CUt
         const int col = nt * p.TN + (item0 + hf) * UNIT;
         if (item0 + hf < item1 && col < g.n[0]) { res[0] = __ldcg(res_row + (col >> 3)); res[1] = __ldcg(res_row + (col >> 3) + 1); }
     }
+    float c[16] = {}, sn[16] = {};         // the first item's waited 1.2 us for memory where they were asked for after the sums
+    auto item_rope = [&](int u) {          // cosines and sines of item u's pairs
+        int col;
+        const int seg = pair_group(g, min(nt * p.n_units + (u >> 1), p.groups - 1), col);
+        if (u < item1 && seg < g.rope_segments) load_rope<16>(g, pos, (col + (u & 1) * 16) & ((g.head_dim >> 1) - 1), c, sn);
+    };
     if (EPI == kEpiQKV && valid) {
         pos = __ldcg(g.row_pos + row);
-        if (g.rope_segments > 0) {
-            const int64_t at = (int64_t)(pos < 0 ? 0 : pos) * (g.head_dim >> 1);
-            for (int i = hf * 32; i < (g.head_dim >> 1); i += 64) { prefetch_l1(g.rope_cos + at + i); prefetch_l1(g.rope_sin + at + i); }
-        }
+        item_rope(item0 + hf);
     }
 
     bool ok = !*abort_flag;
@@ -352,12 +354,12 @@ gemm_rows_kernel(const GemmArgs g, const RowsPlan p, const __grid_constant__ CUt
                 int col;
                 const int seg = pair_group(g, min(grp, p.groups - 1), col);
                 col += (u & 1) * 16;
-                float lo[16], hi[16], c[16], sn[16];
-                if (valid && seg < g.rope_segments) load_rope<16>(g, pos, col & ((g.head_dim >> 1) - 1), c, sn);
+                float lo[16], hi[16];
                 sum_cluster16<S>(taddr + (u >> 1) * 64 + (u & 1) * 16, peers, sc, p.rows_pad, row, lo);
                 sum_cluster16<S>(taddr + (u >> 1) * 64 + (u & 1) * 16 + 32, peers, sc + 16, p.rows_pad, row, hi);
                 if (valid && grp < p.groups) {
                     rope_qkv<16>(g, seg, col, lo, hi, c, sn);
+                    item_rope(u + 2);
                     store_qkv<16>(g, row, pos, seg, col, lo, hi);
                 }
             }
