@@ -121,6 +121,7 @@ struct AttnTcArgs {
     // of four requests into the four 32-row quarters of one tile, so that the shared cache's key tiles are read
     // once per four requests; each request's fresh tiles follow, visible to its own quarter only.  Else 1.
     int group, batch;
+    int split;                // one-tile kernel: CTAs (a cluster) per query tile, each over a part of the key tiles
     const uint32_t* pos_excl;
     const uint32_t* row_keep;
     // Eq. 4-5 taken from this attention's own logits (two-query-tile kernel; the one-shot probe of Section 3.2): for the
@@ -167,10 +168,13 @@ attention_tc_kernel(const AttnTcArgs a, const __grid_constant__ CUtensorMap mapQ
     //           13,14 p_full | 15,16 pv_done (P V of the tile completed: O holds it, its S/P buffer is free)
     auto bar = [&](int i) { return bars + 8 * i; };
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int qt = blockIdx.x, h = blockIdx.y, b = blockIdx.z;
+    // key split: a cluster of C CTAs shares a query tile, each taking a contiguous part of the key tiles
+    const int C = a.split, rank = C > 1 ? (int)cluster_ctarank() : 0;
+    const int qt = blockIdx.x / C, h = blockIdx.y, b = blockIdx.z;
     const int kvh = h / (a.n_heads / a.n_kv_heads);
     const int n_cache_tiles = (a.ctx_len + 127) / 128;
-    const int n_tiles = n_cache_tiles + a.n_fresh_tiles * min(a.group, a.batch - (int)blockIdx.z * a.group);
+    const int all_tiles = n_cache_tiles + a.n_fresh_tiles * min(a.group, a.batch - (int)blockIdx.z * a.group);
+    const int j0 = rank * all_tiles / C, n_tiles = (rank + 1) * all_tiles / C - j0;     // this CTA's first key tile, and how many
     const int kb = a.cache_shared ? 0 : b;          // one cache for the whole batch, or one per request
     const int G = a.group;                          // requests per tile (4: blockIdx.z counts groups of four)
     const int b0 = b * G;                           // first request of the tile
@@ -199,6 +203,8 @@ attention_tc_kernel(const AttnTcArgs a, const __grid_constant__ CUtensorMap mapQ
     pdl_wait();
     pdl_launch_dependents();
 
+    const bool softmax = warp >= 2 && warp < 18 && (warp & 3) < live_q;
+    float m_use = -INFINITY, l = 0.f;               // softmax threads: exponent reference and denominator share of the row
     if (warp == 0 && lane == 0) {
         // ---------------- TMA producer ----------------
         const uint64_t pol_q = policy_evict_first(), pol_kv = policy_evict_last();
@@ -219,11 +225,11 @@ attention_tc_kernel(const AttnTcArgs a, const __grid_constant__ CUtensorMap mapQ
             const int s = j & 1;
             const uint32_t par = ((j >> 1) & 1) ^ 1;
             if (!(ok = mbar_wait(bar(3 + s), par, abort_flag))) break;
-            const bool fresh = j >= n_cache_tiles;
+            const bool fresh = j0 + j >= n_cache_tiles;
             const CUtensorMap* mk = fresh ? &mapKn : &mapK;
             const CUtensorMap* mv = fresh ? &mapVn : &mapV;
-            const int f = j - n_cache_tiles;                          // fresh tiles: request by request
-            const int r0 = (fresh ? f % a.n_fresh_tiles : j) * 128, bz = fresh ? b0 + f / a.n_fresh_tiles : kb;
+            const int f = j0 + j - n_cache_tiles;                     // fresh tiles: request by request
+            const int r0 = (fresh ? f % a.n_fresh_tiles : j0 + j) * 128, bz = fresh ? b0 + f / a.n_fresh_tiles : kb;
             mbar_expect_tx(bar(1 + s), AT_TILE);
             tma_load_3d(sK0 + s * AT_TILE, mk, kvh * 128, r0, bz, bar(1 + s), pol_kv);
             tma_load_3d(sK0 + s * AT_TILE + AT_PANEL, mk, kvh * 128 + 64, r0, bz, bar(1 + s), pol_kv);
@@ -276,7 +282,7 @@ attention_tc_kernel(const AttnTcArgs a, const __grid_constant__ CUtensorMap mapQ
             tc_commit(bar(15 + s));    // pv_done: O holds tiles 0..j, the S/P buffer is free
             tc_commit(bar(7 + s));     // v_empty
         }
-    } else if (warp >= 2 && warp < 18 && (warp & 3) < live_q) {
+    } else if (softmax) {
         // ---------------- softmax: four threads per query row ----------------
         // Warp 2 + 4 c + q' (q = warp & 3 is its TMEM lane quarter) takes keys [32 c, 32 c + 32) of every
         // tile for the 32 rows of quarter q, and columns [32 c, 32 c + 32) of O.  Sixteen warps (four per
@@ -291,19 +297,18 @@ attention_tc_kernel(const AttnTcArgs a, const __grid_constant__ CUtensorMap mapQ
         const uint32_t lane_off = (uint32_t)(q * 32) << 16;
         const uint32_t col_off = (uint32_t)(c4 * 32);
         const int bq = G > 1 ? b0 + q : b;          // the request whose rows this quarter holds
-        float m_use = -INFINITY, l = 0.f;
         bool ok = true;
         for (int j = 0; j < n_tiles; ++j) {
-            const int s = j & 1;
+            const int s = j & 1, jk = j0 + j;         // ring stage, key tile
             // which of this thread's 32 keys count: the cache's positions up to the context end, minus those a
             // fresh row serves; of the fresh rows, those that serve their position
             uint32_t keep;
-            if (j < n_cache_tiles) {
-                const int valid = a.ctx_len - j * 128 - c4 * 32;
+            if (jk < n_cache_tiles) {
+                const int valid = a.ctx_len - jk * 128 - c4 * 32;
                 keep = valid >= 32 ? 0xffffffffu : (valid <= 0 ? 0u : (1u << valid) - 1u);
-                if (a.pos_excl && j * 4 + c4 < a.excl_words) keep &= ~__ldg(a.pos_excl + (int64_t)bq * a.excl_words + j * 4 + c4);
+                if (a.pos_excl && jk * 4 + c4 < a.excl_words) keep &= ~__ldg(a.pos_excl + (int64_t)bq * a.excl_words + jk * 4 + c4);
             } else {
-                const int f = j - n_cache_tiles;
+                const int f = jk - n_cache_tiles;
                 if (G > 1 && f / a.n_fresh_tiles != q) {
                     // another request's fresh rows: none of them is a key of this quarter's rows.  All four warps
                     // of the quarter come here, so none of them goes to the quarter's barrier for this tile.
@@ -406,10 +411,11 @@ attention_tc_kernel(const AttnTcArgs a, const __grid_constant__ CUtensorMap mapQ
         float* row_sum = reinterpret_cast<float*>(base_ptr + AT_TILE);         // the K stages are idle now
         row_sum[c4 * 128 + row] = l;
         asm volatile("bar.sync %0, 128;" ::"r"(1 + q) : "memory");
-        if (ok && !*abort_flag) {
+        l = (row_sum[row] + row_sum[128 + row]) + (row_sum[256 + row] + row_sum[384 + row]);
+        if (C == 1 && ok && !*abort_flag) {
             tc_fence_after();
             const int grow = G > 1 ? lane : qt * 128 + row;     // the row inside its request
-            const float inv = 1.f / ((row_sum[row] + row_sum[128 + row]) + (row_sum[256 + row] + row_sum[384 + row]));
+            const float inv = 1.f / l;
             __nv_bfloat16* out = static_cast<__nv_bfloat16*>(a.o) + (((int64_t)bq * a.n + grow) * a.n_heads + h) * 128 + col_off;
             float v[32];
             tc_ld32(tO + lane_off + col_off, v);
@@ -423,6 +429,69 @@ attention_tc_kernel(const AttnTcArgs a, const __grid_constant__ CUtensorMap mapQ
                 }
             }
         }
+    }
+    if (C > 1) {
+        // ---------------- merge of the cluster's parts through distributed shared memory ----------------
+        // (reference, denominator) of every row meet first; each CTA scales its O to the common reference and lays it out by
+        // the CTA that finishes the columns (128 / C each), which sums the parts in rank order.  The K and V stages are idle
+        // by now.  All threads pass the three cluster barriers, whatever happened before.
+        float2* ml = reinterpret_cast<float2*>(base_ptr + AT_TILE + 4096);             // [128], behind row_sum
+        const uint32_t parts = base + 2 * AT_TILE;                                     // [owner][column / 4][row][4] fp32
+        const int q = warp & 3, c4 = (warp - 2) >> 2, row = q * 32 + lane, width = 128 / C;
+        __syncwarp();
+        if (softmax && c4 == 0) ml[row] = make_float2(m_use, l);
+        __syncwarp();
+        cluster_sync_all();
+        float denom = 0.f;
+        if (softmax) {
+            const uint32_t ml_row = smem_u32(ml + row);
+            float ref = -INFINITY, m_c[8], l_c[8];
+#pragma unroll
+            for (int c = 0; c < 8; ++c)
+                if (c < C) {
+                    asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(m_c[c]), "=f"(l_c[c]) : "r"(mapa_u32(ml_row, c)) : "memory");
+                    ref = fmaxf(ref, m_c[c]);
+                }
+#pragma unroll
+            for (int c = 0; c < 8; ++c)
+                if (c < C && m_c[c] > -INFINITY) denom += l_c[c] * fast_exp2(m_c[c] - ref);
+            const float f = m_use > -INFINITY ? fast_exp2(m_use - ref) : 0.f;
+            tc_fence_after();
+            float v[32];
+            tc_ld32(tO + ((uint32_t)(q * 32) << 16) + c4 * 32, v);
+            const uint32_t dst = parts + ((c4 * 8 * 128 + row) << 4);                  // owners' columns lie one after the other
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+                asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};"
+                             ::"r"(dst + i * 2048), "f"(v[4 * i] * f), "f"(v[4 * i + 1] * f), "f"(v[4 * i + 2] * f), "f"(v[4 * i + 3] * f)
+                             : "memory");
+        }
+        __syncwarp();
+        cluster_sync_all();
+        if (softmax) {
+            const int bq = G > 1 ? b0 + q : b, grow = G > 1 ? lane : qt * 128 + row;
+            const float inv = 1.f / denom;
+            const int col = rank * width + c4 * (width >> 2);                          // width / 4 columns per thread
+            __nv_bfloat16* out = static_cast<__nv_bfloat16*>(a.o) + (((int64_t)bq * a.n + grow) * a.n_heads + h) * 128 + col;
+#pragma unroll 1
+            for (int g4 = 0; g4 < width >> 4; ++g4) {
+                const uint32_t src = parts + (((col >> 2) + g4) * 128 + row) * 16;
+                float4 u[8];
+#pragma unroll
+                for (int c = 0; c < 8; ++c)
+                    if (c < C)
+                        asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
+                                     : "=f"(u[c].x), "=f"(u[c].y), "=f"(u[c].z), "=f"(u[c].w) : "r"(mapa_u32(src, c)) : "memory");
+                float4 o = u[0];
+#pragma unroll
+                for (int c = 1; c < 8; ++c)
+                    if (c < C) { o.x += u[c].x; o.y += u[c].y; o.z += u[c].z; o.w += u[c].w; }
+                if (grow < a.n)
+                    *reinterpret_cast<uint2*>(out + g4 * 4) = make_uint2(pack_bf16(o.x * inv, o.y * inv), pack_bf16(o.z * inv, o.w * inv));
+            }
+        }
+        __syncwarp();
+        cluster_sync_all();
     }
     // ---------------- teardown ----------------
     tc_fence_before();
@@ -1004,12 +1073,33 @@ int launch_attention_tc(const AttnArgs& a, uint32_t* status, cudaStream_t stream
     const bool use_2q = fused_score || mode_2q == 2 || (mode_2q == 1 && a.ctx_len + (two_src ? n_fresh : 0) <= 4096 &&
                                                         (int64_t)((q_tiles + 1) / 2) * a.n_heads * a.batch >= 148);
     cudaError_t err;
-    if (use_2q && (q_tiles >= 2 || fused_score))
+    if (use_2q && (q_tiles >= 2 || fused_score)) {
         err = launch_pdl(attention_tc2q_kernel, dim3((q_tiles + 1) / 2, a.n_heads, a.batch), dim3(AT2_THREADS), AT2_SMEM, stream, t,
                          *mq, *mk, *mv, *mkn, *mvn);
-    else
-        err = launch_pdl(attention_tc_kernel, dim3(q_tiles, a.n_heads, (a.batch + group - 1) / group), dim3(AT_THREADS), AT_SMEM,
-                         stream, t, *mq, *mk, *mv, *mkn, *mvn);
+    } else {
+        // Few query tiles leave most SMs idle, and one SM pulls K and V at 60-100 GB/s: the key tiles of a query tile are split
+        // over a cluster of up to eight CTAs, as many as one wave holds while each still has two tiles.  Layer-step of 103 rows
+        // over 1024 keys (32 query tiles): attention 17.3 -> 13.6 us with four CTAs, the step 153.5 us with one, 152.1 with
+        // two, 150.0 with four; decode pass of 32 rows (4 layers) 679, 675, 665.
+        const int groups = (a.batch + group - 1) / group;
+        const int64_t ctas = (int64_t)q_tiles * a.n_heads * groups;
+        const int tiles = (a.ctx_len + 127) / 128 + t.n_fresh_tiles * (a.batch - (groups - 1) * group);   // of the last group
+        t.split = 1;
+        while (t.split < 8 && ctas * t.split * 2 <= 148 && tiles >= t.split * 4) t.split *= 2;
+        cudaLaunchConfig_t cfg{};
+        cfg.gridDim = dim3(q_tiles * t.split, a.n_heads, groups);
+        cfg.blockDim = dim3(AT_THREADS);
+        cfg.dynamicSmemBytes = AT_SMEM;
+        cfg.stream = stream;
+        cudaLaunchAttribute at[2];
+        at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        at[0].val.programmaticStreamSerializationAllowed = 1;
+        at[1].id = cudaLaunchAttributeClusterDimension;
+        at[1].val.clusterDim.x = t.split; at[1].val.clusterDim.y = 1; at[1].val.clusterDim.z = 1;
+        cfg.attrs = at;
+        cfg.numAttrs = t.split > 1 ? 2 : 1;
+        err = cudaLaunchKernelEx(&cfg, attention_tc_kernel, t, *mq, *mk, *mv, *mkn, *mvn);
+    }
     return err == cudaSuccess ? 1 : -1;
 }
 

@@ -97,3 +97,17 @@ def test_few_row_projections(shape, rows):
     k_new, v_new, y = run_split_calls(dc, torch.from_numpy(anchors).to(DEV), rows)
     assert dc.ctx.poll_status() == 0
     check_against_oracle(dc, anchors, k_new, v_new, y, None, None, rows)
+
+
+# 3, 5, 9, 17 and 40 key tiles: 1, 2, 4, 8 and 8 CTAs per query tile, with unequal shares
+@pytest.mark.parametrize("T,rows,drop", [(300, 33, False), (520, 1, False), (1100, 128, True), (2100, 40, False), (5000, 97, True)])
+def test_attention_key_split(T, rows, drop):
+    lay = wl.make_layout(1, 6, T - 6 - 40, 8, 32, 32, "none")
+    case = wl.make_case(MID128, lay, 0.0, cfg_id=74)
+    dc = DeviceCase(case, max_rows=rows)
+    ratio = (rows - 0.5) / lay.affix_len
+    anchors = np.sort(np.random.default_rng(T).choice(lay.affix_len, rows, replace=False)).astype(np.int32)[None]
+    _, _, _, y = run_layer_step(dc, ratio, ab.F_DROP_NON_ANCHOR if drop else 0, anchors)
+    assert dc.ctx.poll_status() == 0
+    ref = oracle_step(case, 0, anchor_idx=anchors[0], drop_non_anchor=drop)
+    assert_close_bf16(ab.to_host_bits(y[0]), ref["y"], "y")
