@@ -225,7 +225,7 @@ __device__ __forceinline__ FinishItem finish_plan(const GemmArgs& g, const TcPla
     f.pc1 = -1; f.u128 = 0; f.lo_col = 0; f.skip = false;
     if (g.epilogue == kEpiResidual || g.epilogue == kEpiLogits) {
         f.pc0 = item * 4;
-        if (g.epilogue == kEpiLogits && f.nt * 2 + (item >> 3) >= p.units) f.skip = true;   // past the vocabulary's end
+        f.skip = f.nt * 2 + (item >> 3) >= p.units;                           // the tile's second half is past the last column
     } else if (g.epilogue == kEpiSwiGLU) {
         f.pc0 = item * 4; f.pc1 = 32 + f.pc0;
     } else {
@@ -815,7 +815,7 @@ __global__ void __launch_bounds__(256, 2) gemm_finish_kernel(const GemmArgs g, c
     FinishItem f{};
     if (active) {
         f = finish_plan(g, p, t, item, row);
-        if (g.epilogue == kEpiResidual) load_residual16(g, f.grow, f.nt * TC_BN + item * 16, res);
+        if (g.epilogue == kEpiResidual && !f.skip) load_residual16(g, f.grow, f.nt * TC_BN + item * 16, res);
     }
     pdl_wait();
     pdl_launch_dependents();

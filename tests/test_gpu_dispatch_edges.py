@@ -111,3 +111,18 @@ def test_attention_key_split(T, rows, drop):
     assert dc.ctx.poll_status() == 0
     ref = oracle_step(case, 0, anchor_idx=anchors[0], drop_non_anchor=drop)
     assert_close_bf16(ab.to_host_bits(y[0]), ref["y"], "y")
+
+
+# an odd number of 128-column units: the last weight tile is half past the end of the row, whole or cut
+ODD_TILES = wl.LayerShape(1920, 2, 1, 128, 256, 1e-5, False, 5e5, "odd-tiles")
+
+
+@pytest.mark.parametrize("shape,rows", [(ODD_TILES, n) for n in (9, 128, 140, 300)])
+def test_row_counts_of_wide_shapes(shape, rows):
+    lay = wl.make_layout(1, 3, rows + 40, 8, 8, 8, "none")
+    case = wl.make_case(shape, lay, 0.0, cfg_id=75)
+    dc = DeviceCase(case, max_rows=rows)
+    anchors = np.sort(np.random.default_rng(rows).choice(lay.affix_len, rows, replace=False)).astype(np.int32)[None]
+    k_new, v_new, y = run_split_calls(dc, torch.from_numpy(anchors).to(DEV), rows)
+    assert dc.ctx.poll_status() == 0
+    check_against_oracle(dc, anchors, k_new, v_new, y, None, None, rows)
