@@ -113,11 +113,15 @@ def test_attention_key_split(T, rows, drop):
     assert_close_bf16(ab.to_host_bits(y[0]), ref["y"], "y")
 
 
+# rows of 5376 columns take a warp each in the row preparation, narrower ones go through in batches: one row per CTA up to
+# several batches of them
+WIDE128 = wl.LayerShape(5376, 2, 1, 128, 256, 1e-5, False, 5e5, "wide-d128")
 # an odd number of 128-column units: the last weight tile is half past the end of the row, whole or cut
 ODD_TILES = wl.LayerShape(1920, 2, 1, 128, 256, 1e-5, False, 5e5, "odd-tiles")
 
 
-@pytest.mark.parametrize("shape,rows", [(ODD_TILES, n) for n in (9, 128, 140, 300)])
+@pytest.mark.parametrize("shape,rows", [(ODD_TILES, n) for n in (9, 128, 140, 300)]
+                         + [(MID128, 129), (MID128, 257), (MID128, 600), (WIDE128, 140), (WIDE128, 300)])
 def test_row_counts_of_wide_shapes(shape, rows):
     lay = wl.make_layout(1, 3, rows + 40, 8, 8, 8, "none")
     case = wl.make_case(shape, lay, 0.0, cfg_id=75)
