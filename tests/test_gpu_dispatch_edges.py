@@ -130,3 +130,18 @@ def test_row_counts_of_wide_shapes(shape, rows):
     k_new, v_new, y = run_split_calls(dc, torch.from_numpy(anchors).to(DEV), rows)
     assert dc.ctx.poll_status() == 0
     check_against_oracle(dc, anchors, k_new, v_new, y, None, None, rows)
+
+
+# a few keys four times as long, so that the exponents' reference moves on a later key tile: one CTA and a cluster per query
+# tile, with and without masked keys
+@pytest.mark.parametrize("T,rows,drop", [(1100, 40, False), (1100, 40, True), (700, 200, True), (4500, 300, False)])
+def test_attention_reference_moves(T, rows, drop):
+    lay = wl.make_layout(1, 6, T - 6 - 40, 8, 32, 32, "none")
+    case = wl.make_case(MID128, lay, 0.0, cfg_id=76, hot_frac=0.01)
+    dc = DeviceCase(case, max_rows=rows)
+    ratio = (rows - 0.5) / lay.affix_len
+    anchors = np.sort(np.random.default_rng(T).choice(lay.affix_len, rows, replace=False)).astype(np.int32)[None]
+    _, _, _, y = run_layer_step(dc, ratio, ab.F_DROP_NON_ANCHOR if drop else 0, anchors)
+    assert dc.ctx.poll_status() == 0
+    ref = oracle_step(case, 0, anchor_idx=anchors[0], drop_non_anchor=drop)
+    assert_close_bf16(ab.to_host_bits(y[0]), ref["y"], "y")
