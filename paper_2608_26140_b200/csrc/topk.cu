@@ -24,7 +24,7 @@ __device__ __forceinline__ uint32_t score_key(float f) {
 // histogram divide [smallest, largest] in 2048, which sorts out more than the leading bits of the keys do (the scores of a
 // request share their exponents), so one pass mostly leaves few candidates.  Warp w owns the keys of [w seg, (w + 1) seg):
 // loads are coalesced and the ordered output needs ballots and one sum over the warps.  Against a radix select over four
-// bytes with two block scans per 1024 positions (added time in its chain): 512 scores 6.6 -> 6.3 us, 2048 7.9 -> 5.8,
+// bytes with two block scans per 1024 positions (added time in its chain): 512 scores 6.6 -> 6.3 us, 2048 9.8 -> 5.8,
 // 8192 16.0 -> 8.7.
 __global__ void __launch_bounds__(kTopkThreads) topk_kernel(float* scores, int L, int K,
                                                             int32_t* __restrict__ anchor_idx, int use_smem,
