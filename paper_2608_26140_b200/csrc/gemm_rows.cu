@@ -227,29 +227,38 @@ gemm_rows_kernel(const GemmArgs g, const RowsPlan p, const __grid_constant__ CUt
             tma_load_3d(base + stage * p.stage_bytes, &mapA, 0, (blk0 + i) * p.CP, full_bar(stage), pol_a);
             if (++stage == p.stages) { stage = 0; phase ^= 1; }
         }
-    } else if (threadIdx.x == 32) {
-        bool ok = !*abort_flag;
+    } else if (warp == 1) {
+        // What bounds a stage here is this warp, not the data: 4 to 16 instructions of 60-100 cycles (they read A and B from
+        // shared memory, which the TMA fills meanwhile), then about 400 cycles until the next stage's first.  With one thread
+        // in the loop, whose descriptors are no warp-uniform values, the instructions took 94-121 cycles: masked rows' queries
+        // 2030 -> 1590 cycles a stage, layer-step of 103 rows 145.9 -> 144.2 us, of 8 rows 53.1 -> 51.6, decode pass of
+        // 32 rows over 4 layers 656 -> 646.  The next stage's barrier tested before the instructions or before the commit:
+        // 1 us slower.
+        bool ok = __all_sync(0xffffffffu, !*abort_flag);
         int stage = 0;
         uint32_t phase = 0;
         const uint32_t idesc = idesc_bf16(p.mma_n);
         for (int i = 0; i < n_blk && ok; ++i) {
-            if (!(ok = mbar_poll(full_bar(stage), phase, abort_flag))) break;
+            if (!(ok = __all_sync(0xffffffffu, mbar_poll(full_bar(stage), phase, abort_flag)))) break;
             tc_fence_after();
-            const uint32_t sA = base + stage * p.stage_bytes, sB = sA + a_bytes;
-            for (int c = 0; c < p.CP; ++c) {
-                const uint64_t da = smem_desc_sw128(sA + c * p.rows_pad * 128);
-                for (int u = 0; u < p.mma_count; ++u) {
-                    const uint64_t db = smem_desc_sw128(sB + u * box_bytes + c * p.R * 128);
+            if (elect_lane()) {
+                const uint32_t sA = base + stage * p.stage_bytes, sB = sA + a_bytes;
+                for (int c = 0; c < p.CP; ++c) {
+                    const uint64_t da = smem_desc_sw128(sA + c * p.rows_pad * 128);
+                    for (int u = 0; u < p.mma_count; ++u) {
+                        const uint64_t db = smem_desc_sw128(sB + u * box_bytes + c * p.R * 128);
 #pragma unroll
-                    for (int k = 0; k < 4; ++k)
-                        tc_mma(tmem_base + u * p.mma_n, da + (uint64_t)(k * 2), db + (uint64_t)(k * 2), idesc,
-                               (i > 0 || c > 0 || k > 0) ? 1u : 0u);
+                        for (int k = 0; k < 4; ++k)
+                            tc_mma(tmem_base + u * p.mma_n, da + (uint64_t)(k * 2), db + (uint64_t)(k * 2), idesc,
+                                   (i > 0 || c > 0 || k > 0) ? 1u : 0u);
+                    }
                 }
+                tc_commit(empty_bar(stage));
+                if (i + 1 == n_blk) tc_commit(done_bar);
             }
-            tc_commit(empty_bar(stage));
+            __syncwarp();
             if (++stage == p.stages) { stage = 0; phase ^= 1; }
         }
-        if (ok) tc_commit(done_bar);
     }
     __syncwarp();
 
@@ -437,8 +446,8 @@ int resident_clusters() {
 // (6.5 TB/s); a CTA not faster than about 60 GB/s (its weight rows and, once per tile, all rows of A; measured 45-60 with
 // this ring); a split costs an exchange per doubling, 1.5 us where rotary pairs are finished and 1 us otherwise.  A stage
 // takes as many panels as leave three stages in the ring (fewer, larger stages lost, two stages of any size did too).
-// Measured at 103 rows (us per launch, finish included | here): q/k/v 30.2 | 29.6, output 16.3 | 13.0, gate/up 47.7 | 43,
-// down 25.7 | 23.4; at 32 rows output 14.3 | 10.9, down 25.0 | 20.4, masked rows' queries 20.6 | 18.8.
+// Measured when it replaced that kernel, at 103 rows (us per launch, finish included | here): q/k/v 30.2 | 29.6, output
+// 16.3 | 13.0, gate/up 47.7 | 43, down 25.7 | 23.4; at 32 rows output 14.3 | 10.9, down 25.0 | 20.4.
 constexpr int kRingBytes = 200 * 1024;
 bool plan_rows(const GemmArgs& g, RowsPlan& best) {
     if (g.M > 128 || g.epilogue == kEpiLogits || g.K < 64) return false;

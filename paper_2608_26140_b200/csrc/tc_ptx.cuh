@@ -32,6 +32,17 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
         : "memory");
     return ok != 0;
 }
+// One lane of a converged warp, always the same.  The thread that issues the MMAs is taken this way, inside a loop that the
+// whole warp runs: descriptors and counters are then warp-uniform values, which the instruction wants.
+__device__ __forceinline__ bool elect_lane() {
+    uint32_t one;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "elect.sync _|p, 0xffffffff;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(one));
+    return one != 0;
+}
 // Bounded wait: false if the limit ran out or another role already gave up.
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
     for (uint32_t i = 0; i < TC_WAIT_LIMIT; ++i) {
