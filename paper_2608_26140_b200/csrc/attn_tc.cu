@@ -252,7 +252,7 @@ attention_tc_kernel(const AttnTcArgs a, const __grid_constant__ CUtensorMap mapQ
             tma_load_3d(sV0 + s * AT_TILE, mv, kvh * 128, r0, bz, bar(5 + s), pol_kv);
             tma_load_3d(sV0 + s * AT_TILE + AT_PANEL, mv, kvh * 128 + 64, r0, bz, bar(5 + s), pol_kv);
         }
-    } else if (warp == 1 && lane == 0) {
+    } else if (warp == 1) {
         // ---------------- MMA issuer 1: S = Q K^T (M 128, N 128, both operands K-major) ----------------
         // The two products are issued by two threads of different warps: one thread doing both spends
         // more time in its four barrier waits and sixteen issues per tile than the tensor pipe needs
@@ -260,41 +260,47 @@ attention_tc_kernel(const AttnTcArgs a, const __grid_constant__ CUtensorMap mapQ
         // dependencies (P of tile j after S of tile j, S buffer reuse, O in tile order) all go through
         // mbarriers, so no ordering between the two threads is assumed.
         const uint32_t idesc_s = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(128 >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
-        bool ok = mbar_wait(bar(0), 0, abort_flag);
+        bool ok = __all_sync(0xffffffffu, mbar_poll(bar(0), 0, abort_flag));
         for (int j = 0; j < n_tiles && ok; ++j) {
             const int s = j & 1;
             const uint32_t par = (j >> 1) & 1;
-            if (!(ok = mbar_wait(bar(1 + s), par, abort_flag))) break;          // K of tile j landed
+            if (!(ok = __all_sync(0xffffffffu, mbar_poll(bar(1 + s), par, abort_flag)))) break;          // K of tile j landed
             // its S buffer also holds the P of tile j - 2: free once that tile's P V has completed
-            if (j >= 2 && !(ok = mbar_wait(bar(15 + s), ((j - 2) >> 1) & 1, abort_flag))) break;
+            if (j >= 2 && !(ok = __all_sync(0xffffffffu, mbar_poll(bar(15 + s), ((j - 2) >> 1) & 1, abort_flag)))) break;
             tc_fence_after();
             const uint32_t k = sK0 + s * AT_TILE;
+            if (elect_lane()) {
 #pragma unroll
-            for (int ks = 0; ks < 8; ++ks) {
-                const uint64_t da = smem_desc_sw128(sQ + (ks >> 2) * AT_PANEL) + (uint64_t)((ks & 3) * 2);
-                const uint64_t db = smem_desc_sw128(k + (ks >> 2) * AT_PANEL) + (uint64_t)((ks & 3) * 2);
-                tc_mma(tS0 + s * 128, da, db, idesc_s, ks > 0 ? 1u : 0u);
+                for (int ks = 0; ks < 8; ++ks) {
+                    const uint64_t da = smem_desc_sw128(sQ + (ks >> 2) * AT_PANEL) + (uint64_t)((ks & 3) * 2);
+                    const uint64_t db = smem_desc_sw128(k + (ks >> 2) * AT_PANEL) + (uint64_t)((ks & 3) * 2);
+                    tc_mma(tS0 + s * 128, da, db, idesc_s, ks > 0 ? 1u : 0u);
+                }
+                tc_commit(bar(9 + s));     // s_full
+                tc_commit(bar(3 + s));     // k_empty
             }
-            tc_commit(bar(9 + s));     // s_full
-            tc_commit(bar(3 + s));     // k_empty
+            __syncwarp();
         }
-    } else if (warp == AT_THREADS / 32 - 1 && lane == 0) {
+    } else if (warp == AT_THREADS / 32 - 1) {
         // ---------------- MMA issuer 2: O += P V (A = P K-major, B = V MN-major) ----------------
         const uint32_t idesc_o = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 16) | ((uint32_t)(128 >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
         bool ok = true;
         for (int j = 0; j < n_tiles && ok; ++j) {
             const int s = j & 1;
-            if (!(ok = mbar_wait(bar(13 + s), (j >> 1) & 1, abort_flag))) break;    // P of tile j written, O rescaled
-            if (!(ok = mbar_wait(bar(5 + s), (j >> 1) & 1, abort_flag))) break;     // V of tile j landed
+            if (!(ok = __all_sync(0xffffffffu, mbar_poll(bar(13 + s), (j >> 1) & 1, abort_flag)))) break;    // P of tile j written, O rescaled
+            if (!(ok = __all_sync(0xffffffffu, mbar_poll(bar(5 + s), (j >> 1) & 1, abort_flag)))) break;     // V of tile j landed
             tc_fence_after();
             const uint32_t v = sV0 + s * AT_TILE;
+            if (elect_lane()) {
 #pragma unroll
-            for (int ks = 0; ks < 8; ++ks) {
-                const uint64_t db = smem_desc_mn_sw128(v + ks * 2048);
-                tc_mma_ta(tO, tS0 + s * 128 + ks * 8, db, idesc_o, (j > 0 || ks > 0) ? 1u : 0u);   // 16 keys = 8 columns of P
+                for (int ks = 0; ks < 8; ++ks) {
+                    const uint64_t db = smem_desc_mn_sw128(v + ks * 2048);
+                    tc_mma_ta(tO, tS0 + s * 128 + ks * 8, db, idesc_o, (j > 0 || ks > 0) ? 1u : 0u);   // 16 keys = 8 columns of P
+                }
+                tc_commit(bar(15 + s));    // pv_done: O holds tiles 0..j, the S/P buffer is free
+                tc_commit(bar(7 + s));     // v_empty
             }
-            tc_commit(bar(15 + s));    // pv_done: O holds tiles 0..j, the S/P buffer is free
-            tc_commit(bar(7 + s));     // v_empty
+            __syncwarp();
         }
     } else if (softmax) {
         // ---------------- softmax: four threads per query row ----------------
@@ -679,12 +685,16 @@ attention_tc2q_kernel(const AttnTcArgs a, const __grid_constant__ CUtensorMap ma
             tma_load_3d(sK0 + s * AT_TILE, &mapK, kvh * 128, (sw0 + js) * 128, kb, bar(1 + s), pol_kv);
             tma_load_3d(sK0 + s * AT_TILE + AT_PANEL, &mapK, kvh * 128 + 64, (sw0 + js) * 128, kb, bar(1 + s), pol_kv);
         }
-    } else if (warp == 1 && lane == 0) {
-        // ---------------- MMA issuer ----------------
+    } else if (warp == 1) {
+        // ---------------- MMA issuer: the whole warp runs the loop, one lane issues ----------------
+        // (with one lane in the loop, refresh of 14 752 rows 12 579 -> 12 524 us here, layer-step of 103 rows 144.0 -> 143.8 us
+        // in the one-tile kernel)
         const uint32_t idesc_s = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(128 >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
         const uint32_t idesc_o = idesc_s | (1u << 16);       // B = V is MN-major
+        auto wait = [&](int i, uint32_t parity) { return __all_sync(0xffffffffu, mbar_spin(bar(i), parity, abort_flag)); };
         auto issue_s = [&](int t, int j) {                   // S_t = Q_t K_j^T, then s_full of query tile t
             const uint32_t k = sK0 + (j & 1) * AT_TILE;
+            if (!elect_lane()) return;
 #pragma unroll
             for (int ks = 0; ks < 8; ++ks) {
                 const uint64_t da = smem_desc_sw128(sQ + t * AT_TILE + (ks >> 2) * AT_PANEL) + (uint64_t)((ks & 3) * 2);
@@ -693,53 +703,65 @@ attention_tc2q_kernel(const AttnTcArgs a, const __grid_constant__ CUtensorMap ma
             }
             tc_commit(bar(9 + t));
         };
-        bool ok = mbar_spin(bar(0), 0, abort_flag);
-        if (ok && n_tiles > 0 && (ok = mbar_spin(bar(1), 0, abort_flag))) {
+        bool ok = wait(0, 0);
+        if (ok && n_tiles > 0 && (ok = wait(1, 0))) {
             tc_fence_after();
             for (int t = 0; t < n_sets; ++t) issue_s(t, 0);
-            tc_commit(bar(3));                               // k_empty of stage 0
+            if (elect_lane()) tc_commit(bar(3));             // k_empty of stage 0
+            __syncwarp();
         }
         for (int j = 0; j < n_tiles && ok; ++j) {
             const int s = j & 1;
             const bool more = j + 1 < n_tiles;
-            if (!(ok = mbar_spin(bar(5 + s), (j >> 1) & 1, abort_flag))) break;                       // V of tile j landed
-            if (more && !(ok = mbar_spin(bar(1 + (s ^ 1)), ((j + 1) >> 1) & 1, abort_flag))) break;   // K of tile j + 1 landed
+            if (!(ok = wait(5 + s, (j >> 1) & 1))) break;                       // V of tile j landed
+            if (more && !(ok = wait(1 + (s ^ 1), ((j + 1) >> 1) & 1))) break;   // K of tile j + 1 landed
             const uint32_t v = sV0 + s * AT_TILE;
             for (int t = 0; t < n_sets && ok; ++t) {
                 for (int hb = 0; hb < 2 && ok; ++hb) {
-                    if (!(ok = mbar_spin(bar(11 + 2 * t + hb), j & 1, abort_flag))) break;  // P of this half written, O rescaled
+                    if (!(ok = wait(11 + 2 * t + hb, j & 1))) break;  // P of this half written, O rescaled
                     tc_fence_after();
+                    if (elect_lane()) {
 #pragma unroll
-                    for (int k4 = 0; k4 < 4; ++k4) {
-                        const int ks = hb * 4 + k4;          // 16 keys = 8 columns of P
-                        tc_mma_ta(tmem_base + 256 + t * 128, tmem_base + t * 128 + ks * 8, smem_desc_mn_sw128(v + ks * 2048), idesc_o,
-                                  (j > 0 || ks > 0) ? 1u : 0u);
+                        for (int k4 = 0; k4 < 4; ++k4) {
+                            const int ks = hb * 4 + k4;          // 16 keys = 8 columns of P
+                            tc_mma_ta(tmem_base + 256 + t * 128, tmem_base + t * 128 + ks * 8, smem_desc_mn_sw128(v + ks * 2048), idesc_o,
+                                      (j > 0 || ks > 0) ? 1u : 0u);
+                        }
+                        tc_commit(bar(15 + 2 * t + hb));         // pv_done: O holds everything up to this half
                     }
-                    tc_commit(bar(15 + 2 * t + hb));         // pv_done: O holds everything up to this half
+                    __syncwarp();
                 }
                 if (ok && more) issue_s(t, j + 1);           // overwrites P: executes after the P V just issued
+                __syncwarp();
             }
-            tc_commit(bar(7 + s));                           // v_empty
-            if (more) tc_commit(bar(3 + (s ^ 1)));           // k_empty of tile j + 1
+            if (elect_lane()) {
+                tc_commit(bar(7 + s));                           // v_empty
+                if (more) tc_commit(bar(3 + (s ^ 1)));           // k_empty of tile j + 1
+            }
+            __syncwarp();
         }
         // score sweep: D_t = K Q_t^T into the S buffer of query tile t (its last P V was issued above by this thread, and
         // the tensor pipe keeps one thread's instructions in order)
         for (int js = 0; js < n_sw && ok; ++js) {
             const int jj = n_tiles + js, s = jj & 1;
-            if (!(ok = mbar_spin(bar(1 + s), (jj >> 1) & 1, abort_flag))) break;
+            if (!(ok = wait(1 + s, (jj >> 1) & 1))) break;
             const uint32_t k = sK0 + s * AT_TILE;
             for (int t = 0; t < n_sets && ok; ++t) {
-                if (js > 0 && !(ok = mbar_spin(bar(19 + t), (js - 1) & 1, abort_flag))) break;
+                if (js > 0 && !(ok = wait(19 + t, (js - 1) & 1))) break;
                 tc_fence_after();
+                if (elect_lane()) {
 #pragma unroll
-                for (int ks = 0; ks < 8; ++ks) {
-                    const uint64_t da = smem_desc_sw128(k + (ks >> 2) * AT_PANEL) + (uint64_t)((ks & 3) * 2);
-                    const uint64_t db = smem_desc_sw128(sQ + t * AT_TILE + (ks >> 2) * AT_PANEL) + (uint64_t)((ks & 3) * 2);
-                    tc_mma(tmem_base + t * 128, da, db, idesc_s, ks > 0 ? 1u : 0u);
+                    for (int ks = 0; ks < 8; ++ks) {
+                        const uint64_t da = smem_desc_sw128(k + (ks >> 2) * AT_PANEL) + (uint64_t)((ks & 3) * 2);
+                        const uint64_t db = smem_desc_sw128(sQ + t * AT_TILE + (ks >> 2) * AT_PANEL) + (uint64_t)((ks & 3) * 2);
+                        tc_mma(tmem_base + t * 128, da, db, idesc_s, ks > 0 ? 1u : 0u);
+                    }
+                    tc_commit(bar(9 + t));
                 }
-                tc_commit(bar(9 + t));
+                __syncwarp();
             }
-            if (ok) tc_commit(bar(3 + s));                   // k_empty
+            if (ok && elect_lane()) tc_commit(bar(3 + s));   // k_empty
+            __syncwarp();
         }
     } else if (warp >= 2 && warp < 2 + 4 * n_sets) {
       const int t = (warp - 2) >> 2;
