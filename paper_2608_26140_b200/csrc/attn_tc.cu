@@ -507,12 +507,14 @@ attention_tc_kernel(const AttnTcArgs a, const __grid_constant__ CUtensorMap mapQ
 #pragma unroll
                 for (int c = 1; c < 8; ++c)
                     if (c < C) { o.x += u[c].x; o.y += u[c].y; o.z += u[c].z; o.w += u[c].w; }
+                if (g4 + 1 == width >> 4) cluster_arrive();      // the last read: before the stores, which it would wait for
                 if (grow < a.n)
                     *reinterpret_cast<uint2*>(out + g4 * 4) = make_uint2(pack_bf16(o.x * inv, o.y * inv), pack_bf16(o.z * inv, o.w * inv));
             }
         }
         __syncwarp();
-        cluster_sync_all();
+        if (!softmax) cluster_arrive();
+        cluster_wait();
     }
     // ---------------- teardown ----------------
     tc_fence_before();

@@ -74,8 +74,6 @@ __device__ __forceinline__ float4 ld_cluster_f4(uint32_t cluster_addr) {
                  : "memory");
     return v;
 }
-__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
-__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 __device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map, int c1, int c2, uint32_t bar, uint64_t policy) {
     asm volatile(
         "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint "
@@ -335,6 +333,13 @@ gemm_rows_kernel(const GemmArgs g, const RowsPlan p, const __grid_constant__ CUt
             peers[i] = mapa_u32(base + (rank < r ? rank : rank - 1) * region, r);
         }
     }
+    // Once a warp has read its last piece of the peers' staging areas they may leave; it says so before its stores, which the
+    // arrival would otherwise wait for (here, in the scoring and in the attention: layer-step of 8 rows 52.2 -> 51.8 us, of
+    // 103 rows 143.65 -> 143.2).
+    bool arrived = S == 1;
+    auto last_read = [&](bool last) {
+        if (!arrived && last) { cluster_arrive(); arrived = true; }
+    };
     if (ok && live) {
         for (int u = item0 + hf; u < item1; u += 2) {
             const int sc = (u - item0) * UNIT;
@@ -342,6 +347,7 @@ gemm_rows_kernel(const GemmArgs g, const RowsPlan p, const __grid_constant__ CUt
                 const int col = nt * p.TN + u * 16;
                 float v[16];
                 sum_cluster16<S>(taddr + u * 16, peers, sc, p.rows_pad, row, v);
+                last_read(u + 2 >= item1);
                 if (valid && col < g.n[0]) {
                     if (u != item0 + hf) { res[0] = __ldcg(res_row + (col >> 3)); res[1] = __ldcg(res_row + (col >> 3) + 1); }
                     const uint32_t rw[8] = {res[0].x, res[0].y, res[0].z, res[0].w, res[1].x, res[1].y, res[1].z, res[1].w};
@@ -366,6 +372,7 @@ gemm_rows_kernel(const GemmArgs g, const RowsPlan p, const __grid_constant__ CUt
                 float lo[16], hi[16];
                 sum_cluster16<S>(taddr + (u >> 1) * 64 + (u & 1) * 16, peers, sc, p.rows_pad, row, lo);
                 sum_cluster16<S>(taddr + (u >> 1) * 64 + (u & 1) * 16 + 32, peers, sc + 16, p.rows_pad, row, hi);
+                last_read(u + 2 >= item1);
                 if (valid && grp < p.groups) {
                     rope_qkv<16>(g, seg, col, lo, hi, c, sn);
                     item_rope(u + 2);
@@ -374,6 +381,8 @@ gemm_rows_kernel(const GemmArgs g, const RowsPlan p, const __grid_constant__ CUt
             }
         }
     }
+    __syncwarp();
+    last_read(true);
     // ---------------- teardown ----------------
     tc_fence_before();
     __syncthreads();
@@ -390,7 +399,7 @@ gemm_rows_kernel(const GemmArgs g, const RowsPlan p, const __grid_constant__ CUt
         __syncthreads();
     }
     __syncwarp();
-    if (S > 1) { cluster_arrive(); cluster_wait(); }          // no CTA leaves while a peer may still read its staging area
+    if (S > 1) cluster_wait();                                // no CTA leaves while a peer may still read its staging area
     if (warp == 1) {
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(p.tmem_cols) : "memory");

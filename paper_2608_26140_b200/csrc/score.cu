@@ -362,6 +362,7 @@ __global__ void __cluster_dims__(kSmallCluster, 1, 1) __launch_bounds__(128) sco
         s_inv[tid] = 1.f / Dn;
     }
     __syncthreads();
+    cluster.barrier_arrive();      // the neighbours' statistics have been read
 
     // pass 2: column sums of the normalised weights over this CTA's keys, 16 keys of every tile per warp
     for (int kt = 0; kt < ntiles; ++kt) {
@@ -390,7 +391,7 @@ __global__ void __cluster_dims__(kSmallCluster, 1, 1) __launch_bounds__(128) sco
             }
         }
     }
-    cluster.sync();        // no CTA leaves while a neighbour may still read its statistics
+    cluster.barrier_wait();        // no CTA leaves while a neighbour may still read its statistics
 }
 
 // ---- pass 3: ordered sum over heads -------------------------------------------------------
