@@ -136,6 +136,7 @@ struct AttnTcArgs {
     // once per four requests; each request's fresh tiles follow, visible to its own quarter only.  Else 1.
     int group, batch;
     int split;                // one-tile kernel: CTAs (a cluster) per query tile, each over a part of the key tiles
+    int n_items;              // one-tile kernel: query tiles over all heads and requests (or groups)
     const uint32_t* pos_excl;
     const uint32_t* row_keep;
     // Eq. 4-5 taken from this attention's own logits (two-query-tile kernel; the one-shot probe of Section 3.2): for the
@@ -162,12 +163,17 @@ __device__ __forceinline__ bool mbar_spin(uint32_t bar, uint32_t parity, volatil
     return false;
 }
 
+// MANY: many more items than SMs.  A CTA then takes every gridDim.x-th one and keeps its tensor memory and barriers; the loads and
+// the first S of the next item run under the tail of this one (64 requests of 103 rows over 608 keys: attention 184 -> 158 us,
+// layer-step 2774 -> 2757).  With one item per CTA the same code was 1.7 us slower (103 rows over 1024 keys).
+template <bool MANY>
 __global__ void __launch_bounds__(AT_THREADS, 1)
 attention_tc_kernel(const AttnTcArgs a, const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUtensorMap mapK,
                     const __grid_constant__ CUtensorMap mapV, const __grid_constant__ CUtensorMap mapKn,
                     const __grid_constant__ CUtensorMap mapVn) {
     extern __shared__ unsigned char smem_raw[];
-    __shared__ uint16_t row_max[4][128];  // [tile parity][key quarter][row]: upper halves of fp32, rounded up
+    __shared__ uint16_t row_max[4][128];  // [key quarter][row]: upper halves of fp32, rounded up
+    __shared__ float row_sum[4][128];     // [key quarter][row]: shares of the denominator
     const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     unsigned char* base_ptr = smem_raw + (base - smem_u32(smem_raw));
     if (base - smem_u32(smem_raw) > (uint32_t)AT_SLACK) {      // the tiles would not fit: report, touch nothing
@@ -184,22 +190,32 @@ attention_tc_kernel(const AttnTcArgs a, const __grid_constant__ CUtensorMap mapQ
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     // key split: a cluster of C CTAs shares a query tile, each taking a contiguous part of the key tiles
     const int C = a.split, rank = C > 1 ? (int)cluster_ctarank() : 0;
-    const int qt = blockIdx.x / C, h = blockIdx.y, b = blockIdx.z;
-    const int kvh = h / (a.n_heads / a.n_kv_heads);
+    const int first = blockIdx.x / C, stride = gridDim.x;        // items: (query tile, head, request or group of four)
     const int n_cache_tiles = (a.ctx_len + 127) / 128;
-    const int all_tiles = n_cache_tiles + a.n_fresh_tiles * min(a.group, a.batch - (int)blockIdx.z * a.group);
-    const int j0 = rank * all_tiles / C, n_tiles = (rank + 1) * all_tiles / C - j0;     // this CTA's first key tile, and how many
-    const int kb = a.cache_shared ? 0 : b;          // one cache for the whole batch, or one per request
-    const int G = a.group;                          // requests per tile (4: blockIdx.z counts groups of four)
-    const int b0 = b * G;                           // first request of the tile
-    const int n_req = min(G, a.batch - b0);
-    // 32-row quarters of the tile that hold rows: the softmax warps of the others have nothing to do (their
-    // rows of S, P and O are never read), which matters when a decode pass brings 32 rows per request
-    const int live_q = G > 1 ? n_req : min(4, (a.n - qt * 128 + 31) / 32);
+    const int G = a.group;                          // requests per tile (4: b counts groups of four)
+    int qt, h, b, kvh, kb, b0, n_req, live_q, j0, n_tiles;
+    auto set_item = [&](int item) {
+        const int t = item / a.q_tiles;
+        qt = item - t * a.q_tiles;
+        b = t / a.n_heads;
+        h = t - b * a.n_heads;
+        kvh = h / (a.n_heads / a.n_kv_heads);
+        kb = a.cache_shared ? 0 : b;                // one cache for the whole batch, or one per request
+        b0 = b * G;                                 // first request of the tile
+        n_req = min(G, a.batch - b0);
+        const int all_tiles = n_cache_tiles + a.n_fresh_tiles * n_req;
+        j0 = rank * all_tiles / C;                  // this CTA's first key tile, and how many
+        n_tiles = (rank + 1) * all_tiles / C - j0;
+        // 32-row quarters of the tile that hold rows: the softmax warps of the others have nothing to do (their
+        // rows of S, P and O are never read), which matters when a decode pass brings 32 rows per request
+        live_q = G > 1 ? n_req : min(4, (a.n - qt * 128 + 31) / 32);
+    };
+    set_item(first);
+    const int p_warps = MANY ? 16 : 4 * live_q;     // softmax warps that report a tile's P
 
     if (threadIdx.x == 0) {
         for (int i = 0; i <= 10; ++i) mbar_init(bar(i), 1);
-        mbar_init(bar(13), 4 * live_q); mbar_init(bar(14), 4 * live_q);    // p_full: the softmax warps that have rows
+        mbar_init(bar(13), p_warps); mbar_init(bar(14), p_warps);          // p_full
         mbar_init(bar(15), 1); mbar_init(bar(16), 1);      // pv_done
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -217,40 +233,47 @@ attention_tc_kernel(const AttnTcArgs a, const __grid_constant__ CUtensorMap mapQ
     pdl_wait();
     pdl_launch_dependents();
 
-    const bool softmax = warp >= 2 && warp < 18 && (warp & 3) < live_q;
+    const bool softmax = warp >= 2 && warp < 18 && (MANY || (warp & 3) < live_q);
+    int J = 0;                                      // key tiles of the items before: ring stages and phases go on
     float m_use = -INFINITY, l = 0.f;               // softmax threads: exponent reference and denominator share of the row
     if (warp == 0 && lane == 0) {
         // ---------------- TMA producer ----------------
         const uint64_t pol_q = policy_evict_first(), pol_kv = policy_evict_last();
-        if (G > 1) {
-            // 32-row boxes: request b0 + r fills rows [32 r, 32 r + 32) of both panels (rows past its n read as zero)
-            mbar_expect_tx(bar(0), n_req * 8192);
-            for (int r = 0; r < n_req; ++r) {
-                tma_load_3d(sQ + r * 4096, &mapQ, h * 128, 0, b0 + r, bar(0), pol_q);
-                tma_load_3d(sQ + AT_PANEL + r * 4096, &mapQ, h * 128 + 64, 0, b0 + r, bar(0), pol_q);
-            }
-        } else {
-            mbar_expect_tx(bar(0), AT_TILE);
-            tma_load_3d(sQ, &mapQ, h * 128, qt * 128, b, bar(0), pol_q);
-            tma_load_3d(sQ + AT_PANEL, &mapQ, h * 128 + 64, qt * 128, b, bar(0), pol_q);
-        }
         bool ok = true;
-        for (int j = 0; j < n_tiles && ok; ++j) {
-            const int s = j & 1;
-            const uint32_t par = ((j >> 1) & 1) ^ 1;
-            if (!(ok = mbar_wait(bar(3 + s), par, abort_flag))) break;
-            const bool fresh = j0 + j >= n_cache_tiles;
-            const CUtensorMap* mk = fresh ? &mapKn : &mapK;
-            const CUtensorMap* mv = fresh ? &mapVn : &mapV;
-            const int f = j0 + j - n_cache_tiles;                     // fresh tiles: request by request
-            const int r0 = (fresh ? f % a.n_fresh_tiles : j0 + j) * 128, bz = fresh ? b0 + f / a.n_fresh_tiles : kb;
-            mbar_expect_tx(bar(1 + s), AT_TILE);
-            tma_load_3d(sK0 + s * AT_TILE, mk, kvh * 128, r0, bz, bar(1 + s), pol_kv);
-            tma_load_3d(sK0 + s * AT_TILE + AT_PANEL, mk, kvh * 128 + 64, r0, bz, bar(1 + s), pol_kv);
-            if (!(ok = mbar_wait(bar(7 + s), par, abort_flag))) break;
-            mbar_expect_tx(bar(5 + s), AT_TILE);
-            tma_load_3d(sV0 + s * AT_TILE, mv, kvh * 128, r0, bz, bar(5 + s), pol_kv);
-            tma_load_3d(sV0 + s * AT_TILE + AT_PANEL, mv, kvh * 128 + 64, r0, bz, bar(5 + s), pol_kv);
+        for (int item = first; item < a.n_items && ok; item += stride, J += n_tiles) {
+            if (MANY) set_item(item);
+            // the last S of the item before has read Q
+            if (J > 0 && !(ok = mbar_wait(bar(3 + ((J - 1) & 1)), ((J - 1) >> 1) & 1, abort_flag))) break;
+            if (G > 1) {
+                // 32-row boxes: request b0 + r fills rows [32 r, 32 r + 32) of both panels (rows past its n read as zero)
+                mbar_expect_tx(bar(0), n_req * 8192);
+                for (int r = 0; r < n_req; ++r) {
+                    tma_load_3d(sQ + r * 4096, &mapQ, h * 128, 0, b0 + r, bar(0), pol_q);
+                    tma_load_3d(sQ + AT_PANEL + r * 4096, &mapQ, h * 128 + 64, 0, b0 + r, bar(0), pol_q);
+                }
+            } else {
+                mbar_expect_tx(bar(0), AT_TILE);
+                tma_load_3d(sQ, &mapQ, h * 128, qt * 128, b, bar(0), pol_q);
+                tma_load_3d(sQ + AT_PANEL, &mapQ, h * 128 + 64, qt * 128, b, bar(0), pol_q);
+            }
+            for (int j = 0; j < n_tiles && ok; ++j) {
+                const int s = (J + j) & 1;
+                const uint32_t par = (((J + j) >> 1) & 1) ^ 1;
+                if (!(ok = mbar_wait(bar(3 + s), par, abort_flag))) break;
+                const bool fresh = j0 + j >= n_cache_tiles;
+                const CUtensorMap* mk = fresh ? &mapKn : &mapK;
+                const CUtensorMap* mv = fresh ? &mapVn : &mapV;
+                const int f = j0 + j - n_cache_tiles;                     // fresh tiles: request by request
+                const int r0 = (fresh ? f % a.n_fresh_tiles : j0 + j) * 128, bz = fresh ? b0 + f / a.n_fresh_tiles : kb;
+                mbar_expect_tx(bar(1 + s), AT_TILE);
+                tma_load_3d(sK0 + s * AT_TILE, mk, kvh * 128, r0, bz, bar(1 + s), pol_kv);
+                tma_load_3d(sK0 + s * AT_TILE + AT_PANEL, mk, kvh * 128 + 64, r0, bz, bar(1 + s), pol_kv);
+                if (!(ok = mbar_wait(bar(7 + s), par, abort_flag))) break;
+                mbar_expect_tx(bar(5 + s), AT_TILE);
+                tma_load_3d(sV0 + s * AT_TILE, mv, kvh * 128, r0, bz, bar(5 + s), pol_kv);
+                tma_load_3d(sV0 + s * AT_TILE + AT_PANEL, mv, kvh * 128 + 64, r0, bz, bar(5 + s), pol_kv);
+            }
+            if (!MANY) break;
         }
     } else if (warp == 1) {
         // ---------------- MMA issuer 1: S = Q K^T (M 128, N 128, both operands K-major) ----------------
@@ -260,47 +283,59 @@ attention_tc_kernel(const AttnTcArgs a, const __grid_constant__ CUtensorMap mapQ
         // dependencies (P of tile j after S of tile j, S buffer reuse, O in tile order) all go through
         // mbarriers, so no ordering between the two threads is assumed.
         const uint32_t idesc_s = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(128 >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
-        bool ok = __all_sync(0xffffffffu, mbar_poll(bar(0), 0, abort_flag));
-        for (int j = 0; j < n_tiles && ok; ++j) {
-            const int s = j & 1;
-            const uint32_t par = (j >> 1) & 1;
-            if (!(ok = __all_sync(0xffffffffu, mbar_poll(bar(1 + s), par, abort_flag)))) break;          // K of tile j landed
-            // its S buffer also holds the P of tile j - 2: free once that tile's P V has completed
-            if (j >= 2 && !(ok = __all_sync(0xffffffffu, mbar_poll(bar(15 + s), ((j - 2) >> 1) & 1, abort_flag)))) break;
-            tc_fence_after();
-            const uint32_t k = sK0 + s * AT_TILE;
-            if (elect_lane()) {
+        bool ok = true;
+        uint32_t q_par = 0;
+        for (int item = first; item < a.n_items && ok; item += stride, J += n_tiles, q_par ^= 1) {
+            if (MANY) set_item(item);
+            ok = __all_sync(0xffffffffu, mbar_poll(bar(0), q_par, abort_flag));
+            for (int j = 0; j < n_tiles && ok; ++j) {
+                const int s = (J + j) & 1;
+                const uint32_t par = ((J + j) >> 1) & 1;
+                if (!(ok = __all_sync(0xffffffffu, mbar_poll(bar(1 + s), par, abort_flag)))) break;          // K of tile j landed
+                // its S buffer also holds the P of tile j - 2: free once that tile's P V has completed
+                if (J + j >= 2 && !(ok = __all_sync(0xffffffffu, mbar_poll(bar(15 + s), par ^ 1, abort_flag)))) break;
+                tc_fence_after();
+                const uint32_t k = sK0 + s * AT_TILE;
+                if (elect_lane()) {
 #pragma unroll
-                for (int ks = 0; ks < 8; ++ks) {
-                    const uint64_t da = smem_desc_sw128(sQ + (ks >> 2) * AT_PANEL) + (uint64_t)((ks & 3) * 2);
-                    const uint64_t db = smem_desc_sw128(k + (ks >> 2) * AT_PANEL) + (uint64_t)((ks & 3) * 2);
-                    tc_mma(tS0 + s * 128, da, db, idesc_s, ks > 0 ? 1u : 0u);
+                    for (int ks = 0; ks < 8; ++ks) {
+                        const uint64_t da = smem_desc_sw128(sQ + (ks >> 2) * AT_PANEL) + (uint64_t)((ks & 3) * 2);
+                        const uint64_t db = smem_desc_sw128(k + (ks >> 2) * AT_PANEL) + (uint64_t)((ks & 3) * 2);
+                        tc_mma(tS0 + s * 128, da, db, idesc_s, ks > 0 ? 1u : 0u);
+                    }
+                    tc_commit(bar(9 + s));     // s_full
+                    tc_commit(bar(3 + s));     // k_empty
                 }
-                tc_commit(bar(9 + s));     // s_full
-                tc_commit(bar(3 + s));     // k_empty
+                __syncwarp();
             }
-            __syncwarp();
+            if (!MANY) break;
         }
     } else if (warp == AT_THREADS / 32 - 1) {
         // ---------------- MMA issuer 2: O += P V (A = P K-major, B = V MN-major) ----------------
         const uint32_t idesc_o = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 16) | ((uint32_t)(128 >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
+        // (the P of an item's first tile comes from threads that have read the O of the item before)
         bool ok = true;
-        for (int j = 0; j < n_tiles && ok; ++j) {
-            const int s = j & 1;
-            if (!(ok = __all_sync(0xffffffffu, mbar_poll(bar(13 + s), (j >> 1) & 1, abort_flag)))) break;    // P of tile j written, O rescaled
-            if (!(ok = __all_sync(0xffffffffu, mbar_poll(bar(5 + s), (j >> 1) & 1, abort_flag)))) break;     // V of tile j landed
-            tc_fence_after();
-            const uint32_t v = sV0 + s * AT_TILE;
-            if (elect_lane()) {
+        for (int item = first; item < a.n_items && ok; item += stride, J += n_tiles) {
+            if (MANY) set_item(item);
+            for (int j = 0; j < n_tiles && ok; ++j) {
+                const int s = (J + j) & 1;
+                const uint32_t par = ((J + j) >> 1) & 1;
+                if (!(ok = __all_sync(0xffffffffu, mbar_poll(bar(13 + s), par, abort_flag)))) break;    // P of tile j written, O rescaled
+                if (!(ok = __all_sync(0xffffffffu, mbar_poll(bar(5 + s), par, abort_flag)))) break;     // V of tile j landed
+                tc_fence_after();
+                const uint32_t v = sV0 + s * AT_TILE;
+                if (elect_lane()) {
 #pragma unroll
-                for (int ks = 0; ks < 8; ++ks) {
-                    const uint64_t db = smem_desc_mn_sw128(v + ks * 2048);
-                    tc_mma_ta(tO, tS0 + s * 128 + ks * 8, db, idesc_o, (j > 0 || ks > 0) ? 1u : 0u);   // 16 keys = 8 columns of P
+                    for (int ks = 0; ks < 8; ++ks) {
+                        const uint64_t db = smem_desc_mn_sw128(v + ks * 2048);
+                        tc_mma_ta(tO, tS0 + s * 128 + ks * 8, db, idesc_o, (j > 0 || ks > 0) ? 1u : 0u);   // 16 keys = 8 columns of P
+                    }
+                    tc_commit(bar(15 + s));    // pv_done: O holds tiles 0..j, the S/P buffer is free
+                    tc_commit(bar(7 + s));     // v_empty
                 }
-                tc_commit(bar(15 + s));    // pv_done: O holds tiles 0..j, the S/P buffer is free
-                tc_commit(bar(7 + s));     // v_empty
+                __syncwarp();
             }
-            __syncwarp();
+            if (!MANY) break;
         }
     } else if (softmax) {
         // ---------------- softmax: four threads per query row ----------------
@@ -319,136 +354,150 @@ attention_tc_kernel(const AttnTcArgs a, const __grid_constant__ CUtensorMap mapQ
         const int row = q * 32 + lane;
         const uint32_t lane_off = (uint32_t)(q * 32) << 16;
         const uint32_t col_off = (uint32_t)(c4 * 32);
-        const int bq = G > 1 ? b0 + q : b;          // the request whose rows this quarter holds
         bool ok = true;
-        for (int j = 0; j < n_tiles; ++j) {
-            const int s = j & 1, jk = j0 + j;         // ring stage, key tile
-            // which of this thread's 32 keys count: the cache's positions up to the context end, minus those a
-            // fresh row serves; of the fresh rows, those that serve their position
-            uint32_t keep;
-            if (jk < n_cache_tiles) {
-                const int valid = a.ctx_len - jk * 128 - c4 * 32;
-                keep = valid >= 32 ? 0xffffffffu : (valid <= 0 ? 0u : (1u << valid) - 1u);
-                if (a.pos_excl && jk * 4 + c4 < a.excl_words) keep &= ~__ldg(a.pos_excl + (int64_t)bq * a.excl_words + jk * 4 + c4);
-            } else {
-                const int f = jk - n_cache_tiles;
-                if (G > 1 && f / a.n_fresh_tiles != q) {
-                    // another request's fresh rows: none of them is a key of this quarter's rows.  All four warps
-                    // of the quarter come here, so none of them goes to the quarter's barrier for this tile.
-                    if (ok && (ok = mbar_wait(bar(9 + s), (j >> 1) & 1, abort_flag))) {
-                        tc_fence_after();
-                        uint32_t pz[16];
+        for (int item = first; item < a.n_items; item += stride, J += n_tiles) {
+            if (MANY) set_item(item);
+            const int bq = G > 1 ? b0 + q : b;          // the request whose rows this quarter holds
+            if (MANY && q >= live_q) {                  // no rows in this quarter: report its P as written
+                for (int j = 0; j < n_tiles && ok; ++j) {
+                    ok = __all_sync(0xffffffffu, mbar_wait(bar(9 + ((J + j) & 1)), ((J + j) >> 1) & 1, abort_flag));
+                    if (ok && lane == 0) mbar_arrive(bar(13 + ((J + j) & 1)));
+                }
+                if (!ok) break;
+                continue;
+            }
+            m_use = -INFINITY;
+            l = 0.f;
+            for (int j = 0; j < n_tiles; ++j) {
+                const int s = (J + j) & 1, jk = j0 + j;   // ring stage, key tile
+                const uint32_t par = ((J + j) >> 1) & 1;
+                // which of this thread's 32 keys count: the cache's positions up to the context end, minus those a
+                // fresh row serves; of the fresh rows, those that serve their position
+                uint32_t keep;
+                if (jk < n_cache_tiles) {
+                    const int valid = a.ctx_len - jk * 128 - c4 * 32;
+                    keep = valid >= 32 ? 0xffffffffu : (valid <= 0 ? 0u : (1u << valid) - 1u);
+                    if (a.pos_excl && jk * 4 + c4 < a.excl_words) keep &= ~__ldg(a.pos_excl + (int64_t)bq * a.excl_words + jk * 4 + c4);
+                } else {
+                    const int f = jk - n_cache_tiles;
+                    if (G > 1 && f / a.n_fresh_tiles != q) {
+                        // another request's fresh rows: none of them is a key of this quarter's rows.  All four warps
+                        // of the quarter come here, so none of them goes to the quarter's barrier for this tile.
+                        if (ok && (ok = mbar_wait(bar(9 + s), par, abort_flag))) {
+                            tc_fence_after();
+                            uint32_t pz[16];
 #pragma unroll
-                        for (int i = 0; i < 16; ++i) pz[i] = 0u;
-                        tc_st16(tS0 + s * 128 + c4 * 16 + lane_off, pz);
-                        tc_wait_st();
-                        tc_fence_before();
-                        __syncwarp();
-                        if (lane == 0) mbar_arrive(bar(13 + s));
+                            for (int i = 0; i < 16; ++i) pz[i] = 0u;
+                            tc_st16(tS0 + s * 128 + c4 * 16 + lane_off, pz);
+                            tc_wait_st();
+                            tc_fence_before();
+                            __syncwarp();
+                            if (lane == 0) mbar_arrive(bar(13 + s));
+                        }
+                        continue;
                     }
-                    continue;
+                    const int w = (f % a.n_fresh_tiles) * 4 + c4;
+                    keep = w < a.keep_words ? __ldg(a.row_keep + (int64_t)bq * a.keep_words + w) : 0u;
                 }
-                const int w = (f % a.n_fresh_tiles) * 4 + c4;
-                keep = w < a.keep_words ? __ldg(a.row_keep + (int64_t)bq * a.keep_words + w) : 0u;
-            }
-            float sv[32];
-            float mt = -INFINITY;
-            if (ok && (ok = mbar_wait(bar(9 + s), (j >> 1) & 1, abort_flag))) {
-                tc_fence_after();
-                // this thread's quarter row of S into registers, masked keys as -inf
-                tc_ld32(tS0 + s * 128 + col_off + lane_off, sv);
-                if (keep != 0xffffffffu) {
-#pragma unroll
-                    for (int i = 0; i < 32; ++i) sv[i] = ((keep >> i) & 1u) ? sv[i] : -INFINITY;
-                }
-                float m4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
-#pragma unroll
-                for (int i = 0; i < 32; i += 2) m4[(i >> 1) & 3] = fmaxf(fmaxf(m4[(i >> 1) & 3], sv[i]), sv[i + 1]);
-                mt = fmaxf(fmaxf(m4[0], m4[1]), fmaxf(m4[2], m4[3])) * a.scale_log2e;
-            }
-            // The four threads of a row must use the same reference.  It moves on the first tile and seldom after; whether it
-            // has to is one vote of the four warps that share these 32 rows, at the barrier that they need anyway (every
-            // thread of a row must have read its S columns before P overwrites them).  A thread whose wait ran out votes too.
-            bool raise = false;
-            if (quarter_any(1 + q, !ok || mt - m_use > kRescaleGap)) {
-                // all take the largest of the four quarter-row maxima rounded up to 16 significant bits (an upper bound is
-                // all the exponent needs)
-                uint32_t mb = __float_as_uint(mt);
-                if ((mb & 0xFFFFu) && !(mb >> 31)) mb += 0x10000u;
-                mb >>= 16;
-                row_max[c4][row] = (uint16_t)mb;
-                if (quarter_any(1 + q, !ok)) { ok = false; break; }      // the four warps leave together
-                mt = fmaxf(fmaxf(__uint_as_float((uint32_t)row_max[0][row] << 16), __uint_as_float((uint32_t)row_max[1][row] << 16)),
-                           fmaxf(__uint_as_float((uint32_t)row_max[2][row] << 16), __uint_as_float((uint32_t)row_max[3][row] << 16)));
-                if (j == 0) m_use = mt;
-                else raise = mt - m_use > kRescaleGap;
-            }
-            if (__any_sync(0xffffffffu, raise)) {
-                // O may only be touched once the P V of tile j - 1 has completed
-                if ((ok = mbar_wait(bar(15 + ((j - 1) & 1)), ((j - 1) >> 1) & 1, abort_flag))) {
+                float sv[32];
+                float mt = -INFINITY;
+                if (ok && (ok = mbar_wait(bar(9 + s), par, abort_flag))) {
                     tc_fence_after();
-                    const float f = raise ? fast_exp2(m_use - mt) : 1.f;
-                    float v[32];
-                    tc_ld32(tO + lane_off + col_off, v);
+                    // this thread's quarter row of S into registers, masked keys as -inf
+                    tc_ld32(tS0 + s * 128 + col_off + lane_off, sv);
+                    if (keep != 0xffffffffu) {
 #pragma unroll
-                    for (int i = 0; i < 32; ++i) v[i] *= f;
-                    tc_st32(tO + lane_off + col_off, v);
-                    tc_wait_st();
-                    l *= f;
-                    if (raise) m_use = mt;
+                        for (int i = 0; i < 32; ++i) sv[i] = ((keep >> i) & 1u) ? sv[i] : -INFINITY;
+                    }
+                    float m4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+#pragma unroll
+                    for (int i = 0; i < 32; i += 2) m4[(i >> 1) & 3] = fmaxf(fmaxf(m4[(i >> 1) & 3], sv[i]), sv[i + 1]);
+                    mt = fmaxf(fmaxf(m4[0], m4[1]), fmaxf(m4[2], m4[3])) * a.scale_log2e;
+                }
+                // The four threads of a row must use the same reference.  It moves on the first tile and seldom after; whether it
+                // has to is one vote of the four warps that share these 32 rows, at the barrier that they need anyway (every
+                // thread of a row must have read its S columns before P overwrites them).  A thread whose wait ran out votes too.
+                bool raise = false;
+                if (quarter_any(1 + q, !ok || mt - m_use > kRescaleGap)) {
+                    // all take the largest of the four quarter-row maxima rounded up to 16 significant bits (an upper bound is
+                    // all the exponent needs)
+                    uint32_t mb = __float_as_uint(mt);
+                    if ((mb & 0xFFFFu) && !(mb >> 31)) mb += 0x10000u;
+                    mb >>= 16;
+                    row_max[c4][row] = (uint16_t)mb;
+                    if (quarter_any(1 + q, !ok)) { ok = false; break; }      // the four warps leave together
+                    mt = fmaxf(fmaxf(__uint_as_float((uint32_t)row_max[0][row] << 16), __uint_as_float((uint32_t)row_max[1][row] << 16)),
+                               fmaxf(__uint_as_float((uint32_t)row_max[2][row] << 16), __uint_as_float((uint32_t)row_max[3][row] << 16)));
+                    if (j == 0) m_use = mt;
+                    else raise = mt - m_use > kRescaleGap;
+                }
+                if (__any_sync(0xffffffffu, raise)) {
+                    // O may only be touched once the P V of tile j - 1 has completed
+                    if ((ok = mbar_wait(bar(15 + (s ^ 1)), ((J + j - 1) >> 1) & 1, abort_flag))) {
+                        tc_fence_after();
+                        const float f = raise ? fast_exp2(m_use - mt) : 1.f;
+                        float v[32];
+                        tc_ld32(tO + lane_off + col_off, v);
+#pragma unroll
+                        for (int i = 0; i < 32; ++i) v[i] *= f;
+                        tc_st32(tO + lane_off + col_off, v);
+                        tc_wait_st();
+                        l *= f;
+                        if (raise) m_use = mt;
+                    }
+                }
+                if (!ok) continue;
+                // P overwrites the S buffer in tensor memory: 32 keys = 16 columns of two bf16 at column 16 c4
+                // (every thread of the row has read its S columns: they all passed the vote above)
+                const float neg = m_use > -INFINITY ? -m_use : 0.f;      // no key of the row has counted yet: all P are 0
+                const float2 scale2 = make_float2(a.scale_log2e, a.scale_log2e), neg2 = make_float2(neg, neg);
+                float2 l2a = make_float2(0.f, 0.f), l2b = l2a;
+                uint32_t pk[16];
+                auto exps = [&](auto all_kept) {
+#pragma unroll
+                    for (int i = 0; i < 32; i += 4) {
+                        const float2 xa = __ffma2_rn(make_float2(sv[i], sv[i + 1]), scale2, neg2);
+                        const float2 xb = __ffma2_rn(make_float2(sv[i + 2], sv[i + 3]), scale2, neg2);
+                        const float2 pa = make_float2(fast_exp2(xa.x), fast_exp2(xa.y));
+                        const float2 pb = make_float2(fast_exp2(xb.x), all_kept.value ? poly_exp2(xb.y) : fast_exp2(xb.y));
+                        l2a = __fadd2_rn(l2a, pa);
+                        l2b = __fadd2_rn(l2b, pb);
+                        pk[i >> 1] = pack_bf16(pa.x, pa.y);
+                        pk[(i >> 1) + 1] = pack_bf16(pb.x, pb.y);
+                    }
+                };
+                if (keep == 0xffffffffu) exps(std::true_type{});
+                else exps(std::false_type{});
+                tc_st16(tS0 + s * 128 + c4 * 16 + lane_off, pk);
+                tc_wait_st();
+                l += (l2a.x + l2a.y) + (l2b.x + l2b.y);
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(bar(13 + s));   // p_full
+            }
+            // epilogue: O / l once the last P V has completed; the denominators of the four quarters add up
+            if (ok && n_tiles > 0) ok = mbar_wait(bar(15 + ((J + n_tiles - 1) & 1)), ((J + n_tiles - 1) >> 1) & 1, abort_flag);
+            row_sum[c4][row] = l;
+            if (quarter_any(1 + q, !ok)) break;         // the four warps leave together
+            l = (row_sum[0][row] + row_sum[1][row]) + (row_sum[2][row] + row_sum[3][row]);
+            if (C == 1) {
+                tc_fence_after();
+                const int grow = G > 1 ? lane : qt * 128 + row;     // the row inside its request
+                const float inv = 1.f / l;
+                __nv_bfloat16* out = static_cast<__nv_bfloat16*>(a.o) + (((int64_t)bq * a.n + grow) * a.n_heads + h) * 128 + col_off;
+                float v[32];
+                tc_ld32(tO + lane_off + col_off, v);
+                if (grow < a.n) {
+#pragma unroll
+                    for (int k8 = 0; k8 < 4; ++k8) {
+                        const float* pv = v + k8 * 8;
+                        *reinterpret_cast<uint4*>(out + k8 * 8) =
+                            make_uint4(pack_bf16(pv[0] * inv, pv[1] * inv), pack_bf16(pv[2] * inv, pv[3] * inv),
+                                       pack_bf16(pv[4] * inv, pv[5] * inv), pack_bf16(pv[6] * inv, pv[7] * inv));
+                    }
                 }
             }
-            if (!ok) continue;
-            // P overwrites the S buffer in tensor memory: 32 keys = 16 columns of two bf16 at column 16 c4
-            // (every thread of the row has read its S columns: they all passed the vote above)
-            const float neg = m_use > -INFINITY ? -m_use : 0.f;      // no key of the row has counted yet: all P are 0
-            const float2 scale2 = make_float2(a.scale_log2e, a.scale_log2e), neg2 = make_float2(neg, neg);
-            float2 l2a = make_float2(0.f, 0.f), l2b = l2a;
-            uint32_t pk[16];
-            auto exps = [&](auto all_kept) {
-#pragma unroll
-                for (int i = 0; i < 32; i += 4) {
-                    const float2 xa = __ffma2_rn(make_float2(sv[i], sv[i + 1]), scale2, neg2);
-                    const float2 xb = __ffma2_rn(make_float2(sv[i + 2], sv[i + 3]), scale2, neg2);
-                    const float2 pa = make_float2(fast_exp2(xa.x), fast_exp2(xa.y));
-                    const float2 pb = make_float2(fast_exp2(xb.x), all_kept.value ? poly_exp2(xb.y) : fast_exp2(xb.y));
-                    l2a = __fadd2_rn(l2a, pa);
-                    l2b = __fadd2_rn(l2b, pb);
-                    pk[i >> 1] = pack_bf16(pa.x, pa.y);
-                    pk[(i >> 1) + 1] = pack_bf16(pb.x, pb.y);
-                }
-            };
-            if (keep == 0xffffffffu) exps(std::true_type{});
-            else exps(std::false_type{});
-            tc_st16(tS0 + s * 128 + c4 * 16 + lane_off, pk);
-            tc_wait_st();
-            l += (l2a.x + l2a.y) + (l2b.x + l2b.y);
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(bar(13 + s));   // p_full
-        }
-        // epilogue: O / l once the last P V has completed; the denominators of the four quarters add up
-        if (ok && n_tiles > 0) ok = mbar_wait(bar(15 + ((n_tiles - 1) & 1)), ((n_tiles - 1) >> 1) & 1, abort_flag);
-        float* row_sum = reinterpret_cast<float*>(base_ptr + AT_TILE);         // the K stages are idle now
-        row_sum[c4 * 128 + row] = l;
-        asm volatile("bar.sync %0, 128;" ::"r"(1 + q) : "memory");
-        l = (row_sum[row] + row_sum[128 + row]) + (row_sum[256 + row] + row_sum[384 + row]);
-        if (C == 1 && ok && !*abort_flag) {
-            tc_fence_after();
-            const int grow = G > 1 ? lane : qt * 128 + row;     // the row inside its request
-            const float inv = 1.f / l;
-            __nv_bfloat16* out = static_cast<__nv_bfloat16*>(a.o) + (((int64_t)bq * a.n + grow) * a.n_heads + h) * 128 + col_off;
-            float v[32];
-            tc_ld32(tO + lane_off + col_off, v);
-            if (grow < a.n) {
-#pragma unroll
-                for (int k8 = 0; k8 < 4; ++k8) {
-                    const float* pv = v + k8 * 8;
-                    *reinterpret_cast<uint4*>(out + k8 * 8) =
-                        make_uint4(pack_bf16(pv[0] * inv, pv[1] * inv), pack_bf16(pv[2] * inv, pv[3] * inv),
-                                   pack_bf16(pv[4] * inv, pv[5] * inv), pack_bf16(pv[6] * inv, pv[7] * inv));
-                }
-            }
+            if (!MANY) break;
         }
     }
     if (C > 1) {
@@ -456,7 +505,7 @@ attention_tc_kernel(const AttnTcArgs a, const __grid_constant__ CUtensorMap mapQ
         // (reference, denominator) of every row meet first; each CTA scales its O to the common reference and lays it out by
         // the CTA that finishes the columns (128 / C each), which sums the parts in rank order.  The K and V stages are idle
         // by now.  All threads pass the three cluster barriers, whatever happened before.
-        float2* ml = reinterpret_cast<float2*>(base_ptr + AT_TILE + 4096);             // [128], behind row_sum
+        float2* ml = reinterpret_cast<float2*>(base_ptr + AT_TILE + 4096);             // [128]
         const uint32_t parts = base + 2 * AT_TILE;                                     // [owner][column / 4][row][4] fp32
         const int q = warp & 3, c4 = (warp - 2) >> 2, row = q * 32 + lane, width = 128 / C;
         __syncwarp();
@@ -1081,7 +1130,8 @@ int launch_attention_tc(const AttnArgs& a, uint32_t* status, cudaStream_t stream
     if (!mq || !mk || !mv || !mkn || !mvn) return 0;
     static bool attr = false;
     if (!attr) {
-        cudaFuncSetAttribute(attention_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, AT_SMEM);
+        cudaFuncSetAttribute(attention_tc_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, AT_SMEM);
+        cudaFuncSetAttribute(attention_tc_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, AT_SMEM);
         cudaFuncSetAttribute(attention_tc2q_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, AT2_SMEM);
         attr = true;
     }
@@ -1090,7 +1140,7 @@ int launch_attention_tc(const AttnArgs& a, uint32_t* status, cudaStream_t stream
     t.scale_log2e = 1.4426950408889634f / sqrtf(128.f);
     t.status = status;
     t.cache_shared = shared ? 1 : 0;
-    t.group = group; t.batch = a.batch;
+    t.group = group; t.batch = a.batch; t.q_tiles = q_tiles;
     if (two_src) {
         t.n_fresh_tiles = (n_fresh + 127) / 128; t.excl_words = a.excl_words; t.keep_words = a.keep_words;
         t.pos_excl = a.pos_excl; t.row_keep = a.row_keep;      // with key_drop the caller has OR-ed it into pos_excl
@@ -1105,7 +1155,7 @@ int launch_attention_tc(const AttnArgs& a, uint32_t* status, cudaStream_t stream
     static const int mode_2q = [] { const char* e = getenv("ACACHE_ATTN_TC2Q"); return e ? atoi(e) : 1; }();
     const bool fused_score = a.score_rowmask && a.score_partial && group == 1;
     if (fused_score) {
-        t.score_rowmask = a.score_rowmask; t.score_partial = a.score_partial; t.rm_words = a.rm_words; t.q_tiles = q_tiles;
+        t.score_rowmask = a.score_rowmask; t.score_partial = a.score_partial; t.rm_words = a.rm_words;
         t.affix_start = a.affix_start; t.affix_len = a.affix_len; t.score_norm_full = a.score_norm_full;
     }
     // the scores are taken from the logits in the two-query-tile kernel only
@@ -1126,7 +1176,11 @@ int launch_attention_tc(const AttnArgs& a, uint32_t* status, cudaStream_t stream
         t.split = 1;
         while (t.split < 8 && ctas * t.split * 2 <= 148 && tiles >= t.split * 4) t.split *= 2;
         cudaLaunchConfig_t cfg{};
-        cfg.gridDim = dim3(q_tiles * t.split, a.n_heads, groups);
+        t.n_items = (int)ctas;
+        // from six rounds of CTAs on, items share a CTA (13.8 rounds: 1 % of the layer-step; at 1.9 and 2.8 rounds, where
+        // the hardware's assignment evens out the last round, 0.3 and 0.9 % slower)
+        const bool many = t.split == 1 && t.n_items >= 6 * sm_count();
+        cfg.gridDim = dim3(many ? sm_count() : t.n_items * t.split);
         cfg.blockDim = dim3(AT_THREADS);
         cfg.dynamicSmemBytes = AT_SMEM;
         cfg.stream = stream;
@@ -1137,7 +1191,7 @@ int launch_attention_tc(const AttnArgs& a, uint32_t* status, cudaStream_t stream
         at[1].val.clusterDim.x = t.split; at[1].val.clusterDim.y = 1; at[1].val.clusterDim.z = 1;
         cfg.attrs = at;
         cfg.numAttrs = t.split > 1 ? 2 : 1;
-        err = cudaLaunchKernelEx(&cfg, attention_tc_kernel, t, *mq, *mk, *mv, *mkn, *mvn);
+        err = cudaLaunchKernelEx(&cfg, many ? attention_tc_kernel<true> : attention_tc_kernel<false>, t, *mq, *mk, *mv, *mkn, *mvn);
     }
     return err == cudaSuccess ? 1 : -1;
 }

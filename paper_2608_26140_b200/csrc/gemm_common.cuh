@@ -440,7 +440,6 @@ __device__ __forceinline__ void prep_phase_many(const GemmArgs& g, PrepShared<TH
 // gemm_tc.cu; the returned pointer is good until the next lookup (copy the map), under g_map_mutex.
 const CUtensorMap* get_panel_map(const void* ptr, int rows, int cols, int box_rows, int panels, int half);
 extern std::mutex g_map_mutex;
-int sm_count();
 
 // gemm_rows.cu: projections of at most 128 rows whose tiles fit the SMs at once; 0 = not applicable (the caller then uses
 // the kernels of gemm_tc.cu), else the number of kernels launched, -1 if a launch failed.

@@ -5,6 +5,8 @@
 
 namespace acache {
 
+int sm_count();           // of the current device (gemm_tc.cu)
+
 // ---- rows.cu ----------------------------------------------------------------------------
 // cache[b, pos_r] = new[b, r] for K and V; rows with an invalid position are skipped.
 void launch_scatter_kv(void* cache_k, void* cache_v, int64_t batch_stride, int ctx_len,

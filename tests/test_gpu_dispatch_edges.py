@@ -145,3 +145,31 @@ def test_attention_reference_moves(T, rows, drop):
     assert dc.ctx.poll_status() == 0
     ref = oracle_step(case, 0, anchor_idx=anchors[0], drop_non_anchor=drop)
     assert_close_bf16(ab.to_host_bits(y[0]), ref["y"], "y")
+
+
+# many more (query tile, head, request) items than SMs: several per CTA, the last round incomplete; query tiles with empty
+# quarters, and four requests to a tile over a shared cache with a last group of two
+HEADS32 = wl.LayerShape(256, 32, 4, 128, 256, 1e-5, False, 5e5, "heads32")
+
+
+@pytest.mark.parametrize("B,T,rows,shared", [(30, 300, 40, False), (15, 4200, 203, False), (118, 160, 9, True)])
+def test_attention_items_per_cta(B, T, rows, shared):
+    lay = wl.make_layout(B, 3, T - 27, 8, 8, 8, "none")
+    case = wl.make_case(HEADS32, lay, 0.0, cfg_id=77, weights=cached_weights(HEADS32, 77))
+    dc = DeviceCase(case, max_rows=rows)
+    rng = np.random.default_rng(T)
+    anchors = np.stack([np.sort(rng.choice(lay.affix_len, rows, replace=False)) for _ in range(B)]).astype(np.int32)
+    da = torch.from_numpy(anchors).to(DEV)
+    if shared:
+        dsk, dsv = ab.to_device_bf16(case.cache_k[:1].copy(), DEV), ab.to_device_bf16(case.cache_v[:1].copy(), DEV)
+        k_new = torch.zeros((B, rows, 4, 128), dtype=torch.bfloat16, device=DEV)
+        v_new, y = torch.zeros_like(k_new), torch.zeros((B, rows, 256), dtype=torch.bfloat16, device=DEV)
+        dc.ctx.recompute_anchors(dc.lw, dc.req, ab.KV(dsk.data_ptr(), dsv.data_ptr(), 0, T), dc.x, 0, da, rows, k_new, v_new, y)
+    else:
+        y = run_layer_step(dc, (rows - 0.5) / lay.affix_len, 0, anchors)[3]
+    assert dc.ctx.poll_status() == 0
+    for b in (0, 1, B // 2, B - 1):
+        c = 0 if shared else b
+        ref = orc.layer_step(case.weights, HEADS32, case.x[b], case.cache_k[c], case.cache_v[c], T, lay.affix_start, lay.affix_len,
+                             lay.masked_pos[b], lay.extra_rows[b], case.rope_cos, case.rope_sin, anchor_idx=anchors[b])
+        assert_close_bf16(ab.to_host_bits(y[b]), ref["y"], "y")
