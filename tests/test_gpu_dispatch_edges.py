@@ -16,13 +16,17 @@ pytestmark = pytest.mark.gpu
 
 @pytest.mark.parametrize("V,B,n_blk", [
     (1280, 4, 32),        # 128 rows: the last size of the one-SM kernel
-    (1280, 3, 43),        # 129 rows: two SMs per tile, the second row tile nearly empty, K cut between clusters
+    (1280, 3, 43),        # 129 rows: two SMs per tile, the second row tile nearly empty
     (2688, 3, 43),        # an odd number of 128-wide vocabulary units: one SM
     (65536, 5, 29),       # whole tiles, 145 rows
     (16384, 19, 31),      # whole tiles, 589 rows: three row pairs, the last one without a second row tile
 ])
 def test_lm_head_tiles(V, B, n_blk):
     check_predict_commit(wl.TINY, V, B, 64, n_blk)
+
+
+def test_lm_head_cut_tiles():     # ten tiles of 129 rows, K = 2048 cut between the clusters
+    check_predict_commit(wl.LayerShape(2048, 2, 1, 128, 256, 1e-5, False, 5e5, "lm-head-cut"), 2560, 3, 64, 43)
 
 
 @pytest.mark.parametrize("T", [51200, 51201])     # the last context whose position map fits shared memory, the first past it
@@ -116,12 +120,15 @@ def test_attention_key_split(T, rows, drop):
 # rows of 5376 columns take a warp each in the row preparation, narrower ones go through in batches: one row per CTA up to
 # several batches of them
 WIDE128 = wl.LayerShape(5376, 2, 1, 128, 256, 1e-5, False, 5e5, "wide-d128")
+# K long enough for few tiles to be cut between clusters, in the q/k/v and the gate/up projection
+LONGK128 = wl.LayerShape(3584, 4, 1, 128, 1024, 1e-6, True, 1e6, "longk-d128")
 # an odd number of 128-column units: the last weight tile is half past the end of the row, whole or cut
 ODD_TILES = wl.LayerShape(1920, 2, 1, 128, 256, 1e-5, False, 5e5, "odd-tiles")
 
 
 @pytest.mark.parametrize("shape,rows", [(ODD_TILES, n) for n in (9, 128, 140, 300)]
-                         + [(MID128, 129), (MID128, 257), (MID128, 600), (WIDE128, 140), (WIDE128, 300)])
+                         + [(MID128, 129), (MID128, 257), (MID128, 600), (WIDE128, 140), (WIDE128, 300)]
+                         + [(LONGK128, 129), (LONGK128, 385)])
 def test_row_counts_of_wide_shapes(shape, rows):
     lay = wl.make_layout(1, 3, rows + 40, 8, 8, 8, "none")
     case = wl.make_case(shape, lay, 0.0, cfg_id=75)
