@@ -294,10 +294,11 @@ __device__ __forceinline__ void rmsnorm_row_warp(const uint4* __restrict__ xr, c
     }
 }
 
-// Phase 0 of the projection kernels: the rows of R (or compact rows) -> RMSNorm -> the A operand, then a grid-wide barrier;
-// the rows are read back through TMA.  With no more rows than CTAs a whole CTA takes a row (shortest latency); with more
-// every warp takes rows of its own.
-__device__ __forceinline__ void prep_rows_plain(const GemmArgs& g, float* red) {
+// Phase 0 of the projection kernels: the rows of R (or compact rows) -> RMSNorm -> the A operand,
+// then a grid-wide barrier; the rows are read back through TMA.  With no more rows than CTAs a
+// whole CTA takes a row (shortest latency); with many rows every warp takes rows of its own, which
+// keeps six rows in flight per SM instead of one.
+__device__ __forceinline__ void prep_phase(const GemmArgs& g, float* red, volatile int* abort_flag) {
     const RowPrep& rp = g.prep;
     const __nv_bfloat16* x = static_cast<const __nv_bfloat16*>(rp.x);
     __nv_bfloat16* a_out = static_cast<__nv_bfloat16*>(const_cast<void*>(g.a));
@@ -324,114 +325,9 @@ __device__ __forceinline__ void prep_rows_plain(const GemmArgs& g, float* red) {
             src = src_next;
         }
     }
-}
-// More than 128 rows: every CTA takes its share of them, up to kPrepRows at once, with all threads on each row.  The loads of
-// a batch are in flight together, one round through shared memory sums all its rows, and the gain, a constant input, is in
-// registers before the dependency wait (rows of up to two 16-byte pieces per thread; wider ones: a warp per row).  Against a
-// warp per row for all: layer-step of 615 rows 396.7 -> 390.7 us, of 5 x 203 rows 531.0 -> 523.6, decode pass of 512 rows
-// over 4 layers 1952 -> 1929.  In the kernels of at most 128 rows, a row per CTA, the same code was slower (layer-step of 8
-// rows 53.6 -> 55.8 us, of 103 rows 149.7 -> 152.1).
-constexpr int kPrepRows = 6;
-template <int THREADS>
-struct PrepShared {
-    float red[kPrepRows][THREADS / 32];
-    int64_t src[kPrepRows];
-};
-struct PrepGain {
-    uint4 v[2];
-    bool fits;
-};
-__device__ __forceinline__ void prep_gain(const GemmArgs& g, PrepGain& gain) {
-    const int nchunk = g.K >> 3;
-    gain.fits = nchunk <= 2 * (int)blockDim.x;
-#pragma unroll
-    for (int i = 0; i < 2; ++i) {
-        const int c = threadIdx.x + i * blockDim.x;
-        gain.v[i] = gain.fits && c < nchunk ? __ldg(reinterpret_cast<const uint4*>(g.prep.gain) + c) : make_uint4(0u, 0u, 0u, 0u);
-    }
-}
-template <int THREADS>
-__device__ __forceinline__ void prep_rows_batched(const GemmArgs& g, PrepShared<THREADS>& sh, const PrepGain& gain) {
-    const RowPrep& rp = g.prep;
-    const __nv_bfloat16* x = static_cast<const __nv_bfloat16*>(rp.x);
-    const int nchunk = g.K >> 3, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int share = (g.M + gridDim.x - 1) / gridDim.x, batches = (share + kPrepRows - 1) / kPrepRows;
-    const int per = (share + batches - 1) / batches;
-    const int end = min((int)(blockIdx.x + 1) * share, g.M);
-#pragma unroll 1
-    for (int row0 = blockIdx.x * share; row0 < end; row0 += per) {
-        const int n = min(per, end - row0);
-        if ((int)threadIdx.x < n) sh.src[threadIdx.x] = prep_row_source(g, row0 + threadIdx.x, true);
-        __syncthreads();
-        uint4 u[kPrepRows][2];
-        float ss[kPrepRows];
-#pragma unroll
-        for (int r = 0; r < kPrepRows; ++r) {
-            const uint4* xr = reinterpret_cast<const uint4*>(x + (r < n ? sh.src[r] : 0));
-#pragma unroll
-            for (int i = 0; i < 2; ++i) {
-                const int c = threadIdx.x + i * blockDim.x;
-                u[r][i] = r < n && c < nchunk ? __ldcg(xr + c) : make_uint4(0u, 0u, 0u, 0u);
-            }
-        }
-#pragma unroll
-        for (int r = 0; r < kPrepRows; ++r) {
-            ss[r] = 0.f;
-            if (r < n) {
-#pragma unroll
-                for (int i = 0; i < 2; ++i) {
-                    const uint32_t w[4] = {u[r][i].x, u[r][i].y, u[r][i].z, u[r][i].w};
-#pragma unroll
-                    for (int e = 0; e < 4; ++e) { const float p = bf16_lo(w[e]), q = bf16_hi(w[e]); ss[r] += p * p + q * q; }
-                }
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) ss[r] += __shfl_xor_sync(0xffffffffu, ss[r], o);
-                if (lane == 0) sh.red[r][warp] = ss[r];
-            }
-        }
-        __syncthreads();
-#pragma unroll
-        for (int r = 0; r < kPrepRows; ++r) {
-            if (r < n) {
-                float tot = 0.f;
-#pragma unroll
-                for (int i = 0; i < THREADS / 32; ++i) tot += sh.red[r][i];
-                const float rstd = rsqrtf(tot / (float)g.K + rp.eps);
-                uint4* out = static_cast<uint4*>(const_cast<void*>(g.a)) + (int64_t)(row0 + r) * nchunk;
-                uint4* raw = rp.raw_out ? static_cast<uint4*>(rp.raw_out) + (int64_t)(row0 + r) * nchunk : nullptr;
-#pragma unroll
-                for (int i = 0; i < 2; ++i) {
-                    const int c = threadIdx.x + i * blockDim.x;
-                    if (c < nchunk) {
-                        if (raw) raw[c] = u[r][i];
-                        const uint32_t w[4] = {u[r][i].x, u[r][i].y, u[r][i].z, u[r][i].w};
-                        const uint32_t gw[4] = {gain.v[i].x, gain.v[i].y, gain.v[i].z, gain.v[i].w};
-                        uint32_t o[4];
-#pragma unroll
-                        for (int e = 0; e < 4; ++e)
-                            o[e] = pack_bf16(bf16_lo(w[e]) * rstd * bf16_lo(gw[e]), bf16_hi(w[e]) * rstd * bf16_hi(gw[e]));
-                        out[c] = make_uint4(o[0], o[1], o[2], o[3]);
-                    }
-                }
-            }
-        }
-        __syncthreads();
-    }
-}
-__device__ __forceinline__ void prep_barrier(const GemmArgs& g, volatile int* abort_flag) {
     asm volatile("fence.proxy.async;" ::: "memory");   // the rows are read back through TMA
     grid_barrier(g.grid_bar, abort_flag, g.debug_expire != 0);
     asm volatile("fence.proxy.async;" ::: "memory");
-}
-__device__ __forceinline__ void prep_phase(const GemmArgs& g, float* red, volatile int* abort_flag) {
-    prep_rows_plain(g, red);
-    prep_barrier(g, abort_flag);
-}
-template <int THREADS>
-__device__ __forceinline__ void prep_phase_many(const GemmArgs& g, PrepShared<THREADS>& sh, const PrepGain& gain, volatile int* abort_flag) {
-    if (gain.fits) prep_rows_batched<THREADS>(g, sh, gain);
-    else prep_rows_plain(g, sh.red[0]);
-    prep_barrier(g, abort_flag);
 }
 
 // Tensor map over bf16 [rows, cols] row-major with the panel of 64 columns as a dimension: box = 64 columns x box_rows rows x

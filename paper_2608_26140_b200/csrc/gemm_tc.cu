@@ -629,7 +629,7 @@ gemm_tc2_kernel(const GemmArgs g, const TcPlan p, const int clusters, const __gr
                 const __grid_constant__ CUtensorMap mapB0, const __grid_constant__ CUtensorMap mapB1,
                 const __grid_constant__ CUtensorMap mapB2) {
     extern __shared__ unsigned char smem_raw[];
-    __shared__ PrepShared<TC2_THREADS> prep_sh;
+    __shared__ float red[TC2_THREADS / 32];
     const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     unsigned char* base_ptr = smem_raw + (base - smem_u32(smem_raw));
     const uint32_t bars = base + TC2_STAGES * TC2_STAGE_BYTES;
@@ -659,12 +659,10 @@ gemm_tc2_kernel(const GemmArgs g, const TcPlan p, const int clusters, const __gr
     cluster_sync_all();          // the peer's barriers are initialised before anyone signals them
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
-    PrepGain gain{};
-    if (g.prep.enabled) prep_gain(g, gain);
     pdl_wait();
     pdl_launch_dependents();
 
-    if (g.prep.enabled) prep_phase_many(g, prep_sh, gain, abort_flag);
+    if (g.prep.enabled) prep_phase(g, red, abort_flag);
 
     const int m_pairs = (p.m_tiles + 1) >> 1;
     const int tiles = m_pairs * p.n_tiles;

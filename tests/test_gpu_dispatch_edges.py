@@ -117,8 +117,7 @@ def test_attention_key_split(T, rows, drop):
     assert_close_bf16(ab.to_host_bits(y[0]), ref["y"], "y")
 
 
-# rows of 5376 columns take a warp each in the row preparation, narrower ones go through in batches: one row per CTA up to
-# several batches of them
+# rows that no longer fit a warp's registers in the row preparation
 WIDE128 = wl.LayerShape(5376, 2, 1, 128, 256, 1e-5, False, 5e5, "wide-d128")
 # K long enough for few tiles to be cut between clusters, in the q/k/v and the gate/up projection
 LONGK128 = wl.LayerShape(3584, 4, 1, 128, 1024, 1e-6, True, 1e6, "longk-d128")
