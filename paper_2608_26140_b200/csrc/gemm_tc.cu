@@ -1079,10 +1079,11 @@ GemmLaunch plan_gemm(const GemmArgs& g) {
         // Cutting tiles pays up to about two thirds of a wave, unless K is so short that the finish costs what the shorter main
         // loop gains: of a whole tile's time the cut loop took 0.66-0.70 at 0.44 of its K blocks and 0.83-0.90 at 0.65 (partial
         // tiles included), the finish that of about 20 K blocks.  (us, whole | cut + finish: 512 rows output 32.0 | 22.3 + 7.3,
-        // down 67.1 | 43.0 + 7.1; 615 rows output 31.3 | 27.9 + 9.3, down 73.5 | 61.0 + 9.5.)
+        // down 67.1 | 43.0 + 7.1; 615 rows output 31.3 | 27.9 + 9.3, down 73.5 | 61.0 + 9.5.)  Below half a wave always: whole tiles
+        // leave too few CTAs for the row preparation (refresh of 166 rows of 256 columns 199.8 us cut, 203.3 whole).
         static const int stream_k_pct = [] { const char* e = getenv("ACACHE_GEMM_PAIR_STREAMK_PCT"); return e ? atoi(e) : 66; }();
         const int64_t total = (int64_t)tiles * p.KB;
-        if (tiles * 100 <= stream_k_pct * max_clusters && 1.05 * tiles / max_clusters + 20.0 / p.KB < 0.8) {
+        if (tiles * 100 <= stream_k_pct * max_clusters && (tiles * 2 < max_clusters || 1.05 * tiles / max_clusters + 20.0 / p.KB < 0.8)) {
             gl.clusters = (int)std::min<int64_t>(max_clusters, total);
             p.pair_u = (int)((total + gl.clusters - 1) / gl.clusters);
             gl.clusters = (int)((total + p.pair_u - 1) / p.pair_u);
