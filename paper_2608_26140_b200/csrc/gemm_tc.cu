@@ -375,7 +375,7 @@ __global__ void __launch_bounds__(256, 2) prep_rows_kernel(const GemmArgs g) {
     while (row < g.M) {
         const int next = row + gridDim.x * nw;
         const int64_t src_next = next < g.M ? prep_row_source(g, next, lane == 0) : 0;
-        rmsnorm_row_warp(reinterpret_cast<const uint4*>(x + src), reinterpret_cast<const uint4*>(rp.gain),
+        rmsnorm_row_warp<false>(reinterpret_cast<const uint4*>(x + src), reinterpret_cast<const uint4*>(rp.gain),
                          reinterpret_cast<uint4*>(a_out + (int64_t)row * g.K), g.K, rp.eps, lane,
                          raw ? reinterpret_cast<uint4*>(raw + (int64_t)row * g.K) : nullptr);
         row = next;
@@ -662,7 +662,7 @@ gemm_tc2_kernel(const GemmArgs g, const TcPlan p, const int clusters, const __gr
     pdl_wait();
     pdl_launch_dependents();
 
-    if (g.prep.enabled) prep_phase(g, red, abort_flag);
+    if (g.prep.enabled) prep_phase<true>(g, red, abort_flag);
 
     const int m_pairs = (p.m_tiles + 1) >> 1;
     const int tiles = m_pairs * p.n_tiles;
