@@ -302,16 +302,16 @@ __device__ __forceinline__ void rmsnorm_row_warp(const uint4* __restrict__ xr, c
 }
 
 // Phase 0 of the projection kernels: the rows of R (or compact rows) -> RMSNorm -> the A operand,
-// then a grid-wide barrier; the rows are read back through TMA.  With no more rows than CTAs a
+// then a grid-wide barrier; the rows are read back through TMA.  With no more rows than CTAs (cta_rows) a
 // whole CTA takes a row (shortest latency); with many rows every warp takes rows of its own, which
 // keeps six rows in flight per SM instead of one.
 template <bool GAIN_EARLY = false>
-__device__ __forceinline__ void prep_phase(const GemmArgs& g, float* red, volatile int* abort_flag) {
+__device__ __forceinline__ void prep_phase(const GemmArgs& g, float* red, volatile int* abort_flag, int cta_rows) {
     const RowPrep& rp = g.prep;
     const __nv_bfloat16* x = static_cast<const __nv_bfloat16*>(rp.x);
     __nv_bfloat16* a_out = static_cast<__nv_bfloat16*>(const_cast<void*>(g.a));
     __nv_bfloat16* raw = static_cast<__nv_bfloat16*>(rp.raw_out);
-    if (g.M <= (int)gridDim.x) {
+    if (g.M <= cta_rows) {
         for (int row = blockIdx.x; row < g.M; row += gridDim.x) {
             const int64_t src = prep_row_source(g, row, threadIdx.x == 0);
             rmsnorm_row(reinterpret_cast<const uint4*>(x + src), reinterpret_cast<const uint4*>(rp.gain),

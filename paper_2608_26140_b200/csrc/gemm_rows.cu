@@ -6,6 +6,14 @@
 // one CTA or to a cluster of S = 2 or 4 CTAs that split K; the cluster's partial accumulators meet in distributed shared
 // memory, every CTA finishing its share of the columns, and the epilogue follows in the same kernel.
 //
+// Small projections (the general kernel would give every CTA one K block) keep its order of sums: every block of 64 K columns
+// has an accumulator of its own in tensor memory, and they are added in ascending order, a CTA of a cluster handing over its
+// blocks one by one.  A row's result is then what the general kernel gives, whatever the tile, the split and the number of
+// rows: narrow models predict from near ties (2-4 % of the rows of a 256-column model with 2048 tokens have a second choice
+// within 0.02 of the first), which another order of sums, though no less precise, decides differently.  Price: layer-step of
+// 58 rows of 256 columns 51.2 -> 53.1 us (the sums' code is a loop over the blocks: unrolled by four, its instructions' way
+// from L2 made that 54.3).
+//
 // A ring stage holds CP panels of 64 K columns, loaded by one TMA instruction per operand box (3-d and 4-d tensor maps: the
 // panel is a dimension of the box), so that a stage's fixed cost of waits and issue is shared by more bytes.
 //
@@ -13,6 +21,7 @@
 // lane quarter x column half).  All eight take part in the row preparation before (prep_phase).  Every wait on an mbarrier
 // or the grid barrier is bounded as in gemm_tc.cu; the cluster barriers are passed by every CTA whatever happened before.
 #include <algorithm>
+#include <type_traits>
 
 #include "common.cuh"
 #include "gemm_common.cuh"
@@ -33,6 +42,9 @@ struct RowsPlan {
     int rows_pad;             // M rounded up to 8: rows of an A panel
     int R, n_units;           // weight rows per box, boxes per stage
     int mma_n, mma_count;     // columns per instruction, instructions per 16 K columns (one panel: the boxes lie side by side)
+    int KB, apart;            // K blocks of 64; 1: an accumulator per K block, added in order
+    int cta_rows;             // row preparation: a whole CTA per row up to this many rows, a warp above (rows of more than 256
+                              // columns are then summed in another order: apart, as many as the general kernel would take)
     int stages, stage_bytes;
     int tmem_cols;
     int groups;               // q/k/v: groups of 32 rotary pairs over all segments
@@ -114,6 +126,12 @@ struct WeightBoxes {
     }
 };
 
+// K blocks of 64 that rank r of a cluster multiplies.
+template <int S>
+__device__ __forceinline__ int rank_panels(const RowsPlan& p, int r) {
+    return min((r + 1) * p.blocks / S * p.CP, p.KB) - r * p.blocks / S * p.CP;
+}
+
 // 16 adjacent accumulator columns of this thread's row, summed over the cluster: own tensor memory first, then the peers in
 // rank order (fixed, hence bitwise reproducible).  slice_col: the columns' place inside the slice this CTA finishes;
 // peers: where it lies in each peer's staging area (cluster addresses).
@@ -139,7 +157,49 @@ __device__ __forceinline__ void sum_cluster16(uint32_t taddr, const uint32_t (&p
     }
 }
 
-template <int S, int EPI>
+// The same 16 columns where every K block has its own accumulator: all blocks of the tile in ascending order, rank by rank.
+// per_block: bytes between a peer's blocks in the staging area.
+template <int S>
+__device__ __forceinline__ void sum_apart16(const RowsPlan& p, int rank, uint32_t taddr, const uint32_t (&peers)[S > 1 ? S - 1 : 1],
+                                            int slice_col, int per_block, int row, float (&v)[16]) {
+#pragma unroll
+    for (int j = 0; j < 16; ++j) v[j] = 0.f;
+    const int r = min(row, p.rows_pad - 1);
+#pragma unroll
+    for (int c = 0; c < S; ++c) {
+        const int nb = rank_panels<S>(p, c);
+        if (c == rank) {
+#pragma unroll 1
+            for (int i = 0; i < nb; ++i) {
+                float t[16];
+                tc_ld16(taddr + i * p.TN, t);
+#pragma unroll
+                for (int j = 0; j < 16; ++j) v[j] += t[j];
+            }
+        } else if (S > 1) {
+            // (peers holds the other ranks; c < rank: its c-th, else its (c - 1)-th)
+            const uint32_t src = (c < rank ? peers[c < S - 1 ? c : 0] : peers[c > 0 ? c - 1 : 0]) + (((slice_col >> 2) * p.rows_pad + r) << 4);
+#pragma unroll 1
+            for (int i0 = 0; i0 < nb; i0 += 4) {
+                float4 t[4][4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) t[i][j] = ld_cluster_f4(src + min(i0 + i, nb - 1) * per_block + ((j * p.rows_pad) << 4));
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+                    if (i0 + i < nb) {
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) {
+                            v[4 * j] += t[i][j].x; v[4 * j + 1] += t[i][j].y; v[4 * j + 2] += t[i][j].z; v[4 * j + 3] += t[i][j].w;
+                        }
+                    }
+            }
+        }
+    }
+}
+
+template <int S, int EPI, bool APART>
 __global__ void __launch_bounds__(RW_THREADS, 1)
 gemm_rows_kernel(const GemmArgs g, const RowsPlan p, const __grid_constant__ CUtensorMap mapA,
                  const __grid_constant__ CUtensorMap mapB0, const __grid_constant__ CUtensorMap mapB1,
@@ -207,7 +267,7 @@ gemm_rows_kernel(const GemmArgs g, const RowsPlan p, const __grid_constant__ CUt
     pdl_wait();
     pdl_launch_dependents();
 
-    if (g.prep.enabled) prep_phase(g, red, abort_flag);
+    if (g.prep.enabled) prep_phase(g, red, abort_flag, p.cta_rows);
 
     // ---------------- the contraction ----------------
     if (threadIdx.x == 0) {
@@ -241,14 +301,16 @@ gemm_rows_kernel(const GemmArgs g, const RowsPlan p, const __grid_constant__ CUt
             tc_fence_after();
             if (elect_lane()) {
                 const uint32_t sA = base + stage * p.stage_bytes, sB = sA + a_bytes;
-                for (int c = 0; c < p.CP; ++c) {
+                const int panels = APART ? min(p.CP, p.KB - (blk0 + i) * p.CP) : p.CP;     // past K a panel has no accumulator
+                for (int c = 0; c < panels; ++c) {
+                    const uint32_t acc = tmem_base + (APART ? (i * p.CP + c) * p.TN : 0);
                     const uint64_t da = smem_desc_sw128(sA + c * p.rows_pad * 128);
                     for (int u = 0; u < p.mma_count; ++u) {
                         const uint64_t db = smem_desc_sw128(sB + u * box_bytes + c * p.R * 128);
 #pragma unroll
                         for (int k = 0; k < 4; ++k)
-                            tc_mma(tmem_base + u * p.mma_n, da + (uint64_t)(k * 2), db + (uint64_t)(k * 2), idesc,
-                                   (i > 0 || c > 0 || k > 0) ? 1u : 0u);
+                            tc_mma(acc + u * p.mma_n, da + (uint64_t)(k * 2), db + (uint64_t)(k * 2), idesc,
+                                   (k > 0 || (!APART && (i > 0 || c > 0))) ? 1u : 0u);
                     }
                 }
                 tc_commit(empty_bar(stage));
@@ -268,7 +330,9 @@ gemm_rows_kernel(const GemmArgs g, const RowsPlan p, const __grid_constant__ CUt
     // the columns this CTA finishes: items of 16 + 16 rotary pairs (q/k/v), of 16 columns (residual), of 8 + 8 (SwiGLU)
     constexpr int UNIT = EPI == kEpiQKV ? 32 : 16;
     const int items = p.TN / UNIT, item0 = rank * items / S, item1 = (rank + 1) * items / S;
-    const int region = (items + S - 1) / S * UNIT * p.rows_pad * 4;
+    // staging of the slice of one destination: [block (one if not APART)][column / 4][row][4]
+    const int per_block = (items + S - 1) / S * UNIT * p.rows_pad * 4;
+    const int region = per_block * (APART ? (p.blocks + S - 1) / S * p.CP : 1);
 
     // what does not depend on the sums is requested while the weights stream
     int pos = 0;
@@ -297,27 +361,30 @@ gemm_rows_kernel(const GemmArgs g, const RowsPlan p, const __grid_constant__ CUt
     tc_fence_after();
     uint32_t peers[S > 1 ? S - 1 : 1] = {};
     if (S > 1) {
-        // the other CTAs' slices to the staging area (the ring: every MMA that read it has completed), layout
-        // [destination][column / 4][row][4]
+        // the other CTAs' slices to the staging area (the ring: every MMA that read it has completed)
         if (ok && live) {
             int at = 0;
             for (int d = 0; d < S; ++d) {
                 if (d == rank) continue;
                 const int u0 = d * items / S, u1 = (d + 1) * items / S;
+                const int nb = APART ? rank_panels<S>(p, rank) : 1;
                 for (int u = u0 + hf; u < u1; u += 2) {
 #pragma unroll
                     for (int part = 0; part < UNIT / 16; ++part) {
                         const int col = EPI == kEpiQKV ? (u >> 1) * 64 + (u & 1) * 16 + part * 32 : u * 16;
-                        float v[16];
-                        tc_ld16(taddr + col, v);
                         const int sc = ((u - u0) * UNIT + part * 16) >> 2;
-                        if (row < p.rows_pad) {
+#pragma unroll 1
+                        for (int blk = 0; blk < nb; ++blk) {
+                            float v[16];
+                            tc_ld16(taddr + blk * p.TN + col, v);
+                            if (row < p.rows_pad) {
 #pragma unroll
-                            for (int j = 0; j < 4; ++j)
-                                asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};"
-                                             ::"r"(base + at * region + (((sc + j) * p.rows_pad + row) << 4)), "f"(v[4 * j]),
-                                               "f"(v[4 * j + 1]), "f"(v[4 * j + 2]), "f"(v[4 * j + 3])
-                                             : "memory");
+                                for (int j = 0; j < 4; ++j)
+                                    asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};"
+                                                 ::"r"(base + at * region + blk * per_block + (((sc + j) * p.rows_pad + row) << 4)),
+                                                   "f"(v[4 * j]), "f"(v[4 * j + 1]), "f"(v[4 * j + 2]), "f"(v[4 * j + 3])
+                                                 : "memory");
+                            }
                         }
                     }
                 }
@@ -336,6 +403,10 @@ gemm_rows_kernel(const GemmArgs g, const RowsPlan p, const __grid_constant__ CUt
     // Once a warp has read its last piece of the peers' staging areas they may leave; it says so before its stores, which the
     // arrival would otherwise wait for (here, in the scoring and in the attention: layer-step of 8 rows 52.2 -> 51.8 us, of
     // 103 rows 143.65 -> 143.2).
+    auto sum16 = [&](int col, int slice_col, float (&v)[16]) {
+        if (APART) sum_apart16<S>(p, rank, taddr + col, peers, slice_col, per_block, row, v);
+        else sum_cluster16<S>(taddr + col, peers, slice_col, p.rows_pad, row, v);
+    };
     bool arrived = S == 1;
     auto last_read = [&](bool last) {
         if (!arrived && last) { cluster_arrive(); arrived = true; }
@@ -346,7 +417,7 @@ gemm_rows_kernel(const GemmArgs g, const RowsPlan p, const __grid_constant__ CUt
             if (EPI == kEpiResidual) {
                 const int col = nt * p.TN + u * 16;
                 float v[16];
-                sum_cluster16<S>(taddr + u * 16, peers, sc, p.rows_pad, row, v);
+                sum16(u * 16, sc, v);
                 last_read(u + 2 >= item1);
                 if (valid && col < g.n[0]) {
                     if (u != item0 + hf) { res[0] = __ldcg(res_row + (col >> 3)); res[1] = __ldcg(res_row + (col >> 3) + 1); }
@@ -359,6 +430,17 @@ gemm_rows_kernel(const GemmArgs g, const RowsPlan p, const __grid_constant__ CUt
                 const int col = nt * (p.TN >> 1) + u * 8;
                 float gate[8], up[8];
                 tc_ld8x2(taddr + u * 8, taddr + (p.TN >> 1) + u * 8, gate, up);
+                if (APART) {
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) { gate[i] += 0.f; up[i] += 0.f; }        // -0 becomes 0, as in a sum from 0
+#pragma unroll 1
+                    for (int blk = 1; blk < p.KB; ++blk) {
+                        float a[8], b[8];
+                        tc_ld8x2(taddr + blk * p.TN + u * 8, taddr + blk * p.TN + (p.TN >> 1) + u * 8, a, b);
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) { gate[i] += a[i]; up[i] += b[i]; }
+                    }
+                }
                 if (valid && col < g.n[0]) {
 #pragma unroll
                     for (int i = 0; i < 8; ++i) gate[i] = silu(gate[i]) * up[i];
@@ -370,8 +452,8 @@ gemm_rows_kernel(const GemmArgs g, const RowsPlan p, const __grid_constant__ CUt
                 const int seg = pair_group(g, min(grp, p.groups - 1), col);
                 col += (u & 1) * 16;
                 float lo[16], hi[16];
-                sum_cluster16<S>(taddr + (u >> 1) * 64 + (u & 1) * 16, peers, sc, p.rows_pad, row, lo);
-                sum_cluster16<S>(taddr + (u >> 1) * 64 + (u & 1) * 16 + 32, peers, sc + 16, p.rows_pad, row, hi);
+                sum16((u >> 1) * 64 + (u & 1) * 16, sc, lo);
+                sum16((u >> 1) * 64 + (u & 1) * 16 + 32, sc + 16, hi);
                 last_read(u + 2 >= item1);
                 if (valid && grp < p.groups) {
                     rope_qkv<16>(g, seg, col, lo, hi, c, sn);
@@ -409,10 +491,10 @@ gemm_rows_kernel(const GemmArgs g, const RowsPlan p, const __grid_constant__ CUt
 // ---- host side ------------------------------------------------------------------------------
 namespace {
 
-template <int S, int EPI>
+template <int S, int EPI, bool APART>
 cudaError_t launch_rows(const GemmArgs& g, const RowsPlan& p, const CUtensorMap& a, const CUtensorMap* b, cudaStream_t stream) {
     static const cudaError_t attr =
-        cudaFuncSetAttribute(gemm_rows_kernel<S, EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024);
+        cudaFuncSetAttribute(gemm_rows_kernel<S, EPI, APART>, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024);
     if (attr != cudaSuccess) return attr;
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(p.n_tiles * S);
@@ -426,7 +508,7 @@ cudaError_t launch_rows(const GemmArgs& g, const RowsPlan& p, const CUtensorMap&
     at[1].val.clusterDim.x = S; at[1].val.clusterDim.y = 1; at[1].val.clusterDim.z = 1;
     cfg.attrs = at;
     cfg.numAttrs = S > 1 ? 2 : 1;
-    return cudaLaunchKernelEx(&cfg, gemm_rows_kernel<S, EPI>, g, p, a, b[0], b[1], b[2]);
+    return cudaLaunchKernelEx(&cfg, gemm_rows_kernel<S, EPI, APART>, g, p, a, b[0], b[1], b[2]);
 }
 
 // Clusters of S CTAs that are resident at once with one CTA per SM (the SM counts of the GPCs are not multiples of S).
@@ -434,7 +516,7 @@ template <int S>
 int resident_clusters() {
     static const int n = [] {
         if (S == 1) return sm_count();
-        cudaFuncSetAttribute(gemm_rows_kernel<S, kEpiResidual>, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024);
+        cudaFuncSetAttribute(gemm_rows_kernel<S, kEpiResidual, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024);
         cudaLaunchConfig_t cfg{};
         cfg.gridDim = dim3(sm_count() / S * S);
         cfg.blockDim = dim3(RW_THREADS);
@@ -445,7 +527,7 @@ int resident_clusters() {
         cfg.attrs = at;
         cfg.numAttrs = 1;
         int c = 0;
-        if (cudaOccupancyMaxActiveClusters(&c, gemm_rows_kernel<S, kEpiResidual>, &cfg) != cudaSuccess) { (void)cudaGetLastError(); c = 0; }
+        if (cudaOccupancyMaxActiveClusters(&c, gemm_rows_kernel<S, kEpiResidual, false>, &cfg) != cudaSuccess) { (void)cudaGetLastError(); c = 0; }
         return c;
     }();
     return n;
@@ -457,13 +539,18 @@ int resident_clusters() {
 // takes as many panels as leave three stages in the ring (fewer, larger stages lost, two stages of any size did too).
 // Measured when it replaced that kernel, at 103 rows (us per launch, finish included | here): q/k/v 30.2 | 29.6, output
 // 16.3 | 13.0, gate/up 47.7 | 43, down 25.7 | 23.4; at 32 rows output 14.3 | 10.9, down 25.0 | 20.4.
-constexpr int kRingBytes = 200 * 1024;
+// With an accumulator per K block the tile is at most what 256 columns of tensor memory hold (two CTAs then fit an SM), and a
+// doubling of the split costs 2.5 us, for every block is exchanged (58 rows, 1024 -> 256 columns in the chain above: over two
+// CTAs 1.4 us slower than in one).
+constexpr int kRingBytes = 200 * 1024, kApartColumns = 256;
 bool plan_rows(const GemmArgs& g, RowsPlan& best) {
     if (g.M > 128 || g.epilogue == kEpiLogits || g.K < 64) return false;
     const bool qkv = g.epilogue == kEpiQKV, swiglu = g.epilogue == kEpiSwiGLU;
     const int n_total = swiglu ? 2 * g.n[0] : g.n[0] + g.n[1] + g.n[2];
     const int KB = g.K / 64, rows_pad = (g.M + 7) & ~7;
-    const int step = qkv ? 64 : swiglu ? 16 : 32;
+    const int general_iterations = (swiglu ? g.n[0] / 128 : (n_total / 128 + 1) / 2) * KB;      // of the general kernel
+    const bool apart = general_iterations <= sm_count();
+    const int step = qkv ? 64 : swiglu || apart ? 16 : 32;
     const int limit[3] = {resident_clusters<1>(), resident_clusters<2>(), resident_clusters<4>()};
     double t_best = 1e30;
     for (int si = 0; si < (swiglu ? 1 : 3); ++si) {
@@ -478,10 +565,12 @@ bool plan_rows(const GemmArgs& g, RowsPlan& best) {
             const int blocks = (KB + CP - 1) / CP;
             if (blocks < S) continue;
             const int my_blocks = (blocks + S - 1) / S;
+            const int accs = apart ? my_blocks * CP : 1;        // accumulators of a CTA
+            if (apart && accs * TN > kApartColumns) continue;
             const int stages = std::min(std::min(kRingBytes / (CP * panel), RW_MAX_STAGES), my_blocks);
-            const int region = (items + S - 1) / S * (qkv ? 32 : 16) * rows_pad * 4;
+            const int region = (items + S - 1) / S * (qkv ? 32 : 16) * rows_pad * 4 * accs;
             const double t_hbm = 2.0 * n_total * g.K / 6.5e6, t_sm = (double)my_blocks * CP * panel / 60e3;
-            const double t = std::max(std::max(t_hbm, t_sm), my_blocks * 0.15) + si * (qkv ? 1.5 : 1.0);
+            const double t = std::max(std::max(t_hbm, t_sm), my_blocks * 0.15) + si * (apart ? 2.5 : qkv ? 1.5 : 1.0);
             if (t >= t_best * 0.999) continue;
             t_best = t;
             best = RowsPlan{};
@@ -491,7 +580,9 @@ bool plan_rows(const GemmArgs& g, RowsPlan& best) {
             best.mma_n = CP == 1 ? TN : best.R;
             best.mma_count = CP == 1 ? 1 : best.n_units;
             best.stages = stages; best.stage_bytes = CP * panel;
-            best.tmem_cols = TN <= 32 ? 32 : TN <= 64 ? 64 : TN <= 128 ? 128 : 256;
+            best.KB = KB; best.apart = apart;
+            best.cta_rows = apart && g.K > 256 ? general_iterations : n_tiles * S;
+            best.tmem_cols = accs * TN <= 32 ? 32 : accs * TN <= 64 ? 64 : accs * TN <= 128 ? 128 : 256;
             best.groups = n_total / 64;
             // the MMA reads 128 rows of A whatever M is: the last panel's read may run past the ring
             const int ring = std::max(stages * CP * panel, (stages - 1) * CP * panel + (CP - 1) * rows_pad * 128 + 128 * 128);
@@ -520,15 +611,19 @@ int launch_gemm_rows(const GemmArgs& g, cudaStream_t stream) {
         }
     }
     cudaError_t e = cudaErrorInvalidValue;
-    if (g.epilogue == kEpiSwiGLU) e = launch_rows<1, kEpiSwiGLU>(g, p, map_a, map_b, stream);
-    else if (g.epilogue == kEpiResidual)
-        e = p.S == 1 ? launch_rows<1, kEpiResidual>(g, p, map_a, map_b, stream)
-          : p.S == 2 ? launch_rows<2, kEpiResidual>(g, p, map_a, map_b, stream)
-                     : launch_rows<4, kEpiResidual>(g, p, map_a, map_b, stream);
-    else
-        e = p.S == 1 ? launch_rows<1, kEpiQKV>(g, p, map_a, map_b, stream)
-          : p.S == 2 ? launch_rows<2, kEpiQKV>(g, p, map_a, map_b, stream)
-                     : launch_rows<4, kEpiQKV>(g, p, map_a, map_b, stream);
+    auto launch = [&](auto epi, auto apart) {
+        constexpr int EPI = decltype(epi)::value;
+        constexpr bool APART = decltype(apart)::value;
+        if constexpr (EPI == kEpiSwiGLU) return launch_rows<1, EPI, APART>(g, p, map_a, map_b, stream);
+        else
+            return p.S == 1 ? launch_rows<1, EPI, APART>(g, p, map_a, map_b, stream)
+                 : p.S == 2 ? launch_rows<2, EPI, APART>(g, p, map_a, map_b, stream)
+                            : launch_rows<4, EPI, APART>(g, p, map_a, map_b, stream);
+    };
+    auto launch_epi = [&](auto epi) { return p.apart ? launch(epi, std::true_type{}) : launch(epi, std::false_type{}); };
+    if (g.epilogue == kEpiSwiGLU) e = launch_epi(std::integral_constant<int, kEpiSwiGLU>{});
+    else if (g.epilogue == kEpiResidual) e = launch_epi(std::integral_constant<int, kEpiResidual>{});
+    else e = launch_epi(std::integral_constant<int, kEpiQKV>{});
     return e == cudaSuccess ? 1 : -1;
 }
 

@@ -440,7 +440,7 @@ gemm_tc_kernel(const GemmArgs g, const TcPlan p, const __grid_constant__ CUtenso
     pdl_launch_dependents();
 
     // ---------------- phase 0: gather the rows of R and RMSNorm them into A ----------------
-    if (g.prep.enabled) prep_phase(g, red, abort_flag);
+    if (g.prep.enabled) prep_phase(g, red, abort_flag, gridDim.x);
 
     // ---------------- phase 1: the contraction ----------------
 
@@ -662,7 +662,7 @@ gemm_tc2_kernel(const GemmArgs g, const TcPlan p, const int clusters, const __gr
     pdl_wait();
     pdl_launch_dependents();
 
-    if (g.prep.enabled) prep_phase<true>(g, red, abort_flag);
+    if (g.prep.enabled) prep_phase<true>(g, red, abort_flag, gridDim.x);
 
     const int m_pairs = (p.m_tiles + 1) >> 1;
     const int tiles = m_pairs * p.n_tiles;

@@ -179,3 +179,38 @@ def test_attention_items_per_cta(B, T, rows, shared):
         ref = orc.layer_step(case.weights, HEADS32, case.x[b], case.cache_k[c], case.cache_v[c], T, lay.affix_start, lay.affix_len,
                              lay.masked_pos[b], lay.extra_rows[b], case.rope_cos, case.rope_sin, anchor_idx=anchors[b])
         assert_close_bf16(ab.to_host_bits(y[b]), ref["y"], "y")
+
+
+# Small projections sum K in the general kernel's order, block by block: a row's bits do not depend on how many rows are in the
+# call, on the tile or on the split over a cluster (140 rows take the two-SM kernel).  Every product is reached with inputs that
+# the other rows of a call do not change: no queries, hence equal weights over equal values, so that the attention's output is
+# the bias of V exactly.
+NARROW512 = wl.LayerShape(512, 2, 1, 128, 512, 1e-6, True, 1e6, "narrow-512")       # eight blocks: q/k/v over two CTAs
+NARROW1K = wl.LayerShape(1024, 1, 1, 128, 384, 1e-6, True, 1e6, "narrow-1k")        # sixteen: q/k/v on the general kernel
+
+
+@pytest.mark.parametrize("shape,counts", [(wl.TINY_GQA, (1, 9, 60, 128)), (NARROW512, (40, 57, 128)), (NARROW1K, (49, 128))])
+def test_small_projections_do_not_depend_on_the_number_of_rows(shape, counts):
+    lay = wl.make_layout(1, 3, 200, 8, 8, 8, "none")
+    case = wl.make_case(shape, lay, 0.0, cfg_id=78)
+    w = dict(case.weights)
+    for name in ("wq", "bq", "wv"):
+        w[name] = np.zeros_like(w[name])
+    w["bv"] = orc.f64_to_bf16_bits(np.random.default_rng(78).standard_normal(w["bv"].shape))
+    case.weights = w
+    case.cache_v[:] = w["bv"].reshape(case.cache_v.shape[2:])
+    dc = DeviceCase(case, max_rows=140)
+    rows = np.sort(np.random.default_rng(79).choice(200, 140, replace=False)).astype(np.int32)
+
+    def outputs(anchors):
+        k_new, v_new, y = run_split_calls(dc, torch.from_numpy(anchors[None].copy()).to(DEV), len(anchors))
+        assert dc.ctx.poll_status() == 0
+        assert torch.equal(v_new[0], dc.cv[0, :len(anchors)])
+        return k_new[0], y[0]
+
+    k_all, y_all = outputs(rows)
+    for n in counts:
+        pick = np.sort(np.random.default_rng(n).choice(140, n, replace=False))
+        k_new, y = outputs(rows[pick])
+        at = torch.from_numpy(pick).to(DEV)
+        assert torch.equal(k_new, k_all[at]) and torch.equal(y, y_all[at]), n
