@@ -601,6 +601,7 @@ constexpr int TC2_SMEM = TC2_STAGES * TC2_STAGE_BYTES + 1024 + 256;
 // (4, 24, 32, 48 are slower), and cutting the row pairs into L2-sized blocks as well changes nothing more.
 constexpr int kTileGroupN = 16;
 constexpr int kKeepWeightsFromPairs = 3;
+constexpr int kWholeTilesFromKB = 56;     // K blocks from which whole tiles were measured against cut ones (plan_gemm)
 constexpr int kPrepKernelRows = 4096;     // from this many rows the row preparation is a kernel of its own
 __device__ __forceinline__ void tile_coords(int t, int m_pairs, int n_tiles, int group_n, int& nt, int& mp) {
     const int full = n_tiles / group_n, per_group = group_n * m_pairs;
@@ -1081,9 +1082,13 @@ GemmLaunch plan_gemm(const GemmArgs& g) {
         // tiles included), the finish that of about 20 K blocks.  (us, whole | cut + finish: 512 rows output 32.0 | 22.3 + 7.3,
         // down 67.1 | 43.0 + 7.1; 615 rows output 31.3 | 27.9 + 9.3, down 73.5 | 61.0 + 9.5.)  Below half a wave always: whole tiles
         // leave too few CTAs for the row preparation (refresh of 166 rows of 256 columns 199.8 us cut, 203.3 whole).
+        // Below 3584 columns (kWholeTilesFromKB) always too, although whole tiles are faster there (refresh of 1100 rows of 256
+        // columns, 4 layers: 299 us whole, 324 cut): whole tiles add the K blocks in another order, no less precise, but narrow
+        // models predict from near ties (1-2.5 % of the tokens of such passes changed).
         static const int stream_k_pct = [] { const char* e = getenv("ACACHE_GEMM_PAIR_STREAMK_PCT"); return e ? atoi(e) : 66; }();
         const int64_t total = (int64_t)tiles * p.KB;
-        if (tiles * 100 <= stream_k_pct * max_clusters && (tiles * 2 < max_clusters || 1.05 * tiles / max_clusters + 20.0 / p.KB < 0.8)) {
+        if (tiles * 100 <= stream_k_pct * max_clusters &&
+            (p.KB < kWholeTilesFromKB || tiles * 2 < max_clusters || 1.05 * tiles / max_clusters + 20.0 / p.KB < 0.8)) {
             gl.clusters = (int)std::min<int64_t>(max_clusters, total);
             p.pair_u = (int)((total + gl.clusters - 1) / gl.clusters);
             gl.clusters = (int)((total + p.pair_u - 1) / p.pair_u);

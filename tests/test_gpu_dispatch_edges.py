@@ -214,3 +214,19 @@ def test_small_projections_do_not_depend_on_the_number_of_rows(shape, counts):
         k_new, y = outputs(rows[pick])
         at = torch.from_numpy(pick).to(DEV)
         assert torch.equal(k_new, k_all[at]) and torch.equal(y, y_all[at]), n
+
+
+# With 256 columns of K, gate/up of these row counts fills 43, 54 and 65 % of a wave with pair tiles: cut, hence with a finish
+# kernel, in all three (whole tiles would add the K blocks in another order).
+def test_short_contractions_are_cut_up_to_two_thirds_of_a_wave():
+    lay = wl.make_layout(1, 3, 1500, 8, 8, 8, "none")
+    case = wl.make_case(wl.TINY, lay, 0.0, cfg_id=80)
+    launches = []
+    for rows in (1000, 1100, 1500):
+        dc = DeviceCase(case, max_rows=rows)
+        anchors = np.sort(np.random.default_rng(rows).choice(1500, rows, replace=False)).astype(np.int32)[None]
+        k_new, v_new, y = run_split_calls(dc, torch.from_numpy(anchors).to(DEV), rows)
+        assert dc.ctx.poll_status() == 0
+        check_against_oracle(dc, anchors, k_new, v_new, y, None, None, rows)
+        launches.append(dc.ctx.launch_count())
+    assert launches[0] == launches[1] == launches[2]
