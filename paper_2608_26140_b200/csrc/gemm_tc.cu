@@ -602,6 +602,7 @@ constexpr int TC2_SMEM = TC2_STAGES * TC2_STAGE_BYTES + 1024 + 256;
 constexpr int kTileGroupN = 16;
 constexpr int kKeepWeightsFromPairs = 3;
 constexpr int kWholeTilesFromKB = 56;     // K blocks from which whole tiles were measured against cut ones (plan_gemm)
+constexpr int kSmallHeadPairs = 3, kSmallHeadBlocks = 24;   // an LM head stays on the one-SM kernel up to: row pairs, K blocks per CTA
 constexpr int kPrepKernelRows = 4096;     // from this many rows the row preparation is a kernel of its own
 __device__ __forceinline__ void tile_coords(int t, int m_pairs, int n_tiles, int group_n, int& nt, int& mp) {
     const int full = n_tiles / group_n, per_group = group_n * m_pairs;
@@ -1065,13 +1066,19 @@ GemmLaunch plan_gemm(const GemmArgs& g) {
     // contiguous ranges, one per cluster (stream-K), and the cut tiles go through the finish kernel.
     // The LM head comes here as well: on the one-SM kernel, which reads every weight tile once per 128 rows and moves twice
     // the shared-memory bytes per flop, 512 rows x 126 464 x 4096 took 670 us with its finish, here 379 us (decode
-    // pass of 16 requests, 4 layers: 2349 -> 2025 us).
+    // pass of 16 requests, 4 layers: 2349 -> 2025 us).  Except a small one, whose tiles would be cut here, over few rows
+    // (us with its row preparation and reduction, one SM | two: 512 rows x 2048 x 256 21.5 | 24.2, 129 x 2560 x 2048
+    // 22.2 | 27.3, 700 x 2048 x 1024 32.2 | 36.4, 700 x 2048 x 4096 (21 K blocks per CTA) 41.5 | 44.7; but 512 x 4096 x 4096
+    // (28) 43.9 | 42.4, 1300 x 2048 x 256 (six row pairs) 43.7 | 35.4, and whole tiles, 160 x 16384 x 4096, 59.0 | 42.4).
     static const int pair_min_tiles = [] { const char* e = getenv("ACACHE_GEMM_PAIR_MIN_MTILES"); return e ? atoi(e) : 2; }();
     const int max_clusters = pair_max_clusters();
-    if (p.m_tiles >= pair_min_tiles && (p.units % 2 == 0 || swiglu) && max_clusters >= 1) {
+    static const int stream_k_pct = [] { const char* e = getenv("ACACHE_GEMM_PAIR_STREAMK_PCT"); return e ? atoi(e) : 66; }();
+    const int m_pairs = (p.m_tiles + 1) / 2;
+    const int tiles = m_pairs * p.n_tiles;
+    const bool below_cut = tiles * 100 <= stream_k_pct * max_clusters;
+    const bool small_head = g.epilogue == kEpiLogits && below_cut && m_pairs <= kSmallHeadPairs && p.U <= kSmallHeadBlocks;
+    if (p.m_tiles >= pair_min_tiles && (p.units % 2 == 0 || swiglu) && max_clusters >= 1 && !small_head) {
         gl.pair = true;
-        const int m_pairs = (p.m_tiles + 1) / 2;
-        const int tiles = m_pairs * p.n_tiles;
         p.m_pairs = m_pairs;
         static const int group_n = [] { const char* e = getenv("ACACHE_GEMM_GROUP_N"); return e && atoi(e) > 0 ? atoi(e) : kTileGroupN; }();
         p.group_n = group_n;
@@ -1084,11 +1091,11 @@ GemmLaunch plan_gemm(const GemmArgs& g) {
         // leave too few CTAs for the row preparation (refresh of 166 rows of 256 columns 199.8 us cut, 203.3 whole).
         // Below 3584 columns (kWholeTilesFromKB) always too, although whole tiles are faster there (refresh of 1100 rows of 256
         // columns, 4 layers: 299 us whole, 324 cut): whole tiles add the K blocks in another order, no less precise, but narrow
-        // models predict from near ties (1-2.5 % of the tokens of such passes changed).
-        static const int stream_k_pct = [] { const char* e = getenv("ACACHE_GEMM_PAIR_STREAMK_PCT"); return e ? atoi(e) : 66; }();
+        // models predict from near ties (1-2.5 % of the tokens of such passes changed).  (Not the LM head: its logits stay fp32, and
+        // 780 rows x 2560 x 2048 took 35.8 us whole, 41.3 cut.)
         const int64_t total = (int64_t)tiles * p.KB;
-        if (tiles * 100 <= stream_k_pct * max_clusters &&
-            (p.KB < kWholeTilesFromKB || tiles * 2 < max_clusters || 1.05 * tiles / max_clusters + 20.0 / p.KB < 0.8)) {
+        if (below_cut &&
+            ((p.KB < kWholeTilesFromKB && g.epilogue != kEpiLogits) || tiles * 2 < max_clusters || 1.05 * tiles / max_clusters + 20.0 / p.KB < 0.8)) {
             gl.clusters = (int)std::min<int64_t>(max_clusters, total);
             p.pair_u = (int)((total + gl.clusters - 1) / gl.clusters);
             gl.clusters = (int)((total + p.pair_u - 1) / p.pair_u);

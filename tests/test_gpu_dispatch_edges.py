@@ -16,7 +16,9 @@ pytestmark = pytest.mark.gpu
 
 @pytest.mark.parametrize("V,B,n_blk", [
     (1280, 4, 32),        # 128 rows: the last size of the one-SM kernel
-    (1280, 3, 43),        # 129 rows: two SMs per tile, the second row tile nearly empty
+    (1280, 3, 43),        # 129 rows, few tiles: one SM, the second row tile nearly empty
+    (2048, 19, 31),       # 589 rows, three row pairs, few tiles: one SM
+    (2048, 29, 31),       # 899 rows, four row pairs: two SMs, tiles cut between the clusters
     (2688, 3, 43),        # an odd number of 128-wide vocabulary units: one SM
     (65536, 5, 29),       # whole tiles, 145 rows
     (16384, 19, 31),      # whole tiles, 589 rows: three row pairs, the last one without a second row tile
@@ -25,8 +27,10 @@ def test_lm_head_tiles(V, B, n_blk):
     check_predict_commit(wl.TINY, V, B, 64, n_blk)
 
 
-def test_lm_head_cut_tiles():     # ten tiles of 129 rows, K = 2048 cut between the clusters
-    check_predict_commit(wl.LayerShape(2048, 2, 1, 128, 256, 1e-5, False, 5e5, "lm-head-cut"), 2560, 3, 64, 43)
+def test_lm_head_cut_tiles():     # K = 2048: ten pair tiles of 129 rows on one SM, 32 of 780 cut between the clusters
+    shape = wl.LayerShape(2048, 2, 1, 128, 256, 1e-5, False, 5e5, "lm-head-cut")
+    check_predict_commit(shape, 2560, 3, 64, 43)
+    check_predict_commit(shape, 2048, 13, 64, 60)
 
 
 @pytest.mark.parametrize("T", [51200, 51201])     # the last context whose position map fits shared memory, the first past it
