@@ -380,8 +380,8 @@ void launch_copy_out(const void* big, void* big_out, int64_t n_big, const void* 
 
 // A CTA takes 64 affix keys of a request; its four groups of 64 threads take every fourth head each, eight loads in
 // flight per thread, and meet in a fixed order.  Bound by L2 latency: which query tiles wrote sums is found by a
-// warp, a tile per lane (one thread reading the words one after the other and a thread per key over all heads and
-// tiles: 54 us for 32 requests x 28 heads x 2 tiles x 1024 keys; this 13.5).
+// warp, a tile per lane, 256 tiles at a time (one thread reading the words one after the other and a thread per key over
+// all heads and tiles: 54 us for 32 requests x 28 heads x 2 tiles x 1024 keys; this 13.5).
 __global__ void __launch_bounds__(256) score_reduce_tiles_kernel(const float* __restrict__ partial,
                                                                  const uint32_t* __restrict__ rowmask, int rm_words,
                                                                  float* __restrict__ scores, int n_heads, int q_tiles, int L,
@@ -392,35 +392,39 @@ __global__ void __launch_bounds__(256) score_reduce_tiles_kernel(const float* __
     pdl_wait();
     pdl_launch_dependents();
     const int b = blockIdx.y, lane = threadIdx.x & 31;
-    if (threadIdx.x < 32) {
-        int n = 0;
-        for (int q0 = 0; q0 < q_tiles && q0 < 256; q0 += 32) {
-            const int qt = q0 + lane;
-            uint32_t any = 0u;
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-                if (qt * 4 + i < rm_words) any |= __ldg(rowmask + (int64_t)b * rm_words + qt * 4 + i);
-            const bool hit = any != 0u && qt < q_tiles;
-            const uint32_t hits = __ballot_sync(0xffffffffu, hit);
-            if (hit) live[n + __popc(hits & ((1u << lane) - 1u))] = qt;
-            n += __popc(hits);
-        }
-        if (lane == 0) n_live_s = n;
-    }
-    __syncthreads();
-    const int n_live = n_live_s, grp = threadIdx.x >> 6, j = blockIdx.x * 64 + (threadIdx.x & 63);
+    const int grp = threadIdx.x >> 6, j = blockIdx.x * 64 + (threadIdx.x & 63);
     float s = 0.f;
-    if (j < L) {
-        for (int q = 0; q < n_live; ++q) {
-            const float* src = partial + ((int64_t)b * n_heads * q_tiles + live[q]) * L + j;
-            for (int h0 = grp; h0 < n_heads; h0 += 32) {
-                float t[8];
+    for (int first = 0; first < q_tiles; first += 256) {
+        if (threadIdx.x < 32) {
+            int n = 0;
+            for (int q0 = first; q0 < min(q_tiles, first + 256); q0 += 32) {
+                const int qt = q0 + lane;
+                uint32_t any = 0u;
 #pragma unroll
-                for (int u = 0; u < 8; ++u) t[u] = h0 + 4 * u < n_heads ? __ldcg(src + (int64_t)(h0 + 4 * u) * q_tiles * L) : 0.f;
+                for (int i = 0; i < 4; ++i)
+                    if (qt * 4 + i < rm_words) any |= __ldg(rowmask + (int64_t)b * rm_words + qt * 4 + i);
+                const bool hit = any != 0u && qt < q_tiles;
+                const uint32_t hits = __ballot_sync(0xffffffffu, hit);
+                if (hit) live[n + __popc(hits & ((1u << lane) - 1u))] = qt;
+                n += __popc(hits);
+            }
+            if (lane == 0) n_live_s = n;
+        }
+        __syncthreads();
+        const int n_live = n_live_s;
+        if (j < L) {
+            for (int q = 0; q < n_live; ++q) {
+                const float* src = partial + ((int64_t)b * n_heads * q_tiles + live[q]) * L + j;
+                for (int h0 = grp; h0 < n_heads; h0 += 32) {
+                    float t[8];
 #pragma unroll
-                for (int u = 0; u < 8; ++u) s += t[u];
+                    for (int u = 0; u < 8; ++u) t[u] = h0 + 4 * u < n_heads ? __ldcg(src + (int64_t)(h0 + 4 * u) * q_tiles * L) : 0.f;
+#pragma unroll
+                    for (int u = 0; u < 8; ++u) s += t[u];
+                }
             }
         }
+        __syncthreads();
     }
     group_sum[grp][threadIdx.x & 63] = s;
     __syncthreads();

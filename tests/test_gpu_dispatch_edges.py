@@ -71,6 +71,22 @@ def test_probe_row_mask_of_long_contexts(T):
     assert np.all(np.abs(s_gpu[0] - ref) <= 1e-3 * np.maximum(ref, ref.mean()))
 
 
+def test_probe_scores_of_more_than_256_query_tiles():
+    # 32964 rows in 258 tiles, the masked ones in the last: against the scoring kernels on the same cache (Eq. 4-5 from bf16
+    # queries and keys summed in fp32: the bound the other scoring tests use)
+    shape = wl.LayerShape(256, 2, 1, 128, 256, 1e-5, False, 5e5, "probe-many-rows")
+    lay = wl.make_layout(1, 0, 64, 32900, 64, 32, "all")
+    case = wl.make_case(shape, lay, 0.0, cfg_id=81)
+    dc = DeviceCase(case)
+    scores = torch.zeros((2, 64), dtype=torch.float32, device=DEV)
+    y = torch.zeros((1, lay.n_extra, 256), dtype=torch.bfloat16, device=DEV)
+    for i, flags in enumerate((ab.F_SCORE | ab.F_NO_RECOMPUTE, ab.F_SCORE)):
+        dc.ctx.layer_step(dc.lw, dc.req, dc.kv(), dc.x, 0, 0.0, flags, scores[i:i + 1], None, y)
+    assert dc.ctx.poll_status() == 0
+    apart, probe = scores.cpu().numpy().astype(np.float64)
+    assert apart.min() > 0 and np.all(np.abs(probe - apart) <= 1e-3 * np.maximum(apart, apart.mean()))
+
+
 @pytest.mark.parametrize("L", [255, 256, 257, 1025, 2047, 8192, 16385])
 def test_topk_score_distributions(L):
     """Histogram ranges and candidate counts the selection's passes depend on: a few huge scores over many small ones,
