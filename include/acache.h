@@ -464,7 +464,8 @@ acache_status acache_generate_block(acache_ctx *ctx, int32_t n_layers, const aca
  *   its rows, it is not staged: the kernels read
  *   the rows the step needs (the masked rows and the K+e recomputed rows: n_masked + K + e rows of D bf16 per
  *   request, each once) in place over the bus, so x_host must stay valid and unchanged until the
- *   stream has passed this call.  Page-locked results are written by a copy kernel (y up to 4 MB). */
+ *   stream has passed this call.  Page-locked results are written by a copy kernel (y up to 4 MB).
+ *   A buffer that is page-locked at its start must be so to its end (ACACHE_ERR_INVALID_ARG otherwise). */
 acache_status acache_layer_step_host(acache_ctx *ctx, const acache_layer_weights *w,
                                      const acache_request *req, acache_kv *kv,
                                      const void *x_host, double ratio, uint32_t flags,

@@ -308,11 +308,19 @@ acache_status run_recompute(acache_ctx* c, const acache_layer_weights* w, const 
 static thread_local bool g_reuse_maps = false;
 
 namespace {
-// Device-side address of page-locked host memory (nullptr for pageable or unknown memory).
-const void* mapped_device_pointer(const void* host) {
-    cudaPointerAttributes at{};
-    if (!host || cudaPointerGetAttributes(&at, host) != cudaSuccess) { cudaGetLastError(); return nullptr; }
-    return at.type == cudaMemoryTypeHost ? at.devicePointer : nullptr;
+// Device-side address of page-locked host memory (nullptr for pageable or unknown memory).  partial (optional): set when the
+// memory is page-locked at its start but not to its end, where a kernel would leave the mapping.
+const void* mapped_device_pointer(const void* host, size_t bytes = 1, bool* partial = nullptr) {
+    cudaPointerAttributes at{}, end{};
+    if (!host) return nullptr;
+    if (bytes == 0) bytes = 1;
+    if (cudaPointerGetAttributes(&at, host) != cudaSuccess) { cudaGetLastError(); return nullptr; }
+    if (at.type != cudaMemoryTypeHost || !at.devicePointer) return nullptr;
+    if (cudaPointerGetAttributes(&end, static_cast<const char*>(host) + bytes - 1) != cudaSuccess) cudaGetLastError();
+    if (end.type == cudaMemoryTypeHost && static_cast<char*>(end.devicePointer) == static_cast<char*>(at.devicePointer) + bytes - 1)
+        return at.devicePointer;
+    if (partial) *partial = true;
+    return nullptr;
 }
 }  // namespace
 
@@ -984,7 +992,16 @@ acache_status acache_layer_step_host(acache_ctx* ctx, const acache_layer_weights
     // output projection): the row preparation leaves a copy in the staging buffer, which is free then, and the
     // residual is read from there (measured: 290 -> 219 us per step at 103 rows).
     const int64_t pulled = (int64_t)req->n_masked + (int64_t)k + req->n_extra;
-    const void* x_dev = pulled * 4 <= req->ctx_len && acache_host_x_in_place(x_host) ? mapped_device_pointer(x_host) : nullptr;
+    const size_t rows = (size_t)req->batch * ((size_t)k + (req->n_extra > 0 ? req->n_extra : 0));
+    const size_t n_s = (size_t)req->batch * req->affix_len, n_a = (size_t)req->batch * k;
+    const size_t y_bytes = (flags & ACACHE_F_NO_RECOMPUTE) ? 0 : rows * d.hidden * 2;
+    bool partial = false;
+    const void* x_map = mapped_device_pointer(x_host, xb, &partial);
+    void* y_map = const_cast<void*>(mapped_device_pointer(y_host, y_bytes, &partial));
+    void* s_map = const_cast<void*>(mapped_device_pointer(scores_host, n_s * 4, &partial));
+    void* a_map = const_cast<void*>(mapped_device_pointer(anchor_idx_host, n_a * 4, &partial));
+    if (partial) return fail(ctx, ACACHE_ERR_INVALID_ARG, "a host buffer is page-locked only in part");
+    const void* x_dev = pulled * 4 <= req->ctx_len && acache_host_x_in_place(x_host) ? x_map : nullptr;
     if (!x_dev) {
         if (cudaMemcpyAsync(xs, x_host, xb, cudaMemcpyHostToDevice, stream) != cudaSuccess) return check_cuda(ctx, "H2D x");
         x_dev = xs;
@@ -998,15 +1015,9 @@ acache_status acache_layer_step_host(acache_ctx* ctx, const acache_layer_weights
     // 32-byte pieces, y cost 40 us more), unless y is so large that the copy engine's start no longer counts and the SMs
     // have better to do.
     constexpr size_t kCopyKernelBytes = 4u << 20;
-    void* s_map = const_cast<void*>(mapped_device_pointer(scores_host));
-    void* a_map = k ? const_cast<void*>(mapped_device_pointer(anchor_idx_host)) : nullptr;
-    const size_t rows = (size_t)req->batch * (k + req->n_extra);
-    const size_t n_s = (size_t)req->batch * req->affix_len, n_a = (size_t)req->batch * k;
-    const size_t y_bytes = (flags & ACACHE_F_NO_RECOMPUTE) ? 0 : rows * d.hidden * 2;
+    if (y_bytes > kCopyKernelBytes || !aligned16(y_map)) y_map = nullptr;
     bool ok = true;
     if (s_map && (a_map || !k) && n_s + n_a < (1u << 30)) {
-        void* y_map = y_bytes && y_bytes <= kCopyKernelBytes ? const_cast<void*>(mapped_device_pointer(y_host)) : nullptr;
-        if (!aligned16(y_map)) y_map = nullptr;
         launch_copy_out(ys, y_map, y_map ? (int64_t)(y_bytes / 16) : 0, ss, s_map, (int)n_s, as, a_map, (int)n_a, stream);
         ++ctx->launches;
         if (y_bytes && !y_map) ok &= cudaMemcpyAsync(y_host, ys, y_bytes, cudaMemcpyDeviceToHost, stream) == cudaSuccess;

@@ -365,6 +365,33 @@ def test_host_buffer_entry_point(shape, L, extra, ratio):
     assert np.array_equal(ab.to_host_bits(yh2), ab.to_host_bits(y_dev[:, :n]))
 
 
+@pytest.mark.parametrize("which", range(4))
+def test_host_buffers_page_locked_in_part_are_refused(which):
+    lay = wl.make_layout(2, 0, 600, 32, 32, 32, "all")
+    case = wl.make_case(MID128, lay, 0.05, cfg_id=17)
+    dc = DeviceCase(case)
+    n = 30 + lay.n_extra
+    cudart = torch.cuda.cudart()
+    bufs = [torch.from_numpy(case.x.view(np.int16).copy()).view(torch.bfloat16), torch.zeros((2, 600), dtype=torch.float32),
+            torch.zeros((2, 30), dtype=torch.int32), torch.zeros((2, n, MID128.hidden), dtype=torch.bfloat16)]
+    room = torch.zeros(4 * 4096 + bufs[which].numel() * bufs[which].element_size(), dtype=torch.uint8)
+    page = -room.data_ptr() % 4096 + 4096                    # page-locked up to here: all but the buffer's first 64 bytes lie past it
+    t = room[page - 64:page - 64 + bufs[which].numel() * bufs[which].element_size()].view(bufs[which].dtype).view(bufs[which].shape)
+    bufs[which] = t.copy_(bufs[which])
+    assert int(cudart.cudaHostRegister(room.data_ptr() + page - 4096, 4096, 0)) == 0
+    before = dc.ctx.launch_count()
+    try:
+        x, s, a, y = bufs
+        with pytest.raises(ab.AcacheError) as e:
+            dc.ctx.layer_step_host(dc.lw, dc.req, dc.kv(), x, 0.05, 0, s, a, y)
+        assert e.value.status == ab.ERR_INVALID_ARG and dc.ctx.launch_count() == before
+    finally:
+        assert int(cudart.cudaHostUnregister(room.data_ptr() + page - 4096)) == 0
+    dc.ctx.layer_step_host(dc.lw, dc.req, dc.kv(), x, 0.05, 0, s, a, y)          # all pageable: accepted
+    torch.cuda.synchronize()
+    assert dc.ctx.poll_status() == 0 and y.float().abs().max() > 0
+
+
 def test_invalid_arguments_enqueue_nothing():
     lay = wl.make_layout(1, 0, 128, 16, 32, 32, "none")
     case = wl.make_case(wl.TINY, lay, 0.1, cfg_id=18)
