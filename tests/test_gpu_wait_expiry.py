@@ -17,13 +17,21 @@ from test_gpu_parity import MID128, dev_i32
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("B,L,extra", [
-    (1, 300, "none"),      # 60 rows: one CTA per tile, ring stages filled with weights before the barrier
-    (2, 400, "all"),       # several 128-row tiles: the two-SM projection kernel
+# q/k/v of few rows and a long K: cut between the CTAs of a cluster, which pass their barriers whatever ran out
+DEEP128 = wl.LayerShape(3584, 4, 1, 128, 256, 1e-6, True, 1e6, "deep-d128")
+LONG128 = wl.LayerShape(2560, 6, 3, 128, 256, 1e-6, True, 1e6, "long-d128")
+
+
+@pytest.mark.parametrize("shape,B,L,extra,kernel", [
+    (wl.TINY, 1, 300, "none", "gemm_rows_kernel<1, 0, true>"),       # 60 rows: one CTA per tile, ring stages filled with weights
+    (MID128, 1, 300, "none", "gemm_rows_kernel<2, 0, true>"),        # before the barrier; two and four CTAs per tile
+    (LONG128, 1, 160, "none", "gemm_rows_kernel<2, 0, false>"),
+    (DEEP128, 1, 300, "none", "gemm_rows_kernel<4, 0, false>"),
+    (MID128, 2, 400, "all", "gemm_tc2_kernel"),                      # several 128-row tiles: the two-SM projection kernel
 ])
-def test_a_wait_that_runs_out_is_reported_and_the_context_stays_usable(B, L, extra):
+def test_a_wait_that_runs_out_is_reported_and_the_context_stays_usable(shape, B, L, extra, kernel):
     lay = wl.make_layout(B, 4, L, 40, 32, 32, extra)
-    case = wl.make_case(MID128, lay, 0.2, cfg_id=17)
+    case = wl.make_case(shape, lay, 0.2, cfg_id=17)
     dc = DeviceCase(case)
     K = orc.k_from_ratio(L, 0.2)
     n = K + lay.n_extra
@@ -31,12 +39,15 @@ def test_a_wait_that_runs_out_is_reported_and_the_context_stays_usable(B, L, ext
     anchors = dev_i32(np.stack([np.sort(g.choice(L, K, replace=False)) for _ in range(B)]))
 
     def step():
-        y = torch.zeros((B, n, MID128.hidden), dtype=torch.bfloat16, device=DEV)
+        y = torch.zeros((B, n, shape.hidden), dtype=torch.bfloat16, device=DEV)
         dc.ctx.layer_step(dc.lw, dc.req, dc.kv(), dc.x, 0, 0.2, 0, None, anchors, y)
         torch.cuda.synchronize()                     # returns: no kernel of the step is stuck
         return ab.to_host_bits(y), ab.to_host_bits(dc.ck), ab.to_host_bits(dc.cv)
 
-    clean = step()
+    with torch.profiler.profile(activities=[torch.profiler.ProfilerActivity.CUDA]) as prof:
+        clean = step()
+    names = [e.key for e in prof.key_averages()]
+    assert any(kernel in name for name in names), names              # the projection whose barrier runs out is this kernel
     assert dc.ctx.poll_status_code() == (ab.OK, 0)
     dc.reset_cache()
     dc.ctx.debug_expire_next_wait()
