@@ -1089,10 +1089,6 @@ const CUtensorMap* get_map3(const void* ptr, int rows, int cols, int batch, int6
     return &e.map;
 }
 
-
-namespace {
-}  // namespace
-
 // Returns the number of kernels launched, 0 if this problem is not for the tensor-core kernel
 // (the caller then uses the mma.sync kernel), -1 if a launch failed.
 int launch_attention_tc(const AttnArgs& a, uint32_t* status, cudaStream_t stream) {

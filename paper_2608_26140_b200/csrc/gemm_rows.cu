@@ -539,9 +539,9 @@ int resident_clusters() {
 // takes as many panels as leave three stages in the ring (fewer, larger stages lost, two stages of any size did too).
 // Measured when it replaced that kernel, at 103 rows (us per launch, finish included | here): q/k/v 30.2 | 29.6, output
 // 16.3 | 13.0, gate/up 47.7 | 43, down 25.7 | 23.4; at 32 rows output 14.3 | 10.9, down 25.0 | 20.4.
-// With an accumulator per K block the tile is at most what 256 columns of tensor memory hold (two CTAs then fit an SM), and a
-// doubling of the split costs 2.5 us, for every block is exchanged (58 rows, 1024 -> 256 columns in the chain above: over two
-// CTAs 1.4 us slower than in one).
+// With an accumulator per K block the tile is at most what 256 columns of tensor memory hold (two CTAs then fit an SM).  A split
+// costs 2.5 us there, for every block is exchanged (58 rows, 1024 -> 256 columns in the chain above: over two CTAs 1.4 us slower
+// than in one); it is taken for rotary pairs alone, whose tiles of 64 columns hold four blocks to a CTA.
 constexpr int kRingBytes = 200 * 1024, kApartColumns = 256;
 bool plan_rows(const GemmArgs& g, RowsPlan& best) {
     if (g.M > 128 || g.epilogue == kEpiLogits || g.K < 64) return false;
@@ -553,7 +553,7 @@ bool plan_rows(const GemmArgs& g, RowsPlan& best) {
     const int step = qkv ? 64 : swiglu || apart ? 16 : 32;
     const int limit[3] = {resident_clusters<1>(), resident_clusters<2>(), resident_clusters<4>()};
     double t_best = 1e30;
-    for (int si = 0; si < (swiglu ? 1 : 3); ++si) {
+    for (int si = 0; si < (swiglu || (apart && !qkv) ? 1 : apart ? 2 : 3); ++si) {
         const int S = 1 << si;
         for (int TN = step; TN <= 256; TN += step) {
             const int items = TN / (qkv ? 32 : 16);
@@ -614,7 +614,9 @@ int launch_gemm_rows(const GemmArgs& g, cudaStream_t stream) {
     auto launch = [&](auto epi, auto apart) {
         constexpr int EPI = decltype(epi)::value;
         constexpr bool APART = decltype(apart)::value;
-        if constexpr (EPI == kEpiSwiGLU) return launch_rows<1, EPI, APART>(g, p, map_a, map_b, stream);
+        if constexpr (EPI == kEpiSwiGLU || (APART && EPI == kEpiResidual)) return launch_rows<1, EPI, APART>(g, p, map_a, map_b, stream);
+        else if constexpr (APART)
+            return p.S == 1 ? launch_rows<1, EPI, APART>(g, p, map_a, map_b, stream) : launch_rows<2, EPI, APART>(g, p, map_a, map_b, stream);
         else
             return p.S == 1 ? launch_rows<1, EPI, APART>(g, p, map_a, map_b, stream)
                  : p.S == 2 ? launch_rows<2, EPI, APART>(g, p, map_a, map_b, stream)

@@ -53,7 +53,7 @@ constexpr int TC_SMEM = TC_STAGES * TC_STAGE_BYTES + 1024 /*alignment slack*/ + 
 constexpr int TC_SLOT_FLOATS = TC_BM * TC_BN;          // one fp32 partial tile
 
 struct TcPlan {
-    int m_tiles, n_tiles, KB, tiles, U, ctas, smax;
+    int m_tiles, n_tiles, KB, tiles, U, ctas;
     int prefill;          // ring stages whose weight halves are loaded before the dependency wait
     int pair_u;           // two-SM kernel, stream-K mode: (pair tile, K block) iterations per cluster (0: whole tiles)
     int m_pairs;          // 256-row tile rows of the two-SM kernel
@@ -1009,7 +1009,6 @@ TcPlan make_plan(int M, int K, int units, bool swiglu) {
     const int g = (int)(total < sm_count() ? total : sm_count());
     p.U = (int)((total + g - 1) / g);
     p.ctas = (int)((total + p.U - 1) / p.U);
-    p.smax = 2;   // partial slots per CTA
     // measured: 174.9 us per layer-step of 103 rows with no stage prefilled, 169.1 with two, 167.9-168.6 with three or four
     p.prefill = TC_STAGES;
     return p;
