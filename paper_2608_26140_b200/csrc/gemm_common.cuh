@@ -42,6 +42,19 @@ __device__ __forceinline__ bool grid_barrier(unsigned int* bar, volatile int* ab
     return passed;
 }
 
+__device__ __forceinline__ void tc_ld16(uint32_t taddr, float (&v)[16]) {
+    uint32_t r[16];
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
+        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+        : "r"(taddr)
+        : "memory");
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+    for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
+}
 __device__ __forceinline__ uint4 pack8(const float* v) {
     return make_uint4(pack_bf16(v[0], v[1]), pack_bf16(v[2], v[3]), pack_bf16(v[4], v[5]), pack_bf16(v[6], v[7]));
 }
@@ -206,8 +219,9 @@ __device__ __forceinline__ int64_t prep_row_source(const GemmArgs& g, int row, b
 // out = bf16(x * rsqrt(mean(x^2) + eps) * g) for one row, by one warp: rows of up to 4096 values in one pass from
 // registers; longer ones in two passes with eight independent 16-byte loads in flight per lane (the second pass hits
 // L1 / L2).
-// GAIN_EARLY: the gain is asked for beside the row, in 64 more registers, where there are few rows per warp and the trip for
-// it would follow the row's (615 rows: layer-step 384.7 -> 381.6 us, 5 x 203 rows 530.7 -> 527.7).
+// GAIN_EARLY: the first half of the gain is asked for beside the row, in 32 more registers, where there are few rows per warp and
+// the trip for it would follow the row's (615 rows: layer-step 384.7 -> 381.6 us, 5 x 203 rows 530.7 -> 527.7; the whole gain
+// spills, see gemm_tc2_kernel).
 template <bool GAIN_EARLY>
 __device__ __forceinline__ void rmsnorm_row_warp(const uint4* __restrict__ xr, const uint4* __restrict__ gn,
                                                  uint4* __restrict__ out, int hidden, float eps, int lane,
@@ -216,7 +230,7 @@ __device__ __forceinline__ void rmsnorm_row_warp(const uint4* __restrict__ xr, c
     if (nchunk <= 512) {
         // rows of up to 4096 values: one pass, the row stays in registers (sixteen 16-byte loads in flight per lane,
         // one trip to memory per row instead of two), the gain is requested before the warp-wide sum
-        uint4 u[16], early[GAIN_EARLY ? 16 : 1];
+        uint4 u[16], early[GAIN_EARLY ? 8 : 1];
         float s1 = 0.f;
 #pragma unroll
         for (int i = 0; i < 16; ++i) {
@@ -225,7 +239,7 @@ __device__ __forceinline__ void rmsnorm_row_warp(const uint4* __restrict__ xr, c
         }
         if (GAIN_EARLY) {
 #pragma unroll
-            for (int i = 0; i < 16; ++i) early[GAIN_EARLY ? i : 0] = i * 32 + lane < nchunk ? __ldg(gn + i * 32 + lane) : make_uint4(0, 0, 0, 0);
+            for (int i = 0; i < 8; ++i) early[GAIN_EARLY ? i : 0] = i * 32 + lane < nchunk ? __ldg(gn + i * 32 + lane) : make_uint4(0, 0, 0, 0);
         }
         if (raw) {
 #pragma unroll
@@ -247,7 +261,7 @@ __device__ __forceinline__ void rmsnorm_row_warp(const uint4* __restrict__ xr, c
         for (int i = 0; i < 16; ++i) {
             const int c = i * 32 + lane;
             if (c < nchunk) {
-                const uint4 gg = GAIN_EARLY ? early[GAIN_EARLY ? i : 0] : __ldg(gn + c);
+                const uint4 gg = GAIN_EARLY && i < 8 ? early[GAIN_EARLY ? i & 7 : 0] : __ldg(gn + c);
                 const uint32_t w[4] = {u[i].x, u[i].y, u[i].z, u[i].w};
                 const uint32_t gw[4] = {gg.x, gg.y, gg.z, gg.w};
                 uint32_t r[4];
