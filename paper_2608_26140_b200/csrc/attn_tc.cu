@@ -164,8 +164,10 @@ __device__ __forceinline__ bool mbar_spin(uint32_t bar, uint32_t parity, volatil
 }
 
 // MANY: many more items than SMs.  A CTA then takes every gridDim.x-th one and keeps its tensor memory and barriers; the loads and
-// the first S of the next item run under the tail of this one (64 requests of 103 rows over 608 keys: attention 184 -> 158 us,
-// layer-step 2774 -> 2757).  With one item per CTA the same code was 1.7 us slower (103 rows over 1024 keys).
+// the first S of the next item run under the tail of this one (layer-steps of 103 rows and 608 keys, us, one item per CTA | this:
+// 64 requests 2678-2694 | 2659-2668, 40 requests 1756 | 1750; 60 rows and 396 keys, 30 requests 899 | 893; refresh of 90 rows
+// over 192 keys, 64 requests, 2 layers 5841 | 5804; 28 heads, 64 requests of 105 rows 2790 | 2796; two runs differ by 0.3-0.8 %).
+// With one item per CTA the same code was 1.7 us slower (103 rows over 1024 keys).
 template <bool MANY>
 __global__ void __launch_bounds__(AT_THREADS, 1)
 attention_tc_kernel(const AttnTcArgs a, const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUtensorMap mapK,
@@ -1173,8 +1175,8 @@ int launch_attention_tc(const AttnArgs& a, uint32_t* status, cudaStream_t stream
         while (t.split < 8 && ctas * t.split * 2 <= 148 && tiles >= t.split * 4) t.split *= 2;
         cudaLaunchConfig_t cfg{};
         t.n_items = (int)ctas;
-        // from six rounds of CTAs on, items share a CTA (13.8 rounds: 1 % of the layer-step; at 1.9 and 2.8 rounds, where
-        // the hardware's assignment evens out the last round, 0.3 and 0.9 % slower)
+        // from six rounds of CTAs on, items share a CTA (of the layer-step, 0.7-1.0 % at 13.8 rounds, 0.2-0.5 % at 8.6, 0.4-1.0 % at
+        // 6.5; at 1.9 and 2.8 rounds, where the hardware's assignment evens out the last round, 0.3 and 0.9 % slower)
         const bool many = t.split == 1 && t.n_items >= 6 * sm_count();
         cfg.gridDim = dim3(many ? sm_count() : t.n_items * t.split);
         cfg.blockDim = dim3(AT_THREADS);
