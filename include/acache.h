@@ -30,6 +30,13 @@
  *    call on the same stream (a weight copy or a dequantisation): put an event or any
  *    other kernel in between, or synchronise.  Every other input (x, the cache, index
  *    arrays, scores) follows plain stream order.
+ *  - Reproducibility: a call repeated on the same inputs gives the same bits (every sum has a fixed order).  The
+ *    order belongs to the call, though: the number of rows and requests decides how the K range of a projection
+ *    and the keys of an attention are cut between CTAs, so a request's results alone and beside others agree to
+ *    fp32 summation order (then bf16 rounding), not bit for bit, and a near tie between two tokens may be decided
+ *    either way.  Within 128 rows, projections of which (columns / 256, rounded up) x (K / 64) is at most the SM
+ *    count do not depend on the number of rows (a gate/up tile is 128 of the MLP's columns; rows of more than 256
+ *    columns: from that many rows on, where the row preparation no longer takes a CTA per row).
  *  - Errors: every call returns acache_status.  Argument and shape validation happens
  *    on the host before any launch, so a non-OK status means nothing was enqueued.
  *    Faults that depend on device data (an index outside its range) never trap: the

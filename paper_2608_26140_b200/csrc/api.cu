@@ -1027,7 +1027,7 @@ acache_status acache_layer_step_host(acache_ctx* ctx, const acache_layer_weights
         ok &= cudaMemcpyAsync(scores_host, ss, n_s * 4, cudaMemcpyDeviceToHost, stream) == cudaSuccess;
     }
     if (!ok) return check_cuda(ctx, "D2H") == ACACHE_OK ? fail(ctx, ACACHE_ERR_CUDA, "D2H copy failed") : ACACHE_ERR_CUDA;
-    return ACACHE_OK;
+    return check_cuda(ctx, "copy of the results");
 }
 
 }  // extern "C"

@@ -273,7 +273,7 @@ gemm_rows_kernel(const GemmArgs g, const RowsPlan p, const __grid_constant__ CUt
             if (++stage == p.stages) { stage = 0; phase ^= 1; }
         }
     } else if (warp == 1) {
-        // What bounds a stage here is this warp, not the data: 4 to 16 instructions of 60-100 cycles (they read A and B from
+        // What bounds a stage here is this warp, not the data: 4 to 32 instructions of 60-100 cycles (they read A and B from
         // shared memory, which the TMA fills meanwhile), then about 400 cycles until the next stage's first.  With one thread
         // in the loop, whose descriptors are no warp-uniform values, the instructions took 94-121 cycles: masked rows' queries
         // 2030 -> 1590 cycles a stage, layer-step of 103 rows 145.9 -> 144.2 us, of 8 rows 53.1 -> 51.6, decode pass of

@@ -24,8 +24,8 @@ __device__ __forceinline__ uint32_t score_key(float f) {
 // histogram divide [smallest, largest] in 2048, which sorts out more than the leading bits of the keys do (the scores of a
 // request share their exponents), so one pass mostly leaves few candidates.  Warp w owns the keys of [w seg, (w + 1) seg):
 // loads are coalesced and the ordered output needs ballots and one sum over the warps.  Against a radix select over four
-// bytes with two block scans per 1024 positions (added time in its chain): 512 scores 6.6 -> 6.3 us, 2048 9.8 -> 5.8,
-// 8192 16.0 -> 8.7.
+// bytes with two block scans per 1024 positions (launches back to back, one request): 512 scores 7.8 | 8.0 us, 2048 7.8 | 8.0,
+// 8192 19.2 | 8.0, 16 requests of them 19.5 | 8.6.
 __global__ void __launch_bounds__(kTopkThreads) topk_kernel(float* scores, int L, int K,
                                                             int32_t* __restrict__ anchor_idx, int use_smem,
                                                             const float* __restrict__ head_partial, int n_heads,
