@@ -186,6 +186,8 @@ __device__ __forceinline__ void sum_apart16(const RowsPlan& p, int rank, uint32_
     }
 }
 
+// 228 to 232 registers a thread: no CTA of another tensor-memory kernel finds room beside this one.  That matters where calls run on
+// two streams: with clusters on both sides, CTAs that wait for one another's tensor memory and cluster peers would wait for ever.
 template <int S, int EPI, bool APART>
 __global__ void __launch_bounds__(RW_THREADS, 1)
 gemm_rows_kernel(const GemmArgs g, const RowsPlan p, const __grid_constant__ CUtensorMap mapA,
@@ -526,7 +528,7 @@ int resident_clusters() {
 // takes as many panels as leave three stages in the ring (fewer, larger stages lost, two stages of any size did too).
 // Measured when it replaced that kernel, at 103 rows (us per launch, finish included | here): q/k/v 30.2 | 29.6, output
 // 16.3 | 13.0, gate/up 47.7 | 43, down 25.7 | 23.4; at 32 rows output 14.3 | 10.9, down 25.0 | 20.4.
-// With an accumulator per K block the tile is at most what 256 columns of tensor memory hold (two CTAs then fit an SM).  A split
+// With an accumulator per K block the tile is at most what 256 columns of tensor memory hold, as the widest tile does.  A split
 // costs 2.5 us there, for every block is exchanged (58 rows, 1024 -> 256 columns in the chain above: over two CTAs 1.4 us slower
 // than in one); it is taken for rotary pairs alone, whose tiles of 64 columns hold four blocks to a CTA.
 constexpr int kRingBytes = 200 * 1024, kApartColumns = 256;
