@@ -35,8 +35,8 @@ RATIO = 0.2
 
 # dram__bytes_read.sum + dram__bytes_write.sum per launch of the dominant kernel from an ncu capture of the kernel as it
 # stands at the commit named here; None until such a capture exists (a figure from an older kernel is not printed).
-NCU_TRAFFIC = {"kernel": "gemm_tc_kernel, gate/up projection 103 x 24576 x 4096 (one launch; 204.7 MB algorithmic)",
-               "bytes": 207042048, "commit": "c3e8c66"}
+NCU_TRAFFIC = {"kernel": "gemm_rows_kernel, gate/up projection 103 x 24576 x 4096 (one launch; 204.7 MB algorithmic)",
+               "bytes": 207066112, "commit": "2a021a4"}
 
 
 def load_peaks():
