@@ -675,12 +675,11 @@ gemm_tc2_kernel(const GemmArgs g, const TcPlan p, const int clusters, const __gr
     const int m_pairs = (p.m_tiles + 1) >> 1;
     const int tiles = m_pairs * p.n_tiles;
 
-    if (warp == 0 && lane == 0) {
+    if (warp == 0) {
         // TMA producer of this CTA: its 128 rows of A and its half of the weight tile
-        const CUtensorMap* maps[3] = {&mapB0, &mapB1, &mapB2};
         int stage = 0, issued = 0;
         uint32_t phase = 0;
-        bool ok = !*abort_flag;
+        bool ok = __all_sync(0xffffffffu, !*abort_flag);
         const uint64_t pol_a = policy_evict_last();
         const uint64_t pol_w = (g.keep_weights || p.w_keep) ? pol_a : policy_evict_first();
         // work list: whole tiles round-robin (pair_u == 0), or this cluster's contiguous range of
@@ -694,15 +693,19 @@ gemm_tc2_kernel(const GemmArgs g, const TcPlan p, const int clusters, const __gr
             const int kb1 = p.pair_u ? (int)min((long long)p.KB, (long long)(kb0 + (it_end - it))) : p.KB;
             int brow;
             const int bs = half_source(g, p, nt, (int)rank, brow);
+            const CUtensorMap* map_b = bs == 0 ? &mapB0 : bs == 1 ? &mapB1 : &mapB2;
             const int arow = (mp * 2 + (int)rank) * TC_BM;
             for (int kb = kb0; kb < kb1; ++kb) {
-                if (!(ok = mbar_poll(empty_bar(stage), phase ^ 1, abort_flag))) break;
-                const uint32_t sA = base + stage * TC2_STAGE_BYTES, sB = sA + TC_A_BYTES;
-                const uint32_t lead_full = mapa_u32(full_bar(stage), 0);
-                // the leader announces the bytes of both CTAs; the peer's copies only report completion
-                if (rank == 0) mbar_expect_tx(full_bar(stage), 2 * TC2_STAGE_BYTES);
-                tma_load_2d_pair(sA, &mapA, kb * TC_BK, arow, lead_full, pol_a);
-                tma_load_2d_pair(sB, maps[bs], kb * TC_BK, brow, lead_full, pol_w);
+                if (!(ok = __all_sync(0xffffffffu, mbar_poll(empty_bar(stage), phase ^ 1, abort_flag)))) break;
+                if (elect_lane()) {
+                    const uint32_t sA = base + stage * TC2_STAGE_BYTES, sB = sA + TC_A_BYTES;
+                    const uint32_t lead_full = mapa_u32(full_bar(stage), 0);
+                    // the leader announces the bytes of both CTAs; the peer's copies only report completion
+                    if (rank == 0) mbar_expect_tx(full_bar(stage), 2 * TC2_STAGE_BYTES);
+                    tma_load_2d_pair(sA, &mapA, kb * TC_BK, arow, lead_full, pol_a);
+                    tma_load_2d_pair(sB, map_b, kb * TC_BK, brow, lead_full, pol_w);
+                }
+                __syncwarp();
                 ++issued;
                 if (++stage == TC2_STAGES) { stage = 0; phase ^= 1; }
             }
@@ -711,36 +714,44 @@ gemm_tc2_kernel(const GemmArgs g, const TcPlan p, const int clusters, const __gr
         // wait until the MMAs have consumed everything this CTA loaded, so that no signal from the
         // leader can arrive after this CTA has left
         for (int i = 0; i < min(issued, TC2_STAGES) && ok; ++i) {
-            ok = mbar_poll(empty_bar(stage), phase ^ 1, abort_flag);
+            ok = __all_sync(0xffffffffu, mbar_poll(empty_bar(stage), phase ^ 1, abort_flag));
             if (++stage == TC2_STAGES) { stage = 0; phase ^= 1; }
         }
-    } else if (warp == 1 && lane == 0 && rank == 0) {
-        // MMA issuer (leader CTA only)
+    } else if (warp == 1 && rank == 0) {
+        // MMA issuer (leader CTA only): the whole warp runs the loop, an elected lane issues, and the full barrier is polled at
+        // CTA scope (a poll that acquires at cluster scope costs more than the data's own proxy needs).  With one lane in the loop
+        // a K block took 540-630 cycles whatever the tile's width, of which the four instructions need 512: what bounded the loop was
+        // the issue.  Back to back: 64 x 103 rows 2693 -> 2574 us, refresh of 14 752 rows 12 468 -> 12 112 (q/k/v 1209 -> 1043,
+        // output 442 -> 375 a launch), probe of 20 480 rows 16 876 -> 16 341, 615 rows 374.7 -> 368.0; cluster-scope polls in the
+        // same loop: refresh 12 400.
         int stage = 0, acc = 0;
         uint32_t phase = 0, acc_phase = 0;
-        bool ok = !*abort_flag;
+        bool ok = __all_sync(0xffffffffu, !*abort_flag);
         const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(256 >> 3) << 17) | ((uint32_t)(256 >> 4) << 24);
         const long long it_end = p.pair_u ? min((long long)(cluster_id + 1) * p.pair_u, (long long)tiles * p.KB) : 0;
         long long it = p.pair_u ? (long long)cluster_id * p.pair_u : 0;
         for (int t = p.pair_u ? (int)(it / p.KB) : cluster_id; ok && (p.pair_u ? it < it_end : t < tiles);) {
             const int kb0 = p.pair_u ? (int)(it - (long long)t * p.KB) : 0;
             const int kb1 = p.pair_u ? (int)min((long long)p.KB, (long long)(kb0 + (it_end - it))) : p.KB;
-            if (!(ok = mbar_poll_cluster(tempty_bar(acc), acc_phase ^ 1, abort_flag))) break;
+            if (!(ok = __all_sync(0xffffffffu, mbar_poll_cluster(tempty_bar(acc), acc_phase ^ 1, abort_flag)))) break;
             tc_fence_after();
             const uint32_t d_tmem = tmem_base + acc * TC_BN;
             for (int kb = kb0; kb < kb1; ++kb) {
-                if (!(ok = mbar_poll_cluster(full_bar(stage), phase, abort_flag))) break;
+                if (!(ok = __all_sync(0xffffffffu, mbar_poll(full_bar(stage), phase, abort_flag)))) break;
                 tc_fence_after();
-                const uint32_t sA = base + stage * TC2_STAGE_BYTES, sB = sA + TC_A_BYTES;
-                const uint64_t da = smem_desc_sw128(sA), db = smem_desc_sw128(sB);
+                if (elect_lane()) {
+                    const uint32_t sA = base + stage * TC2_STAGE_BYTES, sB = sA + TC_A_BYTES;
+                    const uint64_t da = smem_desc_sw128(sA), db = smem_desc_sw128(sB);
 #pragma unroll
-                for (int k = 0; k < TC_BK / 16; ++k)
-                    tc2_mma(d_tmem, da + (uint64_t)(k * 2), db + (uint64_t)(k * 2), idesc, (kb > kb0 || k > 0) ? 1u : 0u);
-                tc2_commit_both(empty_bar(stage));
+                    for (int k = 0; k < TC_BK / 16; ++k)
+                        tc2_mma(d_tmem, da + (uint64_t)(k * 2), db + (uint64_t)(k * 2), idesc, (kb > kb0 || k > 0) ? 1u : 0u);
+                    tc2_commit_both(empty_bar(stage));
+                    if (kb + 1 == kb1) tc2_commit_both(tfull_bar(acc));
+                }
+                __syncwarp();
                 if (++stage == TC2_STAGES) { stage = 0; phase ^= 1; }
             }
             if (!ok) break;
-            tc2_commit_both(tfull_bar(acc));
             if (++acc == 2) { acc = 0; acc_phase ^= 1; }
             if (p.pair_u) { it += kb1 - kb0; ++t; } else t += clusters;
         }
