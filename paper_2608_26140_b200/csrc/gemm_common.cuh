@@ -353,12 +353,51 @@ __device__ __forceinline__ void prep_phase(const GemmArgs& g, float* red, volati
     asm volatile("fence.proxy.async;" ::: "memory");
 }
 
+// Order of the whole tiles of the two-SM kernels, see kTileGroupN in gemm_tc.cu: groups of group_n weight tiles (nt), inside a
+// group row pairs (mp, or chunks of rows) with the weight tiles innermost.
+__device__ __forceinline__ void tile_coords(int t, int m_pairs, int n_tiles, int group_n, int& nt, int& mp) {
+    const int full = n_tiles / group_n, per_group = group_n * m_pairs;
+    if (t < full * per_group) {
+        const int grp = t / per_group, r = t - grp * per_group;
+        mp = r / group_n;
+        nt = grp * group_n + (r - mp * group_n);
+    } else {
+        const int r = t - full * per_group, gn = n_tiles - full * group_n;
+        mp = r / gn;
+        nt = full * group_n + (r - mp * gn);
+    }
+}
+
+// TMA load into this CTA's shared memory that completes on a barrier of the CTA pair's leader
+__device__ __forceinline__ void tma_load_2d_pair(uint32_t dst, const CUtensorMap* map, int c0, int c1, uint32_t bar_cluster,
+                                                 uint64_t policy) {
+    asm volatile(
+        "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint "
+        "[%0], [%1, {%2, %3}], [%4], %5;"
+        ::"r"(dst), "l"(map), "r"(c0), "r"(c1), "r"(bar_cluster), "l"(policy)
+        : "memory");
+}
 // Tensor map over bf16 [rows, cols] row-major with the panel of 64 columns as a dimension: box = 64 columns x box_rows rows x
 // `panels` panels, 128-byte swizzle, zero fill out of bounds.  half > 0: the rows in groups of `half`, box = box_rows rows of
 // two consecutive groups (the two halves of rotary pairs).  Cached by (pointer, shape, box).  Host side, defined in
 // gemm_tc.cu; the returned pointer is good until the next lookup (copy the map), under g_map_mutex.
 const CUtensorMap* get_panel_map(const void* ptr, int rows, int cols, int box_rows, int panels, int half);
 extern std::mutex g_map_mutex;
+// box = 64 columns x box_rows rows of a bf16 [rows, cols] matrix, like above.
+const CUtensorMap* get_rows_map(const void* ptr, int rows, int cols, int box_rows);
+// Weights for gemm_wm.cu: box = 64 columns x 128 rows, the rows of unit c4 (coordinate of the last dimension) in the order in which
+// the 32 lanes of each quarter want them.  Plain: rows 128 c4 + i.  Rope: 16 rows of the first half of a head, then their partners
+// (head dimension 64: c4 counts heads, two per box).  Pairs: 16 rows of the matrix at ptr, then the same rows of the one `step`
+// bytes further, 64 + 64 rows per unit.
+enum WeightOrder : int { kWeightsPlain = 1, kWeightsRope128, kWeightsRope64, kWeightsPairs };
+const CUtensorMap* get_weight_map(const void* ptr, int rows, int cols, WeightOrder order, int64_t step);
+
+// gemm_wm.cu: projections of more than 128 rows, weights as the product's M.  own_us: what the caller's own kernel would take, as
+// pair_loop_us has it.  0 = not taken (the caller launches its own), 1 = launched, -1 = the launch failed.
+int launch_gemm_wm(const GemmArgs& g, double own_us, int group_n, cudaStream_t stream);
+// Time of the main loop of a two-SM kernel: k_blocks of 64 one after the other, `columns` wide.  Measured at 615 rows (gate/up, 256
+// K blocks in a row): 0.33 us each at 256 columns, 0.285 at 208, 0.24 at 128; the instructions alone would take 0.27, 0.22, 0.14.
+inline double pair_loop_us(double k_blocks, int columns) { return k_blocks * (columns + 200) * 0.0007; }
 
 // gemm_rows.cu: projections of at most 128 rows whose tiles fit the SMs at once; 0 = not applicable (the caller then uses
 // the kernels of gemm_tc.cu), else the number of kernels launched, -1 if a launch failed.

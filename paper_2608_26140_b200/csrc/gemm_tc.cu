@@ -1,8 +1,8 @@
 // C[M, N] = A[M, K] * B[N, K]^T (bf16 in, fp32 accumulate) on the 5th-generation tensor
 // cores for the projections of the selective recomputation (Section 3.3).
 //
-// Projections of at most 128 rows run on gemm_rows.cu where their tiles fit the SMs at once; here, the rest of them (the LM
-// head, very wide ones) and everything above.
+// Projections of at most 128 rows run on gemm_rows.cu where their tiles fit the SMs at once; larger ones on gemm_wm.cu where chunks
+// of rows fill the rounds better than 256-row pairs; here, the rest of both (the LM head, very wide ones, cut tiles).
 //
 // gemm_tc_kernel (at most one CTA per SM):
 //   phase 0 (optional)  gather the rows of R (or take compact rows) and RMSNorm them into the
@@ -607,28 +607,6 @@ constexpr int kKeepWeightsFromPairs = 3;
 constexpr int kWholeTilesFromKB = 56;     // K blocks from which whole tiles were measured against cut ones (plan_gemm)
 constexpr int kSmallHeadPairs = 3, kSmallHeadBlocks = 24;   // an LM head stays on the one-SM kernel up to: row pairs, K blocks per CTA
 constexpr int kPrepKernelRows = 4096;     // from this many rows the row preparation is a kernel of its own
-__device__ __forceinline__ void tile_coords(int t, int m_pairs, int n_tiles, int group_n, int& nt, int& mp) {
-    const int full = n_tiles / group_n, per_group = group_n * m_pairs;
-    if (t < full * per_group) {
-        const int grp = t / per_group, r = t - grp * per_group;
-        mp = r / group_n;
-        nt = grp * group_n + (r - mp * group_n);
-    } else {
-        const int r = t - full * per_group, gn = n_tiles - full * group_n;
-        mp = r / gn;
-        nt = full * group_n + (r - mp * gn);
-    }
-}
-
-// TMA load into this CTA's shared memory that completes on a barrier of the CTA pair's leader
-__device__ __forceinline__ void tma_load_2d_pair(uint32_t dst, const CUtensorMap* map, int c0, int c1, uint32_t bar_cluster,
-                                                 uint64_t policy) {
-    asm volatile(
-        "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint "
-        "[%0], [%1, {%2, %3}], [%4], %5;"
-        ::"r"(dst), "l"(map), "r"(c0), "r"(c1), "r"(bar_cluster), "l"(policy)
-        : "memory");
-}
 // Ten warps leave a thread 168 registers.  With the rotary pairs finished 32 at a time and the whole gain requested early, 300
 // bytes were spilled; 16 at a time and half of the gain, 52: layer-step of 615 rows 369.5 -> 366.4 us, 5 x 203 rows 515 -> 509,
 // 64 x 103 rows 2666 -> 2629, refresh of 14 752 rows 12 286 -> 12 181.
@@ -948,7 +926,7 @@ EncodeTiledFn encode_fn() {
     return fn;
 }
 
-struct MapKey { const void* ptr; int rows, cols, box_rows, panels, half; };
+struct MapKey { const void* ptr; int rows, cols, box_rows, panels, half; int64_t step = 0; };
 struct MapEntry { MapKey key; CUtensorMap map; };
 constexpr int kMapCache = 1024;   // a 32-layer model has over 200 weight matrices
 MapEntry g_maps[kMapCache];
@@ -958,13 +936,13 @@ const CUtensorMap* lookup_map(const MapKey& want, int rank, const cuuint64_t* di
     for (int i = 0; i < g_map_count; ++i) {
         const MapKey& k = g_maps[i].key;
         if (k.ptr == want.ptr && k.rows == want.rows && k.cols == want.cols && k.box_rows == want.box_rows &&
-            k.panels == want.panels && k.half == want.half)
+            k.panels == want.panels && k.half == want.half && k.step == want.step)
             return &g_maps[i].map;
     }
     EncodeTiledFn fn = encode_fn();
     if (!fn) return nullptr;
     MapEntry& e = g_maps[g_map_next];
-    const cuuint32_t estr[4] = {1, 1, 1, 1};
+    const cuuint32_t estr[5] = {1, 1, 1, 1, 1};
     if (fn(&e.map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, rank, const_cast<void*>(want.ptr), dims, strides, box, estr,
            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
@@ -975,17 +953,28 @@ const CUtensorMap* lookup_map(const MapKey& want, int rank, const cuuint64_t* di
     return &e.map;
 }
 
-// bf16 [rows, cols] row-major, box = 128 rows x 64 cols, 128-byte swizzle, zero fill out of bounds; like every lookup here,
-// the pointer is only good until the next one (a miss may replace any entry): callers copy the map.
-const CUtensorMap* get_map(const void* ptr, int rows, int cols) {
-    const cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows}, strides[1] = {(cuuint64_t)cols * 2};
-    const cuuint32_t box[2] = {64, 128};
-    return lookup_map(MapKey{ptr, rows, cols, 128, 0, 0}, 2, dims, strides, box);
-}
-
 }  // namespace
 
 std::mutex g_map_mutex;
+
+// bf16 [rows, cols] row-major, box = box_rows rows x 64 cols, 128-byte swizzle, zero fill out of bounds; like every lookup here,
+// the pointer is only good until the next one (a miss may replace any entry): callers copy the map.
+const CUtensorMap* get_rows_map(const void* ptr, int rows, int cols, int box_rows) {
+    const cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows}, strides[1] = {(cuuint64_t)cols * 2};
+    const cuuint32_t box[2] = {64, (cuuint32_t)box_rows};
+    return lookup_map(MapKey{ptr, rows, cols, box_rows, 0, 0}, 2, dims, strides, box);
+}
+
+const CUtensorMap* get_weight_map(const void* ptr, int rows, int cols, WeightOrder order, int64_t step) {
+    const cuuint64_t row = (cuuint64_t)cols * 2, k = (cuuint64_t)cols, n = (cuuint64_t)rows;
+    const MapKey key{ptr, rows, cols, 128, -(int)order, 0, step};
+    struct Shape { cuuint64_t dims[5], strides[4]; cuuint32_t box[5]; };
+    const Shape s = order == kWeightsPlain   ? Shape{{k, 128, 1, 1, n / 128}, {row, row * 128, row * 128, row * 128}, {64, 128, 1, 1, 1}}
+                  : order == kWeightsRope128 ? Shape{{k, 16, 2, 4, n / 128}, {row, row * 64, row * 16, row * 128}, {64, 16, 2, 4, 1}}
+                  : order == kWeightsRope64  ? Shape{{k, 16, 2, 2, n / 64}, {row, row * 32, row * 16, row * 64}, {64, 16, 2, 2, 2}}
+                                             : Shape{{k, 16, 2, 4, n / 64}, {row, (cuuint64_t)step, row * 16, row * 64}, {64, 16, 2, 4, 1}};
+    return lookup_map(key, 5, s.dims, s.strides, s.box);
+}
 
 const CUtensorMap* get_panel_map(const void* ptr, int rows, int cols, int box_rows, int panels, int half) {
     const cuuint64_t row = (cuuint64_t)cols * 2;
@@ -1035,7 +1024,7 @@ TcPlan make_plan(int M, int K, int units, bool swiglu) {
 struct GemmLaunch {
     TcPlan p;
     bool pair;                // gemm_tc2_kernel
-    int clusters;
+    int clusters, max_clusters;
     SplitTiles split;
 };
 
@@ -1100,6 +1089,7 @@ GemmLaunch plan_gemm(const GemmArgs& g) {
         p.group_n = group_n;
         static const int w_keep_from = [] { const char* e = getenv("ACACHE_GEMM_WKEEP_PAIRS"); return e ? atoi(e) : kKeepWeightsFromPairs; }();
         gl.clusters = std::min(max_clusters, tiles);
+        gl.max_clusters = max_clusters;
         // Cutting tiles pays up to about two thirds of a wave, unless K is so short that the finish costs what the shorter main
         // loop gains: of a whole tile's time the cut loop took 0.66-0.70 at 0.44 of its K blocks and 0.83-0.90 at 0.65 (partial
         // tiles included), the finish that of about 20 K blocks.  (us, whole | cut + finish: 512 rows output 32.0 | 22.3 + 7.3,
@@ -1172,17 +1162,22 @@ static int launch_gemm_impl(const GemmArgs& g, cudaStream_t stream) {
     const bool swiglu = g.epilogue == kEpiSwiGLU;
     const GemmLaunch gl = plan_gemm(g);
     const TcPlan& p = gl.p;
+    if (gl.pair && !p.pair_u) {
+        // whole tiles, which are the same sums with the weights as the product's M, where that takes less time
+        const int tiles = p.m_pairs * p.n_tiles, rounds = (tiles + gl.max_clusters - 1) / gl.max_clusters;
+        if (const int n = launch_gemm_wm(g, pair_loop_us((double)rounds * p.KB, 256), p.group_n, stream)) return n;
+    }
     std::lock_guard<std::mutex> lock(g_map_mutex);
     CUtensorMap map_a, map_b[3];
     {
-        const CUtensorMap* m = get_map(g.a, g.M, g.K);
+        const CUtensorMap* m = get_rows_map(g.a, g.M, g.K, TC_BM);
         if (!m) return -1;
         map_a = *m;
     }
     bool have_b[3] = {false, false, false};
     for (int i = 0; i < 3; ++i)
         if (g.b[i]) {
-            const CUtensorMap* m = get_map(g.b[i], swiglu ? g.n[0] : g.n[i], g.K);
+            const CUtensorMap* m = get_rows_map(g.b[i], swiglu ? g.n[0] : g.n[i], g.K, 128);
             if (m) { map_b[i] = *m; have_b[i] = true; }
         }
     if (!have_b[0]) return -1;

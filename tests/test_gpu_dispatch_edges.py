@@ -254,3 +254,27 @@ def test_short_contractions_are_cut_up_to_two_thirds_of_a_wave():
         check_against_oracle(dc, anchors, k_new, v_new, y, None, None, rows)
         launches.append(dc.ctx.launch_count())
     assert launches[0] == launches[1] == launches[2]
+
+
+# Whole tiles with the weights as the product's M: chunks of 96 to 256 rows, the last one part-filled; both rotary orders, biases and
+# grouped heads, fewer K blocks than ring stages, w_up in memory above and below w_gate; the residual epilogue in the last shape.
+WM128 = wl.LayerShape(256, 40, 5, 128, 3328, 1e-5, True, 5e5, "wm-d128")
+WM64 = wl.LayerShape(256, 80, 10, 64, 3328, 1e-5, True, 5e5, "wm-d64")
+WM_WIDE = wl.LayerShape(6400, 2, 1, 128, 256, 1e-5, False, 5e5, "wm-wide")
+
+
+@pytest.mark.parametrize("shape,rows,up_first", [(WM128, 280, False), (WM128, 333, True), (WM128, 545, False), (WM64, 260, True),
+                                                 (WM64, 417, False), (WM_WIDE, 257, False), (WM_WIDE, 400, False)])
+def test_weights_as_m_projections(shape, rows, up_first):
+    lay = wl.make_layout(1, 3, rows + 30, 8, 8, 8, "none")
+    case = wl.make_case(shape, lay, 0.0, cfg_id=81, weights=cached_weights(shape, 81))
+    dc = DeviceCase(case, max_rows=rows)
+    order = ("w_up", "w_gate") if up_first else ("w_gate", "w_up")
+    both = torch.stack([dc.w_dev[n] for n in order])
+    for i, n in enumerate(order):
+        dc.w_dev[n] = both[i]
+    dc.lw = ab.Context.weights(dc.w_dev)
+    anchors = np.sort(np.random.default_rng(rows).choice(lay.affix_len, rows, replace=False)).astype(np.int32)[None]
+    k_new, v_new, y = run_split_calls(dc, torch.from_numpy(anchors).to(DEV), rows)
+    assert dc.ctx.poll_status() == 0
+    check_against_oracle(dc, anchors, k_new, v_new, y, None, None, rows)

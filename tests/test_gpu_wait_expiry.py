@@ -19,6 +19,7 @@ pytestmark = pytest.mark.gpu
 
 # q/k/v of few rows and a long K: cut between the CTAs of a cluster, which pass their barriers whatever ran out
 DEEP128 = wl.LayerShape(3584, 4, 1, 128, 256, 1e-6, True, 1e6, "deep-d128")
+WIDE_Q128 = wl.LayerShape(256, 40, 5, 128, 256, 1e-5, True, 5e5, "wide-q-d128")
 LONG128 = wl.LayerShape(2560, 6, 3, 128, 256, 1e-6, True, 1e6, "long-d128")
 
 
@@ -28,6 +29,7 @@ LONG128 = wl.LayerShape(2560, 6, 3, 128, 256, 1e-6, True, 1e6, "long-d128")
     (LONG128, 1, 160, "none", "gemm_rows_kernel<2, 0, false>"),
     (DEEP128, 1, 300, "none", "gemm_rows_kernel<4, 0, false>"),
     (MID128, 2, 400, "all", "gemm_tc2_kernel"),                      # several 128-row tiles: the two-SM projection kernel
+    (WIDE_Q128, 2, 400, "all", "gemm_wm_kernel<0>"),                 # the same, more columns: weights as the product's M
 ])
 def test_a_wait_that_runs_out_is_reported_and_the_context_stays_usable(shape, B, L, extra, kernel):
     lay = wl.make_layout(B, 4, L, 40, 32, 32, extra)
