@@ -744,7 +744,7 @@ attention_tc2q_kernel(const AttnTcArgs a, const __grid_constant__ CUtensorMap ma
         // in the one-tile kernel)
         const uint32_t idesc_s = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(128 >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
         const uint32_t idesc_o = idesc_s | (1u << 16);       // B = V is MN-major
-        auto wait = [&](int i, uint32_t parity) { return __all_sync(0xffffffffu, mbar_spin(bar(i), parity, abort_flag)); };
+        auto wait = [&](int i, uint32_t parity) { return __all_sync(0xffffffffu, mbar_poll(bar(i), parity, abort_flag)); };
         auto issue_s = [&](int t, int j) {                   // S_t = Q_t K_j^T, then s_full of query tile t
             const uint32_t k = sK0 + (j & 1) * AT_TILE;
             if (!elect_lane()) return;
@@ -830,35 +830,45 @@ attention_tc2q_kernel(const AttnTcArgs a, const __grid_constant__ CUtensorMap ma
       if (has_rows) {
         // ---------------- softmax: one thread per query row ----------------
         const float2 sc2 = make_float2(a.scale_log2e, a.scale_log2e);
+        // The keys that count are worked out a tile at a time, before the wait for its S, and not at all for tiles that lie whole
+        // inside the context and inside or outside the affix span: worked out per half they took some 400 cycles between the first
+        // half's P and the second half's logits, on the chain of every tile.  With the issuing warp's waits as polls: 14 752 rows
+        // over 2560 keys 790 -> 768 us alone, 1095 -> 1063 back to back under the power cap.  Bound by that chain still (of 5000
+        // cycles per key tile and two query tiles 1900 are issue, 2200 tensor work), not by a unit.
+        uint32_t keep4[4] = {~0u, ~0u, ~0u, ~0u}, aff4[4] = {0u, 0u, 0u, 0u};
+        const int aff0 = a.affix_start, aff1 = a.affix_start + a.affix_len;
         for (int i = 0; i < 2 * n_tiles && ok; ++i) {
             const int hb = i & 1, j = i >> 1;
-            // which of the half's 64 keys count: the cache's positions up to the context end, minus those a
-            // fresh row serves; of the fresh rows, those that serve their position
-            uint32_t keep[2];
+            if (hb == 0) {
+                const int k0 = j * 128;
+                const bool in = !want_lf || (k0 >= aff0 && k0 + 128 <= aff1), out = !want_lf || k0 >= aff1 || k0 + 128 <= aff0;
+                if (!a.pos_excl && k0 + 128 <= a.ctx_len && (in || out)) {
 #pragma unroll
-            for (int c = 0; c < 2; ++c) {
-                const int w = hb * 2 + c;
-                if (j < n_cache_tiles) {
-                    const int valid = a.ctx_len - j * 128 - w * 32;
-                    keep[c] = valid >= 32 ? 0xffffffffu : (valid <= 0 ? 0u : (1u << valid) - 1u);
-                    if (a.pos_excl && j * 4 + w < a.excl_words) keep[c] &= ~__ldg(a.pos_excl + (int64_t)b * a.excl_words + j * 4 + w);
+                    for (int w = 0; w < 4; ++w) { keep4[w] = ~0u; aff4[w] = want_lf && in ? ~0u : 0u; }
                 } else {
-                    const int fw = (j - n_cache_tiles) * 4 + w;
-                    keep[c] = fw < a.keep_words ? __ldg(a.row_keep + (int64_t)b * a.keep_words + fw) : 0u;
-                }
-            }
-            // of those keys, the ones inside the affix span (cache tiles only): all, none, or some (then the slow path)
-            uint32_t aff[2] = {0u, 0u};
-            if (want_lf && j < n_cache_tiles) {
+                    // which of the tile's keys count: the cache's positions up to the context end, minus those a fresh row
+                    // serves; of the fresh rows, those that serve their position
 #pragma unroll
-                for (int c = 0; c < 2; ++c) {
-                    const int k0 = j * 128 + (hb * 2 + c) * 32;
-                    const int lo = max(a.affix_start - k0, 0), hi = min(a.affix_start + a.affix_len - k0, 32);
-                    if (hi > lo) aff[c] = (hi - lo >= 32 ? 0xffffffffu : ((1u << (hi - lo)) - 1u) << lo);
+                    for (int w = 0; w < 4; ++w) {
+                        aff4[w] = 0u;
+                        if (j < n_cache_tiles) {
+                            const int valid = a.ctx_len - k0 - w * 32;
+                            keep4[w] = valid >= 32 ? ~0u : (valid <= 0 ? 0u : (1u << valid) - 1u);
+                            if (a.pos_excl && j * 4 + w < a.excl_words) keep4[w] &= ~__ldg(a.pos_excl + (int64_t)b * a.excl_words + j * 4 + w);
+                            // of those keys, the ones inside the affix span
+                            const int lo = max(aff0 - k0 - w * 32, 0), hi = min(aff1 - k0 - w * 32, 32);
+                            if (want_lf && hi > lo) aff4[w] = (hi - lo >= 32 ? ~0u : ((1u << (hi - lo)) - 1u) << lo);
+                        } else {
+                            const int fw = (j - n_cache_tiles) * 4 + w;
+                            keep4[w] = fw < a.keep_words ? __ldg(a.row_keep + (int64_t)b * a.keep_words + fw) : 0u;
+                        }
+                    }
                 }
             }
-            const bool aff_all = (aff[0] & aff[1]) == 0xffffffffu, aff_none = (aff[0] | aff[1]) == 0u;
-            const bool all = (keep[0] & keep[1]) == 0xffffffffu && (aff_all || aff_none);
+            const uint32_t keep[2] = {hb ? keep4[2] : keep4[0], hb ? keep4[3] : keep4[1]};
+            const uint32_t aff[2] = {hb ? aff4[2] : aff4[0], hb ? aff4[3] : aff4[1]};
+            const bool aff_all = (aff[0] & aff[1]) == ~0u, aff_none = (aff[0] | aff[1]) == 0u;
+            const bool all = (keep[0] & keep[1]) == ~0u && (aff_all || aff_none);
             // warp-uniform: the tensor-memory accesses below are collective
             if (hb == 0) {
                 if (!(ok = __all_sync(0xffffffffu, mbar_spin(bar(9 + t), j & 1, abort_flag)))) break;
@@ -881,19 +891,18 @@ attention_tc2q_kernel(const AttnTcArgs a, const __grid_constant__ CUtensorMap ma
                     sv[c][2 * e] = r.x;
                     sv[c][2 * e + 1] = r.y;
                 }
-            float m4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
-            if (all) {
+            // masked keys as -inf: their P is 0
+            if (!all) {
 #pragma unroll
                 for (int c = 0; c < 2; ++c)
 #pragma unroll
-                    for (int e = 0; e < 32; ++e) m4[e & 3] = fmaxf(m4[e & 3], sv[c][e]);
-            } else {
-#pragma unroll
-                for (int c = 0; c < 2; ++c)
-#pragma unroll
-                    for (int e = 0; e < 32; ++e)
-                        if ((keep[c] >> e) & 1u) m4[e & 3] = fmaxf(m4[e & 3], sv[c][e]);
+                    for (int e = 0; e < 32; ++e) sv[c][e] = ((keep[c] >> e) & 1u) ? sv[c][e] : -INFINITY;
             }
+            float m4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+#pragma unroll
+            for (int c = 0; c < 2; ++c)
+#pragma unroll
+                for (int e = 0; e < 32; e += 2) m4[(e >> 1) & 3] = fmaxf(fmaxf(m4[(e >> 1) & 3], sv[c][e]), sv[c][e + 1]);
             const float mx = fmaxf(fmaxf(m4[0], m4[1]), fmaxf(m4[2], m4[3]));
             const bool raise = mx > kRescaleGap || (first && mx > -INFINITY);
             if (__any_sync(0xffffffffu, raise)) {
@@ -941,8 +950,7 @@ attention_tc2q_kernel(const AttnTcArgs a, const __grid_constant__ CUtensorMap ma
                 } else {
 #pragma unroll
                     for (int e = 0; e < 32; e += 2) {
-                        const float p0 = ((keep[c] >> e) & 1u) ? fast_exp2(sv[c][e]) : 0.f;
-                        const float p1 = ((keep[c] >> (e + 1)) & 1u) ? fast_exp2(sv[c][e + 1]) : 0.f;
+                        const float p0 = fast_exp2(sv[c][e]), p1 = fast_exp2(sv[c][e + 1]);
                         l2a = __fadd2_rn(l2a, make_float2(p0, p1));
                         lf2 = __fadd2_rn(lf2, make_float2(((aff[c] >> e) & 1u) ? p0 : 0.f, ((aff[c] >> (e + 1)) & 1u) ? p1 : 0.f));
                         pk[c * 16 + (e >> 1)] = pack_bf16(p0, p1);
