@@ -320,7 +320,7 @@ int launch_wm(const GemmArgs& g, double own_us, int group_n, cudaStream_t stream
     p.stage_bytes = WM_W_BYTES + p.NC * 64;
     p.stages = std::min(WM_MAX_STAGES, (WM_SMEM_DYN - 1024 - WM_STAGING) / p.stage_bytes);
     p.smem_bytes = 1024 + p.stages * p.stage_bytes + WM_STAGING;
-    p.keep = p.chunks >= 3;
+    p.keep = p.chunks >= 4;       // three chunks (615 rows) keep time by themselves: attention and gate/up behind q/k/v 1-2 us faster without
     CUtensorMap map_x, map_w[3];
     {
         std::lock_guard<std::mutex> lock(g_map_mutex);
