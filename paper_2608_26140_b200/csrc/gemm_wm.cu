@@ -324,20 +324,19 @@ int launch_wm(const GemmArgs& g, double own_us, int group_n, cudaStream_t stream
     CUtensorMap map_x, map_w[3];
     {
         std::lock_guard<std::mutex> lock(g_map_mutex);
+        // a map that cannot be made leaves the projection to the caller's kernel, whose maps have two dimensions
         const CUtensorMap* m = get_rows_map(g.a, g.M, g.K, p.NC / 2);
-        if (!m) return -1;
+        if (!m) return 0;
         map_x = *m;
         const char *gate = static_cast<const char*>(g.b[0]), *up = static_cast<const char*>(g.b[1]);
         p.up_first = EPI == kEpiSwiGLU && up < gate;
+        const int64_t step = p.up_first ? gate - up : up - gate;
+        if (EPI == kEpiSwiGLU && (step <= 0 || step >= ((int64_t)1 << 40))) return 0;
         for (int i = 0; i < 3; ++i) {
-            if (EPI == kEpiSwiGLU) {
-                const int64_t step = p.up_first ? gate - up : up - gate;
-                if (step <= 0 || step >= ((int64_t)1 << 40)) return 0;
-                m = get_weight_map(p.up_first ? up : gate, g.n[0], g.K, kWeightsPairs, step);
-            } else {
-                m = g.b[i] ? get_weight_map(g.b[i], g.n[i], g.K, EPI == kEpiQKV ? (g.head_dim == 128 ? kWeightsRope128 : kWeightsRope64) : kWeightsPlain, 0) : m;
-            }
-            if (!m) return -1;
+            if (EPI == kEpiSwiGLU && i == 0) m = get_weight_map(p.up_first ? up : gate, g.n[0], g.K, kWeightsPairs, step);   // both matrices
+            else if (EPI != kEpiSwiGLU && g.b[i])
+                m = get_weight_map(g.b[i], g.n[i], g.K, EPI != kEpiQKV ? kWeightsPlain : g.head_dim == 128 ? kWeightsRope128 : kWeightsRope64, 0);
+            if (!m) return 0;
             map_w[i] = *m;
         }
     }
