@@ -393,11 +393,15 @@ enum WeightOrder : int { kWeightsPlain = 1, kWeightsRope128, kWeightsRope64, kWe
 const CUtensorMap* get_weight_map(const void* ptr, int rows, int cols, WeightOrder order, int64_t step);
 
 // gemm_wm.cu: projections of more than 128 rows, weights as the product's M.  own_us: what the caller's own kernel would take, as
-// pair_loop_us has it.  0 = not taken (the caller launches its own), 1 = launched, -1 = the launch failed.
+// pair_tile_us has it.  0 = not taken (the caller launches its own), 1 = launched, -1 = the launch failed.
 int launch_gemm_wm(const GemmArgs& g, double own_us, int group_n, cudaStream_t stream);
-// Time of the main loop of a two-SM kernel: k_blocks of 64 one after the other, `columns` wide.  Measured at 615 rows (gate/up, 256
-// K blocks in a row): 0.33 us each at 256 columns, 0.285 at 208, 0.24 at 128; the instructions alone would take 0.27, 0.22, 0.14.
-inline double pair_loop_us(double k_blocks, int columns) { return k_blocks * (columns + 200) * 0.0007; }
+// Time from one tile of a two-SM kernel to the next: its main loop, k_blocks of 64 one after the other, `columns` wide, or the epilogue
+// of the tile before it, if that is longer, and about 1 us for the change of tiles.  Measured at 615 rows (gate/up, 256 K blocks in a
+// row): 0.33 us a K block at 256 columns, 0.285 at 208, 0.24 at 128; the instructions alone would take 0.27, 0.22, 0.14.
+inline double pair_tile_us(int k_blocks, int columns, double epilogue_us) {
+    const double loop_us = k_blocks * (columns + 200) * 0.0007;
+    return 1.0 + (loop_us > epilogue_us ? loop_us : epilogue_us);
+}
 
 // gemm_rows.cu: projections of at most 128 rows whose tiles fit the SMs at once; 0 = not applicable (the caller then uses
 // the kernels of gemm_tc.cu), else the number of kernels launched, -1 if a launch failed.

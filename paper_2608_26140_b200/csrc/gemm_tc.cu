@@ -604,6 +604,7 @@ constexpr int TC2_SMEM = TC2_STAGES * TC2_STAGE_BYTES + 1024 + 256;
 // (4, 24, 32, 48 are slower), and cutting the row pairs into L2-sized blocks as well changes nothing more.
 constexpr int kTileGroupN = 16;
 constexpr int kKeepWeightsFromPairs = 3;
+constexpr double kPairEpilogueUs = 9;     // epilogue of a 256 x 256 tile (1024 columns of K, rounds 1 to 3 of gate/up: 19, 28, 37 us)
 constexpr int kWholeTilesFromKB = 56;     // K blocks from which whole tiles were measured against cut ones (plan_gemm)
 constexpr int kSmallHeadPairs = 3, kSmallHeadBlocks = 24;   // an LM head stays on the one-SM kernel up to: row pairs, K blocks per CTA
 constexpr int kPrepKernelRows = 4096;     // from this many rows the row preparation is a kernel of its own
@@ -1165,7 +1166,7 @@ static int launch_gemm_impl(const GemmArgs& g, cudaStream_t stream) {
     if (gl.pair && !p.pair_u) {
         // whole tiles, which are the same sums with the weights as the product's M, where that takes less time
         const int tiles = p.m_pairs * p.n_tiles, rounds = (tiles + gl.max_clusters - 1) / gl.max_clusters;
-        if (const int n = launch_gemm_wm(g, pair_loop_us((double)rounds * p.KB, 256), p.group_n, stream)) return n;
+        if (const int n = launch_gemm_wm(g, rounds * pair_tile_us(p.KB, 256, kPairEpilogueUs), p.group_n, stream)) return n;
     }
     std::lock_guard<std::mutex> lock(g_map_mutex);
     CUtensorMap map_a, map_b[3];

@@ -30,6 +30,7 @@ constexpr int WM_MAX_STAGES = 8;
 constexpr int WM_PIECE = 32 * 33 * 4;                 // a 32 x 32 piece in shared memory, rows of 33 words
 constexpr int WM_STAGING = 8 * WM_PIECE;
 constexpr int WM_SMEM_DYN = 227 * 1024 - 512;         // beside the barriers and reduction words
+constexpr double kRowEpilogueUs = 0.05, kBehindUs = 0.75;   // the rule's, see launch_wm
 
 struct WmPlan {
     int NC, chunks;           // rows per chunk (a multiple of 16), chunks
@@ -303,14 +304,20 @@ int launch_wm(const GemmArgs& g, double own_us, int group_n, cudaStream_t stream
     p.KB = g.K / 64;
     p.w_tiles = EPI == kEpiSwiGLU ? g.n[0] / 128 : (g.n[0] + g.n[1] + g.n[2]) / 256;
     p.group_n = group_n;
-    // the least time of the main loops, if it is at least 2 % less than the caller's
+    // The least time, if it is 2 % and kBehindUs less than the caller's (behind this kernel a finish kernel takes 0.5-1 us longer, the
+    // attention up to 0.8).  An epilogue takes 0.05 us a row here (1024 columns of K, a round of 208 rows of gate/up: 8-10 us for 4.6
+    // of main loop) and 9 us a tile there; by main loops alone gate/up of short contractions came here and lost (us of a layer-step,
+    // there | here: 2045 rows of 256 columns 83.6 | 87.5, 2700 of 1024 165 | 178, 800 of 2048 160 | 168).  With it, all projections
+    // there | as chosen, 4096 columns: 129 rows 159.7 | 150.6, 300 218.9 | 203.7, 512 232.8 | 232.7, 615 291.5 | 281.0, 800 356 | 332,
+    // 1200 508 | 477, 2045 729 | 727; 3584 columns: 129 146.4 | 143.6, 300 217 | 206, 615 299 | 288, 800 373 | 342, 1200 474 | 459,
+    // 2045 755 | 727.  What is left on the wrong side: down projection of 3496 rows of a 1024-column model 169.5 | 173.0.
     const int first = (g.M + 255) / 256;
-    double best = 0.98 * own_us;
+    double best = 0.98 * own_us - kBehindUs;
     for (int chunks = first; chunks <= first + 6; ++chunks) {
         const int NC = ((g.M + chunks - 1) / chunks + 15) & ~15;
         if (NC < 64) break;
         const int tiles = p.w_tiles * chunks, rounds = (tiles + max_clusters - 1) / max_clusters;
-        const double t = pair_loop_us((double)rounds * p.KB, NC);
+        const double t = rounds * pair_tile_us(p.KB, NC, NC * kRowEpilogueUs);
         if (t >= best) continue;
         best = t;
         p.NC = NC; p.chunks = chunks;
@@ -320,7 +327,10 @@ int launch_wm(const GemmArgs& g, double own_us, int group_n, cudaStream_t stream
     p.stage_bytes = WM_W_BYTES + p.NC * 64;
     p.stages = std::min(WM_MAX_STAGES, (WM_SMEM_DYN - 1024 - WM_STAGING) / p.stage_bytes);
     p.smem_bytes = 1024 + p.stages * p.stage_bytes + WM_STAGING;
-    p.keep = p.chunks >= 4;       // three chunks (615 rows) keep time by themselves: attention and gate/up behind q/k/v 1-2 us faster without
+    // From four chunks on the next round reads the weights again (16 weight tiles of a group x 4 chunks are a round).  Layer-step, us,
+    // kept | not: one chunk (129 rows) 165 | 151, two (300) 213 | 204, three (615) 283 | 281; four (800) 332 | 333, 3584 columns 342 | 345;
+    // six and nine (1200) 477 | 480, (1800) 648 | 663.
+    p.keep = p.chunks >= 4;
     CUtensorMap map_x, map_w[3];
     {
         std::lock_guard<std::mutex> lock(g_map_mutex);

@@ -278,3 +278,21 @@ def test_weights_as_m_projections(shape, rows, up_first):
     k_new, v_new, y = run_split_calls(dc, torch.from_numpy(anchors).to(DEV), rows)
     assert dc.ctx.poll_status() == 0
     check_against_oracle(dc, anchors, k_new, v_new, y, None, None, rows)
+
+
+def split_calls_and_kernels(dc, anchors):
+    with torch.profiler.profile(activities=[torch.profiler.ProfilerActivity.CUDA]) as prof:
+        out = run_split_calls(dc, torch.from_numpy(anchors[None].copy()).to(DEV), len(anchors))
+        torch.cuda.synchronize()
+    assert dc.ctx.poll_status() == 0
+    return out, " ".join(e.key for e in prof.key_averages())
+
+
+# Gate/up with few K blocks is bound by its epilogue, which is the longer one with the weights as M, whatever the chunks save.
+@pytest.mark.parametrize("shape,rows", [(wl.TINY, 2045), (wl.LayerShape(1024, 2, 1, 128, 3072, 1e-5, False, 5e5, "gate-up-1k"), 615)])
+def test_short_contractions_stay_on_whole_tiles(shape, rows):
+    lay = wl.make_layout(1, 3, rows + 30, 8, 8, 8, "none")
+    dc = DeviceCase(wl.make_case(shape, lay, 0.0, cfg_id=82), max_rows=rows)
+    anchors = np.sort(np.random.default_rng(rows).choice(lay.affix_len, rows, replace=False)).astype(np.int32)
+    _, kernels = split_calls_and_kernels(dc, anchors)
+    assert "gemm_tc2_kernel" in kernels and "gemm_wm_kernel" not in kernels, kernels
