@@ -675,7 +675,9 @@ gemm_tc2_kernel(const GemmArgs g, const TcPlan p, const int clusters, const __gr
             const CUtensorMap* map_b = bs == 0 ? &mapB0 : bs == 1 ? &mapB1 : &mapB2;
             const int arow = (mp * 2 + (int)rank) * TC_BM;
             for (int kb = kb0; kb < kb1; ++kb) {
-                if (!(ok = __all_sync(0xffffffffu, mbar_poll(empty_bar(stage), phase ^ 1, abort_flag)))) break;
+                // The first round of the ring and the first two accumulators are free: polled all the same, by the whole warp, they cost
+                // a launch of a few K blocks 0.05-0.1 us (refresh of 4 x 307 rows of 256 columns, 4 layers, 313.8 -> 312.8).
+                if (issued >= TC2_STAGES && !(ok = __all_sync(0xffffffffu, mbar_poll(empty_bar(stage), phase ^ 1, abort_flag)))) break;
                 if (elect_lane()) {
                     const uint32_t sA = base + stage * TC2_STAGE_BYTES, sB = sA + TC_A_BYTES;
                     const uint32_t lead_full = mapa_u32(full_bar(stage), 0);
@@ -703,7 +705,7 @@ gemm_tc2_kernel(const GemmArgs g, const TcPlan p, const int clusters, const __gr
         // the issue.  Back to back: 64 x 103 rows 2693 -> 2574 us, refresh of 14 752 rows 12 468 -> 12 112 (q/k/v 1209 -> 1043,
         // output 442 -> 375 a launch), probe of 20 480 rows 16 876 -> 16 341, 615 rows 374.7 -> 368.0; cluster-scope polls in the
         // same loop: refresh 12 400.
-        int stage = 0, acc = 0;
+        int stage = 0, acc = 0, started = 0;
         uint32_t phase = 0, acc_phase = 0;
         bool ok = __all_sync(0xffffffffu, !*abort_flag);
         const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(256 >> 3) << 17) | ((uint32_t)(256 >> 4) << 24);
@@ -712,7 +714,7 @@ gemm_tc2_kernel(const GemmArgs g, const TcPlan p, const int clusters, const __gr
         for (int t = p.pair_u ? (int)(it / p.KB) : cluster_id; ok && (p.pair_u ? it < it_end : t < tiles);) {
             const int kb0 = p.pair_u ? (int)(it - (long long)t * p.KB) : 0;
             const int kb1 = p.pair_u ? (int)min((long long)p.KB, (long long)(kb0 + (it_end - it))) : p.KB;
-            if (!(ok = __all_sync(0xffffffffu, mbar_poll_cluster(tempty_bar(acc), acc_phase ^ 1, abort_flag)))) break;
+            if (started++ >= 2 && !(ok = __all_sync(0xffffffffu, mbar_poll_cluster(tempty_bar(acc), acc_phase ^ 1, abort_flag)))) break;
             tc_fence_after();
             const uint32_t d_tmem = tmem_base + acc * TC_BN;
             for (int kb = kb0; kb < kb1; ++kb) {
