@@ -694,6 +694,7 @@ gemm_tc2_kernel(const GemmArgs g, const TcPlan p, const int clusters, const __gr
         }
         // wait until the MMAs have consumed everything this CTA loaded, so that no signal from the
         // leader can arrive after this CTA has left
+        if (issued < TC2_STAGES) { stage = 0; phase = 1; }
         for (int i = 0; i < min(issued, TC2_STAGES) && ok; ++i) {
             ok = __all_sync(0xffffffffu, mbar_poll(empty_bar(stage), phase ^ 1, abort_flag));
             if (++stage == TC2_STAGES) { stage = 0; phase ^= 1; }
