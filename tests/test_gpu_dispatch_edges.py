@@ -8,6 +8,7 @@ from paper_2608_26140_b200 import binding as ab
 from paper_2608_26140_b200 import workloads as wl
 
 from helpers import DEV, DeviceCase, assert_close_bf16, cached_weights, oracle_step
+from launched_kernels import launched_kernels
 from test_gpu_parity import MID128, check_against_oracle, run_layer_step, run_split_calls
 from test_gpu_predict_commit import test_predict_commit as check_predict_commit
 
@@ -256,43 +257,71 @@ def test_short_contractions_are_cut_up_to_two_thirds_of_a_wave():
     assert launches[0] == launches[1] == launches[2]
 
 
-# Whole tiles with the weights as the product's M: chunks of 96 to 256 rows, the last one part-filled; both rotary orders, biases and
-# grouped heads, fewer K blocks than ring stages, w_up in memory above and below w_gate; the residual epilogue in the last shape.
+# Whole tiles with the weights as the product's M (gemm_wm_kernel), both rotary orders, biases and grouped heads, w_up in memory above
+# and below w_gate, the residual epilogue in the WIDE shapes.  256 columns: fewer K blocks than ring stages, chunks of 64 to 144
+# rows, the last one part-filled or full (288); where chunks save too little, whole tiles.  1024 columns: the ring wraps; 140 rows are
+# one chunk of 144, 540 rows four, three tiles to a cluster, so that an accumulator is taken again.
 WM128 = wl.LayerShape(256, 40, 5, 128, 3328, 1e-5, True, 5e5, "wm-d128")
 WM64 = wl.LayerShape(256, 80, 10, 64, 3328, 1e-5, True, 5e5, "wm-d64")
 WM_WIDE = wl.LayerShape(6400, 2, 1, 128, 256, 1e-5, False, 5e5, "wm-wide")
+WM128_DEEP = wl.LayerShape(1024, 92, 4, 128, 6400, 1e-5, True, 5e5, "wm-d128-deep")
+WM64_DEEP = wl.LayerShape(1024, 184, 8, 64, 6400, 1e-5, True, 5e5, "wm-d64-deep")
+WM_WIDE_DEEP = wl.LayerShape(12800, 8, 1, 128, 1024, 1e-5, True, 5e5, "wm-wide-deep")
+WM_CASES = [(WM128, 280, False), (WM128, 288, True), (WM128, 333, True), (WM128, 545, False), (WM64, 260, True), (WM64, 300, False),
+            (WM64, 417, False), (WM_WIDE, 257, False), (WM_WIDE, 400, False), (WM_WIDE, 545, False), (WM128_DEEP, 140, True),
+            (WM128_DEEP, 540, False), (WM64_DEEP, 140, False), (WM64_DEEP, 540, True)]
+WM_TOO_LITTLE = [(WM128, 333), (WM64, 417), (WM_WIDE, 400)]
 
 
-@pytest.mark.parametrize("shape,rows,up_first", [(WM128, 280, False), (WM128, 333, True), (WM128, 545, False), (WM64, 260, True),
-                                                 (WM64, 417, False), (WM_WIDE, 257, False), (WM_WIDE, 400, False)])
-def test_weights_as_m_projections(shape, rows, up_first):
-    lay = wl.make_layout(1, 3, rows + 30, 8, 8, 8, "none")
+def wm_case(shape, rows, max_rows, up_first):
+    lay = wl.make_layout(1, 3, max_rows + 30, 8, 8, 8, "none")
     case = wl.make_case(shape, lay, 0.0, cfg_id=81, weights=cached_weights(shape, 81))
-    dc = DeviceCase(case, max_rows=rows)
+    dc = DeviceCase(case, max_rows=max_rows)
     order = ("w_up", "w_gate") if up_first else ("w_gate", "w_up")
     both = torch.stack([dc.w_dev[n] for n in order])
     for i, n in enumerate(order):
         dc.w_dev[n] = both[i]
     dc.lw = ab.Context.weights(dc.w_dev)
-    anchors = np.sort(np.random.default_rng(rows).choice(lay.affix_len, rows, replace=False)).astype(np.int32)[None]
-    k_new, v_new, y = run_split_calls(dc, torch.from_numpy(anchors).to(DEV), rows)
+    return dc, np.sort(np.random.default_rng(rows).choice(lay.affix_len, max_rows, replace=False)).astype(np.int32)
+
+
+def wm_split_calls(dc, anchors):
+    out = run_split_calls(dc, torch.from_numpy(anchors[None].copy()).to(DEV), len(anchors))
     assert dc.ctx.poll_status() == 0
-    check_against_oracle(dc, anchors, k_new, v_new, y, None, None, rows)
+    return out
 
 
-def split_calls_and_kernels(dc, anchors):
-    with torch.profiler.profile(activities=[torch.profiler.ProfilerActivity.CUDA]) as prof:
-        out = run_split_calls(dc, torch.from_numpy(anchors[None].copy()).to(DEV), len(anchors))
-        torch.cuda.synchronize()
-    assert dc.ctx.poll_status() == 0
-    return out, " ".join(e.key for e in prof.key_averages())
+# The next two tests compare results; this one says that the kernel they mean is the one that runs.  Gate/up with few K blocks is
+# bound by its epilogue, which is the longer one with the weights as M, whatever the chunks save: the last two.
+def test_which_projections_take_the_weights_as_m():
+    short = [(wl.TINY, 2045), (wl.LayerShape(1024, 2, 1, 128, 3072, 1e-5, False, 5e5, "gate-up-1k"), 615)]
+    whole = [(s, n) for s in (WM128_DEEP, WM64_DEEP, WM_WIDE_DEEP) for n in (256, 768)] + WM_TOO_LITTLE + short
+    taken = [c[:2] for c in WM_CASES if c[:2] not in WM_TOO_LITTLE] + [(s, n) for s in (WM128_DEEP, WM64_DEEP, WM_WIDE_DEEP) for n in (150, 540)]
+    launched = launched_kernels(taken + whole)
+    for (shape, rows), kernels in zip(taken, launched):
+        for epilogue in (1,) if shape in (WM_WIDE, WM_WIDE_DEEP) else (0, 2):            # residual; q/k/v and gate/up
+            assert f"gemm_wm_kernel<{epilogue}>" in kernels, (shape.name, rows, kernels)
+    for (shape, rows), kernels in zip(whole, launched[len(taken):]):
+        assert "gemm_tc2_kernel" in kernels and "gemm_wm_kernel" not in kernels, (shape.name, rows, kernels)
 
 
-# Gate/up with few K blocks is bound by its epilogue, which is the longer one with the weights as M, whatever the chunks save.
-@pytest.mark.parametrize("shape,rows", [(wl.TINY, 2045), (wl.LayerShape(1024, 2, 1, 128, 3072, 1e-5, False, 5e5, "gate-up-1k"), 615)])
-def test_short_contractions_stay_on_whole_tiles(shape, rows):
-    lay = wl.make_layout(1, 3, rows + 30, 8, 8, 8, "none")
-    dc = DeviceCase(wl.make_case(shape, lay, 0.0, cfg_id=82), max_rows=rows)
-    anchors = np.sort(np.random.default_rng(rows).choice(lay.affix_len, rows, replace=False)).astype(np.int32)
-    _, kernels = split_calls_and_kernels(dc, anchors)
-    assert "gemm_tc2_kernel" in kernels and "gemm_wm_kernel" not in kernels, kernels
+@pytest.mark.parametrize("shape,rows,up_first", WM_CASES)
+def test_weights_as_m_projections(shape, rows, up_first):
+    dc, anchors = wm_case(shape, rows, rows, up_first)
+    check_against_oracle(dc, anchors[None], *wm_split_calls(dc, anchors), None, None, rows)
+
+
+# The same rows at the head of a call of whole 256 x 256 tiles have the same bits (as many row pairs, so that cut projections are cut
+# alike).  k_new and v_new as they are; y with inputs that the other rows do not change (as above: no queries, equal values).
+@pytest.mark.parametrize("shape,up_first", [(WM128_DEEP, False), (WM64_DEEP, True), (WM_WIDE_DEEP, False)])
+@pytest.mark.parametrize("rows,more", [(150, 256), (540, 768)])
+def test_weights_as_m_projections_have_the_bits_of_whole_tiles(shape, up_first, rows, more):
+    dc, anchors = wm_case(shape, rows, more, up_first)
+    few, many = wm_split_calls(dc, anchors[:rows]), wm_split_calls(dc, anchors)
+    assert torch.equal(few[0], many[0][:, :rows]) and torch.equal(few[1], many[1][:, :rows])
+    for name in ("wq", "bq", "wv"):
+        dc.w_dev[name].zero_()
+    dc.cv[:] = dc.w_dev["bv"].view(shape.n_kv_heads, shape.head_dim)
+    few, many = wm_split_calls(dc, anchors[:rows]), wm_split_calls(dc, anchors)
+    assert torch.equal(few[1][0], dc.cv[0, :rows])
+    assert torch.equal(few[2], many[2][:, :rows])
