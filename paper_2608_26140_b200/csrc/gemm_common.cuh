@@ -1,4 +1,4 @@
-// Parts shared by the projection kernels (gemm_rows.cu, gemm_tc.cu): the row preparation in front of a contraction
+// Parts shared by the projection kernels (gemm_rows.cu, gemm_tc.cu, gemm_wm.cu): the row preparation in front of a contraction
 // with its grid-wide barrier, and the epilogues on adjacent fp32 accumulator columns of one row.
 #pragma once
 #include "common.cuh"

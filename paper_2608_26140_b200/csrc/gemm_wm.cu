@@ -2,18 +2,21 @@
 //
 // gemm_tc2_kernel (gemm_tc.cu) gives the rows the M side of its instruction: they come in pairs of 128-row tiles, 615 rows cost
 // what 768 do, and a launch is a whole number of rounds of 256 x 256 tiles.  Here a cluster of two CTAs multiplies 256 rows of the
-// weights by a chunk of NC rows of the input, NC any multiple of 16 up to 256, chosen with the number of chunks so that rounds x
-// time of a chunk is least (launch_wm).  Everything else is that kernel's: cta_group::2, one producer and one issuing warp, two
-// accumulators, eight epilogue warps, whole tiles walked in groups of weight tiles; and so are the results, bit for bit.
+// weights by a chunk of NC rows of the input, NC a multiple of 16 from 64 to 256 (in use up to 240: chunks of 256 save nothing), chosen
+// with the number of chunks so that rounds x time of a chunk is least (launch_wm).  Everything else is that kernel's: cta_group::2, one
+// producer and one issuing warp, two accumulators, eight epilogue warps, whole tiles walked in groups of weight tiles; and so are the
+// results, bit for bit.
 //
-// us per launch, gemm_tc2_kernel | this: 615 rows (three chunks of 208) q/k/v 60.6 | 55.0, gate/up 101 | 92, output 26.9 | 25.4;
-// 1015 rows of a 3584-column model (five chunks of 208 for four row pairs) down 113 | 95; 1639 rows gate/up 239 | 230, down 140 | 118.
-// Bound, at these sizes, by the operands' way from L2 and HBM rather than by the instructions (0.285 us per K block of 208 columns
-// against 0.22), then by power.
+// us per launch, gemm_tc2_kernel | this: 615 rows (three chunks of 208) q/k/v 60.6 | 55.0, gate/up 101 | 92, output (four chunks of 160)
+// 26.9 | 25.4; 512 rows (three of 176) q/k/v 59.6 | 56.4, which the kernels behind it pay back; 1015 rows of a 3584-column model (five
+// chunks of 208 for four row pairs) down 113 | 95; 1639 rows gate/up 239 | 230, down 140 | 118.
+// Bound at these sizes by no unit: gate/up of 615 rows has the tensor pipe busy 66 % of the launch, L2 at 41 % and HBM at 33 % of their
+// peaks (1.57 GHz); what is left is the launch's edges and waits for operands in the ring.  From about 1500 rows by power.
 //
 // The accumulator lies the other way round (tensor-memory lane = output column, column = row of the input), so the epilogue turns
-// 32 x 32 pieces round in shared memory and then works on one row per thread like the others.  Which weight rows a warp's 32 lanes are is the tensor map's choice: of a rotary head 16 pairs (i and i + d/2 side by side), of gate/up 16 columns
-// of each (the two matrices are one map whose third dimension steps from one to the other), else 32 adjacent columns.
+// 32 x 32 pieces round in shared memory and then works on one row per thread like the others.  Which weight rows a warp's 32 lanes are
+// is the tensor map's choice: of a rotary head 16 pairs (i and i + d/2 side by side), of gate/up 16 columns of each (the two matrices
+// are one map whose third dimension steps from one to the other), else 32 adjacent columns.
 #include <algorithm>
 
 #include "common.cuh"
