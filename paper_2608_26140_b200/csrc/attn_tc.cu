@@ -17,9 +17,10 @@
 // TMEM) when the true maximum has grown by more than 2^8, which keeps P within bf16 range and
 // makes rescales rare.  Every mbarrier wait is bounded (status flag kFlagWaitExpired on expiry).
 // With two key sources (a cache shared by the batch + each request's private rows, Section 4.1) the
-// private rows' tiles follow the cache's, and key masks tell which of the two serves a position; when
-// every request brings at most 32 rows (decode passes), four requests share one tile, one per 32-row
-// quarter, so that the shared cache's tiles are read once per four requests.
+// private rows' tiles follow the cache's, and key masks tell which of the two serves a position.  When
+// every request brings at most 64 rows (decode passes), two or four requests share one query tile
+// (attention_group_kernel, below the one-tile kernel).
+#include <climits>
 #include <type_traits>
 #include <cuda.h>
 
@@ -98,6 +99,25 @@ __device__ __forceinline__ void tc_mma_ta(uint32_t d_tmem, uint32_t a_tmem, uint
         ::"r"(d_tmem), "r"(a_tmem), "l"(bdesc), "r"(idesc), "r"(acc)
         : "memory");
 }
+// The two products with D written only in the 32-lane quarters of `lanes` (bit q = quarter q).
+__device__ __forceinline__ void tc_mma_lanes(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t acc, uint32_t lanes) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "setp.ne.b32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, {%5, %6, %7, %8}, p;\n\t}"
+        ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(acc), "r"((lanes & 1u) - 1u), "r"(((lanes >> 1) & 1u) - 1u),
+          "r"(((lanes >> 2) & 1u) - 1u), "r"(((lanes >> 3) & 1u) - 1u)
+        : "memory");
+}
+__device__ __forceinline__ void tc_mma_ta_lanes(uint32_t d_tmem, uint32_t a_tmem, uint64_t bdesc, uint32_t idesc, uint32_t acc, uint32_t lanes) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "setp.ne.b32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, {%5, %6, %7, %8}, p;\n\t}"
+        ::"r"(d_tmem), "r"(a_tmem), "l"(bdesc), "r"(idesc), "r"(acc), "r"((lanes & 1u) - 1u), "r"(((lanes >> 1) & 1u) - 1u),
+          "r"(((lanes >> 2) & 1u) - 1u), "r"(((lanes >> 3) & 1u) - 1u)
+        : "memory");
+}
 __device__ __forceinline__ void tc_st16(uint32_t taddr, const uint32_t (&v)[16]) {
     asm volatile(
         "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], "
@@ -131,12 +151,9 @@ struct AttnTcArgs {
     // still name cache positions that do not exist as keys (the DropNA layout of Section 5.3).
     int n_fresh_tiles, excl_words, keep_words, cache_shared;
     int kv_prefetch;          // two-query-tile kernel: K/V tiles requested into L2 ahead of the rings
-    // one-tile kernel over a shared cache with at most 32 rows per request (decode passes): group = 4 puts the rows
-    // of four requests into the four 32-row quarters of one tile, so that the shared cache's key tiles are read
-    // once per four requests; each request's fresh tiles follow, visible to its own quarter only.  Else 1.
-    int group, batch;
-    int split;                // one-tile kernel: CTAs (a cluster) per query tile, each over a part of the key tiles
-    int n_items;              // one-tile kernel: query tiles over all heads and requests (or groups)
+    int group, batch;         // attention_group_kernel: requests per query tile, requests in all
+    int split;                // one-tile kernels: CTAs (a cluster) per query tile, each over a part of the key tiles
+    int n_items;              // one-tile kernels: query tiles over all heads and requests (or groups)
     const uint32_t* pos_excl;
     const uint32_t* row_keep;
     // Eq. 4-5 taken from this attention's own logits (two-query-tile kernel; the one-shot probe of Section 3.2): for the
@@ -161,6 +178,196 @@ __device__ __forceinline__ bool mbar_spin(uint32_t bar, uint32_t parity, volatil
     }
     *abort_flag = 1;
     return false;
+}
+
+// A key tile of one query row's quarter (32 keys per thread): S from tensor memory at tS, P written back over its low columns, O
+// at tO rescaled when the reference moves.  Four threads share a row; their warps (one lane quarter, one scheduler) meet at a vote
+// every tile and only ever leave the loop together: a thread whose wait ran out (ok = false) skips its work and votes for the
+// exchange, where all four learn of it and this returns false.  row_max: this row's entry of the first of four arrays, `stride` apart.
+// The softmax is on the chain of every tile; with the maxima of all tiles exchanged through shared memory and one fp32 operation
+// per element at a time it took 2000 cycles of a tile's 2600-3100 (maximum 280, 500 with masked keys; exchange 350; exponentials
+// 1200-1300).  With the vote, masks applied once and packed fp32 arithmetic: attention of 1639 rows over 8288 keys 260 -> 235 us.
+template <class WaitS, class WaitPrevious>
+__device__ __forceinline__ bool softmax_tile(uint32_t keep, bool first, float scale_log2e, uint32_t tS, uint32_t tO, int c4, int vote,
+                                             uint16_t* row_max, int stride, uint32_t p_full, float& m_use, float& l, bool& ok,
+                                             WaitS wait_s, WaitPrevious wait_previous) {
+    float sv[32];
+    float mt = -INFINITY;
+    if (ok && (ok = wait_s())) {
+        tc_fence_after();
+        // this thread's quarter row of S into registers, masked keys as -inf
+        tc_ld32(tS + c4 * 32, sv);
+        if (keep != 0xffffffffu) {
+#pragma unroll
+            for (int i = 0; i < 32; ++i) sv[i] = ((keep >> i) & 1u) ? sv[i] : -INFINITY;
+        }
+        float m4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+#pragma unroll
+        for (int i = 0; i < 32; i += 2) m4[(i >> 1) & 3] = fmaxf(fmaxf(m4[(i >> 1) & 3], sv[i]), sv[i + 1]);
+        mt = fmaxf(fmaxf(m4[0], m4[1]), fmaxf(m4[2], m4[3])) * scale_log2e;
+    }
+    // The four threads of a row must use the same reference.  It moves on the first tile and seldom after; whether it
+    // has to is one vote of the four warps that share these 32 rows, at the barrier that they need anyway (every
+    // thread of a row must have read its S columns before P overwrites them).  A thread whose wait ran out votes too.
+    bool raise = false;
+    if (quarter_any(vote, !ok || mt - m_use > kRescaleGap)) {
+        // all take the largest of the four quarter-row maxima rounded up to 16 significant bits (an upper bound is
+        // all the exponent needs)
+        uint32_t mb = __float_as_uint(mt);
+        if ((mb & 0xFFFFu) && !(mb >> 31)) mb += 0x10000u;
+        mb >>= 16;
+        row_max[c4 * stride] = (uint16_t)mb;
+        if (quarter_any(vote, !ok)) { ok = false; return false; }      // the four warps leave together
+        mt = fmaxf(fmaxf(__uint_as_float((uint32_t)row_max[0] << 16), __uint_as_float((uint32_t)row_max[stride] << 16)),
+                   fmaxf(__uint_as_float((uint32_t)row_max[2 * stride] << 16), __uint_as_float((uint32_t)row_max[3 * stride] << 16)));
+        if (first) m_use = mt;
+        else raise = mt - m_use > kRescaleGap;
+    }
+    if (__any_sync(0xffffffffu, raise)) {
+        // O may only be touched once the P V of the tile before has completed
+        if ((ok = wait_previous())) {
+            tc_fence_after();
+            const float f = raise ? fast_exp2(m_use - mt) : 1.f;
+            float v[32];
+            tc_ld32(tO + c4 * 32, v);
+#pragma unroll
+            for (int i = 0; i < 32; ++i) v[i] *= f;
+            tc_st32(tO + c4 * 32, v);
+            tc_wait_st();
+            l *= f;
+            if (raise) m_use = mt;
+        }
+    }
+    if (!ok) return true;
+    // P overwrites the S buffer in tensor memory: 32 keys = 16 columns of two bf16 at column 16 c4
+    // (every thread of the row has read its S columns: they all passed the vote above)
+    const float neg = m_use > -INFINITY ? -m_use : 0.f;      // no key of the row has counted yet: all P are 0
+    const float2 scale2 = make_float2(scale_log2e, scale_log2e), neg2 = make_float2(neg, neg);
+    float2 l2a = make_float2(0.f, 0.f), l2b = l2a;
+    uint32_t pk[16];
+    auto exps = [&](auto all_kept) {
+#pragma unroll
+        for (int i = 0; i < 32; i += 4) {
+            const float2 xa = __ffma2_rn(make_float2(sv[i], sv[i + 1]), scale2, neg2);
+            const float2 xb = __ffma2_rn(make_float2(sv[i + 2], sv[i + 3]), scale2, neg2);
+            const float2 pa = make_float2(fast_exp2(xa.x), fast_exp2(xa.y));
+            const float2 pb = make_float2(fast_exp2(xb.x), all_kept.value ? poly_exp2(xb.y) : fast_exp2(xb.y));
+            l2a = __fadd2_rn(l2a, pa);
+            l2b = __fadd2_rn(l2b, pb);
+            pk[i >> 1] = pack_bf16(pa.x, pa.y);
+            pk[(i >> 1) + 1] = pack_bf16(pb.x, pb.y);
+        }
+    };
+    if (keep == 0xffffffffu) exps(std::true_type{});
+    else exps(std::false_type{});
+    tc_st16(tS + c4 * 16, pk);
+    tc_wait_st();
+    l += (l2a.x + l2a.y) + (l2b.x + l2b.y);
+    tc_fence_before();
+    __syncwarp();
+    if ((threadIdx.x & 31) == 0) mbar_arrive(p_full);
+    return true;
+}
+// 32 columns of a finished row: O / l as bf16, 16 bytes a store.
+__device__ __forceinline__ void store_o32(__nv_bfloat16* out, const float (&v)[32], float inv) {
+#pragma unroll
+    for (int k8 = 0; k8 < 4; ++k8) {
+        const float* pv = v + k8 * 8;
+        *reinterpret_cast<uint4*>(out + k8 * 8) =
+            make_uint4(pack_bf16(pv[0] * inv, pv[1] * inv), pack_bf16(pv[2] * inv, pv[3] * inv),
+                       pack_bf16(pv[4] * inv, pv[5] * inv), pack_bf16(pv[6] * inv, pv[7] * inv));
+    }
+}
+
+// The cache's key tiles that hold a key for any of the requests [b0, b0 + n_req): tiles [x, y).  Private rows serve whatever
+// lies outside the affix, so the tiles in front of it and behind it often hold none (a context of 2560 positions with 2048 affix
+// rows: 4 of 20).  Where a cluster shares the key tiles they are all visited: most CTAs of it would gain nothing, and the look at the
+// masks takes 1.5 us.  Called by all threads; lo_hi in shared memory holds (INT_MAX, 0) before the block's last barrier.
+__device__ __forceinline__ int2 kept_tiles(const AttnTcArgs& a, int b0, int n_req, int* lo_hi) {
+    const int n = (a.ctx_len + 127) / 128;
+    if (!a.pos_excl) return make_int2(0, n);
+    int first = INT_MAX, end = 0;                  // a word (32 positions of one request) per thread and round
+    for (int i = threadIdx.x; i < n * 4 * n_req; i += blockDim.x) {
+        const int r = i / (n * 4), w = i - r * n * 4, valid = a.ctx_len - w * 32;
+        uint32_t in = valid >= 32 ? ~0u : (valid <= 0 ? 0u : (1u << valid) - 1u);
+        if (w < a.excl_words) in &= ~__ldg(a.pos_excl + (int64_t)(b0 + r) * a.excl_words + w);
+        if (in) {
+            first = min(first, w >> 2);
+            end = max(end, (w >> 2) + 1);
+        }
+    }
+    first = __reduce_min_sync(0xffffffffu, first);
+    end = __reduce_max_sync(0xffffffffu, end);
+    if ((threadIdx.x & 31) == 0 && end > 0) {
+        atomicMin(lo_hi, first);
+        atomicMax(lo_hi + 1, end);
+    }
+    __syncthreads();
+    const int lo = lo_hi[0], hi = lo_hi[1];
+    return lo < hi ? make_int2(lo, hi) : make_int2(0, 0);
+}
+// Merge of a cluster's parts through distributed shared memory: (reference, denominator) of every row meet first; each CTA scales
+// its O to the common reference and lays it out by the CTA that finishes the columns (128 / C each), which sums the parts in rank
+// order.  The K and V stages are idle by now.  All threads pass the three cluster barriers, whatever happened before.  out: the
+// row's 128 columns, null for a row that does not exist; any: this CTA had key tiles (else its O holds nothing).
+__device__ __forceinline__ void merge_parts(uint32_t base, unsigned char* base_ptr, int C, int rank, bool softmax, bool any, int c4,
+                                            int row, uint32_t tO, float m_use, float l, __nv_bfloat16* out) {
+    float2* ml = reinterpret_cast<float2*>(base_ptr + AT_TILE + 4096);             // [128]
+    const uint32_t parts = base + 2 * AT_TILE;                                     // [owner][column / 4][row][4] fp32
+    const int width = 128 / C;
+    __syncwarp();
+    if (softmax && c4 == 0) ml[row] = make_float2(m_use, l);
+    __syncwarp();
+    cluster_sync_all();
+    float denom = 0.f;
+    if (softmax) {
+        const uint32_t ml_row = smem_u32(ml + row);
+        float ref = -INFINITY, m_c[8], l_c[8];
+#pragma unroll
+        for (int c = 0; c < 8; ++c)
+            if (c < C) {
+                asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(m_c[c]), "=f"(l_c[c]) : "r"(mapa_u32(ml_row, c)) : "memory");
+                ref = fmaxf(ref, m_c[c]);
+            }
+#pragma unroll
+        for (int c = 0; c < 8; ++c)
+            if (c < C && m_c[c] > -INFINITY) denom += l_c[c] * fast_exp2(m_c[c] - ref);
+        const float f = m_use > -INFINITY ? fast_exp2(m_use - ref) : 0.f;
+        tc_fence_after();
+        float v[32];
+        tc_ld32(tO + c4 * 32, v);
+        const uint32_t dst = parts + ((c4 * 8 * 128 + row) << 4);                  // owners' columns lie one after the other
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const float4 p = any ? make_float4(v[4 * i] * f, v[4 * i + 1] * f, v[4 * i + 2] * f, v[4 * i + 3] * f) : make_float4(0.f, 0.f, 0.f, 0.f);
+            asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(dst + i * 2048), "f"(p.x), "f"(p.y), "f"(p.z), "f"(p.w) : "memory");
+        }
+    }
+    __syncwarp();
+    cluster_sync_all();
+    if (softmax) {
+        const float inv = 1.f / denom;
+        const int col = rank * width + c4 * (width >> 2);                          // width / 4 columns per thread
+#pragma unroll 1
+        for (int g4 = 0; g4 < width >> 4; ++g4) {
+            const uint32_t src = parts + (((col >> 2) + g4) * 128 + row) * 16;
+            float4 u[8];
+#pragma unroll
+            for (int c = 0; c < 8; ++c)
+                if (c < C)
+                    asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
+                                 : "=f"(u[c].x), "=f"(u[c].y), "=f"(u[c].z), "=f"(u[c].w) : "r"(mapa_u32(src, c)) : "memory");
+            float4 o = u[0];
+#pragma unroll
+            for (int c = 1; c < 8; ++c)
+                if (c < C) { o.x += u[c].x; o.y += u[c].y; o.z += u[c].z; o.w += u[c].w; }
+            if (g4 + 1 == width >> 4) cluster_arrive();      // the last read: before the stores, which it would wait for
+            if (out) *reinterpret_cast<uint2*>(out + col + g4 * 4) = make_uint2(pack_bf16(o.x * inv, o.y * inv), pack_bf16(o.z * inv, o.w * inv));
+        }
+    }
+    __syncwarp();
+    if (!softmax) cluster_arrive();
+    cluster_wait();
 }
 
 // MANY: many more items than SMs.  A CTA then takes every gridDim.x-th one and keeps its tensor memory and barriers; the loads and
@@ -188,14 +395,16 @@ attention_tc_kernel(const AttnTcArgs a, const __grid_constant__ CUtensorMap mapQ
     volatile int* abort_flag = reinterpret_cast<volatile int*>(base_ptr + 5 * AT_TILE + 200);
     // barriers: 0 q_full | 1,2 k_full | 3,4 k_empty | 5,6 v_full | 7,8 v_empty | 9,10 s_full | 11,12 unused |
     //           13,14 p_full | 15,16 pv_done (P V of the tile completed: O holds it, its S/P buffer is free)
+    int* kept = reinterpret_cast<int*>(base_ptr + 5 * AT_TILE + 208);
     auto bar = [&](int i) { return bars + 8 * i; };
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     // key split: a cluster of C CTAs shares a query tile, each taking a contiguous part of the key tiles
     const int C = a.split, rank = C > 1 ? (int)cluster_ctarank() : 0;
     const int first = blockIdx.x / C, stride = gridDim.x;        // items: (query tile, head, request or group of four)
     const int n_cache_tiles = (a.ctx_len + 127) / 128;
-    const int G = a.group;                          // requests per tile (4: b counts groups of four)
-    int qt, h, b, kvh, kb, b0, n_req, live_q, j0, n_tiles;
+    int2 visited = make_int2(0, n_cache_tiles);     // the cache's key tiles that hold keys
+    // this CTA's key tiles: n_c of the cache from c0 on, then fresh ones from f0 on
+    int qt, h, b, kvh, kb, live_q, c0, n_c, f0, n_tiles;
     auto set_item = [&](int item) {
         const int t = item / a.q_tiles;
         qt = item - t * a.q_tiles;
@@ -203,14 +412,15 @@ attention_tc_kernel(const AttnTcArgs a, const __grid_constant__ CUtensorMap mapQ
         h = t - b * a.n_heads;
         kvh = h / (a.n_heads / a.n_kv_heads);
         kb = a.cache_shared ? 0 : b;                // one cache for the whole batch, or one per request
-        b0 = b * G;                                 // first request of the tile
-        n_req = min(G, a.batch - b0);
-        const int all_tiles = n_cache_tiles + a.n_fresh_tiles * n_req;
-        j0 = rank * all_tiles / C;                  // this CTA's first key tile, and how many
-        n_tiles = (rank + 1) * all_tiles / C - j0;
+        const int all_tiles = n_cache_tiles + a.n_fresh_tiles;
+        const int j0 = rank * all_tiles / C, j1 = (rank + 1) * all_tiles / C;
+        c0 = max(j0, visited.x);
+        n_c = max(min(j1, visited.y) - c0, 0);
+        f0 = max(j0 - n_cache_tiles, 0);
+        n_tiles = n_c + max(j1 - n_cache_tiles, 0) - f0;
         // 32-row quarters of the tile that hold rows: the softmax warps of the others have nothing to do (their
         // rows of S, P and O are never read), which matters when a decode pass brings 32 rows per request
-        live_q = G > 1 ? n_req : min(4, (a.n - qt * 128 + 31) / 32);
+        live_q = min(4, (a.n - qt * 128 + 31) / 32);
     };
     set_item(first);
     const int p_warps = MANY ? 16 : 4 * live_q;     // softmax warps that report a tile's P
@@ -220,6 +430,7 @@ attention_tc_kernel(const AttnTcArgs a, const __grid_constant__ CUtensorMap mapQ
         mbar_init(bar(13), p_warps); mbar_init(bar(14), p_warps);          // p_full
         mbar_init(bar(15), 1); mbar_init(bar(16), 1);      // pv_done
         *abort_flag = 0;
+        kept[0] = INT_MAX; kept[1] = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 1) {
@@ -234,6 +445,10 @@ attention_tc_kernel(const AttnTcArgs a, const __grid_constant__ CUtensorMap mapQ
     const uint32_t tS0 = tmem_base, tO = tmem_base + 256;
     pdl_wait();
     pdl_launch_dependents();
+    if (!MANY && C == 1 && a.pos_excl) {
+        visited = kept_tiles(a, b, 1, kept);
+        set_item(first);
+    }
 
     const bool softmax = warp >= 2 && warp < 18 && (MANY || (warp & 3) < live_q);
     int J = 0;                                      // key tiles of the items before: ring stages and phases go on
@@ -246,27 +461,17 @@ attention_tc_kernel(const AttnTcArgs a, const __grid_constant__ CUtensorMap mapQ
             if (MANY) set_item(item);
             // the last S of the item before has read Q
             if (J > 0 && !(ok = mbar_wait(bar(3 + ((J - 1) & 1)), ((J - 1) >> 1) & 1, abort_flag))) break;
-            if (G > 1) {
-                // 32-row boxes: request b0 + r fills rows [32 r, 32 r + 32) of both panels (rows past its n read as zero)
-                mbar_expect_tx(bar(0), n_req * 8192);
-                for (int r = 0; r < n_req; ++r) {
-                    tma_load_3d(sQ + r * 4096, &mapQ, h * 128, 0, b0 + r, bar(0), pol_q);
-                    tma_load_3d(sQ + AT_PANEL + r * 4096, &mapQ, h * 128 + 64, 0, b0 + r, bar(0), pol_q);
-                }
-            } else {
-                mbar_expect_tx(bar(0), AT_TILE);
-                tma_load_3d(sQ, &mapQ, h * 128, qt * 128, b, bar(0), pol_q);
-                tma_load_3d(sQ + AT_PANEL, &mapQ, h * 128 + 64, qt * 128, b, bar(0), pol_q);
-            }
+            mbar_expect_tx(bar(0), AT_TILE);
+            tma_load_3d(sQ, &mapQ, h * 128, qt * 128, b, bar(0), pol_q);
+            tma_load_3d(sQ + AT_PANEL, &mapQ, h * 128 + 64, qt * 128, b, bar(0), pol_q);
             for (int j = 0; j < n_tiles && ok; ++j) {
                 const int s = (J + j) & 1;
                 const uint32_t par = (((J + j) >> 1) & 1) ^ 1;
                 if (!(ok = mbar_wait(bar(3 + s), par, abort_flag))) break;
-                const bool fresh = j0 + j >= n_cache_tiles;
+                const bool fresh = j >= n_c;
                 const CUtensorMap* mk = fresh ? &mapKn : &mapK;
                 const CUtensorMap* mv = fresh ? &mapVn : &mapV;
-                const int f = j0 + j - n_cache_tiles;                     // fresh tiles: request by request
-                const int r0 = (fresh ? f % a.n_fresh_tiles : j0 + j) * 128, bz = fresh ? b0 + f / a.n_fresh_tiles : kb;
+                const int r0 = (fresh ? f0 + j - n_c : c0 + j) * 128, bz = fresh ? b : kb;
                 mbar_expect_tx(bar(1 + s), AT_TILE);
                 tma_load_3d(sK0 + s * AT_TILE, mk, kvh * 128, r0, bz, bar(1 + s), pol_kv);
                 tma_load_3d(sK0 + s * AT_TILE + AT_PANEL, mk, kvh * 128 + 64, r0, bz, bar(1 + s), pol_kv);
@@ -344,13 +549,7 @@ attention_tc_kernel(const AttnTcArgs a, const __grid_constant__ CUtensorMap mapQ
         // Warp 2 + 4 c + q' (q = warp & 3 is its TMEM lane quarter) takes keys [32 c, 32 c + 32) of every
         // tile for the 32 rows of quarter q, and columns [32 c, 32 c + 32) of O.  Sixteen warps (four per
         // scheduler) keep the exponential, conversion and TMEM-load latencies of one warp hidden behind
-        // the others.  The four warps of a row quarter, which share a scheduler, meet at a vote every tile and only ever
-        // leave the loop together: a thread whose wait ran out skips its work and votes for the exchange, where all four
-        // learn of it.  The softmax is on the chain of every tile; with the maxima of all tiles exchanged through shared
-        // memory and one fp32 operation per element at a time it took 2000 cycles of a tile's 2600-3100 (maximum 280, 500
-        // with masked keys; exchange 350; exponentials 1200-1300).  With the vote, masks applied once and packed fp32
-        // arithmetic: attention of 1639 rows over 8288 keys 260 -> 235 us, decode layer of 512 rows over shared storage
-        // 88 -> 83 us (layer-step 1015 -> 995, pass over 4 layers 1913 -> 1877).
+        // the others.
         const int c4 = (warp - 2) >> 2;
         const int q = warp & 3;
         const int row = q * 32 + lane;
@@ -359,7 +558,6 @@ attention_tc_kernel(const AttnTcArgs a, const __grid_constant__ CUtensorMap mapQ
         bool ok = true;
         for (int item = first; item < a.n_items; item += stride, J += n_tiles) {
             if (MANY) set_item(item);
-            const int bq = G > 1 ? b0 + q : b;          // the request whose rows this quarter holds
             if (MANY && q >= live_q) {                  // no rows in this quarter: report its P as written
                 for (int j = 0; j < n_tiles && ok; ++j) {
                     ok = __all_sync(0xffffffffu, mbar_wait(bar(9 + ((J + j) & 1)), ((J + j) >> 1) & 1, abort_flag));
@@ -371,111 +569,23 @@ attention_tc_kernel(const AttnTcArgs a, const __grid_constant__ CUtensorMap mapQ
             m_use = -INFINITY;
             l = 0.f;
             for (int j = 0; j < n_tiles; ++j) {
-                const int s = (J + j) & 1, jk = j0 + j;   // ring stage, key tile
+                const int s = (J + j) & 1;                // ring stage
                 const uint32_t par = ((J + j) >> 1) & 1;
                 // which of this thread's 32 keys count: the cache's positions up to the context end, minus those a
                 // fresh row serves; of the fresh rows, those that serve their position
                 uint32_t keep;
-                if (jk < n_cache_tiles) {
-                    const int valid = a.ctx_len - jk * 128 - c4 * 32;
+                if (j < n_c) {
+                    const int w = (c0 + j) * 4 + c4, valid = a.ctx_len - w * 32;
                     keep = valid >= 32 ? 0xffffffffu : (valid <= 0 ? 0u : (1u << valid) - 1u);
-                    if (a.pos_excl && jk * 4 + c4 < a.excl_words) keep &= ~__ldg(a.pos_excl + (int64_t)bq * a.excl_words + jk * 4 + c4);
+                    if (a.pos_excl && w < a.excl_words) keep &= ~__ldg(a.pos_excl + (int64_t)b * a.excl_words + w);
                 } else {
-                    const int f = jk - n_cache_tiles;
-                    if (G > 1 && f / a.n_fresh_tiles != q) {
-                        // another request's fresh rows: none of them is a key of this quarter's rows.  All four warps
-                        // of the quarter come here, so none of them goes to the quarter's barrier for this tile.
-                        if (ok && (ok = mbar_wait(bar(9 + s), par, abort_flag))) {
-                            tc_fence_after();
-                            uint32_t pz[16];
-#pragma unroll
-                            for (int i = 0; i < 16; ++i) pz[i] = 0u;
-                            tc_st16(tS0 + s * 128 + c4 * 16 + lane_off, pz);
-                            tc_wait_st();
-                            tc_fence_before();
-                            __syncwarp();
-                            if (lane == 0) mbar_arrive(bar(13 + s));
-                        }
-                        continue;
-                    }
-                    const int w = (f % a.n_fresh_tiles) * 4 + c4;
-                    keep = w < a.keep_words ? __ldg(a.row_keep + (int64_t)bq * a.keep_words + w) : 0u;
+                    const int w = (f0 + j - n_c) * 4 + c4;
+                    keep = w < a.keep_words ? __ldg(a.row_keep + (int64_t)b * a.keep_words + w) : 0u;
                 }
-                float sv[32];
-                float mt = -INFINITY;
-                if (ok && (ok = mbar_wait(bar(9 + s), par, abort_flag))) {
-                    tc_fence_after();
-                    // this thread's quarter row of S into registers, masked keys as -inf
-                    tc_ld32(tS0 + s * 128 + col_off + lane_off, sv);
-                    if (keep != 0xffffffffu) {
-#pragma unroll
-                        for (int i = 0; i < 32; ++i) sv[i] = ((keep >> i) & 1u) ? sv[i] : -INFINITY;
-                    }
-                    float m4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
-#pragma unroll
-                    for (int i = 0; i < 32; i += 2) m4[(i >> 1) & 3] = fmaxf(fmaxf(m4[(i >> 1) & 3], sv[i]), sv[i + 1]);
-                    mt = fmaxf(fmaxf(m4[0], m4[1]), fmaxf(m4[2], m4[3])) * a.scale_log2e;
-                }
-                // The four threads of a row must use the same reference.  It moves on the first tile and seldom after; whether it
-                // has to is one vote of the four warps that share these 32 rows, at the barrier that they need anyway (every
-                // thread of a row must have read its S columns before P overwrites them).  A thread whose wait ran out votes too.
-                bool raise = false;
-                if (quarter_any(1 + q, !ok || mt - m_use > kRescaleGap)) {
-                    // all take the largest of the four quarter-row maxima rounded up to 16 significant bits (an upper bound is
-                    // all the exponent needs)
-                    uint32_t mb = __float_as_uint(mt);
-                    if ((mb & 0xFFFFu) && !(mb >> 31)) mb += 0x10000u;
-                    mb >>= 16;
-                    row_max[c4][row] = (uint16_t)mb;
-                    if (quarter_any(1 + q, !ok)) { ok = false; break; }      // the four warps leave together
-                    mt = fmaxf(fmaxf(__uint_as_float((uint32_t)row_max[0][row] << 16), __uint_as_float((uint32_t)row_max[1][row] << 16)),
-                               fmaxf(__uint_as_float((uint32_t)row_max[2][row] << 16), __uint_as_float((uint32_t)row_max[3][row] << 16)));
-                    if (j == 0) m_use = mt;
-                    else raise = mt - m_use > kRescaleGap;
-                }
-                if (__any_sync(0xffffffffu, raise)) {
-                    // O may only be touched once the P V of tile j - 1 has completed
-                    if ((ok = mbar_wait(bar(15 + (s ^ 1)), ((J + j - 1) >> 1) & 1, abort_flag))) {
-                        tc_fence_after();
-                        const float f = raise ? fast_exp2(m_use - mt) : 1.f;
-                        float v[32];
-                        tc_ld32(tO + lane_off + col_off, v);
-#pragma unroll
-                        for (int i = 0; i < 32; ++i) v[i] *= f;
-                        tc_st32(tO + lane_off + col_off, v);
-                        tc_wait_st();
-                        l *= f;
-                        if (raise) m_use = mt;
-                    }
-                }
-                if (!ok) continue;
-                // P overwrites the S buffer in tensor memory: 32 keys = 16 columns of two bf16 at column 16 c4
-                // (every thread of the row has read its S columns: they all passed the vote above)
-                const float neg = m_use > -INFINITY ? -m_use : 0.f;      // no key of the row has counted yet: all P are 0
-                const float2 scale2 = make_float2(a.scale_log2e, a.scale_log2e), neg2 = make_float2(neg, neg);
-                float2 l2a = make_float2(0.f, 0.f), l2b = l2a;
-                uint32_t pk[16];
-                auto exps = [&](auto all_kept) {
-#pragma unroll
-                    for (int i = 0; i < 32; i += 4) {
-                        const float2 xa = __ffma2_rn(make_float2(sv[i], sv[i + 1]), scale2, neg2);
-                        const float2 xb = __ffma2_rn(make_float2(sv[i + 2], sv[i + 3]), scale2, neg2);
-                        const float2 pa = make_float2(fast_exp2(xa.x), fast_exp2(xa.y));
-                        const float2 pb = make_float2(fast_exp2(xb.x), all_kept.value ? poly_exp2(xb.y) : fast_exp2(xb.y));
-                        l2a = __fadd2_rn(l2a, pa);
-                        l2b = __fadd2_rn(l2b, pb);
-                        pk[i >> 1] = pack_bf16(pa.x, pa.y);
-                        pk[(i >> 1) + 1] = pack_bf16(pb.x, pb.y);
-                    }
-                };
-                if (keep == 0xffffffffu) exps(std::true_type{});
-                else exps(std::false_type{});
-                tc_st16(tS0 + s * 128 + c4 * 16 + lane_off, pk);
-                tc_wait_st();
-                l += (l2a.x + l2a.y) + (l2b.x + l2b.y);
-                tc_fence_before();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(bar(13 + s));   // p_full
+                if (!softmax_tile(keep, j == 0, a.scale_log2e, tS0 + s * 128 + lane_off, tO + lane_off, c4, 1 + q, &row_max[0][row], 128,
+                                  bar(13 + s), m_use, l, ok, [&] { return mbar_wait(bar(9 + s), par, abort_flag); },
+                                  [&] { return mbar_wait(bar(15 + (s ^ 1)), ((J + j - 1) >> 1) & 1, abort_flag); }))
+                    break;
             }
             // epilogue: O / l once the last P V has completed; the denominators of the four quarters add up
             if (ok && n_tiles > 0) ok = mbar_wait(bar(15 + ((J + n_tiles - 1) & 1)), ((J + n_tiles - 1) >> 1) & 1, abort_flag);
@@ -484,88 +594,274 @@ attention_tc_kernel(const AttnTcArgs a, const __grid_constant__ CUtensorMap mapQ
             l = (row_sum[0][row] + row_sum[1][row]) + (row_sum[2][row] + row_sum[3][row]);
             if (C == 1) {
                 tc_fence_after();
-                const int grow = G > 1 ? lane : qt * 128 + row;     // the row inside its request
-                const float inv = 1.f / l;
-                __nv_bfloat16* out = static_cast<__nv_bfloat16*>(a.o) + (((int64_t)bq * a.n + grow) * a.n_heads + h) * 128 + col_off;
+                const int grow = qt * 128 + row;
                 float v[32];
                 tc_ld32(tO + lane_off + col_off, v);
-                if (grow < a.n) {
-#pragma unroll
-                    for (int k8 = 0; k8 < 4; ++k8) {
-                        const float* pv = v + k8 * 8;
-                        *reinterpret_cast<uint4*>(out + k8 * 8) =
-                            make_uint4(pack_bf16(pv[0] * inv, pv[1] * inv), pack_bf16(pv[2] * inv, pv[3] * inv),
-                                       pack_bf16(pv[4] * inv, pv[5] * inv), pack_bf16(pv[6] * inv, pv[7] * inv));
-                    }
-                }
+                if (grow < a.n)
+                    store_o32(static_cast<__nv_bfloat16*>(a.o) + (((int64_t)b * a.n + grow) * a.n_heads + h) * 128 + col_off, v, 1.f / l);
             }
             if (!MANY) break;
         }
     }
     if (C > 1) {
-        // ---------------- merge of the cluster's parts through distributed shared memory ----------------
-        // (reference, denominator) of every row meet first; each CTA scales its O to the common reference and lays it out by
-        // the CTA that finishes the columns (128 / C each), which sums the parts in rank order.  The K and V stages are idle
-        // by now.  All threads pass the three cluster barriers, whatever happened before.
-        float2* ml = reinterpret_cast<float2*>(base_ptr + AT_TILE + 4096);             // [128]
-        const uint32_t parts = base + 2 * AT_TILE;                                     // [owner][column / 4][row][4] fp32
-        const int q = warp & 3, c4 = (warp - 2) >> 2, row = q * 32 + lane, width = 128 / C;
-        __syncwarp();
-        if (softmax && c4 == 0) ml[row] = make_float2(m_use, l);
-        __syncwarp();
-        cluster_sync_all();
-        float denom = 0.f;
-        if (softmax) {
-            const uint32_t ml_row = smem_u32(ml + row);
-            float ref = -INFINITY, m_c[8], l_c[8];
-#pragma unroll
-            for (int c = 0; c < 8; ++c)
-                if (c < C) {
-                    asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(m_c[c]), "=f"(l_c[c]) : "r"(mapa_u32(ml_row, c)) : "memory");
-                    ref = fmaxf(ref, m_c[c]);
-                }
-#pragma unroll
-            for (int c = 0; c < 8; ++c)
-                if (c < C && m_c[c] > -INFINITY) denom += l_c[c] * fast_exp2(m_c[c] - ref);
-            const float f = m_use > -INFINITY ? fast_exp2(m_use - ref) : 0.f;
-            tc_fence_after();
-            float v[32];
-            tc_ld32(tO + ((uint32_t)(q * 32) << 16) + c4 * 32, v);
-            const uint32_t dst = parts + ((c4 * 8 * 128 + row) << 4);                  // owners' columns lie one after the other
-#pragma unroll
-            for (int i = 0; i < 8; ++i)
-                asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};"
-                             ::"r"(dst + i * 2048), "f"(v[4 * i] * f), "f"(v[4 * i + 1] * f), "f"(v[4 * i + 2] * f), "f"(v[4 * i + 3] * f)
-                             : "memory");
+        const int c4 = (warp - 2) >> 2, row = (warp & 3) * 32 + lane, grow = qt * 128 + row;
+        merge_parts(base, base_ptr, C, rank, softmax, n_tiles > 0, c4, row, tO + ((uint32_t)(warp & 3) << 21), m_use, l,
+                    grow < a.n ? static_cast<__nv_bfloat16*>(a.o) + (((int64_t)b * a.n + grow) * a.n_heads + h) * 128 : nullptr);
+    }
+    // ---------------- teardown ----------------
+    tc_fence_before();
+    __syncthreads();
+    if (*abort_flag) {
+        if (threadIdx.x == 0) {
+            atomicOr(a.status, kFlagWaitExpired);
+            for (int i = 0; i < 4096; ++i) __nanosleep(64);   // let copies already in flight land
         }
-        __syncwarp();
-        cluster_sync_all();
-        if (softmax) {
-            const int bq = G > 1 ? b0 + q : b, grow = G > 1 ? lane : qt * 128 + row;
-            const float inv = 1.f / denom;
-            const int col = rank * width + c4 * (width >> 2);                          // width / 4 columns per thread
-            __nv_bfloat16* out = static_cast<__nv_bfloat16*>(a.o) + (((int64_t)bq * a.n + grow) * a.n_heads + h) * 128 + col;
-#pragma unroll 1
-            for (int g4 = 0; g4 < width >> 4; ++g4) {
-                const uint32_t src = parts + (((col >> 2) + g4) * 128 + row) * 16;
-                float4 u[8];
+        __syncthreads();
+    }
+    if (warp == 1) {
+        tc_fence_after();
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem_base) : "memory");
+    }
+}
+
+// ---- few rows per request over a shared cache ----------------------------------------------------
+// Decode passes: the rows of `group` requests (four of at most 32 rows, or two of at most 64) share one 128-row query tile of one
+// head, so that the shared cache's key tiles are read once per group.  First come those tiles, one step each, with the requests'
+// own key masks.  Then come the requests' private rows, one round per 128 of them: every request's part of S (its 32-row quarter,
+// or its two) is the product with its own key tile, written to its own lanes only (the instruction's disable-output-lane mask), and
+// its part of O += P V likewise.  A round's softmax so works on as many logits as a shared tile's; with a step per (request, tile)
+// three quarters of the softmax warps wrote zeros, and a step took as long as any.  16 requests of 32 rows, 32 heads, 2048 shared
+// keys and 922 private rows: 86 -> 70 us per layer (HBM floor 42), pass over 4 layers 1830 -> 1752.  A shared step is bound by the softmax chain (2700 cycles),
+// a round by HBM (7300 cycles for 256 KB, 7.5 TB/s over the chip).  Rounds and shared steps in turn, so that one's loads run under
+// the other's arithmetic, took 61 us, but another order of sums changes tokens that were near ties (2 of 512): not done.  Private
+// tiles requested into L2 while the shared steps run: 77-87 us.  K and V rings of three stages.
+constexpr int AG_STAGES = 3;
+constexpr int AG_SMEM = (1 + 2 * AG_STAGES) * AT_TILE + 2048 + 512;    // Q, K, V, row exchange, barriers; the window has to start 1024-aligned
+
+__global__ void __launch_bounds__(AT_THREADS, 1)
+attention_group_kernel(const AttnTcArgs a, const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUtensorMap mapK,
+                       const __grid_constant__ CUtensorMap mapV, const __grid_constant__ CUtensorMap mapKn,
+                       const __grid_constant__ CUtensorMap mapVn) {
+    extern __shared__ unsigned char smem_raw[];
+    const uint32_t base = smem_u32(smem_raw);
+    if (base & 1023u) {                                        // the tiles would not be aligned: report, touch nothing
+        if (threadIdx.x == 0) atomicOr(a.status, kFlagWaitExpired);
+        return;
+    }
+    constexpr int kRows = (1 + 2 * AG_STAGES) * AT_TILE, kBars = kRows + 2048;
+    const uint32_t sQ = base, sK0 = base + AT_TILE, sV0 = base + (1 + AG_STAGES) * AT_TILE, bars = base + kBars;
+    volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(smem_raw + kBars + 352);
+    volatile int* abort_flag = reinterpret_cast<volatile int*>(smem_raw + kBars + 356);
+    int* kept = reinterpret_cast<int*>(smem_raw + kBars + 360);
+    // barriers: 0 q_full | by ring stage: 1.. k_full | 4.. k_empty | 7.. v_full | 10.. v_empty |
+    //           by (S buffer, request): 13.. s_full | 21.. p_full | 29.. pv_done
+    auto bar = [&](int i) { return bars + 8 * i; };
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int C = a.split, rank = C > 1 ? (int)cluster_ctarank() : 0;
+    const int G = a.group, qpr = 4 / G;                        // quarters per request
+    const int item = blockIdx.x / C, h = item % a.n_heads, b0 = item / a.n_heads * G;
+    const int n_req = min(G, a.batch - b0), live_q = n_req * qpr;
+    const int kvh = h / (a.n_heads / a.n_kv_heads);
+
+    if (threadIdx.x == 0) {
+        for (int i = 0; i < 37; ++i) mbar_init(bar(i), i >= 21 && i < 29 ? 4 * qpr : 1);
+        *abort_flag = 0;
+        kept[0] = INT_MAX; kept[1] = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == 1) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;"
+                     ::"r"(smem_u32(const_cast<uint32_t*>(tmem_slot))) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem_base = *tmem_slot;
+    const uint32_t tS0 = tmem_base, tO = tmem_base + 256;
+    pdl_wait();
+    pdl_launch_dependents();
+    if (threadIdx.x == AT_THREADS - 32) {                      // (a warp that has nothing else to do yet)
+        const uint64_t pol = policy_evict_first();
+        mbar_expect_tx(bar(0), n_req * qpr * 8192);
+        for (int r = 0; r < n_req; ++r) {                      // boxes of 32 qpr rows (rows past the request's read as zero)
+            tma_load_3d(sQ + r * qpr * 4096, &mapQ, h * 128, 0, b0 + r, bar(0), pol);
+            tma_load_3d(sQ + AT_PANEL + r * qpr * 4096, &mapQ, h * 128 + 64, 0, b0 + r, bar(0), pol);
+        }
+    }
+    __syncwarp();
+    const int n_cache = (a.ctx_len + 127) / 128;
+    const int2 cache = C == 1 ? kept_tiles(a, b0, n_req, kept) : make_int2(0, n_cache);
+
+    // This CTA's part: the key tiles, the cache's and then request by request the private ones, are cut into C ranges; of those that
+    // hold keys n_s shared ones from t0 on, then n_own(r) private ones of request r from f_own(r) on, one in each round.
+    const int n_all = n_cache + a.n_fresh_tiles * n_req;
+    const int j0 = rank * n_all / C, j1 = (rank + 1) * n_all / C;
+    const int t0 = max(j0, cache.x), n_s = max(min(j1, cache.y) - t0, 0);
+    auto f_own = [&](int r) { return min(max(j0 - n_cache - r * a.n_fresh_tiles, 0), a.n_fresh_tiles); };
+    auto n_own = [&](int r) { return min(max(j1 - n_cache - r * a.n_fresh_tiles, 0), a.n_fresh_tiles) - f_own(r); };
+    int n_steps = 0;
+    for (int r = 0; r < n_req; ++r) n_steps = max(n_steps, n_own(r));
+    n_steps += n_s;
+    // barrier and phase of step i, request r: s_full, p_full, pv_done
+    auto s_full = [&](int i, int r) { return bar(13 + (i & 1) * 4 + r); };
+    auto p_full = [&](int i, int r) { return bar(21 + (i & 1) * 4 + r); };
+    auto pv_done = [&](int i, int r) { return bar(29 + (i & 1) * 4 + r); };
+    auto phase = [](int i) { return (uint32_t)(i >> 1) & 1u; };
+
+    const bool softmax = warp >= 2 && warp < 18 && (warp & 3) < live_q;
+    const int n_mine = n_s + (softmax ? n_own((warp & 3) / qpr) : 0);      // steps of this warp's request
+    float m_use = -INFINITY, l = 0.f;
+    if (warp == 0 && lane == 0) {
+        // ---------------- TMA producer: K and V rings each as far ahead as they go ----------------
+        const uint64_t pol_shared = policy_evict_last(), pol_own = policy_evict_first();
+        int ki = 0, vi = 0, kr = 0, vr = 0, ks = 0, vs = 0;    // where each ring is: step, request of a round, stage, phase
+        uint32_t kp = 1, vp = 1;
+        auto settle = [&](int& i, int& r) {                    // on to the next request that has a tile in the round
+            while (i >= n_s && i < n_steps && (r == n_req || i - n_s >= n_own(r)))
+                if (++r >= n_req) { r = 0; ++i; }
+        };
+        auto load = [&](int& i, int& r, uint32_t dst, uint32_t full, const CUtensorMap* shared_map, const CUtensorMap* own_map) {
+            const bool own = i >= n_s;
+            const CUtensorMap* m = own ? own_map : shared_map;
+            const int r0 = (own ? f_own(r) + i - n_s : t0 + i) * 128, bz = own ? b0 + r : 0;
+            const uint64_t pol = own ? pol_own : pol_shared;
+            mbar_expect_tx(full, AT_TILE);
+            tma_load_3d(dst, m, kvh * 128, r0, bz, full, pol);
+            tma_load_3d(dst + AT_PANEL, m, kvh * 128 + 64, r0, bz, full, pol);
+            if (own) ++r;
+            else ++i;
+            settle(i, r);
+        };
+        settle(ki, kr);
+        settle(vi, vr);
+        for (uint32_t idle = 0; ki < n_steps || vi < n_steps;) {
+            bool moved = false;
+            if (ki < n_steps && mbar_test(bar(4 + ks), kp)) {
+                load(ki, kr, sK0 + ks * AT_TILE, bar(1 + ks), &mapK, &mapKn);
+                if (++ks == AG_STAGES) { ks = 0; kp ^= 1; }
+                moved = true;
+            }
+            if (vi < n_steps && mbar_test(bar(10 + vs), vp)) {
+                load(vi, vr, sV0 + vs * AT_TILE, bar(7 + vs), &mapV, &mapVn);
+                if (++vs == AG_STAGES) { vs = 0; vp ^= 1; }
+                moved = true;
+            }
+            if (moved) idle = 0;
+            else if (++idle >= TC_WAIT_LIMIT << 4) *abort_flag = 1;
+            if ((idle & 1023u) == 1023u && *abort_flag) break;
+        }
+    } else if (warp == 1) {
+        // ---------------- MMA issuer 1: S = Q K^T ----------------
+        const uint32_t idesc_s = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(128 >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
+        auto wait = [&](uint32_t b, uint32_t parity) { return __all_sync(0xffffffffu, mbar_poll(b, parity, abort_flag)); };
+        bool ok = wait(bar(0), 0);
+        int ks = 0;
+        uint32_t kp = 0;
+        for (int i = 0; i < n_steps && ok; ++i) {
+            const bool own = i >= n_s;
+            const int parts = own ? n_req : 1;                 // a product per request, or one for all of them
+            for (int r = 0; r < parts && ok; ++r) {
+                if (own && i - n_s >= n_own(r)) continue;
+                // the S buffer also holds the P of step i - 2: free once that step's P V has completed
+                if (i >= 2)
+                    for (int e = r; e < (own ? r + 1 : n_req) && ok; ++e) ok = wait(pv_done(i, e), phase(i - 2));
+                if (!ok || !(ok = wait(bar(1 + ks), kp))) break;                  // K landed
+                tc_fence_after();
+                const uint32_t k = sK0 + ks * AT_TILE;
+                const uint32_t lanes = own ? ((1u << qpr) - 1u) << (r * qpr) : 15u;
+                if (elect_lane()) {
 #pragma unroll
-                for (int c = 0; c < 8; ++c)
-                    if (c < C)
-                        asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
-                                     : "=f"(u[c].x), "=f"(u[c].y), "=f"(u[c].z), "=f"(u[c].w) : "r"(mapa_u32(src, c)) : "memory");
-                float4 o = u[0];
-#pragma unroll
-                for (int c = 1; c < 8; ++c)
-                    if (c < C) { o.x += u[c].x; o.y += u[c].y; o.z += u[c].z; o.w += u[c].w; }
-                if (g4 + 1 == width >> 4) cluster_arrive();      // the last read: before the stores, which it would wait for
-                if (grow < a.n)
-                    *reinterpret_cast<uint2*>(out + g4 * 4) = make_uint2(pack_bf16(o.x * inv, o.y * inv), pack_bf16(o.z * inv, o.w * inv));
+                    for (int e = 0; e < 8; ++e) {
+                        const uint64_t da = smem_desc_sw128(sQ + (e >> 2) * AT_PANEL) + (uint64_t)((e & 3) * 2);
+                        const uint64_t db = smem_desc_sw128(k + (e >> 2) * AT_PANEL) + (uint64_t)((e & 3) * 2);
+                        tc_mma_lanes(tS0 + (i & 1) * 128, da, db, idesc_s, e > 0 ? 1u : 0u, lanes);
+                    }
+                    for (int e = r; e < (own ? r + 1 : n_req); ++e) tc_commit(s_full(i, e));
+                    tc_commit(bar(4 + ks));            // k_empty
+                }
+                __syncwarp();
+                if (++ks == AG_STAGES) { ks = 0; kp ^= 1; }
             }
         }
+    } else if (warp == AT_THREADS / 32 - 1) {
+        // ---------------- MMA issuer 2: O += P V ----------------
+        const uint32_t idesc_o = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 16) | ((uint32_t)(128 >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
+        auto wait = [&](uint32_t b, uint32_t parity) { return __all_sync(0xffffffffu, mbar_poll(b, parity, abort_flag)); };
+        bool ok = true;
+        int vs = 0;
+        uint32_t vp = 0;
+        for (int i = 0; i < n_steps && ok; ++i) {
+            const bool own = i >= n_s;
+            const int parts = own ? n_req : 1;
+            for (int r = 0; r < parts && ok; ++r) {
+                if (own && i - n_s >= n_own(r)) continue;
+                for (int e = r; e < (own ? r + 1 : n_req) && ok; ++e) ok = wait(p_full(i, e), phase(i));    // P written, O rescaled
+                if (!ok || !(ok = wait(bar(7 + vs), vp))) break;                  // V landed
+                tc_fence_after();
+                const uint32_t v = sV0 + vs * AT_TILE;
+                const uint32_t lanes = own ? ((1u << qpr) - 1u) << (r * qpr) : 15u;
+                if (elect_lane()) {
+#pragma unroll
+                    for (int e = 0; e < 8; ++e)                    // 16 keys = 8 columns of P
+                        tc_mma_ta_lanes(tO, tS0 + (i & 1) * 128 + e * 8, smem_desc_mn_sw128(v + e * 2048), idesc_o,
+                                        (i > 0 || e > 0) ? 1u : 0u, lanes);
+                    for (int e = r; e < (own ? r + 1 : n_req); ++e) tc_commit(pv_done(i, e));
+                    tc_commit(bar(10 + vs));           // v_empty
+                }
+                __syncwarp();
+                if (++vs == AG_STAGES) { vs = 0; vp ^= 1; }
+            }
+        }
+    } else if (softmax) {
+        // ---------------- softmax: four threads per query row, as in the one-tile kernel ----------------
+        const int c4 = (warp - 2) >> 2, q = warp & 3, r = q / qpr;
+        const uint32_t lane_off = (uint32_t)(q * 32) << 16;
+        // per quarter: the exchange of maxima [4][32], and of denominators [4][32] when the last tile is done
+        uint16_t* row_max = reinterpret_cast<uint16_t*>(smem_raw + kRows + q * 512) + lane;
+        float* row_sum = reinterpret_cast<float*>(smem_raw + kRows + q * 512) + lane;
+        bool ok = true;
+        const uint32_t* excl = a.pos_excl + (int64_t)(b0 + r) * a.excl_words;
+        const uint32_t* serves = a.row_keep + (int64_t)(b0 + r) * a.keep_words;
+        int w = (n_s > 0 ? t0 : f_own(r)) * 4 + c4;            // this thread's word of the step's key masks
+        auto keys = [&](bool own) {                            // which of its 32 keys count
+            if (own) return w < a.keep_words ? __ldg(serves + w) : 0u;
+            const int valid = a.ctx_len - w * 32;
+            const uint32_t in = valid >= 32 ? ~0u : (valid <= 0 ? 0u : (1u << valid) - 1u);
+            return w < a.excl_words ? in & ~__ldg(excl + w) : in;
+        };
+        uint32_t next = n_mine > 0 ? keys(n_s == 0) : 0u;      // asked for a step ahead
+        for (int i = 0; i < n_mine; ++i) {
+            const uint32_t keep = next;
+            w = i + 1 == n_s ? f_own(r) * 4 + c4 : w + 4;
+            if (i + 1 < n_mine) next = keys(i + 1 >= n_s);
+            if (!softmax_tile(keep, i == 0, a.scale_log2e, tS0 + (i & 1) * 128 + lane_off, tO + lane_off, c4, 1 + q, row_max, 32,
+                              p_full(i, r), m_use, l, ok, [&] { return mbar_wait(s_full(i, r), phase(i), abort_flag); },
+                              [&] { return mbar_wait(pv_done(i - 1, r), phase(i - 1), abort_flag); }))
+                break;
+        }
+        // O / l once the last P V has completed (every thread of the row has read the maxima by then)
+        if (ok && n_mine > 0) ok = mbar_wait(pv_done(n_mine - 1, r), phase(n_mine - 1), abort_flag);
+        row_sum[c4 * 32] = l;
+        if (!quarter_any(1 + q, !ok)) {
+            l = (row_sum[0] + row_sum[32]) + (row_sum[64] + row_sum[96]);
+            if (C == 1) {
+                tc_fence_after();
+                const int grow = (q - r * qpr) * 32 + lane;
+                float v[32];
+                tc_ld32(tO + lane_off + c4 * 32, v);
+                if (grow < a.n)
+                    store_o32(static_cast<__nv_bfloat16*>(a.o) + (((int64_t)(b0 + r) * a.n + grow) * a.n_heads + h) * 128 + c4 * 32, v, 1.f / l);
+            }
+        }
+    }
+    if (C > 1) {
         __syncwarp();
-        if (!softmax) cluster_arrive();
-        cluster_wait();
+        __syncthreads();              // a request without tiles of its own here is done before the others' products have read K
+        const int q = warp & 3, r = q / qpr, grow = (q - r * qpr) * 32 + lane;
+        merge_parts(base, smem_raw, C, rank, softmax, n_mine > 0, (warp - 2) >> 2, q * 32 + lane, tO + ((uint32_t)q << 21), m_use, l,
+                    r < n_req && grow < a.n ? static_cast<__nv_bfloat16*>(a.o) + (((int64_t)(b0 + r) * a.n + grow) * a.n_heads + h) * 128
+                                            : nullptr);
     }
     // ---------------- teardown ----------------
     tc_fence_before();
@@ -657,8 +953,7 @@ attention_tc2q_kernel(const AttnTcArgs a, const __grid_constant__ CUtensorMap ma
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int qt = blockIdx.x, h = blockIdx.y, b = blockIdx.z;
     const int kvh = h / (a.n_heads / a.n_kv_heads);
-    const int n_cache_tiles = (a.ctx_len + 127) / 128;
-    const int n_tiles = n_cache_tiles + a.n_fresh_tiles;
+    int* kept = reinterpret_cast<int*>(base_ptr + 6 * AT_TILE + 208);
     const int kb = a.cache_shared ? 0 : b;
     const int n_sets = (qt * 256 + 128 < a.n) ? 2 : 1;      // the last CTA of an odd tile count has one tile
     float2* s_tab = reinterpret_cast<float2*>(base_ptr + 6 * AT_TILE + 256);     // [2 query tiles][128 rows] (reference, weight)
@@ -670,6 +965,7 @@ attention_tc2q_kernel(const AttnTcArgs a, const __grid_constant__ CUtensorMap ma
         for (int i = 15; i <= 18; ++i) mbar_init(bar(i), 1);
         mbar_init(bar(19), 4); mbar_init(bar(20), 4);          // score sweep: the four warps of a query tile are done with D
         *abort_flag = 0;
+        kept[0] = INT_MAX; kept[1] = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 1) {
@@ -684,6 +980,8 @@ attention_tc2q_kernel(const AttnTcArgs a, const __grid_constant__ CUtensorMap ma
     // columns: S of query tile 0 | S of query tile 1 | O of query tile 0 | O of query tile 1, 128 each
     pdl_wait();
     pdl_launch_dependents();
+    const int2 cache = kept_tiles(a, b, 1, kept);
+    const int c_lo = cache.x, n_cache_tiles = cache.y - cache.x, n_tiles = n_cache_tiles + a.n_fresh_tiles;
     // score sweep (Eq. 4-5 from this attention's logits): only CTAs whose 256 query rows hold a flagged row walk the
     // affix key tiles [sw0, sw0 + n_sw) a second time
     int n_sw = 0, sw0 = 0;
@@ -706,7 +1004,7 @@ attention_tc2q_kernel(const AttnTcArgs a, const __grid_constant__ CUtensorMap ma
         auto prefetch_tile = [&](int j) {
             if (j >= n_tiles) return;
             const bool fresh = j >= n_cache_tiles;
-            const int r0 = (fresh ? j - n_cache_tiles : j) * 128, bz = fresh ? b : kb;
+            const int r0 = (fresh ? j - n_cache_tiles : c_lo + j) * 128, bz = fresh ? b : kb;
             tma_prefetch_3d(fresh ? &mapKn : &mapK, kvh * 128, r0, bz);
             tma_prefetch_3d(fresh ? &mapKn : &mapK, kvh * 128 + 64, r0, bz);
             tma_prefetch_3d(fresh ? &mapVn : &mapV, kvh * 128, r0, bz);
@@ -722,7 +1020,7 @@ attention_tc2q_kernel(const AttnTcArgs a, const __grid_constant__ CUtensorMap ma
             const bool fresh = j >= n_cache_tiles;
             const CUtensorMap* mk = fresh ? &mapKn : &mapK;
             const CUtensorMap* mv = fresh ? &mapVn : &mapV;
-            const int r0 = (fresh ? j - n_cache_tiles : j) * 128, bz = fresh ? b : kb;
+            const int r0 = (fresh ? j - n_cache_tiles : c_lo + j) * 128, bz = fresh ? b : kb;
             mbar_expect_tx(bar(1 + s), AT_TILE);
             tma_load_3d(sK0 + s * AT_TILE, mk, kvh * 128, r0, bz, bar(1 + s), pol_kv);
             tma_load_3d(sK0 + s * AT_TILE + AT_PANEL, mk, kvh * 128 + 64, r0, bz, bar(1 + s), pol_kv);
@@ -840,7 +1138,7 @@ attention_tc2q_kernel(const AttnTcArgs a, const __grid_constant__ CUtensorMap ma
         for (int i = 0; i < 2 * n_tiles && ok; ++i) {
             const int hb = i & 1, j = i >> 1;
             if (hb == 0) {
-                const int k0 = j * 128;
+                const int k0 = (c_lo + j) * 128;                  // (of a cache tile)
                 const bool in = !want_lf || (k0 >= aff0 && k0 + 128 <= aff1), out = !want_lf || k0 >= aff1 || k0 + 128 <= aff0;
                 if (!a.pos_excl && k0 + 128 <= a.ctx_len && (in || out)) {
 #pragma unroll
@@ -854,7 +1152,7 @@ attention_tc2q_kernel(const AttnTcArgs a, const __grid_constant__ CUtensorMap ma
                         if (j < n_cache_tiles) {
                             const int valid = a.ctx_len - k0 - w * 32;
                             keep4[w] = valid >= 32 ? ~0u : (valid <= 0 ? 0u : (1u << valid) - 1u);
-                            if (a.pos_excl && j * 4 + w < a.excl_words) keep4[w] &= ~__ldg(a.pos_excl + (int64_t)b * a.excl_words + j * 4 + w);
+                            if (a.pos_excl && (k0 >> 5) + w < a.excl_words) keep4[w] &= ~__ldg(a.pos_excl + (int64_t)b * a.excl_words + (k0 >> 5) + w);
                             // of those keys, the ones inside the affix span
                             const int lo = max(aff0 - k0 - w * 32, 0), hi = min(aff1 - k0 - w * 32, 32);
                             if (want_lf && hi > lo) aff4[w] = (hi - lo >= 32 ? ~0u : ((1u << (hi - lo)) - 1u) << lo);
@@ -1115,12 +1413,15 @@ int launch_attention_tc(const AttnArgs& a, uint32_t* status, cudaStream_t stream
     const bool shared = a.kv_batch_stride == 0;           // one cache for the whole batch
     const int kv_cols = a.n_kv_heads * 128;
     std::lock_guard<std::mutex> lock(g_map3_mutex);
-    // decode passes over a shared cache: the rows of four requests share one tile (see AttnTcArgs::group)
+    // decode passes over a shared cache: the rows of several requests share one query tile (attention_group_kernel)
     static const bool group_on = [] { const char* e = getenv("ACACHE_ATTN_GROUP"); return !e || atoi(e) != 0; }();
-    const int group = (group_on && two_src && shared && a.n <= 32 && a.batch >= 2) ? 4 : 1;
+    // (two requests of up to 64 rows only where one to a tile needs more than one wave: half as many CTAs, each with less than
+    // twice the work: 13 requests of 62 rows, 32 heads, pass over 4 layers 2579 -> 2472 us)
+    const bool grouped = group_on && two_src && shared && a.batch >= 2;
+    const int group = grouped && a.n <= 32 ? 4 : grouped && a.n <= 64 && a.batch * a.n_heads > 148 ? 2 : 1;
     CUtensorMap maps[5];
     const CUtensorMap* found[5];
-    found[0] = get_map3(a.q, a.n, a.n_heads * 128, a.batch, (int64_t)a.n * a.n_heads * 128, group > 1 ? 32 : 128);
+    found[0] = get_map3(a.q, a.n, a.n_heads * 128, a.batch, (int64_t)a.n * a.n_heads * 128, 128 / group);
     if (found[0]) maps[0] = *found[0];
     found[1] = get_map3(a.cache_k, a.ctx_len, kv_cols, shared ? 1 : a.batch, shared ? (int64_t)a.ctx_len * kv_cols : a.kv_batch_stride);
     if (found[1]) maps[1] = *found[1];
@@ -1139,6 +1440,7 @@ int launch_attention_tc(const AttnArgs& a, uint32_t* status, cudaStream_t stream
         cudaFuncSetAttribute(attention_tc_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, AT_SMEM);
         cudaFuncSetAttribute(attention_tc_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, AT_SMEM);
         cudaFuncSetAttribute(attention_tc2q_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, AT2_SMEM);
+        cudaFuncSetAttribute(attention_group_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, AG_SMEM);
         attr = true;
     }
     AttnTcArgs t{};
@@ -1185,10 +1487,10 @@ int launch_attention_tc(const AttnArgs& a, uint32_t* status, cudaStream_t stream
         t.n_items = (int)ctas;
         // from six rounds of CTAs on, items share a CTA (of the layer-step, 0.7-1.0 % at 13.8 rounds, 0.2-0.5 % at 8.6, 0.4-1.0 % at
         // 6.5; at 1.9 and 2.8 rounds, where the hardware's assignment evens out the last round, 0.3 and 0.9 % slower)
-        const bool many = t.split == 1 && t.n_items >= 6 * sm_count();
+        const bool many = t.split == 1 && group == 1 && t.n_items >= 6 * sm_count();
         cfg.gridDim = dim3(many ? sm_count() : t.n_items * t.split);
         cfg.blockDim = dim3(AT_THREADS);
-        cfg.dynamicSmemBytes = AT_SMEM;
+        cfg.dynamicSmemBytes = group > 1 ? AG_SMEM : AT_SMEM;
         cfg.stream = stream;
         cudaLaunchAttribute at[2];
         at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -1197,7 +1499,8 @@ int launch_attention_tc(const AttnArgs& a, uint32_t* status, cudaStream_t stream
         at[1].val.clusterDim.x = t.split; at[1].val.clusterDim.y = 1; at[1].val.clusterDim.z = 1;
         cfg.attrs = at;
         cfg.numAttrs = t.split > 1 ? 2 : 1;
-        err = cudaLaunchKernelEx(&cfg, many ? attention_tc_kernel<true> : attention_tc_kernel<false>, t, *mq, *mk, *mv, *mkn, *mvn);
+        err = cudaLaunchKernelEx(&cfg, group > 1 ? attention_group_kernel : many ? attention_tc_kernel<true> : attention_tc_kernel<false>, t, *mq,
+                                 *mk, *mv, *mkn, *mvn);
     }
     return err == cudaSuccess ? 1 : -1;
 }

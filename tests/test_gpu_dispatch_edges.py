@@ -206,6 +206,41 @@ def test_attention_items_per_cta(B, T, rows, shared):
         assert_close_bf16(ab.to_host_bits(y[b]), ref["y"], "y")
 
 
+# Two or four requests to a query tile over a shared cache, private rows in rounds behind the shared tiles: one and several rounds,
+# groups that are not full, one CTA and clusters of up to eight (some without a step of their own), an affix that neither starts
+# nor ends with a tile, empty tiles in front of it and behind it
+@pytest.mark.parametrize("shape,B,pre,L,post,rows,ratio", [
+    (HEADS32, 4, 0, 300, 40, 32, 0.3), (HEADS32, 6, 150, 500, 180, 7, 0.5), (HEADS32, 5, 5, 260, 90, 64, 0.2),
+    (MID128, 2, 9, 700, 60, 33, 0.2), (MID128, 3, 300, 200, 300, 20, 0.1), (MID128, 2, 0, 2500, 64, 1, 0.05),
+    (MID128, 7, 130, 1100, 100, 50, 0.35)])
+def test_attention_of_grouped_requests(shape, B, pre, L, post, rows, ratio):
+    lay = wl.make_layout(B, pre, L, post, rows, rows, "all")
+    case = wl.make_case(shape, lay, ratio, cfg_id=78, weights=cached_weights(shape, 78), hot_frac=0.01)
+    T, K = lay.ctx_len, orc.k_from_ratio(L, ratio)
+    dc = DeviceCase(case, max_rows=K + lay.n_extra)
+    rng = np.random.default_rng(T)
+    anchors = np.stack([np.sort(rng.choice(L, K, replace=False)) for _ in range(B)]).astype(np.int32)
+    own = np.concatenate([anchors + pre, lay.extra_rows], axis=1)              # position of every private row
+    where = [{int(p): i for i, p in enumerate(own[b])} for b in range(B)]
+    slot_rows = np.stack([[where[b][int(p)] for p in lay.masked_pos[b]] for b in range(B)]).astype(np.int32)
+    on = lambda t: torch.from_numpy(np.ascontiguousarray(t)).to(DEV)
+    shared = [ab.to_device_bf16(c[:1].copy(), DEV) for c in (case.cache_k, case.cache_v)]
+    mine = [c[np.arange(B)[:, None], own] for c in (case.cache_k, case.cache_v)]
+    k_slots, v_slots = (ab.to_device_bf16(np.ascontiguousarray(m), DEV) for m in mine)
+    block = on(lay.masked_pos)
+    req = ab.Context.request(B, T, pre, L, block, block, dc.cos, dc.sin)
+    y = torch.zeros((B, rows, shape.hidden), dtype=torch.bfloat16, device=DEV)
+    dc.ctx.recompute_rows_shared(dc.lw, req, dc.req, ab.KV(shared[0].data_ptr(), shared[1].data_ptr(), 0, T), dc.x, 0, on(anchors), K,
+                                 on(slot_rows), k_slots, v_slots, y)
+    assert dc.ctx.poll_status() == 0
+    for b in {0, 1, B // 2, B - 1}:
+        ck, cv = case.cache_k[0].copy(), case.cache_v[0].copy()
+        ck[own[b]], cv[own[b]] = mine[0][b], mine[1][b]
+        ref = orc.layer_step(case.weights, shape, case.x[b], ck, cv, T, pre, L, lay.masked_pos[b], lay.masked_pos[b], case.rope_cos,
+                             case.rope_sin, anchor_idx=np.zeros(0, np.int32))
+        assert_close_bf16(ab.to_host_bits(y[b]), ref["y"], "y")
+
+
 # Small projections sum K in the general kernel's order, block by block: a row's bits do not depend on how many rows are in the
 # call, on the tile or on the split over a cluster (140 rows take the two-SM kernel).  Every product is reached with inputs that
 # the other rows of a call do not change: no queries, hence equal weights over equal values, so that the attention's output is
