@@ -349,17 +349,19 @@ score_colsum_tc_kernel(const ScoreTcArgs a, const int n_pad, const __grid_consta
 constexpr int S1_CLUSTER = 8;
 constexpr int S1_THREADS = 192;                 // warp 0 TMA, warp 1 MMA, warps 2-5 one thread per key
 constexpr int S1_MAX_TILES = 16;
-// query tile (NP rows x 128: 8 or 16 KB) | key ring, 3 or 2 stages (after the last tile: the transposition buffer [128][65]
-// fp32) | tables | barriers.  About 105 KB / 85 KB: two CTAs per SM, which is also what tensor memory allows at up to 256
-// columns per CTA; a CTA that needs all 512 columns asks for S1_SMEM_WIDE so that no second CTA can be resident beside it
-// (a CTA waiting for tensor memory inside a cluster whose peers wait for it at a cluster barrier would never get it).
-template <int NP> struct S1 {
+// query tile (NP rows x 128: 8 or 16 KB) | key ring (after the last tile: the transposition buffer [128][65] fp32) | tables |
+// barriers.  With three stages of keys two CTAs fit on an SM, which is also what tensor memory allows at up to 256 columns per
+// CTA; with two stages three CTAs do, for up to 128 columns: a CTA spends as long after its last tile as it does loading (7000
+// and 8000 cycles for 512 keys).  2048 (head, request) pairs of 512 keys and 32 rows: 102 -> 85 us, and 74 without the cluster
+// barriers of a CTA that has no peers (1000-3500 cycles each, they wait for memory).  Four CTAs with one stage 89.  A CTA
+// that needs all 512 columns asks for S1_SMEM_WIDE so that no second CTA can be resident beside it (a CTA waiting for
+// tensor memory inside a cluster whose peers wait for it at a cluster barrier would never get it).
+template <int NP, int STAGES> struct S1 {
     static constexpr int Q_BYTES = 2 * NP * 128;
-    static constexpr int STAGES = NP == 32 ? 3 : 2;
-    static constexpr int TAB_OFF = Q_BYTES + STAGES * ST_K_BYTES;
+    static constexpr int RING = STAGES * ST_K_BYTES > 128 * 65 * 4 ? STAGES * ST_K_BYTES : 128 * 65 * 4;
+    static constexpr int TAB_OFF = Q_BYTES + RING;
     static constexpr int BAR_OFF = TAB_OFF + 2048;
-    static constexpr int SMEM = BAR_OFF + 512 + 1024;
-    static_assert(128 * 65 * 4 <= STAGES * ST_K_BYTES, "the transposition buffer reuses the key ring");
+    static constexpr int SMEM = BAR_OFF + 512;              // the window has to start 1024-aligned
 };
 constexpr int S1_SMEM_WIDE = 120 * 1024;
 
@@ -388,17 +390,22 @@ __device__ __forceinline__ float2 ld_cluster_f2(uint32_t local_addr, uint32_t ra
 
 // NP: columns per key tile (the masked rows rounded up to 32 or 64); tpc: 128-key tiles per CTA
 // csize: CTAs per cluster (1, 2, 4 or 8; the launch sets the cluster dimension to the same number)
-template <int NP>
-__global__ void __launch_bounds__(S1_THREADS, 2)
+template <int NP, int S1_STAGES, int CTAS>
+__global__ void __launch_bounds__(S1_THREADS, CTAS)
 score_onepass_tc_kernel(const ScoreTcArgs a, const int tpc, const uint32_t tmem_cols, const int csize,
                         const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUtensorMap mapK) {
     extern __shared__ unsigned char smem_raw[];
-    const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
-    unsigned char* base_ptr = smem_raw + (base - smem_u32(smem_raw));
-    constexpr int S1_STAGES = S1<NP>::STAGES, S1_BAR_OFF = S1<NP>::BAR_OFF;
-    const uint32_t sQ = base, sK0 = base + S1<NP>::Q_BYTES;
-    float* s_t = reinterpret_cast<float*>(base_ptr + S1<NP>::Q_BYTES);          // [128 keys][65]: per-thread column values
-    float* s_w = reinterpret_cast<float*>(base_ptr + S1<NP>::TAB_OFF);          // [64] per-row scalar handed to the key threads
+    using Layout = S1<NP, S1_STAGES>;
+    constexpr int S1_BAR_OFF = Layout::BAR_OFF;
+    const uint32_t base = smem_u32(smem_raw);
+    if (base & 1023u) {                                                          // the tiles would not be aligned: report, touch nothing
+        if (threadIdx.x == 0) atomicOr(a.status, kFlagWaitExpired);
+        return;
+    }
+    unsigned char* base_ptr = smem_raw;
+    const uint32_t sQ = base, sK0 = base + Layout::Q_BYTES;
+    float* s_t = reinterpret_cast<float*>(base_ptr + Layout::Q_BYTES);          // [128 keys][65]: per-thread column values
+    float* s_w = reinterpret_cast<float*>(base_ptr + Layout::TAB_OFF);          // [64] per-row scalar handed to the key threads
     float* s_part = s_w + 64;                                                   // [4 warps][64] partial column reductions
     float2* s_x = reinterpret_cast<float2*>(s_part + 256);                      // [64] (maximum, denominator share) for the peers
     const uint32_t bars = base + S1_BAR_OFF;
@@ -548,8 +555,9 @@ score_onepass_tc_kernel(const ScoreTcArgs a, const int tpc, const uint32_t tmem_
         for (int g = 0; g < GROUPS; ++g) d += s_part[g * 64 + threadIdx.x];
         s_x[threadIdx.x] = make_float2(s_w[threadIdx.x], d);
     }
-    // (iii) the eight CTAs' statistics meet: one weight per masked row
-    cluster_sync_s1();
+    // (iii) the CTAs' statistics meet: one weight per masked row
+    if (csize > 1) cluster_sync_s1();
+    else __syncthreads();
     if (threadIdx.x < NP) {
         float2 st[S1_CLUSTER];
 #pragma unroll
@@ -565,6 +573,7 @@ score_onepass_tc_kernel(const ScoreTcArgs a, const int tpc, const uint32_t tmem_
         s_part[threadIdx.x] = ((int)threadIdx.x < a.m && mine > -INFINITY && Dn > 0.f) ? ex2(mine - M) / Dn : 0.f;
     }
     __syncthreads();
+    if (csize > 1) cluster_arrive();         // the peers' statistics have been read: before the stores, which it would wait for
     // (iv) the key's column sum
     if (keyw) {
         for (int t = 0; t < n_tiles && ok; ++t) {
@@ -582,7 +591,8 @@ score_onepass_tc_kernel(const ScoreTcArgs a, const int tpc, const uint32_t tmem_
         }
     }
     tc_fence_before();
-    cluster_sync_s1();            // no CTA leaves while a peer may still read its statistics
+    if (csize > 1) cluster_wait();           // no CTA leaves while a peer may still read its statistics
+    __syncthreads();
     if (*abort_flag) {
         if (threadIdx.x == 0) {
             atomicOr(a.status, kFlagWaitExpired);
@@ -651,12 +661,15 @@ int launch_score_tc(const ScoreArgs& a, uint32_t* status, cudaStream_t stream) {
             const CUtensorMap* mq1 = get_map3(a.q_mask, a.m, a.n_heads * 128, a.batch, (int64_t)a.m * a.n_heads * 128, np);
             if (mq1) {
                 const CUtensorMap map_q1 = *mq1;
-                static bool attr1 = false;
-                if (!attr1) {
-                    cudaFuncSetAttribute(score_onepass_tc_kernel<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, S1_SMEM_WIDE);
-                    cudaFuncSetAttribute(score_onepass_tc_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, S1_SMEM_WIDE);
-                    attr1 = true;
-                }
+                // three CTAs per SM where tensor memory allows it and there are more than two per SM
+                const bool three = np == 32 && cols <= 128 && (int64_t)a.n_heads * a.batch * csize > 2 * 148;
+                auto kernel = three ? score_onepass_tc_kernel<32, 2, 3> : np == 32 ? score_onepass_tc_kernel<32, 3, 2> : score_onepass_tc_kernel<64, 2, 2>;
+                const int need = three ? S1<32, 2>::SMEM : np == 32 ? S1<32, 3>::SMEM : S1<64, 2>::SMEM;
+                static std::once_flag once;
+                std::call_once(once, [] {
+                    for (auto k : {score_onepass_tc_kernel<32, 2, 3>, score_onepass_tc_kernel<32, 3, 2>, score_onepass_tc_kernel<64, 2, 2>})
+                        cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, S1_SMEM_WIDE);
+                });
                 ScoreTcArgs t1{};
                 t1.row_stats = a.row_stats; t1.head_partial = a.head_partial;
                 t1.m = a.m; t1.n_heads = a.n_heads; t1.n_kv_heads = a.n_kv_heads;
@@ -667,7 +680,7 @@ int launch_score_tc(const ScoreArgs& a, uint32_t* status, cudaStream_t stream) {
                 cudaLaunchConfig_t cfg{};
                 cfg.gridDim = dim3(a.n_heads * csize, a.batch);
                 cfg.blockDim = dim3(S1_THREADS);
-                cfg.dynamicSmemBytes = cols > 256 ? (size_t)S1_SMEM_WIDE : (size_t)(np == 32 ? S1<32>::SMEM : S1<64>::SMEM);
+                cfg.dynamicSmemBytes = cols > 256 ? S1_SMEM_WIDE : need;
                 cfg.stream = stream;
                 cudaLaunchAttribute at[2];
                 at[0].id = cudaLaunchAttributeClusterDimension;
@@ -676,9 +689,7 @@ int launch_score_tc(const ScoreArgs& a, uint32_t* status, cudaStream_t stream) {
                 at[1].val.programmaticStreamSerializationAllowed = 1;
                 cfg.attrs = at;
                 cfg.numAttrs = 2;
-                const cudaError_t e1 = np == 32
-                    ? cudaLaunchKernelEx(&cfg, score_onepass_tc_kernel<32>, t1, tpc, cols, csize, map_q1, *mk)
-                    : cudaLaunchKernelEx(&cfg, score_onepass_tc_kernel<64>, t1, tpc, cols, csize, map_q1, *mk);
+                const cudaError_t e1 = cudaLaunchKernelEx(&cfg, kernel, t1, tpc, cols, csize, map_q1, *mk);
                 return e1 == cudaSuccess ? 1 : -1;
             }
         }
