@@ -306,61 +306,72 @@ __device__ __forceinline__ int2 kept_tiles(const AttnTcArgs& a, int b0, int n_re
     const int lo = lo_hi[0], hi = lo_hi[1];
     return lo < hi ? make_int2(lo, hi) : make_int2(0, 0);
 }
-// Merge of a cluster's parts through distributed shared memory: (reference, denominator) of every row meet first; each CTA scales
-// its O to the common reference and lays it out by the CTA that finishes the columns (128 / C each), which sums the parts in rank
-// order.  The K and V stages are idle by now.  All threads pass the three cluster barriers, whatever happened before.  out: the
-// row's 128 columns, null for a row that does not exist; any: this CTA had key tiles (else its O holds nothing).
+// Merge of a cluster's parts through distributed shared memory: every CTA leaves (reference, denominator) of its rows and its O as it
+// is, laid out by the CTA that finishes the columns (128 / C each); behind one barrier that CTA scales the parts to the common
+// reference and sums them in rank order.  (With the references met first and the parts scaled before they were laid out there
+// was a barrier more: layer-step of 103 rows over 1024 keys 146.2 -> 145.7 us.)  The K and V stages are idle by now.  All threads pass the two cluster
+// barriers, whatever happened before.  out: the row's 128 columns, null for a row that does not exist; any: this CTA had key
+// tiles (else its O holds nothing).
 __device__ __forceinline__ void merge_parts(uint32_t base, unsigned char* base_ptr, int C, int rank, bool softmax, bool any, int c4,
                                             int row, uint32_t tO, float m_use, float l, __nv_bfloat16* out) {
     float2* ml = reinterpret_cast<float2*>(base_ptr + AT_TILE + 4096);             // [128]
     const uint32_t parts = base + 2 * AT_TILE;                                     // [owner][column / 4][row][4] fp32
     const int width = 128 / C;
     __syncwarp();
-    if (softmax && c4 == 0) ml[row] = make_float2(m_use, l);
-    __syncwarp();
-    cluster_sync_all();
-    float denom = 0.f;
     if (softmax) {
-        const uint32_t ml_row = smem_u32(ml + row);
-        float ref = -INFINITY, m_c[8], l_c[8];
-#pragma unroll
-        for (int c = 0; c < 8; ++c)
-            if (c < C) {
-                asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(m_c[c]), "=f"(l_c[c]) : "r"(mapa_u32(ml_row, c)) : "memory");
-                ref = fmaxf(ref, m_c[c]);
-            }
-#pragma unroll
-        for (int c = 0; c < 8; ++c)
-            if (c < C && m_c[c] > -INFINITY) denom += l_c[c] * fast_exp2(m_c[c] - ref);
-        const float f = m_use > -INFINITY ? fast_exp2(m_use - ref) : 0.f;
+        if (c4 == 0) ml[row] = make_float2(m_use, l);
         tc_fence_after();
         float v[32];
         tc_ld32(tO + c4 * 32, v);
         const uint32_t dst = parts + ((c4 * 8 * 128 + row) << 4);                  // owners' columns lie one after the other
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
-            const float4 p = any ? make_float4(v[4 * i] * f, v[4 * i + 1] * f, v[4 * i + 2] * f, v[4 * i + 3] * f) : make_float4(0.f, 0.f, 0.f, 0.f);
+            const float4 p = any ? make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]) : make_float4(0.f, 0.f, 0.f, 0.f);
             asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(dst + i * 2048), "f"(p.x), "f"(p.y), "f"(p.z), "f"(p.w) : "memory");
         }
     }
     __syncwarp();
     cluster_sync_all();
     if (softmax) {
-        const float inv = 1.f / denom;
         const int col = rank * width + c4 * (width >> 2);                          // width / 4 columns per thread
+        const uint32_t ml_row = smem_u32(ml + row);
+        float ref = -INFINITY, denom = 0.f, f[8], l_c[8];
+        float4 u[8];
+        const uint32_t src0 = parts + ((col >> 2) * 128 + row) * 16;
+#pragma unroll
+        for (int c = 0; c < 8; ++c)
+            if (c < C) {
+                asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(f[c]), "=f"(l_c[c]) : "r"(mapa_u32(ml_row, c)) : "memory");
+                asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
+                             : "=f"(u[c].x), "=f"(u[c].y), "=f"(u[c].z), "=f"(u[c].w) : "r"(mapa_u32(src0, c)) : "memory");
+            }
+#pragma unroll
+        for (int c = 0; c < 8; ++c)
+            if (c < C) ref = fmaxf(ref, f[c]);
+#pragma unroll
+        for (int c = 0; c < 8; ++c)
+            if (c < C) {
+                f[c] = f[c] > -INFINITY ? fast_exp2(f[c] - ref) : 0.f;             // no key of the row has counted there: its part is 0
+                denom += l_c[c] * f[c];
+            }
+        const float inv = 1.f / denom;
 #pragma unroll 1
         for (int g4 = 0; g4 < width >> 4; ++g4) {
-            const uint32_t src = parts + (((col >> 2) + g4) * 128 + row) * 16;
-            float4 u[8];
+            if (g4 > 0) {
+                const uint32_t src = src0 + g4 * 128 * 16;
 #pragma unroll
-            for (int c = 0; c < 8; ++c)
-                if (c < C)
-                    asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
-                                 : "=f"(u[c].x), "=f"(u[c].y), "=f"(u[c].z), "=f"(u[c].w) : "r"(mapa_u32(src, c)) : "memory");
-            float4 o = u[0];
+                for (int c = 0; c < 8; ++c)
+                    if (c < C)
+                        asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
+                                     : "=f"(u[c].x), "=f"(u[c].y), "=f"(u[c].z), "=f"(u[c].w) : "r"(mapa_u32(src, c)) : "memory");
+            }
+            float4 o = make_float4(__fmul_rn(u[0].x, f[0]), __fmul_rn(u[0].y, f[0]), __fmul_rn(u[0].z, f[0]), __fmul_rn(u[0].w, f[0]));
 #pragma unroll
             for (int c = 1; c < 8; ++c)
-                if (c < C) { o.x += u[c].x; o.y += u[c].y; o.z += u[c].z; o.w += u[c].w; }
+                if (c < C) {
+                    o.x += __fmul_rn(u[c].x, f[c]); o.y += __fmul_rn(u[c].y, f[c]);
+                    o.z += __fmul_rn(u[c].z, f[c]); o.w += __fmul_rn(u[c].w, f[c]);
+                }
             if (g4 + 1 == width >> 4) cluster_arrive();      // the last read: before the stores, which it would wait for
             if (out) *reinterpret_cast<uint2*>(out + col + g4 * 4) = make_uint2(pack_bf16(o.x * inv, o.y * inv), pack_bf16(o.z * inv, o.w * inv));
         }
