@@ -3,8 +3,9 @@
 // At these sizes the weights' stream from HBM is the floor and everything around it is latency.  The general one-SM kernel
 // (gemm_tc.cu) cuts (tile, K block) ranges so that every SM streams the same bytes, and pays with fp32 partial tiles through
 // L2 and a finish kernel behind every projection.  Here a tile of TN weight rows (TN chosen from N, not fixed) belongs to
-// one CTA or to a cluster of S = 2 or 4 CTAs that split K; the cluster's partial accumulators meet in distributed shared
-// memory, every CTA finishing its share of the columns, and the epilogue follows in the same kernel.
+// one CTA or to a cluster of S = 2 or 4 CTAs that split K; every CTA sends its partial accumulators to the CTA that finishes
+// their columns (asynchronous stores into its shared memory, counted by an mbarrier there), and the epilogue follows in the same
+// kernel.
 //
 // Small projections (the general kernel would give every CTA one K block) keep its order of sums: every block of 64 K columns
 // has an accumulator of its own in tensor memory, and they are added in ascending order, a CTA of a cluster handing over its
@@ -48,6 +49,7 @@ struct RowsPlan {
     int stages, stage_bytes;
     int tmem_cols;
     int groups;               // q/k/v: groups of 32 rotary pairs over all segments
+    int recv_off, recv_late;  // where the peers' partial accumulators arrive, from the ring's start on; 1: in the ring itself
     int smem_bytes;
 };
 
@@ -65,13 +67,16 @@ __device__ __forceinline__ void tc_ld8x2(uint32_t ta, uint32_t tb, float (&a)[8]
 #pragma unroll
     for (int i = 0; i < 8; ++i) { a[i] = __uint_as_float(r[i]); b[i] = __uint_as_float(r[8 + i]); }
 }
-__device__ __forceinline__ float4 ld_cluster_f4(uint32_t cluster_addr) {
+__device__ __forceinline__ float4 ld_shared_f4(uint32_t addr) {
     float4 v;
-    asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
-                 : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
-                 : "r"(cluster_addr)
-                 : "memory");
+    asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr) : "memory");
     return v;
+}
+// Four floats into another CTA's shared memory; its mbarrier counts the bytes as they arrive.
+__device__ __forceinline__ void send_f4(uint32_t cluster_addr, const float* v, uint32_t cluster_bar) {
+    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.f32 [%0], {%1, %2, %3, %4}, [%5];"
+                 ::"r"(cluster_addr), "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]), "r"(cluster_bar)
+                 : "memory");
 }
 __device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map, int c1, int c2, uint32_t bar, uint64_t policy) {
     asm volatile(
@@ -119,36 +124,28 @@ __device__ __forceinline__ int rank_panels(const RowsPlan& p, int r) {
     return min((r + 1) * p.blocks / S * p.CP, p.KB) - r * p.blocks / S * p.CP;
 }
 
-// 16 adjacent accumulator columns of this thread's row, summed over the cluster: own tensor memory first, then the peers in
-// rank order (fixed, hence bitwise reproducible).  slice_col: the columns' place inside the slice this CTA finishes;
-// peers: where it lies in each peer's staging area (cluster addresses).
+// 16 adjacent accumulator columns of this thread's row, summed over the cluster: own tensor memory first, then the peers' parts in
+// rank order (fixed, hence bitwise reproducible).  slice_col: the columns' place inside the slice this CTA finishes; recv: where
+// the first peer's part of it lies in shared memory, `region` bytes from one peer to the next.
 template <int S>
-__device__ __forceinline__ void sum_cluster16(uint32_t taddr, const uint32_t (&peers)[S > 1 ? S - 1 : 1], int slice_col, int rows_pad,
-                                              int row, float (&v)[16]) {
-    float4 t[S > 1 ? S - 1 : 1][4];
-    if (S > 1) {
-        const int r = min(row, rows_pad - 1);
-#pragma unroll
-        for (int i = 0; i < S - 1; ++i)
-#pragma unroll
-            for (int j = 0; j < 4; ++j) t[i][j] = ld_cluster_f4(peers[i] + ((((slice_col >> 2) + j) * rows_pad + r) << 4));
-    }
+__device__ __forceinline__ void sum_cluster16(uint32_t taddr, uint32_t recv, int region, int slice_col, int rows_pad, int row,
+                                              float (&v)[16]) {
     tc_ld16(taddr, v);
-    if (S > 1) {
+    const int r = min(row, rows_pad - 1);
 #pragma unroll
-        for (int i = 0; i < S - 1; ++i)
+    for (int i = 0; i < S - 1; ++i)
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                v[4 * j] += t[i][j].x; v[4 * j + 1] += t[i][j].y; v[4 * j + 2] += t[i][j].z; v[4 * j + 3] += t[i][j].w;
-            }
-    }
+        for (int j = 0; j < 4; ++j) {
+            const float4 t = ld_shared_f4(recv + i * region + ((((slice_col >> 2) + j) * rows_pad + r) << 4));
+            v[4 * j] += t.x; v[4 * j + 1] += t.y; v[4 * j + 2] += t.z; v[4 * j + 3] += t.w;
+        }
 }
 
 // The same 16 columns where every K block has its own accumulator: all blocks of the tile in ascending order, rank by rank.
-// per_block: bytes between a peer's blocks in the staging area.
+// per_block: bytes between a peer's blocks.
 template <int S>
-__device__ __forceinline__ void sum_apart16(const RowsPlan& p, int rank, uint32_t taddr, const uint32_t (&peers)[S > 1 ? S - 1 : 1],
-                                            int slice_col, int per_block, int row, float (&v)[16]) {
+__device__ __forceinline__ void sum_apart16(const RowsPlan& p, int rank, uint32_t taddr, uint32_t recv, int region, int slice_col,
+                                            int per_block, int row, float (&v)[16]) {
 #pragma unroll
     for (int j = 0; j < 16; ++j) v[j] = 0.f;
     const int r = min(row, p.rows_pad - 1);
@@ -164,15 +161,14 @@ __device__ __forceinline__ void sum_apart16(const RowsPlan& p, int rank, uint32_
                 for (int j = 0; j < 16; ++j) v[j] += t[j];
             }
         } else if (S > 1) {
-            // (peers holds the other ranks; c < rank: its c-th, else its (c - 1)-th)
-            const uint32_t src = (c < rank ? peers[c < S - 1 ? c : 0] : peers[c > 0 ? c - 1 : 0]) + (((slice_col >> 2) * p.rows_pad + r) << 4);
+            const uint32_t src = recv + (c < rank ? c : c - 1) * region + (((slice_col >> 2) * p.rows_pad + r) << 4);
 #pragma unroll 1
             for (int i0 = 0; i0 < nb; i0 += 4) {
                 float4 t[4][4];
 #pragma unroll
                 for (int i = 0; i < 4; ++i)
 #pragma unroll
-                    for (int j = 0; j < 4; ++j) t[i][j] = ld_cluster_f4(src + min(i0 + i, nb - 1) * per_block + ((j * p.rows_pad) << 4));
+                    for (int j = 0; j < 4; ++j) t[i][j] = ld_shared_f4(src + min(i0 + i, nb - 1) * per_block + ((j * p.rows_pad) << 4));
 #pragma unroll
                 for (int i = 0; i < 4; ++i)
                     if (i0 + i < nb) {
@@ -186,7 +182,7 @@ __device__ __forceinline__ void sum_apart16(const RowsPlan& p, int rank, uint32_
     }
 }
 
-// 228 to 232 registers a thread: no CTA of another tensor-memory kernel finds room beside this one.  That matters where calls run on
+// 228 to 252 registers a thread: no CTA of another tensor-memory kernel finds room beside this one.  That matters where calls run on
 // two streams: with clusters on both sides, CTAs that wait for one another's tensor memory and cluster peers would wait for ever.
 template <int S, int EPI, bool APART>
 __global__ void __launch_bounds__(RW_THREADS, 1)
@@ -194,7 +190,7 @@ gemm_rows_kernel(const GemmArgs g, const RowsPlan p, const __grid_constant__ CUt
                  const __grid_constant__ CUtensorMap mapB0, const __grid_constant__ CUtensorMap mapB1,
                  const __grid_constant__ CUtensorMap mapB2) {
     extern __shared__ unsigned char smem_raw[];
-    __shared__ uint64_t bar_s[2 * RW_MAX_STAGES + 1];
+    __shared__ uint64_t bar_s[2 * RW_MAX_STAGES + 2];
     __shared__ uint32_t tmem_slot;
     __shared__ volatile int abort_s;
     __shared__ float red[RW_THREADS / 32];
@@ -203,18 +199,34 @@ gemm_rows_kernel(const GemmArgs g, const RowsPlan p, const __grid_constant__ CUt
     const uint32_t bars = smem_u32(bar_s);
     auto full_bar = [&](int s) { return bars + 8 * s; };
     auto empty_bar = [&](int s) { return bars + 8 * (RW_MAX_STAGES + s); };
-    const uint32_t done_bar = bars + 8 * 2 * RW_MAX_STAGES;
+    const uint32_t done_bar = bars + 8 * 2 * RW_MAX_STAGES, recv_bar = done_bar + 8;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int rank = S > 1 ? (int)cluster_ctarank() : 0;
     const int nt = blockIdx.x / S;
     const int blk0 = rank * p.blocks / S, blk1 = (rank + 1) * p.blocks / S;
     const int n_blk = blk1 - blk0;
+    // the columns this CTA finishes: items of 16 + 16 rotary pairs (q/k/v), of 16 columns (residual), of 8 + 8 (SwiGLU)
+    constexpr int UNIT = EPI == kEpiQKV ? 32 : 16;
+    const int items = p.TN / UNIT, item0 = rank * items / S, item1 = (rank + 1) * items / S;
+    // a peer's part of them: [block (one if not APART)][column / 4][row][4]
+    const int per_block = (items + S - 1) / S * UNIT * p.rows_pad * 4;
+    const int region = per_block * (APART ? (p.blocks + S - 1) / S * p.CP : 1);
+    const uint32_t recv = base + p.recv_off;
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < p.stages; ++s) { mbar_init(full_bar(s), 1); mbar_init(empty_bar(s), 1); }
         mbar_init(done_bar, 1);
+        if (S > 1) mbar_init(recv_bar, 1);
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        if (S > 1) {              // what the peers will send
+            int from = S - 1;
+            if (APART) {
+                from = 0;
+                for (int c = 0; c < S; ++c) from += c == rank ? 0 : rank_panels<S>(p, c);
+            }
+            mbar_expect_tx(recv_bar, from * (item1 - item0) * UNIT * p.rows_pad * 4);
+        }
     }
     // The weights are constant inputs: the ring's weight halves are requested before the previous kernel has finished; the
     // activation rows follow once they are there.
@@ -252,6 +264,7 @@ gemm_rows_kernel(const GemmArgs g, const RowsPlan p, const __grid_constant__ CUt
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    if (S > 1) cluster_arrive_relaxed();                   // the peers may send once all have come this far
     const uint32_t tmem_base = tmem_slot;
     pdl_wait();
     pdl_launch_dependents();
@@ -316,13 +329,6 @@ gemm_rows_kernel(const GemmArgs g, const RowsPlan p, const __grid_constant__ CUt
     const bool live = q * 32 < p.rows_pad;                 // warp-uniform: the tensor-memory accesses are collective
     const bool valid = row < g.M;
     const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16);
-    // the columns this CTA finishes: items of 16 + 16 rotary pairs (q/k/v), of 16 columns (residual), of 8 + 8 (SwiGLU)
-    constexpr int UNIT = EPI == kEpiQKV ? 32 : 16;
-    const int items = p.TN / UNIT, item0 = rank * items / S, item1 = (rank + 1) * items / S;
-    // staging of the slice of one destination: [block (one if not APART)][column / 4][row][4]
-    const int per_block = (items + S - 1) / S * UNIT * p.rows_pad * 4;
-    const int region = per_block * (APART ? (p.blocks + S - 1) / S * p.CP : 1);
-
     // what does not depend on the sums is requested while the weights stream
     int pos = 0;
     uint4 res[2] = {make_uint4(0u, 0u, 0u, 0u), make_uint4(0u, 0u, 0u, 0u)};
@@ -348,15 +354,21 @@ gemm_rows_kernel(const GemmArgs g, const RowsPlan p, const __grid_constant__ CUt
     if (ok) ok = mbar_wait(done_bar, 0, abort_flag);
     ok = __all_sync(0xffffffffu, ok);
     tc_fence_after();
-    uint32_t peers[S > 1 ? S - 1 : 1] = {};
     if (S > 1) {
-        // the other CTAs' slices to the staging area (the ring: every MMA that read it has completed)
+        // Every other CTA's columns straight from tensor memory into its shared memory; it waits for the bytes alone.  With the
+        // parts staged here, a cluster barrier and loads from the peers: layer-step of 103 rows 145.7 -> 143.3 us, decode pass of
+        // 32 rows over 4 layers 622 -> 618; a launch of 103 rows ended 3.0 us after its last MMA, now 2.0.
+        cluster_wait();
+        if (p.recv_late) {                                 // every CTA's MMAs have read its ring
+            cluster_arrive_relaxed();
+            cluster_wait();
+        }
         if (ok && live) {
-            int at = 0;
+            const int nb = APART ? rank_panels<S>(p, rank) : 1;
             for (int d = 0; d < S; ++d) {
                 if (d == rank) continue;
                 const int u0 = d * items / S, u1 = (d + 1) * items / S;
-                const int nb = APART ? rank_panels<S>(p, rank) : 1;
+                const uint32_t dst = mapa_u32(recv + (rank < d ? rank : rank - 1) * region, d), bar = mapa_u32(recv_bar, d);
                 for (int u = u0 + hf; u < u1; u += 2) {
 #pragma unroll
                     for (int part = 0; part < UNIT / 16; ++part) {
@@ -368,37 +380,20 @@ gemm_rows_kernel(const GemmArgs g, const RowsPlan p, const __grid_constant__ CUt
                             tc_ld16(taddr + blk * p.TN + col, v);
                             if (row < p.rows_pad) {
 #pragma unroll
-                                for (int j = 0; j < 4; ++j)
-                                    asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};"
-                                                 ::"r"(base + at * region + blk * per_block + (((sc + j) * p.rows_pad + row) << 4)),
-                                                   "f"(v[4 * j]), "f"(v[4 * j + 1]), "f"(v[4 * j + 2]), "f"(v[4 * j + 3])
-                                                 : "memory");
+                                for (int j = 0; j < 4; ++j) send_f4(dst + blk * per_block + (((sc + j) * p.rows_pad + row) << 4), v + 4 * j, bar);
                             }
                         }
                     }
                 }
-                ++at;
             }
         }
         __syncwarp();
-        cluster_arrive();
-        cluster_wait();
-#pragma unroll
-        for (int i = 0; i < S - 1; ++i) {
-            const int r = i < rank ? i : i + 1;            // peer; its staging area holds this CTA's slice at place ...
-            peers[i] = mapa_u32(base + (rank < r ? rank : rank - 1) * region, r);
-        }
+        cluster_arrive_relaxed();                          // the last word to the peers: they may leave when they have theirs
+        if (live) ok = __all_sync(0xffffffffu, ok && mbar_wait_cluster(recv_bar, 0, abort_flag));
     }
-    // Once a warp has read its last piece of the peers' staging areas they may leave; it says so before its stores, which the
-    // arrival would otherwise wait for (here, in the scoring and in the attention: layer-step of 8 rows 52.2 -> 51.8 us, of
-    // 103 rows 143.65 -> 143.2).
     auto sum16 = [&](int col, int slice_col, float (&v)[16]) {
-        if (APART) sum_apart16<S>(p, rank, taddr + col, peers, slice_col, per_block, row, v);
-        else sum_cluster16<S>(taddr + col, peers, slice_col, p.rows_pad, row, v);
-    };
-    bool arrived = S == 1;
-    auto last_read = [&](bool last) {
-        if (!arrived && last) { cluster_arrive(); arrived = true; }
+        if (APART) sum_apart16<S>(p, rank, taddr + col, recv, region, slice_col, per_block, row, v);
+        else sum_cluster16<S>(taddr + col, recv, region, slice_col, p.rows_pad, row, v);
     };
     if (ok && live) {
         for (int u = item0 + hf; u < item1; u += 2) {
@@ -407,7 +402,6 @@ gemm_rows_kernel(const GemmArgs g, const RowsPlan p, const __grid_constant__ CUt
                 const int col = nt * p.TN + u * 16;
                 float v[16];
                 sum16(u * 16, sc, v);
-                last_read(u + 2 >= item1);
                 if (valid && col < g.n[0]) {
                     if (u != item0 + hf) { res[0] = __ldcg(res_row + (col >> 3)); res[1] = __ldcg(res_row + (col >> 3) + 1); }
                     const uint32_t rw[8] = {res[0].x, res[0].y, res[0].z, res[0].w, res[1].x, res[1].y, res[1].z, res[1].w};
@@ -443,7 +437,6 @@ gemm_rows_kernel(const GemmArgs g, const RowsPlan p, const __grid_constant__ CUt
                 float lo[16], hi[16];
                 sum16((u >> 1) * 64 + (u & 1) * 16, sc, lo);
                 sum16((u >> 1) * 64 + (u & 1) * 16 + 32, sc + 16, hi);
-                last_read(u + 2 >= item1);
                 if (valid && grp < p.groups) {
                     rope_qkv<16>(g, seg, col, lo, hi, c, sn);
                     item_rope(u + 2);
@@ -453,7 +446,6 @@ gemm_rows_kernel(const GemmArgs g, const RowsPlan p, const __grid_constant__ CUt
         }
     }
     __syncwarp();
-    last_read(true);
     // ---------------- teardown ----------------
     tc_fence_before();
     __syncthreads();
@@ -470,7 +462,7 @@ gemm_rows_kernel(const GemmArgs g, const RowsPlan p, const __grid_constant__ CUt
         __syncthreads();
     }
     __syncwarp();
-    if (S > 1) cluster_wait();                                // no CTA leaves while a peer may still read its staging area
+    if (S > 1) cluster_wait();                                // no CTA leaves before its peers have sent what they will send
     if (warp == 1) {
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(p.tmem_cols) : "memory");
@@ -480,10 +472,12 @@ gemm_rows_kernel(const GemmArgs g, const RowsPlan p, const __grid_constant__ CUt
 // ---- host side ------------------------------------------------------------------------------
 namespace {
 
+constexpr int kSmemBytes = 226 * 1024;
+
 template <int S, int EPI, bool APART>
 cudaError_t launch_rows(const GemmArgs& g, const RowsPlan& p, const CUtensorMap& a, const CUtensorMap* b, cudaStream_t stream) {
     static const cudaError_t attr =
-        cudaFuncSetAttribute(gemm_rows_kernel<S, EPI, APART>, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024);
+        cudaFuncSetAttribute(gemm_rows_kernel<S, EPI, APART>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
     if (attr != cudaSuccess) return attr;
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(p.n_tiles * S);
@@ -505,7 +499,7 @@ template <int S>
 int resident_clusters() {
     static const int n = [] {
         if (S == 1) return sm_count();
-        cudaFuncSetAttribute(gemm_rows_kernel<S, kEpiResidual, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024);
+        cudaFuncSetAttribute(gemm_rows_kernel<S, kEpiResidual, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
         cudaLaunchConfig_t cfg{};
         cfg.gridDim = dim3(sm_count() / S * S);
         cfg.blockDim = dim3(RW_THREADS);
@@ -575,7 +569,12 @@ bool plan_rows(const GemmArgs& g, RowsPlan& best) {
             best.groups = n_total / 64;
             // the MMA reads 128 rows of A whatever M is: the last panel's read may run past the ring
             const int ring = std::max(stages * CP * panel, (stages - 1) * CP * panel + (CP - 1) * rows_pad * 128 + 128 * 128);
-            best.smem_bytes = std::max(ring, (S - 1) * region) + 1024;
+            // The peers' parts arrive behind the ring, or where they do not fit there (more than 112 rows of tiles of 128 columns over
+            // four CTAs) in it, once everyone is done with it: a ring of two stages less made the down projection of 124
+            // rows of 18 944 columns 30.5 -> 33.1 us.
+            best.recv_late = S > 1 && ring + (S - 1) * region + 1024 > kSmemBytes;
+            best.recv_off = best.recv_late ? 0 : ring;
+            best.smem_bytes = (best.recv_late ? std::max(ring, (S - 1) * region) : ring + (S - 1) * region) + 1024;
         }
     }
     return t_best < 1e29;

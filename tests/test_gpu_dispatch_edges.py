@@ -108,7 +108,8 @@ def test_topk_score_distributions(L):
             assert np.array_equal(out[0].cpu().numpy(), orc.select_topk(s, K)[0]), (name, L, K)
 
 
-# K is cut between 1, 2 or 4 CTAs of a cluster depending on rows and shape; a ring stage takes 1 to 8 panels of K
+# K is cut between 1, 2 or 4 CTAs of a cluster depending on rows and shape; a ring stage takes 1 to 8 panels of K; up to 112 rows the
+# cluster's parts arrive beside the ring, above in it (tiles of 128 columns over four CTAs)
 DEEP128 = wl.LayerShape(3584, 4, 1, 128, 8192, 1e-6, True, 1e6, "deep-d128")
 ODD64 = wl.LayerShape(1024, 6, 2, 64, 640, 1e-5, False, 5e5, "odd-d64")
 DEEP64 = wl.LayerShape(2048, 12, 4, 64, 256, 1e-5, False, 5e5, "deep-d64")
@@ -116,7 +117,7 @@ DEEP64 = wl.LayerShape(2048, 12, 4, 64, 256, 1e-5, False, 5e5, "deep-d64")
 WIDE_FFN = wl.LayerShape(256, 2, 1, 128, 19200, 1e-5, False, 5e5, "wide-ffn")
 
 
-@pytest.mark.parametrize("shape,rows", [(DEEP128, n) for n in (1, 8, 33, 103, 128, 129)] + [(ODD64, n) for n in (1, 7, 9, 64, 127)]
+@pytest.mark.parametrize("shape,rows", [(DEEP128, n) for n in (1, 8, 33, 103, 112, 113, 128, 129)] + [(ODD64, n) for n in (1, 7, 9, 64, 127)]
                          + [(DEEP64, n) for n in (7, 127)] + [(WIDE_FFN, n) for n in (1, 40, 128)])
 def test_few_row_projections(shape, rows):
     lay = wl.make_layout(1, 3, 160, 8, 8, 8, "none")
