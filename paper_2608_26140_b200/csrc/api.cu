@@ -200,7 +200,7 @@ acache_status run_recompute(acache_ctx* c, const acache_layer_weights* w, const 
     if (!x_is_compact && r->token_ids) { g.prep.token_ids = r->token_ids; g.prep.table_rows = r->n_embed; }
     // x in page-locked host memory: the gathered rows are kept on the device for the residual of the output projection
     void* x_rows = (c->stash_rows && !r->token_ids) ? c->stash_rows : nullptr;
-    g.prep.raw_out = x_rows;
+    g.prep.raw_out = x_rows; g.prep.x_far = c->stash_rows != nullptr;
     g.b[0] = w->wq; g.b[1] = w->wk; g.b[2] = w->wv;
     g.n[0] = qd; g.n[1] = kvd; g.n[2] = kvd;
     g.epilogue = kEpiQKV;
@@ -608,7 +608,7 @@ acache_status layer_step_impl(acache_ctx* ctx, const acache_layer_weights* w, co
                 void* xnm = wsp<void>(ctx, ctx->o_xn_mask);
                 GemmArgs g{};
                 g.a = xnm; g.M = req->batch * req->n_masked; g.K = d.hidden;
-                g.prep.enabled = 1; g.prep.x = x; g.prep.x_is_compact = x_is_compact;
+                g.prep.enabled = 1; g.prep.x = x; g.prep.x_is_compact = x_is_compact; g.prep.x_far = ctx->stash_rows != nullptr;
                 if (x_is_compact) {
                     // the masked rows are among the extra rows of the compact input: find where
                     int32_t* cidx = wsp<int32_t>(ctx, ctx->o_mcidx);

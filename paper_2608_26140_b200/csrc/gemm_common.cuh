@@ -176,7 +176,7 @@ __device__ __forceinline__ void qkv_unit(const GemmArgs& g, int u128, int& seg, 
 
 // Where row `row` of the A operand comes from (element offset inside rp.x); `writer` (one thread per
 // row) records the row's position and source for the later kernels and raises the bad-index flag.
-__device__ __forceinline__ int64_t prep_row_source(const GemmArgs& g, int row, bool writer) {
+__device__ __forceinline__ int64_t prep_row_source(const GemmArgs& g, int row, bool writer, int* position = nullptr) {
     const RowPrep& rp = g.prep;
     const int rows_per_req = rp.k + rp.e;
     int64_t src = (int64_t)row * g.K;
@@ -207,6 +207,7 @@ __device__ __forceinline__ int64_t prep_row_source(const GemmArgs& g, int row, b
             const int ci = rp.compact_idx[row];
             src = ((int64_t)b * rp.compact_rows + (ci < 0 ? 0 : ci)) * g.K;
         }
+        if (position) *position = pos;
         if (writer) {
             rp.row_pos[row] = pos;
             rp.row_src[row] = src;

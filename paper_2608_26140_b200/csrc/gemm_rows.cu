@@ -49,6 +49,7 @@ struct RowsPlan {
     int stages, stage_bytes;
     int tmem_cols;
     int groups;               // q/k/v: groups of 32 rotary pairs over all segments
+    int own_rows;             // every CTA prepares all rows itself, straight into its ring (own_row_prep)
     int recv_off, recv_late;  // where the peers' partial accumulators arrive, from the ring's start on; 1: in the ring itself
     int smem_bytes;
 };
@@ -182,18 +183,69 @@ __device__ __forceinline__ void sum_apart16(const RowsPlan& p, int rank, uint32_
     }
 }
 
-// 228 to 252 registers a thread: no CTA of another tensor-memory kernel finds room beside this one.  That matters where calls run on
+// Few rows of narrow models (up to 256 columns, 16 bytes a lane): every CTA gathers and normalises all rows itself and writes
+// them into the ring where the TMA would put them.  The rows are 32 KB at most, from L2, and nobody waits for anybody: prepared
+// once for all behind a grid-wide barrier, a row's way was a store to global memory, the barrier (1.5-2.1 us) and the TMA's load
+// of it (0.8).  Layer-step of 58 rows of 256 columns 53.5 -> 46.2 us.  The sum of a row's squares is the shared preparation's, in its order.
+__device__ __forceinline__ void own_row_prep(const GemmArgs& g, const RowsPlan& p, uint32_t base, int* s_pos) {
+    const RowPrep& rp = g.prep;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nchunk = g.K >> 3;
+    constexpr int NW = RW_THREADS / 32;
+    // warp w takes rows w, w + 8, ..; lane i looks up the place of its i-th
+    int64_t src = 0;
+    const int mine = warp + lane * NW;
+    if (mine < g.M) {
+        int pos = 0;
+        src = prep_row_source(g, mine, blockIdx.x == 0, &pos);
+        s_pos[mine] = pos;
+    }
+    const __nv_bfloat16* x = static_cast<const __nv_bfloat16*>(rp.x);
+    const bool in = lane < nchunk;
+    const uint4 gain = in ? __ldg(static_cast<const uint4*>(rp.gain) + lane) : make_uint4(0u, 0u, 0u, 0u);
+    const uint32_t gw[4] = {gain.x, gain.y, gain.z, gain.w};
+    const int panel = lane >> 3;                              // 64 columns, as eight chunks
+    const uint32_t dst = base + panel / p.CP * p.stage_bytes + panel % p.CP * p.rows_pad * 128;
+    auto at = [&](int row) { return dst + row * 128 + (((lane & 7) ^ (row & 7)) << 4); };
+    // All rows of the warp are asked for at once, each lane's 16 bytes to where its result goes.  Loops rather than registers: the
+    // instructions come from L2 on a first pass (eight rows unrolled took 1.9 us after the loads).
+#pragma unroll 1
+    for (int i = 0; warp + i * NW < g.M; ++i) {
+        const int64_t from = __shfl_sync(0xffffffffu, src, i);
+        if (in) asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(at(warp + i * NW)), "l"(x + from + lane * 8) : "memory");
+    }
+    asm volatile("cp.async.wait_all;" ::: "memory");
+#pragma unroll 2
+    for (int row = warp; row < g.M; row += NW) {
+        uint32_t w[4] = {0u, 0u, 0u, 0u};
+        if (in) asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3]) : "r"(at(row)) : "memory");
+        float ss = 0.f;
+#pragma unroll
+        for (int e = 0; e < 4; ++e) { const float a = bf16_lo(w[e]), b = bf16_hi(w[e]); ss += a * a + b * b; }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
+        const float rstd = rsqrtf(ss / (float)g.K + rp.eps);
+        uint32_t r[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) r[e] = pack_bf16(bf16_lo(w[e]) * rstd * bf16_lo(gw[e]), bf16_hi(w[e]) * rstd * bf16_hi(gw[e]));
+        if (in) asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(at(row)), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]) : "memory");
+    }
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");      // the tensor core reads them
+    __syncthreads();
+}
+
+// 229 to 234 registers a thread: no CTA of another tensor-memory kernel finds room beside this one.  That matters where calls run on
 // two streams: with clusters on both sides, CTAs that wait for one another's tensor memory and cluster peers would wait for ever.
-template <int S, int EPI, bool APART>
-__global__ void __launch_bounds__(RW_THREADS, 1)
-gemm_rows_kernel(const GemmArgs g, const RowsPlan p, const __grid_constant__ CUtensorMap mapA,
-                 const __grid_constant__ CUtensorMap mapB0, const __grid_constant__ CUtensorMap mapB1,
-                 const __grid_constant__ CUtensorMap mapB2) {
+// OWN: own_row_prep instead of the shared preparation, in a kernel of its own (with both in one, calls that take the shared one were
+// 3 % slower, their instructions come from further away).
+template <int S, int EPI, bool APART, bool OWN>
+__device__ __forceinline__ void rows_body(const GemmArgs& g, const RowsPlan& p, const CUtensorMap& mapA, const CUtensorMap& mapB0,
+                                          const CUtensorMap& mapB1, const CUtensorMap& mapB2) {
     extern __shared__ unsigned char smem_raw[];
     __shared__ uint64_t bar_s[2 * RW_MAX_STAGES + 2];
     __shared__ uint32_t tmem_slot;
     __shared__ volatile int abort_s;
     __shared__ float red[RW_THREADS / 32];
+    __shared__ int s_pos[OWN ? 128 : 1];
     const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     volatile int* abort_flag = &abort_s;
     const uint32_t bars = smem_u32(bar_s);
@@ -251,7 +303,7 @@ gemm_rows_kernel(const GemmArgs g, const RowsPlan p, const __grid_constant__ CUt
     int prefilled = 0;
     if (threadIdx.x == 0) {
         for (; prefilled < p.stages && prefilled < n_blk; ++prefilled) {
-            mbar_expect_tx(full_bar(prefilled), p.stage_bytes);
+            mbar_expect_tx(full_bar(prefilled), OWN ? p.stage_bytes - a_bytes : p.stage_bytes);
             load_weights(prefilled, blk0 + prefilled);
         }
     }
@@ -269,14 +321,15 @@ gemm_rows_kernel(const GemmArgs g, const RowsPlan p, const __grid_constant__ CUt
     pdl_wait();
     pdl_launch_dependents();
 
-    if (g.prep.enabled) prep_phase(g, red, abort_flag, p.cta_rows);
+    if constexpr (OWN) own_row_prep(g, p, base, s_pos);
+    else if (g.prep.enabled) prep_phase(g, red, abort_flag, p.cta_rows);
 
     // ---------------- the contraction ----------------
     if (threadIdx.x == 0) {
         bool ok = !*abort_flag;
         int stage = 0;
         uint32_t phase = 0;
-        for (int i = 0; i < n_blk && ok; ++i) {
+        for (int i = 0; i < n_blk && ok && !OWN; ++i) {           // (OWN: the whole of K is in the ring)
             if (prefilled > 0) {
                 --prefilled;              // this stage's weights are already on their way
             } else {
@@ -346,7 +399,7 @@ gemm_rows_kernel(const GemmArgs g, const RowsPlan p, const __grid_constant__ CUt
         if (u < item1 && seg < g.rope_segments) load_rope<16>(g, pos, (col + (u & 1) * 16) & ((g.head_dim >> 1) - 1), c, sn);
     };
     if (EPI == kEpiQKV && valid) {
-        pos = __ldcg(g.row_pos + row);
+        pos = OWN ? s_pos[OWN ? row : 0] : __ldcg(g.row_pos + row);
         item_rope(item0 + hf);
     }
 
@@ -454,7 +507,7 @@ gemm_rows_kernel(const GemmArgs g, const RowsPlan p, const __grid_constant__ CUt
             atomicOr(g.status, kFlagWaitExpired);
             // ring stages whose weights were requested before the dependency wait but whose activation rows never were:
             // send those now, so that each stage's full barrier completes when all of its copies have landed
-            for (int i = 0; i < prefilled; ++i) tma_load_3d(base + i * p.stage_bytes, &mapA, 0, 0, full_bar(i), pol_a);
+            for (int i = 0; i < prefilled && !OWN; ++i) tma_load_3d(base + i * p.stage_bytes, &mapA, 0, 0, full_bar(i), pol_a);
             for (int i = 0; i < prefilled; ++i)
                 for (uint32_t n = 0; n < TC_WAIT_LIMIT && !mbar_try_wait(full_bar(i), 0); ++n) __nanosleep(40);
             for (int i = 0; i < 4096; ++i) __nanosleep(64);   // copies of stages that were complete when a role gave up
@@ -469,15 +522,33 @@ gemm_rows_kernel(const GemmArgs g, const RowsPlan p, const __grid_constant__ CUt
     }
 }
 
+template <int S, int EPI, bool APART>
+__global__ void __launch_bounds__(RW_THREADS, 1)
+gemm_rows_kernel(const GemmArgs g, const RowsPlan p, const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB0,
+                 const __grid_constant__ CUtensorMap mapB1, const __grid_constant__ CUtensorMap mapB2) {
+    rows_body<S, EPI, APART, false>(g, p, mapA, mapB0, mapB1, mapB2);
+}
+namespace own_rows {
+template <int S, int EPI, bool APART>
+__global__ void __launch_bounds__(RW_THREADS, 1)
+gemm_rows_kernel(const GemmArgs g, const RowsPlan p, const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB0,
+                 const __grid_constant__ CUtensorMap mapB1, const __grid_constant__ CUtensorMap mapB2) {
+    rows_body<S, EPI, APART, true>(g, p, mapA, mapB0, mapB1, mapB2);
+}
+}  // namespace own_rows
+
 // ---- host side ------------------------------------------------------------------------------
 namespace {
 
 constexpr int kSmemBytes = 226 * 1024;
 
-template <int S, int EPI, bool APART>
+template <int S, int EPI, bool APART, bool OWN = false>
 cudaError_t launch_rows(const GemmArgs& g, const RowsPlan& p, const CUtensorMap& a, const CUtensorMap* b, cudaStream_t stream) {
-    static const cudaError_t attr =
-        cudaFuncSetAttribute(gemm_rows_kernel<S, EPI, APART>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
+    const auto kernel = [] {
+        if constexpr (OWN) return own_rows::gemm_rows_kernel<S, EPI, APART>;
+        else return gemm_rows_kernel<S, EPI, APART>;
+    }();
+    static const cudaError_t attr = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
     if (attr != cudaSuccess) return attr;
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(p.n_tiles * S);
@@ -491,7 +562,7 @@ cudaError_t launch_rows(const GemmArgs& g, const RowsPlan& p, const CUtensorMap&
     at[1].val.clusterDim.x = S; at[1].val.clusterDim.y = 1; at[1].val.clusterDim.z = 1;
     cfg.attrs = at;
     cfg.numAttrs = S > 1 ? 2 : 1;
-    return cudaLaunchKernelEx(&cfg, gemm_rows_kernel<S, EPI, APART>, g, p, a, b[0], b[1], b[2]);
+    return cudaLaunchKernelEx(&cfg, kernel, g, p, a, b[0], b[1], b[2]);
 }
 
 // Clusters of S CTAs that are resident at once with one CTA per SM (the SM counts of the GPCs are not multiples of S).
@@ -564,6 +635,11 @@ bool plan_rows(const GemmArgs& g, RowsPlan& best) {
             best.mma_count = CP == 1 ? 1 : best.n_units;
             best.stages = stages; best.stage_bytes = CP * panel;
             best.KB = KB; best.apart = apart;
+            // Own rows up to eight a warp, where the whole of K is in the ring, and not from host memory (decode pass over 4 layers of
+            // 256 columns, us, shared preparation | own: 16 rows 140 | 116, 32 142 | 120, 64 149 | 136; with both in one kernel, 78
+            // 151 | 151, 96 153 | 157, 128 166 | 172).  The self-test of the grid barrier wants the barrier.
+            best.own_rows = apart && S == 1 && g.prep.enabled && !g.prep.x_far && !g.debug_expire && g.K <= 256 && g.M <= 64 &&
+                            stages == my_blocks && KB % CP == 0;
             best.cta_rows = apart && g.K > 256 ? general_iterations : n_tiles * S;
             best.tmem_cols = accs * TN <= 32 ? 32 : accs * TN <= 64 ? 64 : accs * TN <= 128 ? 128 : 256;
             best.groups = n_total / 64;
@@ -602,6 +678,8 @@ int launch_gemm_rows(const GemmArgs& g, cudaStream_t stream) {
     auto launch = [&](auto epi, auto apart) {
         constexpr int EPI = decltype(epi)::value;
         constexpr bool APART = decltype(apart)::value;
+        if constexpr (APART && EPI != kEpiResidual)
+            if (p.own_rows) return launch_rows<1, EPI, APART, true>(g, p, map_a, map_b, stream);
         if constexpr (EPI == kEpiSwiGLU || (APART && EPI == kEpiResidual)) return launch_rows<1, EPI, APART>(g, p, map_a, map_b, stream);
         else if constexpr (APART)
             return p.S == 1 ? launch_rows<1, EPI, APART>(g, p, map_a, map_b, stream) : launch_rows<2, EPI, APART>(g, p, map_a, map_b, stream);

@@ -116,6 +116,7 @@ struct RowPrep {
     int affix_start, affix_len, ctx_len;
     const void* gain;
     float eps;
+    int x_far;                // x lies in host memory: every row is to be read once
     void* raw_out;            // optional bf16 [M, K]: the gathered rows as read (x far away, e.g. in host memory: read it once)
     int32_t* row_pos;
     int64_t* row_src;
