@@ -115,14 +115,13 @@ ODD64 = wl.LayerShape(1024, 6, 2, 64, 640, 1e-5, False, 5e5, "odd-d64")
 DEEP64 = wl.LayerShape(2048, 12, 4, 64, 256, 1e-5, False, 5e5, "deep-d64")
 # gate/up of more 256-column tiles than SMs: the general one-SM kernel, whole and cut tiles
 WIDE_FFN = wl.LayerShape(256, 2, 1, 128, 19200, 1e-5, False, 5e5, "wide-ffn")
-# rows of up to 256 columns: every CTA prepares them itself up to 64 rows; three K blocks fill no stage of two
+# rows of up to 256 columns: every CTA prepares them itself up to 64 rows
 NARROW128 = wl.LayerShape(128, 2, 2, 64, 384, 1e-6, True, 1e6, "narrow-128")
-NARROW192 = wl.LayerShape(192, 3, 1, 64, 256, 1e-5, False, 5e5, "narrow-192")
 
 
 @pytest.mark.parametrize("shape,rows", [(DEEP128, n) for n in (1, 8, 33, 103, 112, 113, 128, 129)] + [(ODD64, n) for n in (1, 7, 9, 64, 127)]
                          + [(DEEP64, n) for n in (7, 127)] + [(WIDE_FFN, n) for n in (1, 40, 64, 65, 128)]
-                         + [(NARROW128, n) for n in (1, 9, 63, 64, 65)] + [(NARROW192, n) for n in (8, 64)])
+                         + [(NARROW128, n) for n in (1, 9, 63, 64, 65)])
 def test_few_row_projections(shape, rows):
     lay = wl.make_layout(1, 3, 160, 8, 8, 8, "none")
     case = wl.make_case(shape, lay, 0.0, cfg_id=73, weights=cached_weights(shape, 73))
