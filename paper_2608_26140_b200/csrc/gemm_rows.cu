@@ -183,6 +183,25 @@ __device__ __forceinline__ void sum_apart16(const RowsPlan& p, int rank, uint32_
     }
 }
 
+// The shared preparation of the usual case (a CTA per row, a row of up to three 16-byte pieces a thread) and, out of the way of its
+// instructions, the rest: a launch runs most of its instructions once, from L2, and waits for them.  With all of it inline the
+// kernels had 228-252 registers, now 52-212 (layer-step of 103 rows 142.6 -> 139.1 us, decode pass of 32 rows over 4 layers 638 -> 631).
+__device__ __forceinline__ void prep_phase_short(const GemmArgs& g, float* red, volatile int* abort_flag) {
+    const RowPrep& rp = g.prep;
+    for (int row = blockIdx.x; row < g.M; row += gridDim.x) {
+        const int64_t src = prep_row_source(g, row, threadIdx.x == 0);
+        rmsnorm_row_short(reinterpret_cast<const uint4*>(static_cast<const __nv_bfloat16*>(rp.x) + src), static_cast<const uint4*>(rp.gain),
+                          reinterpret_cast<uint4*>(static_cast<__nv_bfloat16*>(const_cast<void*>(g.a)) + (int64_t)row * g.K), g.K, rp.eps, red,
+                          rp.raw_out ? reinterpret_cast<uint4*>(static_cast<__nv_bfloat16*>(rp.raw_out) + (int64_t)row * g.K) : nullptr);
+    }
+    asm volatile("fence.proxy.async;" ::: "memory");   // the rows are read back through TMA
+    grid_barrier(g.grid_bar, abort_flag, g.debug_expire != 0);
+    asm volatile("fence.proxy.async;" ::: "memory");
+}
+__device__ __noinline__ void prep_phase_long(const GemmArgs& g, float* red, volatile int* abort_flag, int cta_rows) {
+    prep_phase(g, red, abort_flag, cta_rows);
+}
+
 // Few rows of narrow models (up to 256 columns, 16 bytes a lane): every CTA gathers and normalises all rows itself and writes
 // them into the ring where the TMA would put them.  The rows are 32 KB at most, from L2, and nobody waits for anybody: prepared
 // once for all behind a grid-wide barrier, a row's way was a store to global memory, the barrier (1.5-2.1 us) and the TMA's load
@@ -233,8 +252,6 @@ __device__ __forceinline__ void own_row_prep(const GemmArgs& g, const RowsPlan& 
     __syncthreads();
 }
 
-// 229 to 234 registers a thread: no CTA of another tensor-memory kernel finds room beside this one.  That matters where calls run on
-// two streams: with clusters on both sides, CTAs that wait for one another's tensor memory and cluster peers would wait for ever.
 // OWN: own_row_prep instead of the shared preparation, in a kernel of its own (with both in one, calls that take the shared one were
 // 3 % slower, their instructions come from further away).
 template <int S, int EPI, bool APART, bool OWN>
@@ -322,7 +339,11 @@ __device__ __forceinline__ void rows_body(const GemmArgs& g, const RowsPlan& p, 
     pdl_launch_dependents();
 
     if constexpr (OWN) own_row_prep(g, p, base, s_pos);
-    else if (g.prep.enabled) prep_phase(g, red, abort_flag, p.cta_rows);
+    else if (EPI != kEpiResidual && g.prep.enabled) {
+        if constexpr (APART) prep_phase(g, red, abort_flag, p.cta_rows);     // (few tiles: mostly the long way, 3-5 % slower as a call)
+        else if (g.M <= p.cta_rows && g.K <= 3 * RW_THREADS * 8) prep_phase_short(g, red, abort_flag);
+        else prep_phase_long(g, red, abort_flag, p.cta_rows);
+    }
 
     // ---------------- the contraction ----------------
     if (threadIdx.x == 0) {
@@ -524,14 +545,14 @@ __device__ __forceinline__ void rows_body(const GemmArgs& g, const RowsPlan& p, 
 
 template <int S, int EPI, bool APART>
 __global__ void __launch_bounds__(RW_THREADS, 1)
-gemm_rows_kernel(const GemmArgs g, const RowsPlan p, const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB0,
+gemm_rows_kernel(const __grid_constant__ GemmArgs g, const __grid_constant__ RowsPlan p, const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB0,
                  const __grid_constant__ CUtensorMap mapB1, const __grid_constant__ CUtensorMap mapB2) {
     rows_body<S, EPI, APART, false>(g, p, mapA, mapB0, mapB1, mapB2);
 }
 namespace own_rows {
 template <int S, int EPI, bool APART>
 __global__ void __launch_bounds__(RW_THREADS, 1)
-gemm_rows_kernel(const GemmArgs g, const RowsPlan p, const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB0,
+gemm_rows_kernel(const __grid_constant__ GemmArgs g, const __grid_constant__ RowsPlan p, const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB0,
                  const __grid_constant__ CUtensorMap mapB1, const __grid_constant__ CUtensorMap mapB2) {
     rows_body<S, EPI, APART, true>(g, p, mapA, mapB0, mapB1, mapB2);
 }
@@ -541,6 +562,10 @@ gemm_rows_kernel(const GemmArgs g, const RowsPlan p, const __grid_constant__ CUt
 namespace {
 
 constexpr int kSmemBytes = 226 * 1024;
+// With this much shared memory no CTA of another tensor-memory kernel with clusters or a grid barrier (76 KB at least) finds room
+// beside this one.  That matters where calls run on two streams: with clusters on both sides, CTAs that wait for one another's
+// tensor memory and cluster peers would wait for ever.  (CTAs that prepare their own rows wait for no other of their launch.)
+constexpr int kAloneBytes = 160 * 1024;
 
 template <int S, int EPI, bool APART, bool OWN = false>
 cudaError_t launch_rows(const GemmArgs& g, const RowsPlan& p, const CUtensorMap& a, const CUtensorMap* b, cudaStream_t stream) {
@@ -651,6 +676,7 @@ bool plan_rows(const GemmArgs& g, RowsPlan& best) {
             best.recv_late = S > 1 && ring + (S - 1) * region + 1024 > kSmemBytes;
             best.recv_off = best.recv_late ? 0 : ring;
             best.smem_bytes = (best.recv_late ? std::max(ring, (S - 1) * region) : ring + (S - 1) * region) + 1024;
+            if (!best.own_rows) best.smem_bytes = std::max(best.smem_bytes, kAloneBytes);
         }
     }
     return t_best < 1e29;

@@ -32,54 +32,60 @@ __device__ __forceinline__ float block_sum(float v, float* red) {
     return t;
 }
 
-// out = bf16(x * rsqrt(mean(x^2) + eps) * g) for one row of `hidden` bf16 values; all threads
-// of the block take part.  raw (optional): the row as it was read is stored there too.
+// out = bf16(x * rsqrt(mean(x^2) + eps) * g) for one row of `hidden` bf16 values, at most three 16-byte pieces per thread; all
+// threads of the block take part.  raw (optional): the row as it was read is stored there too.
+__device__ __forceinline__ void rmsnorm_row_short(const uint4* __restrict__ xr, const uint4* __restrict__ g, uint4* __restrict__ out,
+                                                  int hidden, float eps, float* red, uint4* __restrict__ raw) {
+    const int nchunk = hidden >> 3;
+    // one pass, the row stays in registers, and the gain is
+    // requested before the block-wide sum so that it arrives meanwhile
+    uint4 u[3], gg[3];
+    float ss1 = 0.f;
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        const int c = threadIdx.x + i * blockDim.x;
+        u[i] = c < nchunk ? __ldcg(xr + c) : make_uint4(0u, 0u, 0u, 0u);
+    }
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        const int c = threadIdx.x + i * blockDim.x;
+        gg[i] = c < nchunk ? g[c] : make_uint4(0u, 0u, 0u, 0u);
+    }
+    if (raw) {
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+            const int c = threadIdx.x + i * blockDim.x;
+            if (c < nchunk) raw[c] = u[i];
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        const uint32_t w[4] = {u[i].x, u[i].y, u[i].z, u[i].w};
+#pragma unroll
+        for (int e = 0; e < 4; ++e) { const float a = bf16_lo(w[e]), b = bf16_hi(w[e]); ss1 += a * a + b * b; }
+    }
+    const float rstd1 = rsqrtf(block_sum(ss1, red) / (float)hidden + eps);
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        const int c = threadIdx.x + i * blockDim.x;
+        if (c < nchunk) {
+            const uint32_t w[4] = {u[i].x, u[i].y, u[i].z, u[i].w};
+            const uint32_t gw[4] = {gg[i].x, gg[i].y, gg[i].z, gg[i].w};
+            uint32_t r[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e)
+                r[e] = pack_bf16(bf16_lo(w[e]) * rstd1 * bf16_lo(gw[e]), bf16_hi(w[e]) * rstd1 * bf16_hi(gw[e]));
+            out[c] = make_uint4(r[0], r[1], r[2], r[3]);
+        }
+    }
+}
+// The same for rows of any length.
 __device__ __forceinline__ void rmsnorm_row(const uint4* __restrict__ xr, const uint4* __restrict__ g,
                                             uint4* __restrict__ out, int hidden, float eps, float* red,
                                             uint4* __restrict__ raw = nullptr) {
     const int nchunk = hidden >> 3;
     if (nchunk <= 3 * (int)blockDim.x) {
-        // the row fits in three 16-byte pieces per thread: one pass, the row stays in registers, and the gain is
-        // requested before the block-wide sum so that it arrives meanwhile
-        uint4 u[3], gg[3];
-        float ss1 = 0.f;
-#pragma unroll
-        for (int i = 0; i < 3; ++i) {
-            const int c = threadIdx.x + i * blockDim.x;
-            u[i] = c < nchunk ? __ldcg(xr + c) : make_uint4(0u, 0u, 0u, 0u);
-        }
-#pragma unroll
-        for (int i = 0; i < 3; ++i) {
-            const int c = threadIdx.x + i * blockDim.x;
-            gg[i] = c < nchunk ? g[c] : make_uint4(0u, 0u, 0u, 0u);
-        }
-        if (raw) {
-#pragma unroll
-            for (int i = 0; i < 3; ++i) {
-                const int c = threadIdx.x + i * blockDim.x;
-                if (c < nchunk) raw[c] = u[i];
-            }
-        }
-#pragma unroll
-        for (int i = 0; i < 3; ++i) {
-            const uint32_t w[4] = {u[i].x, u[i].y, u[i].z, u[i].w};
-#pragma unroll
-            for (int e = 0; e < 4; ++e) { const float a = bf16_lo(w[e]), b = bf16_hi(w[e]); ss1 += a * a + b * b; }
-        }
-        const float rstd1 = rsqrtf(block_sum(ss1, red) / (float)hidden + eps);
-#pragma unroll
-        for (int i = 0; i < 3; ++i) {
-            const int c = threadIdx.x + i * blockDim.x;
-            if (c < nchunk) {
-                const uint32_t w[4] = {u[i].x, u[i].y, u[i].z, u[i].w};
-                const uint32_t gw[4] = {gg[i].x, gg[i].y, gg[i].z, gg[i].w};
-                uint32_t r[4];
-#pragma unroll
-                for (int e = 0; e < 4; ++e)
-                    r[e] = pack_bf16(bf16_lo(w[e]) * rstd1 * bf16_lo(gw[e]), bf16_hi(w[e]) * rstd1 * bf16_hi(gw[e]));
-                out[c] = make_uint4(r[0], r[1], r[2], r[3]);
-            }
-        }
+        rmsnorm_row_short(xr, g, out, hidden, eps, red, raw);
         return;
     }
     float ss = 0.f;
