@@ -254,23 +254,22 @@ __global__ void __launch_bounds__(128) score_colsum_kernel(ScoreArgs a, int n_sp
 
 // ---- both passes in one launch: short affixes, one request or a few ----------------------------------
 // With at most 1024 affix keys a head's work is cut over a cluster of eight CTAs, 64 or 128 keys each: every CTA takes
-// the softmax statistics of all masked rows over its own keys and sends them to all eight (asynchronous stores into their shared
-// memory, counted by an mbarrier), and each CTA then takes the column sums of its own keys from the tiles it already holds.  One launch
+// the softmax statistics of all masked rows over its own keys and stores them into the shared memory of all eight, and behind a cluster
+// barrier each CTA takes the column sums of its own keys from the tiles it already holds.  One launch
 // instead of two, and the statistics never leave the cluster.  Only when the normaliser runs over the affix
 // keys themselves and the grid fits the SMs in one wave.
+// The barrier is the hardware's, which cannot run out: a bounded wait would have nobody to report to in the scoring without a context,
+// and a CTA that gave up would leave while its peers still store into its shared memory.
 constexpr int kSmallCluster = 8;
 
 template <int D, int kSmallTiles>          // key tiles per CTA: 1 (up to 512 affix keys) or 2 (up to 1024)
 __global__ void __cluster_dims__(kSmallCluster, 1, 1) __launch_bounds__(128) score_small_kernel(ScoreArgs a, float scale_log2e) {
     extern __shared__ __align__(128) unsigned char smem[];
-    __shared__ uint64_t recv_bar;
-    __shared__ volatile int abort_s;
     constexpr int TILE = 64 * D * 2;
     const uint32_t sQ = smem_u32(smem), sK0 = sQ + TILE;
     float2* s_stat = reinterpret_cast<float2*>(smem + (1 + kSmallTiles) * TILE);   // [CTA of the cluster][tile][64 rows] (max, den)
     float* s_max = reinterpret_cast<float*>(s_stat + kSmallCluster * kSmallTiles * 64);
     float* s_inv = s_max + 64;
-    const uint32_t bar = smem_u32(&recv_bar);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int rank = blockIdx.x % kSmallCluster, h = blockIdx.x / kSmallCluster, b = blockIdx.y;
     const int kvh = h / (a.n_heads / a.n_kv_heads);
@@ -286,14 +285,7 @@ __global__ void __cluster_dims__(kSmallCluster, 1, 1) __launch_bounds__(128) sco
             load_tile64<D>(sK0 + t * TILE, kbase + (int64_t)t * 64 * kstride, kstride, min(64, nkeys - t * 64), tid, 128);
     };
     const int groups = (a.m + 15) / 16;
-    if (tid == 0) {
-        mbar_init(bar, 1);
-        abort_s = 0;
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        mbar_expect_tx(bar, kSmallCluster * kSmallTiles * groups * 16 * 8);
-    }
-    __syncwarp();
-    cluster_arrive_relaxed();            // the others may send once all have come this far
+    cluster_arrive_relaxed();            // the others may store once all have started
     if (a.early_k) load_keys();          // see ScoreArgs::early_k
     pdl_wait();
     pdl_launch_dependents();
@@ -346,15 +338,12 @@ __global__ void __cluster_dims__(kSmallCluster, 1, 1) __launch_bounds__(128) sco
                 const uint32_t at = smem_u32(s_stat + (rank * kSmallTiles + t) * 64 + rg * 16 + (lane >> 2) + r * 8);
 #pragma unroll
                 for (int c = 0; c < kSmallCluster; ++c)
-                    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v2.f32 [%0], {%1, %2}, [%3];"
-                                 ::"r"(mapa_u32(at, c)), "f"(mx[r]), "f"(den[r]), "r"(mapa_u32(bar, c))
-                                 : "memory");
+                    asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(mapa_u32(at, c)), "f"(mx[r]), "f"(den[r]) : "memory");
             }
         }
     }
-    // (with the statistics read from the peers behind a cluster barrier, and another one at the end, the layer-step of 103 rows took
-    // 144.2 us, now 143.8; 58 rows of 256 columns 53.3, now 53.1)
-    if (!mbar_poll_cluster(bar, 0, &abort_s) && a.status) atomicOr(a.status, kFlagWaitExpired);
+    __syncwarp();
+    cluster_sync_all();                  // after it nobody touches a peer's shared memory: a CTA may leave when it is done
     if (tid < groups * 16) {
         float ms[kSmallCluster * kSmallTiles], ds[kSmallCluster * kSmallTiles];
 #pragma unroll

@@ -88,3 +88,10 @@ def test_k_from_ratio_host_function(lib):
     for L in (1, 7, 100, 512, 8192):
         for r in (0.0, 0.05, 0.1, 0.2, 0.35, 0.5, 1.0):
             assert f(L, r) == orc.k_from_ratio(L, r)
+
+
+def test_kernels_without_a_status_word_wait_at_hardware_barriers_only():
+    """acache_score_anchors_static launches the kernels of score.cu with nobody to tell that a bounded wait ran out, and a CTA
+    that left after one could still be stored into by its cluster: they hold no such wait."""
+    src = open(os.path.join(ROOT, "paper_2608_26140_b200", "csrc", "score.cu")).read()
+    assert not re.findall(r"\bmbar_\w+\s*\(|\babort_\w+|kFlagWaitExpired|st\.async", src)
