@@ -38,6 +38,7 @@ constexpr int AT_TILE = 128 * 128 * 2;           // 32 KB: a [128 x 128] bf16 ti
 constexpr int AT_PANEL = 128 * 64 * 2;           // 16 KB
 constexpr int AT_SLACK = 256;                    // the dynamic window starts 1024-aligned in practice; checked at run time
 constexpr int AT_SMEM = 5 * AT_TILE + AT_SLACK + 256;   // Q, K x2, V x2 (P lives in tensor memory)
+static_assert(AT_SMEM >= kAloneBytes);
 constexpr float kRescaleGap = 8.f;               // log2 units
 
 __device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map, int c0, int c1, int c2, uint32_t bar,

@@ -562,11 +562,6 @@ gemm_rows_kernel(const __grid_constant__ GemmArgs g, const __grid_constant__ Row
 namespace {
 
 constexpr int kSmemBytes = 226 * 1024;
-// With this much shared memory no CTA of another tensor-memory kernel with clusters or a grid barrier (76 KB at least) finds room
-// beside this one.  That matters where calls run on two streams: with clusters on both sides, CTAs that wait for one another's
-// tensor memory and cluster peers would wait for ever.  (CTAs that prepare their own rows wait for no other of their launch.)
-constexpr int kAloneBytes = 160 * 1024;
-
 template <int S, int EPI, bool APART, bool OWN = false>
 cudaError_t launch_rows(const GemmArgs& g, const RowsPlan& p, const CUtensorMap& a, const CUtensorMap* b, cudaStream_t stream) {
     const auto kernel = [] {
@@ -676,7 +671,7 @@ bool plan_rows(const GemmArgs& g, RowsPlan& best) {
             best.recv_late = S > 1 && ring + (S - 1) * region + 1024 > kSmemBytes;
             best.recv_off = best.recv_late ? 0 : ring;
             best.smem_bytes = (best.recv_late ? std::max(ring, (S - 1) * region) : ring + (S - 1) * region) + 1024;
-            if (!best.own_rows) best.smem_bytes = std::max(best.smem_bytes, kAloneBytes);
+            if (!best.own_rows) best.smem_bytes = std::max(best.smem_bytes, kAloneBytes);    // (own rows wait for nobody)
         }
     }
     return t_best < 1e29;

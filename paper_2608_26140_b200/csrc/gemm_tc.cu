@@ -50,6 +50,7 @@ constexpr int TC_HALF_BYTES = 128 * TC_BK * 2;         // 16 KB: one 128-row hal
 constexpr int TC_STAGE_BYTES = TC_A_BYTES + 2 * TC_HALF_BYTES;
 constexpr int TC_THREADS = 192;                        // warp 0: TMA, warp 1: MMA, warps 2-5: drain; all six warps do phase 0
 constexpr int TC_SMEM = TC_STAGES * TC_STAGE_BYTES + 1024 /*alignment slack*/ + 256 /*barriers*/;
+static_assert(TC_SMEM >= kAloneBytes);
 constexpr int TC_SLOT_FLOATS = TC_BM * TC_BN;          // one fp32 partial tile
 
 struct TcPlan {
@@ -592,6 +593,7 @@ constexpr int TC2_THREADS = 320;                                // warp 0: TMA, 
 constexpr int TC2_STAGES = 6;
 constexpr int TC2_STAGE_BYTES = TC_A_BYTES + TC_HALF_BYTES;     // 32 KB per CTA and stage
 constexpr int TC2_SMEM = TC2_STAGES * TC2_STAGE_BYTES + 1024 + 256;
+static_assert(TC2_SMEM >= kAloneBytes);
 
 // Tile order of the two-SM kernel: groups of kTileGroupN weight tiles; inside a group the row
 // pairs are walked with the group's weight tiles innermost.  The ~74 clusters running at any

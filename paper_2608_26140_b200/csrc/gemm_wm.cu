@@ -329,7 +329,7 @@ int launch_wm(const GemmArgs& g, double own_us, int group_n, cudaStream_t stream
     if (!p.NC) return 0;
     p.stage_bytes = WM_W_BYTES + p.NC * 64;
     p.stages = std::min(WM_MAX_STAGES, (WM_SMEM_DYN - 1024 - WM_STAGING) / p.stage_bytes);
-    p.smem_bytes = 1024 + p.stages * p.stage_bytes + WM_STAGING;
+    p.smem_bytes = std::max(kAloneBytes, 1024 + p.stages * p.stage_bytes + WM_STAGING);
     // From four chunks on the next round reads the weights again (16 weight tiles of a group x 4 chunks are a round).  Layer-step, us,
     // kept | not: one chunk (129 rows) 165 | 151, two (300) 213 | 204, three (615) 283 | 281; four (800) 332 | 333, 3584 columns 342 | 345;
     // six and nine (1200) 477 | 480, (1800) 648 | 663.

@@ -354,8 +354,7 @@ constexpr int S1_MAX_TILES = 16;
 // CTA; with two stages three CTAs do, for up to 128 columns: a CTA spends as long after its last tile as it does loading (7000
 // and 8000 cycles for 512 keys).  2048 (head, request) pairs of 512 keys and 32 rows: 102 -> 85 us, and 74 without the cluster
 // barriers of a CTA that has no peers (1000-3500 cycles each, they wait for memory).  Four CTAs with one stage 89.  A CTA
-// that needs all 512 columns asks for S1_SMEM_WIDE so that no second CTA can be resident beside it (a CTA waiting for
-// tensor memory inside a cluster whose peers wait for it at a cluster barrier would never get it).
+// that needs all 512 columns asks for kAloneBytes.
 template <int NP, int STAGES> struct S1 {
     static constexpr int Q_BYTES = 2 * NP * 128;
     static constexpr int RING = STAGES * ST_K_BYTES > 128 * 65 * 4 ? STAGES * ST_K_BYTES : 128 * 65 * 4;
@@ -363,7 +362,10 @@ template <int NP, int STAGES> struct S1 {
     static constexpr int BAR_OFF = TAB_OFF + 2048;
     static constexpr int SMEM = BAR_OFF + 512;              // the window has to start 1024-aligned
 };
-constexpr int S1_SMEM_WIDE = 120 * 1024;
+static_assert(!can_share_sm(kAloneBytes, S1<32, 2>::SMEM) && !can_share_sm(kAloneBytes, S1<32, 3>::SMEM) &&
+              !can_share_sm(kAloneBytes, S1<64, 2>::SMEM), "tensor memory: one of these beside a CTA that needs all of it");
+// the first takes up to 128 columns, the others 256: no third CTA beside two of those
+static_assert(S1<32, 3>::SMEM >= S1<64, 2>::SMEM && !can_share_sm(2 * S1<64, 2>::SMEM + 1024, S1<32, 2>::SMEM));
 
 __device__ __forceinline__ void tc_st32f(uint32_t taddr, const float (&v)[32]) {
     asm volatile(
@@ -668,7 +670,7 @@ int launch_score_tc(const ScoreArgs& a, uint32_t* status, cudaStream_t stream) {
                 static std::once_flag once;
                 std::call_once(once, [] {
                     for (auto k : {score_onepass_tc_kernel<32, 2, 3>, score_onepass_tc_kernel<32, 3, 2>, score_onepass_tc_kernel<64, 2, 2>})
-                        cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, S1_SMEM_WIDE);
+                        cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kAloneBytes);
                 });
                 ScoreTcArgs t1{};
                 t1.row_stats = a.row_stats; t1.head_partial = a.head_partial;
@@ -680,7 +682,7 @@ int launch_score_tc(const ScoreArgs& a, uint32_t* status, cudaStream_t stream) {
                 cudaLaunchConfig_t cfg{};
                 cfg.gridDim = dim3(a.n_heads * csize, a.batch);
                 cfg.blockDim = dim3(S1_THREADS);
-                cfg.dynamicSmemBytes = cols > 256 ? S1_SMEM_WIDE : need;
+                cfg.dynamicSmemBytes = cols > 256 ? kAloneBytes : need;
                 cfg.stream = stream;
                 cudaLaunchAttribute at[2];
                 at[0].id = cudaLaunchAttributeClusterDimension;

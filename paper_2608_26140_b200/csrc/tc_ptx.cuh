@@ -114,6 +114,13 @@ __device__ __forceinline__ bool mbar_poll_cluster(uint32_t bar, uint32_t parity,
     *abort_flag = 1;
     return false;
 }
+// Shared memory decides which CTAs share an SM, and tensor memory (512 columns) has to be enough for all that do: a CTA of a cluster
+// that waits for columns while its peers wait for it, beside one of another stream's launch in the same place, would wait for ever.
+// CTAs that hold tensor memory while they wait for others (a cluster barrier, a grid barrier) therefore either take kAloneBytes or
+// more, or at most 256 columns and enough shared memory to stay off the SM of one that does (and three of them together never need
+// more than there is: asserted where they are defined).  CTAs that wait for nobody may be of any size.
+constexpr int kAloneBytes = 160 * 1024;
+constexpr bool can_share_sm(int a, int b) { return a + b + 2 * 1024 <= 228 * 1024; }       // 1 KB of each CTA is the system's
 // L2 eviction policies: the weights stream through once (evict first); the activation rows
 // every CTA re-reads and the partial tiles the finish phase reads back should stay (evict last).
 __device__ __forceinline__ uint64_t policy_evict_first() {
