@@ -1427,10 +1427,13 @@ int launch_attention_tc(const AttnArgs& a, uint32_t* status, cudaStream_t stream
     std::lock_guard<std::mutex> lock(g_map3_mutex);
     // decode passes over a shared cache: the rows of several requests share one query tile (attention_group_kernel)
     static const bool group_on = [] { const char* e = getenv("ACACHE_ATTN_GROUP"); return !e || atoi(e) != 0; }();
-    // (two requests of up to 64 rows only where one to a tile needs more than one wave: half as many CTAs, each with less than
-    // twice the work: 13 requests of 62 rows, 32 heads, pass over 4 layers 2579 -> 2472 us)
+    // Two requests of up to 64 rows where that saves rounds of CTAs.  A pair takes 1 to 5 % longer than one request, and half as many
+    // rounds are less from two on, except two against two.  One | two to a tile, us, 48 rows, 32 heads, 2048 shared keys and 64 to 500
+    // private rows per request: 7 requests (2 rounds | 1) 71-91 | 46-60, 9 (2 | 2) 73-94 | 75-95, 10 (3 | 2) 102-129 | 77-105,
+    // 13 (3 | 2) 104-134 | 80-108, 19 (5 | 3) 172-218 | 121-161; 4096 shared keys, 9 requests 117 | 122; 28 heads, 9 (2 | 1) 111 | 66.
     const bool grouped = group_on && two_src && shared && a.batch >= 2;
-    const int group = grouped && a.n <= 32 ? 4 : grouped && a.n <= 64 && a.batch * a.n_heads > 148 ? 2 : 1;
+    auto rounds = [&](int requests) { return ((a.batch + requests - 1) / requests * a.n_heads + sm_count() - 1) / sm_count(); };
+    const int group = grouped && a.n <= 32 ? 4 : grouped && a.n <= 64 && rounds(2) < rounds(1) ? 2 : 1;
     CUtensorMap maps[5];
     const CUtensorMap* found[5];
     found[0] = get_map3(a.q, a.n, a.n_heads * 128, a.batch, (int64_t)a.n * a.n_heads * 128, 128 / group);

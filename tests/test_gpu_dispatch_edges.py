@@ -245,6 +245,17 @@ def test_attention_of_grouped_requests(shape, B, pre, L, post, rows, ratio):
         assert_close_bf16(ab.to_host_bits(y[b]), ref["y"], "y")
 
 
+# Two requests of 33 to 64 rows share a tile where that saves rounds of CTAs (on 148 SMs): 2 | 1, 3 | 2, 5 | 3 rounds, but not 1 | 1
+# nor 2 | 2.  Up to 32 rows four always do; more than 64 never.
+def test_which_decode_passes_share_query_tiles():
+    cases = [(5, 48, 1), (9, 48, 0), (9, 33, 0), (9, 64, 0), (10, 48, 1), (13, 64, 1), (19, 33, 1), (4, 48, 0), (4, 32, 1), (9, 32, 1),
+             (2, 7, 1), (10, 65, 0)]
+    launched = launched_kernels([(HEADS32, B, 5, 150, 20, rows, 10) for B, rows, _ in cases], "shared_decode")
+    for (B, rows, grouped), kernels in zip(cases, launched):
+        assert ("attention_group_kernel" in kernels) == bool(grouped), (B, rows, kernels)
+        assert ("attention_tc_kernel<false>" in kernels) != bool(grouped), (B, rows, kernels)
+
+
 # Small projections sum K in the general kernel's order, block by block: a row's bits do not depend on how many rows are in the
 # call, on the tile or on the split over a cluster (140 rows take the two-SM kernel).  Every product is reached with inputs that
 # the other rows of a call do not change: no queries, hence equal weights over equal values, so that the attention's output is
