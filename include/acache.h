@@ -163,7 +163,8 @@ acache_status acache_poll_status(acache_ctx *ctx, acache_stream_t stream, uint32
  * This call makes that happen once, on purpose: the next Q/K/V projection this context launches
  * (acache_recompute_anchors, acache_layer_step, ...) gives the grid-wide barrier that ends its row-preparation
  * phase a target one arrival beyond what its grid can deliver and a short poll limit (about a millisecond),
- * so the wait runs out before any tensor-core work was issued.  The call that contains it still enqueues its
+ * so the wait runs out before any tensor-core work was issued (a projection of so few rows and columns that it
+ * needs no such barrier takes the kernel that has one, this once).  The call that contains it still enqueues its
  * later kernels, whose outputs are then meaningless; acache_poll_status afterwards returns ACACHE_ERR_TIMEOUT
  * and re-arms the barrier, and the next call on the context runs normally.  Nothing faults, traps or spins
  * without a bound. */
