@@ -82,6 +82,17 @@ def shared_decode(shape, B, pre, L, post, n, K):
     return names(ctx, lambda: ctx.recompute_rows_shared(ab.Context.weights(w), req, owned, kv, x, 0, anchors, K, slot_rows, *slots, y))
 
 
+def scoring(shape, B, L, m, shared, norm_full):
+    """score_anchors of m masked rows over L affix keys, 7 rows in front of them"""
+    lay = wl.make_layout(B, 7, L, 20, max(m, 8), m)
+    cache, q = zeros(1 if shared else B, lay.ctx_len, shape.n_kv_heads, shape.head_dim), zeros(B, m, shape.n_heads, shape.head_dim)
+    masked, scores = on_device(lay.masked_pos), torch.zeros((B, L), device="cuda:0")
+    ctx = ab.Context.for_shape(shape, B, lay.ctx_len, L, 1, m, "cuda:0")
+    req = ab.Context.request(B, lay.ctx_len, 7, L, masked, None, None, None)
+    kv = ab.KV(cache.data_ptr(), cache.data_ptr(), 0, lay.ctx_len) if shared else ab.Context.kv(cache, cache)
+    return names(ctx, lambda: ctx.score_anchors(req, q, kv, scores, accumulate=False, norm_full=norm_full))
+
+
 if __name__ == "__main__":
     import os
     import numpy as np

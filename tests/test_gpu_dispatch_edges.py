@@ -183,7 +183,7 @@ def test_attention_reference_moves(T, rows, drop):
 
 
 # many more (query tile, head, request) items than SMs: several per CTA, the last round incomplete; query tiles with empty
-# quarters, and four requests to a tile over a shared cache with a last group of two
+# quarters; and four requests to a tile over a shared cache, an item per CTA, with a last group of two
 HEADS32 = wl.LayerShape(256, 32, 4, 128, 256, 1e-5, False, 5e5, "heads32")
 
 
@@ -210,13 +210,30 @@ def test_attention_items_per_cta(B, T, rows, shared):
         assert_close_bf16(ab.to_host_bits(y[b]), ref["y"], "y")
 
 
-# Two or four requests to a query tile over a shared cache, private rows in rounds behind the shared tiles: one and several rounds,
-# groups that are not full, one CTA and clusters of up to eight (some without a step of their own), an affix that neither starts
-# nor ends with a tile, empty tiles in front of it and behind it
-@pytest.mark.parametrize("shape,B,pre,L,post,rows,ratio", [
-    (HEADS32, 4, 0, 300, 40, 32, 0.3), (HEADS32, 6, 150, 500, 180, 7, 0.5), (HEADS32, 5, 5, 260, 90, 64, 0.2),
-    (MID128, 2, 9, 700, 60, 33, 0.2), (MID128, 3, 300, 200, 300, 20, 0.1), (MID128, 2, 0, 2500, 64, 1, 0.05),
-    (MID128, 7, 130, 1100, 100, 50, 0.35)])
+# Decode passes over a shared cache: groups of four in clusters of 4, 2, 8 and 8 CTAs (some without a step of their own), a pair on
+# one CTA, and one request to a tile in clusters of 8 and 4.  An affix that neither starts nor ends with a tile; one and several
+# private tiles; groups that are not full.
+GROUPED = [(HEADS32, 4, 0, 300, 40, 32, 0.3), (HEADS32, 6, 150, 500, 180, 7, 0.5), (MID128, 3, 300, 200, 300, 20, 0.1),
+           (MID128, 2, 0, 2500, 64, 1, 0.05), (HEADS32, 5, 5, 260, 90, 64, 0.2)]
+APART = [(MID128, 2, 9, 700, 60, 33, 0.2), (MID128, 7, 130, 1100, 100, 50, 0.35)]
+# One CTA per query tile, which leaves out the shared tiles without a key: two in front of the affix, one or more behind it, several
+# private rounds.  Groups of four, two and three of them part-filled; pairs; one request to a tile; two tiles of one request.
+SKIP_GROUPED = [(HEADS32, 12, 300, 300, 150, 20, 0.2), (HEADS32, 9, 290, 200, 140, 31, 0.5), (HEADS32, 6, 300, 260, 290, 50, 0.2),
+                (HEADS32, 5, 270, 270, 150, 33, 0.2)]
+SKIP_ONE_TILE = [(HEADS32, 3, 300, 260, 150, 70, 0.2)]
+SKIP_TWO_TILES = [(HEADS32, 5, 300, 260, 150, 140, 0.2)]
+
+
+# The next test compares results; this one says that the kernel they mean is the one that runs.
+def test_which_kernel_decodes_over_a_shared_cache():
+    for cases, kernel in ((GROUPED + SKIP_GROUPED, "attention_group_kernel"), (APART + SKIP_ONE_TILE, "attention_tc_kernel<false>"),
+                          (SKIP_TWO_TILES, "attention_tc2q_kernel")):
+        asked = [(shape, B, pre, L, post, rows, orc.k_from_ratio(L, ratio)) for shape, B, pre, L, post, rows, ratio in cases]
+        for case, kernels in zip(cases, launched_kernels(asked, "shared_decode")):
+            assert [k for k in kernels.split() if "attention" in k and kernel not in k] == [] and kernel in kernels, (case, kernels)
+
+
+@pytest.mark.parametrize("shape,B,pre,L,post,rows,ratio", GROUPED + APART + SKIP_GROUPED + SKIP_ONE_TILE + SKIP_TWO_TILES)
 def test_attention_of_grouped_requests(shape, B, pre, L, post, rows, ratio):
     lay = wl.make_layout(B, pre, L, post, rows, rows, "all")
     case = wl.make_case(shape, lay, ratio, cfg_id=78, weights=cached_weights(shape, 78), hot_frac=0.01)
@@ -254,6 +271,34 @@ def test_which_decode_passes_share_query_tiles():
     for (B, rows, grouped), kernels in zip(cases, launched):
         assert ("attention_group_kernel" in kernels) == bool(grouped), (B, rows, kernels)
         assert ("attention_tc_kernel<false>" in kernels) != bool(grouped), (B, rows, kernels)
+
+
+# One-pass scoring with three CTAs per SM: one CTA per (request, head) and clusters of two, four and eight; 2 to 4 key tiles per CTA, the
+# last one ragged; 1 to 32 masked rows; both normalisers; one cache for the batch.
+THREE_CTAS = [(HEADS32, 10, 300, 32, False, False), (HEADS32, 12, 385, 29, False, True), (HEADS32, 5, 700, 29, True, False),
+              (HEADS32, 3, 1500, 1, False, False), (MID128, 10, 3990, 30, False, True), (MID128, 10, 3990, 17, True, False)]
+
+
+def test_scoring_with_three_ctas_per_sm():
+    launched = launched_kernels([(s, B, L, m, shared, norm_full) for s, B, L, m, shared, norm_full in THREE_CTAS], "scoring")
+    for case, kernels in zip(THREE_CTAS, launched):
+        assert "score_onepass_tc_kernel<32, 2, 3>" in kernels, (case, kernels)
+    for shape, B, L, m, shared, norm_full in THREE_CTAS:
+        lay = wl.make_layout(B, 7, L, 20, max(m, 8), m)
+        ck, q = wl.random_kv_cache(shape, lay, 83)[0], wl.random_q_mask(shape, lay, 84)
+        dk, dq = ab.to_device_bf16(ck, DEV), ab.to_device_bf16(q, DEV)
+        masked = torch.from_numpy(lay.masked_pos.copy()).to(DEV)
+        ctx = ab.Context.for_shape(shape, B, lay.ctx_len, L, 1, m, DEV)
+        req = ab.Context.request(B, lay.ctx_len, 7, L, masked, None, None, None)
+        scores = torch.zeros((B, L), dtype=torch.float32, device=DEV)
+        kv = ab.KV(dk.data_ptr(), dk.data_ptr(), 0, lay.ctx_len) if shared else ab.Context.kv(dk, dk)
+        ctx.score_anchors(req, dq, kv, scores, accumulate=False, norm_full=norm_full)
+        assert ctx.poll_status() == 0
+        for b in (0, B // 2, B - 1):
+            keys = orc.bf16_bits_to_f64(ck[0 if shared else b, :lay.ctx_len])
+            ref = orc.score_anchors(orc.bf16_bits_to_f64(q[b]), keys[7:7 + L], keys, 7, norm_full)
+            got = scores[b].cpu().numpy().astype(np.float64)
+            assert (np.abs(got - ref) / np.maximum(ref, ref.mean())).max() < 1e-3, (shape.name, B, L, m)
 
 
 # Small projections sum K in the general kernel's order, block by block: a row's bits do not depend on how many rows are in the
