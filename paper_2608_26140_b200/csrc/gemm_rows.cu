@@ -551,7 +551,7 @@ gemm_rows_kernel(const __grid_constant__ GemmArgs g, const __grid_constant__ Row
 }
 template <int S, int EPI, bool APART>
 __global__ void __launch_bounds__(RW_THREADS, 1)
-gemm_own_rows_kernel(const __grid_constant__ GemmArgs g, const __grid_constant__ RowsPlan p, const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB0,
+own_gemm_rows_kernel(const __grid_constant__ GemmArgs g, const __grid_constant__ RowsPlan p, const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB0,
                  const __grid_constant__ CUtensorMap mapB1, const __grid_constant__ CUtensorMap mapB2) {
     rows_body<S, EPI, APART, true>(g, p, mapA, mapB0, mapB1, mapB2);
 }
@@ -563,7 +563,7 @@ constexpr int kSmemBytes = 226 * 1024;
 template <int S, int EPI, bool APART, bool OWN = false>
 cudaError_t launch_rows(const GemmArgs& g, const RowsPlan& p, const CUtensorMap& a, const CUtensorMap* b, cudaStream_t stream) {
     const auto kernel = [] {
-        if constexpr (OWN) return gemm_own_rows_kernel<S, EPI, APART>;
+        if constexpr (OWN) return own_gemm_rows_kernel<S, EPI, APART>;
         else return gemm_rows_kernel<S, EPI, APART>;
     }();
     static const cudaError_t attr = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);

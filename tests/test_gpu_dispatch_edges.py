@@ -183,7 +183,7 @@ def test_attention_reference_moves(T, rows, drop):
 
 
 # many more (query tile, head, request) items than SMs: several per CTA, the last round incomplete; query tiles with empty
-# quarters; and four requests to a tile over a shared cache, an item per CTA, with a last group of two
+# quarters; and over a shared cache four requests to a tile, an item per CTA, with a last group of two
 HEADS32 = wl.LayerShape(256, 32, 4, 128, 256, 1e-5, False, 5e5, "heads32")
 
 
@@ -210,30 +210,13 @@ def test_attention_items_per_cta(B, T, rows, shared):
         assert_close_bf16(ab.to_host_bits(y[b]), ref["y"], "y")
 
 
-# Decode passes over a shared cache: groups of four in clusters of 4, 2, 8 and 8 CTAs (some without a step of their own), a pair on
-# one CTA, and one request to a tile in clusters of 8 and 4.  An affix that neither starts nor ends with a tile; one and several
-# private tiles; groups that are not full.
-GROUPED = [(HEADS32, 4, 0, 300, 40, 32, 0.3), (HEADS32, 6, 150, 500, 180, 7, 0.5), (MID128, 3, 300, 200, 300, 20, 0.1),
-           (MID128, 2, 0, 2500, 64, 1, 0.05), (HEADS32, 5, 5, 260, 90, 64, 0.2)]
-APART = [(MID128, 2, 9, 700, 60, 33, 0.2), (MID128, 7, 130, 1100, 100, 50, 0.35)]
-# One CTA per query tile, which leaves out the shared tiles without a key: two in front of the affix, one or more behind it, several
-# private rounds.  Groups of four, two and three of them part-filled; pairs; one request to a tile; two tiles of one request.
-SKIP_GROUPED = [(HEADS32, 12, 300, 300, 150, 20, 0.2), (HEADS32, 9, 290, 200, 140, 31, 0.5), (HEADS32, 6, 300, 260, 290, 50, 0.2),
-                (HEADS32, 5, 270, 270, 150, 33, 0.2)]
-SKIP_ONE_TILE = [(HEADS32, 3, 300, 260, 150, 70, 0.2)]
-SKIP_TWO_TILES = [(HEADS32, 5, 300, 260, 150, 140, 0.2)]
-
-
-# The next test compares results; this one says that the kernel they mean is the one that runs.
-def test_which_kernel_decodes_over_a_shared_cache():
-    for cases, kernel in ((GROUPED + SKIP_GROUPED, "attention_group_kernel"), (APART + SKIP_ONE_TILE, "attention_tc_kernel<false>"),
-                          (SKIP_TWO_TILES, "attention_tc2q_kernel")):
-        asked = [(shape, B, pre, L, post, rows, orc.k_from_ratio(L, ratio)) for shape, B, pre, L, post, rows, ratio in cases]
-        for case, kernels in zip(cases, launched_kernels(asked, "shared_decode")):
-            assert [k for k in kernels.split() if "attention" in k and kernel not in k] == [] and kernel in kernels, (case, kernels)
-
-
-@pytest.mark.parametrize("shape,B,pre,L,post,rows,ratio", GROUPED + APART + SKIP_GROUPED + SKIP_ONE_TILE + SKIP_TWO_TILES)
+# Decode passes over a shared cache, private rows in rounds behind the shared tiles: groups of four in clusters of 4, 2, 8 and 8 CTAs
+# (some without a step of their own), a pair on one CTA (the third case), and one request to a tile in clusters of 8 and 4 (the fourth
+# and the last).  Groups that are not full; an affix that neither starts nor ends with a tile.
+@pytest.mark.parametrize("shape,B,pre,L,post,rows,ratio", [
+    (HEADS32, 4, 0, 300, 40, 32, 0.3), (HEADS32, 6, 150, 500, 180, 7, 0.5), (HEADS32, 5, 5, 260, 90, 64, 0.2),
+    (MID128, 2, 9, 700, 60, 33, 0.2), (MID128, 3, 300, 200, 300, 20, 0.1), (MID128, 2, 0, 2500, 64, 1, 0.05),
+    (MID128, 7, 130, 1100, 100, 50, 0.35)])
 def test_attention_of_grouped_requests(shape, B, pre, L, post, rows, ratio):
     lay = wl.make_layout(B, pre, L, post, rows, rows, "all")
     case = wl.make_case(shape, lay, ratio, cfg_id=78, weights=cached_weights(shape, 78), hot_frac=0.01)
@@ -260,6 +243,22 @@ def test_attention_of_grouped_requests(shape, B, pre, L, post, rows, ratio):
         ref = orc.layer_step(case.weights, shape, case.x[b], ck, cv, T, pre, L, lay.masked_pos[b], lay.masked_pos[b], case.rope_cos,
                              case.rope_sin, anchor_idx=np.zeros(0, np.int32))
         assert_close_bf16(ab.to_host_bits(y[b]), ref["y"], "y")
+
+
+# One CTA per query tile, which leaves out the shared tiles without a key: two in front of the affix, one or more behind it, several
+# private rounds.  Groups of four, two and three of them part-filled; pairs; one request to a tile; two tiles of one request.
+UNSPLIT = {"attention_group_kernel": [(HEADS32, 12, 300, 300, 150, 20, 0.2), (HEADS32, 9, 290, 200, 140, 31, 0.5),
+                                      (HEADS32, 6, 300, 260, 290, 50, 0.2), (HEADS32, 5, 270, 270, 150, 33, 0.2)],
+           "attention_tc_kernel<false>": [(HEADS32, 3, 300, 260, 150, 70, 0.2)],
+           "attention_tc2q_kernel": [(HEADS32, 5, 300, 260, 150, 140, 0.2)]}
+
+
+@pytest.mark.parametrize("kernel", UNSPLIT)
+def test_attention_without_the_empty_tiles_of_a_shared_cache(kernel):
+    asked = [(shape, B, pre, L, post, rows, orc.k_from_ratio(L, ratio)) for shape, B, pre, L, post, rows, ratio in UNSPLIT[kernel]]
+    for case, kernels in zip(UNSPLIT[kernel], launched_kernels(asked, "shared_decode")):
+        assert kernel in kernels and kernels.count("attention") == kernels.count(kernel), (case, kernels)
+        test_attention_of_grouped_requests(*case)
 
 
 # Two requests of 33 to 64 rows share a tile where that saves rounds of CTAs (on 148 SMs): 2 | 1, 3 | 2, 5 | 3 rounds, but not 1 | 1

@@ -24,10 +24,9 @@ LONG128 = wl.LayerShape(2560, 6, 3, 128, 256, 1e-6, True, 1e6, "long-d128")
 
 
 @pytest.mark.parametrize("shape,B,L,extra,kernel", [
-    (wl.TINY, 1, 400, "none", "gemm_rows_kernel<1, 0, true>"),       # 80 rows: one CTA per tile, ring stages filled with weights
-    (wl.TINY, 1, 300, "none", "gemm_own_rows_kernel<1, 0, true>"),   # before the barrier; 60 rows: no barrier, but for the step that
-    (MID128, 1, 300, "none", "gemm_rows_kernel<2, 0, true>"),        # is to run out, which takes the kernel that has one
-    (LONG128, 1, 160, "none", "gemm_rows_kernel<2, 0, false>"),      # two and four CTAs per tile
+    (wl.TINY, 1, 300, "none", "gemm_rows_kernel<1, 0, true>"),       # 60 rows: one CTA per tile, ring stages filled with weights
+    (MID128, 1, 300, "none", "gemm_rows_kernel<2, 0, true>"),        # before the barrier; two and four CTAs per tile
+    (LONG128, 1, 160, "none", "gemm_rows_kernel<2, 0, false>"),
     (DEEP128, 1, 300, "none", "gemm_rows_kernel<4, 0, false>"),
     (MID128, 2, 400, "all", "gemm_tc2_kernel"),                      # several 128-row tiles: the two-SM projection kernel
     (WIDE_Q128, 2, 400, "all", "gemm_wm_kernel<0>"),                 # the same, more columns: weights as the product's M
@@ -50,7 +49,7 @@ def test_a_wait_that_runs_out_is_reported_and_the_context_stays_usable(shape, B,
     with torch.profiler.profile(activities=[torch.profiler.ProfilerActivity.CUDA]) as prof:
         clean = step()
     names = [e.key for e in prof.key_averages()]
-    assert any(kernel in name for name in names), names              # the q/k/v projection is this kernel
+    assert any(kernel in name for name in names), names              # the projection whose barrier runs out is this kernel
     assert dc.ctx.poll_status_code() == (ab.OK, 0)
     dc.reset_cache()
     dc.ctx.debug_expire_next_wait()
@@ -63,3 +62,10 @@ def test_a_wait_that_runs_out_is_reported_and_the_context_stays_usable(shape, B,
     assert dc.ctx.poll_status_code() == (ab.OK, 0)
     for a, b in zip(clean, again):
         assert np.array_equal(a, b)
+
+
+# Up to 64 rows of up to 256 columns the clean steps take a kernel without a grid-wide barrier; the step that is to run out takes the one
+# that has it, as the clean steps of more rows do.
+@pytest.mark.parametrize("L,kernel", [(300, "acache::own_gemm_rows_kernel<1, 0, true>"), (400, "acache::gemm_rows_kernel<1, 0, true>")])
+def test_a_wait_that_runs_out_with_and_without_the_barrier_in_clean_steps(L, kernel):
+    test_a_wait_that_runs_out_is_reported_and_the_context_stays_usable(wl.TINY, 1, L, "none", kernel)
