@@ -185,7 +185,11 @@ __device__ __forceinline__ void sum_apart16(const RowsPlan& p, int rank, uint32_
 
 // The shared preparation of the usual case (a CTA per row, a row of up to three 16-byte pieces a thread) and, out of the way of its
 // instructions, the rest: a launch runs most of its instructions once, from L2, and waits for them.  With all of it inline the
-// kernels had 228-252 registers, now 52-212 (layer-step of 103 rows 142.6 -> 139.1 us, decode pass of 32 rows over 4 layers 638 -> 631).
+// kernels had 228-252 registers; those with one accumulator per tile now have 48-210, those with one per block keep it inline and
+// have 230-252 (layer-step of 103 rows 142.6 -> 139.1 us, decode pass of 32 rows over 4 layers 638 -> 631).  The call gets a copy of the
+// arguments, made on that way only: it takes their address, and a kernel whose parameter has one (as __grid_constant__) reads it more
+// slowly everywhere (decode pass of 78 rows of 256 columns over 2 layers 89.4 -> 88.2 us, layer-step of 58 such rows 46.6 -> 46.0, of
+// 103 rows of 4096 columns 134.8 -> 134.3; one that copies it at its start: the last 138.6).
 __device__ __forceinline__ void prep_phase_short(const GemmArgs& g, float* red, volatile int* abort_flag) {
     const RowPrep& rp = g.prep;
     for (int row = blockIdx.x; row < g.M; row += gridDim.x) {
@@ -342,7 +346,10 @@ __device__ __forceinline__ void rows_body(const GemmArgs& g, const RowsPlan& p, 
     else if (EPI != kEpiResidual && g.prep.enabled) {
         if constexpr (APART) prep_phase(g, red, abort_flag, p.cta_rows);     // (few tiles: mostly the long way, 3-5 % slower as a call)
         else if (g.M <= p.cta_rows && g.K <= 3 * RW_THREADS * 8) prep_phase_short(g, red, abort_flag);
-        else prep_phase_long(g, red, abort_flag, p.cta_rows);
+        else {
+            const GemmArgs args = g;
+            prep_phase_long(args, red, abort_flag, p.cta_rows);
+        }
     }
 
     // ---------------- the contraction ----------------
@@ -545,13 +552,13 @@ __device__ __forceinline__ void rows_body(const GemmArgs& g, const RowsPlan& p, 
 
 template <int S, int EPI, bool APART>
 __global__ void __launch_bounds__(RW_THREADS, 1)
-gemm_rows_kernel(const __grid_constant__ GemmArgs g, const __grid_constant__ RowsPlan p, const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB0,
+gemm_rows_kernel(const GemmArgs g, const RowsPlan p, const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB0,
                  const __grid_constant__ CUtensorMap mapB1, const __grid_constant__ CUtensorMap mapB2) {
     rows_body<S, EPI, APART, false>(g, p, mapA, mapB0, mapB1, mapB2);
 }
 template <int S, int EPI, bool APART>
 __global__ void __launch_bounds__(RW_THREADS, 1)
-own_gemm_rows_kernel(const __grid_constant__ GemmArgs g, const __grid_constant__ RowsPlan p, const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB0,
+own_gemm_rows_kernel(const GemmArgs g, const RowsPlan p, const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB0,
                  const __grid_constant__ CUtensorMap mapB1, const __grid_constant__ CUtensorMap mapB2) {
     rows_body<S, EPI, APART, true>(g, p, mapA, mapB0, mapB1, mapB2);
 }
