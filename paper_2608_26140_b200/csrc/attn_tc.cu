@@ -1,7 +1,8 @@
 // Bidirectional attention of many recomputed rows over the whole context (Section 4.3) on the
-// 5th-generation tensor cores.  Two kernels share the scheme below: attention_tc_kernel (one CTA = 128
-// query rows of one head; used when a request has at most 128 rows) and attention_tc2q_kernel (one CTA
-// = 256 query rows, described where it is defined).  Key/value tiles of 128 keys stream through shared
+// 5th-generation tensor cores.  Three kernels share the scheme below: attention_tc_kernel (one CTA = 128
+// query rows of one head; used when a request has at most 128 rows), attention_group_kernel (the same rows
+// from several requests) and attention_tc2q_kernel (one CTA = 256 query rows), the last two described
+// where they are defined.  Key/value tiles of 128 keys stream through shared
 // memory by TMA (3-d tensor maps: positions past the context end and rows past the request's row count
 // read as zero).
 //
@@ -412,7 +413,7 @@ attention_tc_kernel(const AttnTcArgs a, const __grid_constant__ CUtensorMap mapQ
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     // key split: a cluster of C CTAs shares a query tile, each taking a contiguous part of the key tiles
     const int C = a.split, rank = C > 1 ? (int)cluster_ctarank() : 0;
-    const int first = blockIdx.x / C, stride = gridDim.x;        // items: (query tile, head, request or group of four)
+    const int first = blockIdx.x / C, stride = gridDim.x;        // items: (query tile, head, request)
     const int n_cache_tiles = (a.ctx_len + 127) / 128;
     int2 visited = make_int2(0, n_cache_tiles);     // the cache's key tiles that hold keys
     // this CTA's key tiles: n_c of the cache from c0 on, then fresh ones from f0 on
@@ -643,10 +644,12 @@ attention_tc_kernel(const AttnTcArgs a, const __grid_constant__ CUtensorMap mapQ
 // or its two) is the product with its own key tile, written to its own lanes only (the instruction's disable-output-lane mask), and
 // its part of O += P V likewise.  A round's softmax so works on as many logits as a shared tile's; with a step per (request, tile)
 // three quarters of the softmax warps wrote zeros, and a step took as long as any.  16 requests of 32 rows, 32 heads, 2048 shared
-// keys and 922 private rows: 86 -> 70 us per layer (HBM floor 42), pass over 4 layers 1830 -> 1752.  A shared step is bound by the softmax chain (2700 cycles),
-// a round by HBM (7300 cycles for 256 KB, 7.5 TB/s over the chip).  Rounds and shared steps in turn, so that one's loads run under
-// the other's arithmetic, took 61 us, but another order of sums changes tokens that were near ties (2 of 512): not done.  Private
-// tiles requested into L2 while the shared steps run: 77-87 us.  K and V rings of three stages.
+// keys and 922 private rows, us a layer from the end of the launch before: 89 -> 75, with one barrier of a kind per shared step 72;
+// 280 MB come from DRAM (42 us at the copy rate), 68 us for the launch alone.  A shared step is bound by the softmax chain (2700 cycles).
+// What bounds a round (7300 cycles for 256 KB in one CTA's stamps: above the copy rate, part of it is there already) has not been separated:
+// the loads, or the chain K, S, P, P V of a round.  Rounds and shared steps in turn, so that one's loads run under the other's
+// arithmetic, were 9 us shorter, but another order of sums changes tokens that were near ties (2 of 512): not done.  Private
+// tiles requested into L2 while the shared steps run: 7 to 17 us longer.  K and V rings of three stages.  96 registers, 8 bytes spilled.
 constexpr int AG_STAGES = 3;
 constexpr int AG_SMEM = (1 + 2 * AG_STAGES) * AT_TILE + 2048 + 512;    // Q, K, V, row exchange, barriers; the window has to start 1024-aligned
 
